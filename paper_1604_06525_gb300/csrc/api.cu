@@ -883,7 +883,7 @@ static opt_status create_graph_impl(const opt_graph_desc* d, int D, opt_problem*
                                     const EmbedExtra* ed = nullptr) {
   // unknown planes, distinct-diagonal planes, geometry and vector records per vertex
   const int NXg = ed ? 12 : (D == 3 ? 6 : 3), NMg = ed ? 10 : (D == 3 ? 4 : 2);
-  const int NGR = ed ? 1 : (D == 3 ? 3 : 1), NVR = ed ? 3 : (D == 3 ? 2 : 1);
+  const int NGR = ed ? 1 : (D == 3 ? 3 : 1), NVR = ed || D == 3 ? 3 : 1;
   float* const* ux = ed ? ed->unknowns : d ? d->unknowns : nullptr;
   if (!out) return OPT_ERR_INVALID_ARG;
   *out = nullptr;
@@ -1072,6 +1072,7 @@ static opt_status create_graph_impl(const opt_graph_desc* d, int D, opt_problem*
 
   MeshProb& g = q->hm;
   g.V = V; g.E = E; g.Vp = Vp;
+  g.sym = orow == irow && e1 == isrc;
   g.vchunk_begin = 0; g.vchunk_end = q->nvchunks;
   g.echunk_begin = 0; g.echunk_end = q->nechunks;
   g.tchunk_begin = 0; g.tchunk_end = q->ntchunks;

@@ -13,20 +13,33 @@
 // order.  What a thread reads of a neighbour sits in two per-vertex records
 // (array of structures, a few 32-byte sectors per gather instead of one
 // sector per plane):
-//   grec[v] = (U_x, U_y, U_z, cos a_x), (sin a_x, cos a_y, sin a_y, cos a_z),
-//             (sin a_z, 0, 0, 0)          written by PCGInit's vertex pass
-//   vrec[v] = the vertex's 6-vector (x in PCGInit, p in applyJTJ), 2 float4
+//   grec[v] = (U_x, U_y, U_z, q_w), (q_x, q_y, q_z, 0): rest position and the
+//             rotation R(A_v) as a unit quaternion; behind the 2 V of them, own
+//             vertex only, (cos a_y, sin a_y, cos a_z, sin a_z)
+//                                                   written by PCGInit's vertex pass
+//   vrec[v] = x's displacement in PCGInit; (p_d, w) in applyJTJ, 2 float4;
+//             (x_d, U, delta_d) in the energies, 3 float4
 //
 // ARAP mesh algebra per edge e = (a, b), v = U_a - U_b, d = O - U:
 //   r_e       = s_w [(d_a - d_b) + (v - R(A_a) v)]              (= Fig. 25)
-//   dr/dd_a   = s_w I,  dr/dd_b = -s_w I,
-//   dr/dA_a,m = g_m = -s_w (dR/dA_m)(A_a) v,  R = Rz(az) Ry(ay) Rx(ax).
+//   dr/dd_a   = s_w I,  dr/dd_b = -s_w I.
+// R = Rz(az) Ry(ay) Rx(ax), so dR/dA_m = [beta_m]x R with the unit axes
+//   beta_z = e_z, beta_y = Rz e_y, beta_x = Rz Ry e_x, and with y = R(A_a) v
+//   dr/dA_a,m = -s_w beta_m x y.
+// A direction's angles therefore enter a residual only through the angular
+// velocity w_a = sum_m p_a,m beta_m, formed once per vertex:
+//   J_e p = s_w [(p_a,d - p_b,d) - w_a x y],
+// and the angle rows of J^T t are -s_w beta_m . sum_e y x t_e: one torque per
+// vertex.  (Three derivative vectors per edge end, as the rows are printed,
+// cost three times the arithmetic: 128^3 volume, gather 110 -> 90 us, energies
+// 186 -> 120 us, LM 3 x 10 solve 7.88 -> 7.37 ms; the gather is now bound by the
+// records it moves through L1 / L2, 64 B per neighbour.)
 //
-// Per outer iteration (PCGInit): k_mesh_init_v (cos / sin of the angles, the
-// records), k_mesh_init_pull (J^T F, diag, M^-1, r, delta, float64 r.z and E).
-// Per PCG iteration: k_mesh_apply_v (p = z + beta p into the planes and the
-// records), k_mesh_apply_pull (J^T J p + fit + damping, float64 p.q -> alpha),
-// k_mesh_update (vector update -> beta).
+// Per outer iteration (PCGInit): k_mesh_init_v (quaternions, axes, records),
+// k_mesh_init_pull (J^T F, diag, M^-1, r, delta, float64 r.z and E).
+// Per PCG iteration: k_mesh_apply_v (p = z + beta p into the planes, p_d and w
+// into the records), k_mesh_apply_pull (J^T J p + fit + damping, float64 p.q ->
+// alpha), k_mesh_update (vector update -> beta).
 #include "opt_internal.cuh"
 #include "opt_launch.h"
 
@@ -71,33 +84,138 @@ __device__ __forceinline__ Stencil3 stencil3(const MeshProb& pr, int i) {
   return st;
 }
 
-// A vertex's geometry record and 6-vector record.
+// --- rotations -------------------------------------------------------------
 struct GeoRec {
   float U[3];
-  float cs[6];      // cos ax, sin ax, cos ay, sin ay, cos az, sin az
+  float q[4];       // unit quaternion (w, x, y, z) of R(A)
 };
 __device__ __forceinline__ GeoRec load_geo(const float4* __restrict__ grec, int v) {
-  const float4 a = __ldg(grec + 3 * v), b = __ldg(grec + 3 * v + 1), c = __ldg(grec + 3 * v + 2);
+  const float4 a = __ldg(grec + 2 * (size_t)v), b = __ldg(grec + 2 * (size_t)v + 1);
   GeoRec g;
   g.U[0] = a.x; g.U[1] = a.y; g.U[2] = a.z;
-  g.cs[0] = a.w; g.cs[1] = b.x; g.cs[2] = b.y; g.cs[3] = b.z; g.cs[4] = b.w; g.cs[5] = c.x;
+  g.q[0] = a.w; g.q[1] = b.x; g.q[2] = b.y; g.q[3] = b.z;
   return g;
 }
-// 6-vector record written in the same launch chain (plain loads, not the
-// read-only path)
-__device__ __forceinline__ void load_vec(const float4* vrec, int v, float (&o)[6]) {
-  const float4 a = vrec[2 * v], b = vrec[2 * v + 1];
-  o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y;
+// (cos a_y, sin a_y, cos a_z, sin a_z) of a vertex: what its axes beta_m need
+__device__ __forceinline__ float4 load_axes(const MeshProb& pr, int v) {
+  return __ldg(pr.grec + 2 * (size_t)pr.V + v);
 }
+// Quaternion and axes of Rz(az) Ry(ay) Rx(ax), from the half angles.
+__device__ __forceinline__ void angles_to_quat(const float* a, float (&q)[4], float4& axes) {
+  float sx, cx, sy, cy, sz, cz;
+  sincosf(0.5f * a[0], &sx, &cx);
+  sincosf(0.5f * a[1], &sy, &cy);
+  sincosf(0.5f * a[2], &sz, &cz);
+  const float cc = cy * cz, ss = sy * sz, sc = sy * cz, cs = cy * sz;
+  q[0] = fmaf(cx, cc, sx * ss);
+  q[1] = fmaf(sx, cc, -cx * ss);
+  q[2] = fmaf(cx, sc, sx * cs);
+  q[3] = fmaf(cx, cs, -sx * sc);
+  axes = make_float4(fmaf(-2.f * sy, sy, 1.f), 2.f * sy * cy, fmaf(-2.f * sz, sz, 1.f), 2.f * sz * cz);
+}
+// D = R - I (no cancellation for small angles)
+__device__ __forceinline__ void quat_delta_matrix(const float (&q)[4], float (&D)[3][3]) {
+  const float w = q[0], x2 = 2.f * q[1], y2 = 2.f * q[2], z2 = 2.f * q[3];
+  const float xx = x2 * q[1], yy = y2 * q[2], zz = z2 * q[3];
+  D[0][0] = -(yy + zz);                 D[0][1] = fmaf(x2, q[2], -z2 * w);  D[0][2] = fmaf(x2, q[3], y2 * w);
+  D[1][0] = fmaf(x2, q[2], z2 * w);     D[1][1] = -(xx + zz);               D[1][2] = fmaf(y2, q[3], -x2 * w);
+  D[2][0] = fmaf(x2, q[3], -y2 * w);    D[2][1] = fmaf(y2, q[3], x2 * w);   D[2][2] = -(xx + yy);
+}
+__device__ __forceinline__ void mat_vec(const float (&D)[3][3], const float (&v)[3], float (&o)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) o[i] = fmaf(D[i][0], v[0], fmaf(D[i][1], v[1], D[i][2] * v[2]));
+}
+// (R - I) v of a quaternion used once: t = 2 u x v, then w t + u x t
+__device__ __forceinline__ void quat_delta(const float (&q)[4], const float (&v)[3], float (&o)[3]) {
+  const float x2 = 2.f * q[1], y2 = 2.f * q[2], z2 = 2.f * q[3];
+  const float t0 = fmaf(y2, v[2], -z2 * v[1]), t1 = fmaf(z2, v[0], -x2 * v[2]), t2 = fmaf(x2, v[1], -y2 * v[0]);
+  o[0] = fmaf(q[0], t0, fmaf(q[2], t2, -q[3] * t1));
+  o[1] = fmaf(q[0], t1, fmaf(q[3], t0, -q[1] * t2));
+  o[2] = fmaf(q[0], t2, fmaf(q[1], t1, -q[2] * t0));
+}
+// o -= a x b
+__device__ __forceinline__ void sub_cross(float (&o)[3], const float (&a)[3], const float (&b)[3]) {
+  o[0] = fmaf(-a[1], b[2], fmaf(a[2], b[1], o[0]));
+  o[1] = fmaf(-a[2], b[0], fmaf(a[0], b[2], o[1]));
+  o[2] = fmaf(-a[0], b[1], fmaf(a[1], b[0], o[2]));
+}
+// o += a x b
+__device__ __forceinline__ void add_cross(float (&o)[3], const float (&a)[3], const float (&b)[3]) {
+  o[0] = fmaf(a[1], b[2], fmaf(-a[2], b[1], o[0]));
+  o[1] = fmaf(a[2], b[0], fmaf(-a[0], b[2], o[1]));
+  o[2] = fmaf(a[0], b[1], fmaf(-a[1], b[0], o[2]));
+}
+// w = sum_m p_m beta_m
+__device__ __forceinline__ void angular_velocity(const float4& ax, float pa, float pb, float pc, float (&w)[3]) {
+  const float h = pa * ax.x;
+  w[0] = fmaf(ax.z, h, -ax.w * pb);
+  w[1] = fmaf(ax.w, h, ax.z * pb);
+  w[2] = fmaf(-ax.y, pa, pc);
+}
+// (beta_x . t, beta_y . t, beta_z . t)
+__device__ __forceinline__ void axis_rows(const float4& ax, const float (&t)[3], float (&o)[3]) {
+  const float t1 = fmaf(ax.z, t[0], ax.w * t[1]);
+  o[0] = fmaf(ax.x, t1, -ax.y * t[2]);
+  o[1] = fmaf(ax.z, t[1], -ax.w * t[0]);
+  o[2] = t[2];
+}
+// o_m += |beta_m x y|^2
+__device__ __forceinline__ void axis_squares(const float4& ax, const float (&y)[3], float (&o)[3]) {
+  const float y1 = fmaf(ax.z, y[0], ax.w * y[1]), y2 = fmaf(ax.z, y[1], -ax.w * y[0]);
+  const float t = fmaf(ax.y, y1, ax.x * y[2]);
+  o[0] = fmaf(t, t, fmaf(y2, y2, o[0]));
+  o[1] = fmaf(y1, y1, fmaf(y[2], y[2], o[1]));
+  o[2] = fmaf(y1, y1, fmaf(y2, y2, o[2]));
+}
+
+// Records written in the same launch chain (plain loads, not the read-only
+// path): a displacement, or (p_d, w).
 __device__ __forceinline__ void load_vec3(const float4* vrec, int v, float (&o)[3]) {
-  const float4 a = vrec[2 * v];
+  const float4 a = vrec[2 * (size_t)v];
   o[0] = a.x; o[1] = a.y; o[2] = a.z;
+}
+__device__ __forceinline__ void load_pw(const float4* vrec, int v, float (&p)[3], float (&w)[3]) {
+  const float4 a = vrec[2 * (size_t)v], b = vrec[2 * (size_t)v + 1];
+  p[0] = a.x; p[1] = a.y; p[2] = a.z;
+  w[0] = a.w; w[1] = b.x; w[2] = b.y;
+}
+
+// Runs edge(j, own, in) for the neighbours j of vertex i: own for the far end of
+// every out-edge, in for the source of every in-edge.  Where both lists are
+// equal (every undirected edge given both ways: pr.sym, and the voxel stencil)
+// each neighbour is visited once with both; the first KB neighbour indices are
+// loaded together.
+template <bool G3, typename Edge>
+__device__ __forceinline__ void for_neighbours(const MeshProb& pr, int i, Edge edge) {
+  if (G3) {
+    const Stencil3 st = stencil3(pr, i);
+#pragma unroll
+    for (int t = 0; t < 6; ++t)
+      if (st.ok[t]) edge(i + st.off[t], true, true);
+    return;
+  }
+  const int o0 = pr.orow[i], o1 = pr.orow[i + 1];
+  const bool sym = pr.sym != 0;
+  int jo[KB];
+#pragma unroll
+  for (int t = 0; t < KB; ++t) jo[t] = o0 + t < o1 ? pr.e1[o0 + t] : 0;
+#pragma unroll
+  for (int t = 0; t < KB; ++t)
+    if (o0 + t < o1) edge(jo[t], true, sym);
+  // longer rows; then, one-way edges, the in-edge list
+  const int lists = sym ? 1 : 2;
+  for (int l = 0; l < lists; ++l) {
+    const int k1 = l ? pr.irow[i + 1] : o1;
+    const int* __restrict__ src = l ? pr.isrc : pr.e1;
+#pragma unroll 1
+    for (int k = l ? pr.irow[i] : o0 + KB; k < k1; ++k) edge(src[k], l == 0, sym || l == 1);
+  }
 }
 
 // ---------------------------------------------------------------------------
 // PCGInit
 // ---------------------------------------------------------------------------
-// Vertex pass: cos / sin of the angles and both records of every vertex.
+// Vertex pass: the quaternion and axes of every vertex and both records.
 __global__ void __launch_bounds__(NT) k_mesh_init_v(const MeshProb* __restrict__ probs,
                                                     const Chunk* __restrict__ chunks) {
   pdl_begin();
@@ -106,25 +224,25 @@ __global__ void __launch_bounds__(NT) k_mesh_init_v(const MeshProb* __restrict__
   if (pr.s->done) return;
   const long long pl = pr.Vp;
   for (int v = ch.begin + threadIdx.x; v < ch.end; v += NT) {
-    float x[6], U[3], cs[6];
+    float x[6], U[3], q[4];
 #pragma unroll
     for (int c = 0; c < 6; ++c) x[c] = pr.x[c * pl + v];
 #pragma unroll
     for (int c = 0; c < 3; ++c) U[c] = __ldg(pr.U + c * pl + v);
-#pragma unroll
-    for (int m = 0; m < 3; ++m) sincosf(x[3 + m], &cs[2 * m + 1], &cs[2 * m]);
-    pr.grec[3 * v] = make_float4(U[0], U[1], U[2], cs[0]);
-    pr.grec[3 * v + 1] = make_float4(cs[1], cs[2], cs[3], cs[4]);
-    pr.grec[3 * v + 2] = make_float4(cs[5], 0.f, 0.f, 0.f);
-    pr.vrec[2 * v] = make_float4(x[0], x[1], x[2], x[3]);
-    pr.vrec[2 * v + 1] = make_float4(x[4], x[5], 0.f, 0.f);
+    float4 axes;
+    angles_to_quat(x + 3, q, axes);
+    pr.grec[2 * (size_t)v] = make_float4(U[0], U[1], U[2], q[0]);
+    pr.grec[2 * (size_t)v + 1] = make_float4(q[1], q[2], q[3], 0.f);
+    pr.grec[2 * (size_t)pr.V + v] = axes;
+    pr.vrec[2 * (size_t)v] = make_float4(x[0], x[1], x[2], 0.f);
   }
 }
 
 // Gather pass: per vertex i the rows of J^T F (fit, own edge residuals with
 // their angle rows, incoming edge residuals), diag(J^T J) (displacement:
-// planned w_reg * degree + w_fit; angles: sum |g_m|^2 over the out-edges),
-// the energy of the own residuals, then b = -J^T F, M^-1, r = b, delta = 0.
+// planned w_reg * degree + w_fit; angles: w_reg sum |beta_m x y|^2 over the
+// out-edges), the energy of the own residuals, then b = -J^T F, M^-1, r = b,
+// delta = 0.
 // resident blocks per SM the gather PCGInit is compiled for (85 registers;
 // measured against 2 and 4: level-9 PCGInit 330 -> 316 us, level 7 39.8 -> 36.1 us)
 #ifndef MESH_INIT_MIN_BLOCKS
@@ -141,65 +259,72 @@ __global__ void __launch_bounds__(NT, MESH_INIT_MIN_BLOCKS) k_mesh_init_pull(con
   Scalars* s = pr.s;
   if (s->done) return;
   const long long pl = pr.Vp;
-  const float sw = pr.s_w;
   const float lam = pr.lm ? s->lambda_f : 0.0f;
   F2 acc_rz = f2_zero(), acc_E = f2_zero();
   for (int i = ch.begin + threadIdx.x; i < ch.end; i += NT) {
-    float xi[6];
-    load_vec(pr.vrec, i, xi);
+    float xi[3];
+    load_vec3(pr.vrec, i, xi);
     const GeoRec gi = load_geo(pr.grec, i);
-    float g[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // J^T F
-    float da[3] = {0.f, 0.f, 0.f};                 // angle diagonal
-    float e = 0.f;
+    const float4 axes = load_axes(pr, i);
+    float D[3][3];
+    quat_delta_matrix(gi.q, D);
+    float g[6];                                    // J^T F
+    float f[3] = {0.f, 0.f, 0.f};                  // sum of the residuals / s_w, in-edges negative
+    float tq[3] = {0.f, 0.f, 0.f};                 // torque
+    float da[3] = {0.f, 0.f, 0.f};                 // angle diagonal / w_reg
+    float es = 0.f, e = 0.f;
+    auto own_edge = [&](const float (&d)[3], const float (&v)[3]) {
+      float dv[3], r[3], y[3];
+      mat_vec(D, v, dv);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        r[c] = d[c] - dv[c];
+        y[c] = v[c] + dv[c];
+        f[c] += r[c];
+        es = fmaf(r[c], r[c], es);
+      }
+      add_cross(tq, y, r);
+      axis_squares(axes, y, da);
+    };
+    // residual of (j, i) / s_w: -(d + (R_j - I) (U_j - U_i)) with d = x_i - x_j
+    auto in_edge = [&](const GeoRec& gj, const float (&d)[3], const float (&v)[3]) {
+      float dv[3];
+      quat_delta(gj.q, v, dv);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) f[c] += d[c] - dv[c];
+    };
+    for_neighbours<G3>(pr, i, [&](int j, bool own, bool in) {
+      const GeoRec gj = load_geo(pr.grec, j);
+      float xj[3], d[3], v[3];
+      load_vec3(pr.vrec, j, xj);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        d[c] = xi[c] - xj[c];
+        v[c] = gi.U[c] - gj.U[c];
+      }
+      if (own) own_edge(d, v);
+      if (in) in_edge(gj, d, v);
+    });
+    {
+      float ga[3];
+      axis_rows(axes, tq, ga);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        g[c] = pr.w_reg * f[c];
+        g[3 + c] = -pr.w_reg * ga[c];
+        da[c] *= pr.w_reg;
+      }
+    }
     const int h = handle_of(pr, i);
     if (h >= 0) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const float f = pr.s_f * (xi[c] - pr.htgt[3 * h + c]);
-        g[c] += pr.s_f * f;
-        e += f * f;
+        const float fh = pr.s_f * (xi[c] - pr.htgt[3 * h + c]);
+        g[c] = fmaf(pr.s_f, fh, g[c]);
+        e = fmaf(fh, fh, e);
       }
     }
-    auto own_edge = [&](int j) {
-      float xj[3];
-      load_vec3(pr.vrec, j, xj);
-      const float4 uj = __ldg(pr.grec + 3 * j);
-      const float vx = gi.U[0] - uj.x, vy = gi.U[1] - uj.y, vz = gi.U[2] - uj.z;
-      const RotV R = rot_apply_cs(gi.cs[0], gi.cs[1], gi.cs[2], gi.cs[3], gi.cs[4], gi.cs[5], vx, vy, vz);
-      const float r0 = sw * ((xi[0] - xj[0]) + (vx - R.rv[0]));
-      const float r1 = sw * ((xi[1] - xj[1]) + (vy - R.rv[1]));
-      const float r2 = sw * ((xi[2] - xj[2]) + (vz - R.rv[2]));
-      g[0] += sw * r0; g[1] += sw * r1; g[2] += sw * r2;
-#pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        const float g0 = -sw * R.g[m][0], g1 = -sw * R.g[m][1], g2 = -sw * R.g[m][2];
-        g[3 + m] += g0 * r0 + g1 * r1 + g2 * r2;
-        da[m] += g0 * g0 + g1 * g1 + g2 * g2;
-      }
-      e += r0 * r0 + r1 * r1 + r2 * r2;
-    };
-    auto in_edge = [&](int j) {
-      float xj[3];
-      load_vec3(pr.vrec, j, xj);
-      const GeoRec gj = load_geo(pr.grec, j);
-      const float vx = gj.U[0] - gi.U[0], vy = gj.U[1] - gi.U[1], vz = gj.U[2] - gi.U[2];
-      const RotV R = rot_apply_cs(gj.cs[0], gj.cs[1], gj.cs[2], gj.cs[3], gj.cs[4], gj.cs[5], vx, vy, vz);
-      g[0] -= sw * (sw * ((xj[0] - xi[0]) + (vx - R.rv[0])));
-      g[1] -= sw * (sw * ((xj[1] - xi[1]) + (vy - R.rv[1])));
-      g[2] -= sw * (sw * ((xj[2] - xi[2]) + (vz - R.rv[2])));
-    };
-    if (G3) {
-      const Stencil3 st = stencil3(pr, i);
-#pragma unroll
-      for (int t = 0; t < 6; ++t)
-        if (st.ok[t]) own_edge(i + st.off[t]);
-#pragma unroll
-      for (int t = 0; t < 6; ++t)
-        if (st.ok[t]) in_edge(i + st.off[t]);
-    } else {
-      for (int k = pr.orow[i]; k < pr.orow[i + 1]; ++k) own_edge(pr.e1[k]);
-      for (int k = pr.irow[i]; k < pr.irow[i + 1]; ++k) in_edge(pr.isrc[k]);
-    }
+    e = fmaf(pr.w_reg, es, e);
     const float dg[4] = {pr.degw[i], da[0], da[1], da[2]};
     float mv[4];
 #pragma unroll
@@ -289,108 +414,87 @@ __global__ void __launch_bounds__(NT) k_mesh_apply_v(const MeshProb* __restrict_
     for (int k = 0; k < 4; ++k) {
       const int v = v0 + k;
       if (v < pr.V) {
-        pr.vrec[2 * v] = make_float4(c4(pv[0], k), c4(pv[1], k), c4(pv[2], k), c4(pv[3], k));
-        pr.vrec[2 * v + 1] = make_float4(c4(pv[4], k), c4(pv[5], k), 0.f, 0.f);
+        float w[3];
+        angular_velocity(load_axes(pr, v), c4(pv[3], k), c4(pv[4], k), c4(pv[5], k), w);
+        pr.vrec[2 * (size_t)v] = make_float4(c4(pv[0], k), c4(pv[1], k), c4(pv[2], k), w[0]);
+        pr.vrec[2 * (size_t)v + 1] = make_float4(w[1], w[2], 0.f, 0.f);
       }
     }
   }
 }
 
 // Gather pass: q_i = (fit + damping) p_i + sum over out-edges (i, j) of the
-// own rows s_w J_e p (displacement) and g_m . J_e p (angles) + sum over
-// in-edges (j, i) of -s_w J_e p (displacement), with
-//   J_e p = s_w (p_a,d - p_b,d) + sum_m g_m p_a,m   for e = (a, b);
-// float64 p.q -> alpha.  The neighbour indices of the first KB out- and
-// in-edges are loaded together before any record is needed; the kernel is
-// bound by these dependent load chains, so it is compiled for
-// MESH_PULL_MIN_BLOCKS resident blocks per SM (measured best at 4).
+// own rows s_w J_e p (displacement) and the torque rows (angles) + sum over
+// in-edges (j, i) of -s_w J_e p (displacement); float64 p.q -> alpha.  The
+// kernel is bound by its dependent index -> record loads, so it is compiled for
+// MESH_PULL_MIN_BLOCKS resident blocks per SM.
 template <bool G3>
 __global__ void __launch_bounds__(NT, MESH_PULL_MIN_BLOCKS) k_mesh_apply_pull(const MeshProb* __restrict__ probs,
                                                                              const Chunk* __restrict__ chunks,
-                                                                             double* __restrict__ part) {
+                                                                             double* __restrict__ part,
+                                                                             const float* __restrict__ p_override,
+                                                                             int pcur) {
   pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;
   const long long pl = pr.Vp;
-  const float sw = pr.s_w;
   const float lam = pr.lm ? s->lambda_f : 0.0f;
+  const float* __restrict__ pa = (p_override ? p_override : pr.p + (long long)(pcur & 1) * 6 * pl) + 3 * pl;
   F2 acc = f2_zero();
   for (int i = ch.begin + threadIdx.x; i < ch.end; i += NT) {
-    int o0 = 0, o1 = 0, n0 = 0, n1 = 0;
-    int jo[KB], ji[KB];
-    if (!G3) {
-      o0 = pr.orow[i]; o1 = pr.orow[i + 1];
-      n0 = pr.irow[i]; n1 = pr.irow[i + 1];
-#pragma unroll
-      for (int t = 0; t < KB; ++t) {
-        jo[t] = o0 + t < o1 ? pr.e1[o0 + t] : 0;
-        ji[t] = n0 + t < n1 ? pr.isrc[n0 + t] : 0;
-      }
-    }
-    float pi[6];
-    load_vec(pr.vrec, i, pi);
+    float pd[3], wi[3];
+    load_pw(pr.vrec, i, pd, wi);
     const GeoRec gi = load_geo(pr.grec, i);
-    float q[6];
+    float D[3][3];
+    quat_delta_matrix(gi.q, D);
+    float f[3] = {0.f, 0.f, 0.f}, tq[3] = {0.f, 0.f, 0.f};
+    auto own_edge = [&](const float (&d)[3], const float (&v)[3]) {
+      float y[3], t[3] = {d[0], d[1], d[2]};
+      mat_vec(D, v, y);
 #pragma unroll
-    for (int c = 0; c < 6; ++c) q[c] = pr.lm ? lam * pr.dc[(c < 3 ? 0 : c - 2) * pl + i] * pi[c] : 0.f;
-    if (handle_of(pr, i) >= 0) {
+      for (int c = 0; c < 3; ++c) y[c] += v[c];
+      sub_cross(t, wi, y);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) q[c] += pr.w_fit * pi[c];
-    }
-    auto own_edge = [&](int j) {
-      float pj[3];
-      load_vec3(pr.vrec, j, pj);
-      const float4 uj = __ldg(pr.grec + 3 * j);
-      const float vx = gi.U[0] - uj.x, vy = gi.U[1] - uj.y, vz = gi.U[2] - uj.z;
-      const RotV R = rot_apply_cs(gi.cs[0], gi.cs[1], gi.cs[2], gi.cs[3], gi.cs[4], gi.cs[5], vx, vy, vz);
-      float j0 = sw * (pi[0] - pj[0]), j1 = sw * (pi[1] - pj[1]), j2 = sw * (pi[2] - pj[2]);
-#pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        j0 -= sw * R.g[m][0] * pi[3 + m];
-        j1 -= sw * R.g[m][1] * pi[3 + m];
-        j2 -= sw * R.g[m][2] * pi[3 + m];
-      }
-      q[0] += sw * j0; q[1] += sw * j1; q[2] += sw * j2;
-#pragma unroll
-      for (int m = 0; m < 3; ++m) q[3 + m] -= sw * (R.g[m][0] * j0 + R.g[m][1] * j1 + R.g[m][2] * j2);
+      for (int c = 0; c < 3; ++c) f[c] += t[c];
+      add_cross(tq, y, t);
     };
-    auto in_edge = [&](int j) {
-      float pj[6];
-      load_vec(pr.vrec, j, pj);
+    // -J_e p / s_w of (j, i): d + w_j x (R_j (U_j - U_i)), d = p_i - p_j
+    auto in_edge = [&](const GeoRec& gj, const float (&wj)[3], const float (&d)[3], const float (&v)[3]) {
+      float y[3], t[3] = {d[0], d[1], d[2]};
+      quat_delta(gj.q, v, y);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) y[c] += v[c];
+      sub_cross(t, wj, y);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) f[c] += t[c];
+    };
+    for_neighbours<G3>(pr, i, [&](int j, bool own, bool in) {
       const GeoRec gj = load_geo(pr.grec, j);
-      const float vx = gj.U[0] - gi.U[0], vy = gj.U[1] - gi.U[1], vz = gj.U[2] - gi.U[2];
-      const RotV R = rot_apply_cs(gj.cs[0], gj.cs[1], gj.cs[2], gj.cs[3], gj.cs[4], gj.cs[5], vx, vy, vz);
-      float j0 = sw * (pj[0] - pi[0]), j1 = sw * (pj[1] - pi[1]), j2 = sw * (pj[2] - pi[2]);
+      float pj[3], wj[3], d[3], v[3];
+      load_pw(pr.vrec, j, pj, wj);
 #pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        j0 -= sw * R.g[m][0] * pj[3 + m];
-        j1 -= sw * R.g[m][1] * pj[3 + m];
-        j2 -= sw * R.g[m][2] * pj[3 + m];
+      for (int c = 0; c < 3; ++c) {
+        d[c] = pd[c] - pj[c];
+        v[c] = gi.U[c] - gj.U[c];
       }
-      q[0] -= sw * j0; q[1] -= sw * j1; q[2] -= sw * j2;
-    };
-    if (G3) {
-      const Stencil3 st = stencil3(pr, i);
+      if (own) own_edge(d, v);
+      if (in) in_edge(gj, wj, d, v);
+    });
+    float q[6], ga[3];
+    axis_rows(load_axes(pr, i), tq, ga);
+    const float pi[6] = {pd[0], pd[1], pd[2], pa[i], pa[pl + i], pa[2 * pl + i]};
+    const bool hit = handle_of(pr, i) >= 0;
 #pragma unroll
-      for (int t = 0; t < 6; ++t)
-        if (st.ok[t]) own_edge(i + st.off[t]);
+    for (int c = 0; c < 3; ++c) {
+      q[c] = pr.w_reg * f[c];
+      if (hit) q[c] = fmaf(pr.w_fit, pd[c], q[c]);
+      q[3 + c] = -pr.w_reg * ga[c];
+    }
+    if (pr.lm) {
 #pragma unroll
-      for (int t = 0; t < 6; ++t)
-        if (st.ok[t]) in_edge(i + st.off[t]);
-    } else {
-#pragma unroll
-      for (int t = 0; t < KB + 1; ++t) {
-        // t < KB: one prefetched out-edge (if the row has it); t == KB: the rest of a longer row
-        const int kb = t < KB ? o0 + t : o0 + KB, ke = t < KB ? min(o0 + t + 1, o1) : o1;
-        for (int k = kb; k < ke; ++k) own_edge(t < KB ? jo[t] : pr.e1[k]);
-      }
-#pragma unroll
-      for (int t = 0; t < KB + 1; ++t) {
-        const int kb = t < KB ? n0 + t : n0 + KB, ke = t < KB ? min(n0 + t + 1, n1) : n1;
-        for (int k = kb; k < ke; ++k) in_edge(t < KB ? ji[t] : pr.isrc[k]);
-      }
+      for (int c = 0; c < 6; ++c) q[c] = fmaf(lam * pr.dc[(c < 3 ? 0 : c - 2) * pl + i], pi[c], q[c]);
     }
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
@@ -423,61 +527,15 @@ __global__ void __launch_bounds__(NT, MESH_PULL_MIN_BLOCKS) k_mesh_apply_pull(co
 // out-of-tile neighbours, a table built at planning) in shared memory: the
 // displacement rows of the direction p = M^-1 r + beta p_old (formed here,
 // halo included, with the same roundings everywhere) and the rest position U.
-// With M_i = sum_m p_i,m dR/dA_m(A_i) formed once per vertex (rot3 /
-// rot3_dir), the linearized residual of an out-edge e = (i, j) is
-//   t_e = J_e p = s_w [(p_i,d - p_j,d) - M_i v],   v = U_i - U_j;
-// it adds s_w t_e to i's displacement rows and its angle rows
-// -s_w (dR/dA_m v) . t_e are summed through S_i = sum_e t_e v^T, one
-// contraction per vertex (rot3_contract) instead of three derivative vectors
-// per edge.  Each t_e goes to a shared-memory slot; in-edges that start
+// With R_i and w_i formed once per vertex, the linearized residual of an
+// out-edge e = (i, j) is
+//   t_e = J_e p = s_w [(p_i,d - p_j,d) - w_i x y],   y = R_i (U_i - U_j);
+// it adds s_w t_e to i's displacement rows and y x t_e to i's torque.  Each t_e goes to a shared-memory slot; in-edges that start
 // outside the tile are evaluated edge-parallel from their source's data into
 // further slots; every vertex then subtracts s_w t_e of its in-edges, read
 // from their slots (a slot table built at planning).  So each residual is
 // evaluated once inside a tile and once more per tile border it crosses, no
 // atomic is used, and every row is summed in a fixed order.
-
-// Rotation R = Rz(az) Ry(ay) Rx(ax) from the angles' cos / sin, with
-// u' = dR_:0 / day; the angle derivatives are then
-//   dR/dax = [0 | R_:2 | -R_:1],  dR/day = [u' | sin ax R_:0 | cos ax R_:0],
-//   dR/daz = rows (-R_1:, R_0:, 0).
-struct Rot3 {
-  float r[3][3];
-  float ud[3];
-  float ca, sa;
-};
-__device__ __forceinline__ Rot3 rot3(const float cs[6]) {
-  const float ca = cs[0], sa = cs[1], cb = cs[2], sb = cs[3], cc = cs[4], sc = cs[5];
-  const float a1 = sa * sb, a2 = ca * sb;
-  Rot3 o;
-  o.r[0][0] = cb * cc; o.r[0][1] = fmaf(a1, cc, -ca * sc); o.r[0][2] = fmaf(a2, cc, sa * sc);
-  o.r[1][0] = cb * sc; o.r[1][1] = fmaf(a1, sc, ca * cc);  o.r[1][2] = fmaf(a2, sc, -sa * cc);
-  o.r[2][0] = -sb;     o.r[2][1] = sa * cb;                o.r[2][2] = ca * cb;
-  o.ud[0] = -sb * cc; o.ud[1] = -sb * sc; o.ud[2] = -cb;
-  o.ca = ca; o.sa = sa;
-  return o;
-}
-// M = pa dR/dax + pb dR/day + pc dR/daz
-__device__ __forceinline__ void rot3_dir(const Rot3& R, float pa, float pb, float pc, float (&M)[3][3]) {
-  const float dz[3][3] = {{-R.r[1][0], -R.r[1][1], -R.r[1][2]}, {R.r[0][0], R.r[0][1], R.r[0][2]}, {0.f, 0.f, 0.f}};
-  const float bs = pb * R.sa, bc = pb * R.ca;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    M[i][0] = fmaf(pb, R.ud[i], pc * dz[i][0]);
-    M[i][1] = fmaf(pa, R.r[i][2], fmaf(bs, R.r[i][0], pc * dz[i][1]));
-    M[i][2] = fmaf(-pa, R.r[i][1], fmaf(bc, R.r[i][0], pc * dz[i][2]));
-  }
-}
-// (<dR/dax, S>, <dR/day, S>, <dR/daz, S>), <A, B> = sum_ij A_ij B_ij
-__device__ __forceinline__ void rot3_contract(const Rot3& R, const float (&S)[3][3], float (&o)[3]) {
-  float a = 0.f, b = 0.f, c = 0.f;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    a = fmaf(R.r[i][2], S[i][1], fmaf(-R.r[i][1], S[i][2], a));
-    b = fmaf(R.ud[i], S[i][0], fmaf(R.r[i][0], fmaf(R.sa, S[i][1], R.ca * S[i][2]), b));
-    c = fmaf(-R.r[1][i], S[0][i], fmaf(R.r[0][i], S[1][i], c));
-  }
-  o[0] = a; o[1] = b; o[2] = c;
-}
 
 // The direction of vertex v, components [0, NC): p = M^-1 r + beta p_old
 // (update) or the given p; the same roundings wherever it is formed.
@@ -496,16 +554,6 @@ __device__ __forceinline__ void mesh_direction(const MeshProb& pr, int v, long l
   } else {
 #pragma unroll
     for (int c = 0; c < NC; ++c) o[c] = pin[c * pl + v];
-  }
-}
-
-// J_e p of an edge (a, b) from a's matrix M_a: s_w [(p_a - p_b) - M_a v], v = U_a - U_b
-__device__ __forceinline__ void edge_jp(float sw, const float (&M)[3][3], const float* pa, const float* pb,
-                                        const float (&v)[3], float (&t)[3]) {
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const float mv = fmaf(M[a][0], v[0], fmaf(M[a][1], v[1], M[a][2] * v[2]));
-    t[a] = sw * ((pa[a] - pb[a]) - mv);
   }
 }
 
@@ -538,7 +586,8 @@ __global__ void __launch_bounds__(NT, MESH_TILED_MIN_BLOCKS) k_mesh_apply_tiled(
   int o0 = 0, o1 = 0, n0 = 0, n1 = 0;
   int ln[KB], sl[KB];
   float pi[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  float ui[3] = {0.f, 0.f, 0.f}, cs[6] = {1.f, 0.f, 1.f, 0.f, 1.f, 0.f};
+  float ui[3] = {0.f, 0.f, 0.f}, qi[4] = {1.f, 0.f, 0.f, 0.f};
+  float4 axes = make_float4(1.f, 0.f, 1.f, 0.f);
   if (own) {
     o0 = pr.orow[i]; o1 = pr.orow[i + 1];
     n0 = pr.irow[i]; n1 = pr.irow[i + 1];
@@ -556,7 +605,8 @@ __global__ void __launch_bounds__(NT, MESH_TILED_MIN_BLOCKS) k_mesh_apply_tiled(
 #pragma unroll
     for (int c = 0; c < 3; ++c) ui[c] = g.U[c];
 #pragma unroll
-    for (int c = 0; c < 6; ++c) cs[c] = g.cs[c];
+    for (int c = 0; c < 4; ++c) qi[c] = g.q[c];
+    axes = load_axes(pr, i);
   }
 #pragma unroll
   for (int c = 0; c < 3; ++c) { spu[c][tid] = pi[c]; spu[3 + c][tid] = ui[c]; }
@@ -566,7 +616,7 @@ __global__ void __launch_bounds__(NT, MESH_TILED_MIN_BLOCKS) k_mesh_apply_tiled(
       const int j = pr.hvtx[h0 + l];
       float pj[3];
       mesh_direction<3>(pr, j, pl, update, beta, pin, pj);
-      const float4 g = __ldg(pr.grec + 3 * j);
+      const float4 g = __ldg(pr.grec + 2 * (size_t)j);
       spu[0][VT + l] = pj[0]; spu[1][VT + l] = pj[1]; spu[2][VT + l] = pj[2];
       spu[3][VT + l] = g.x; spu[4][VT + l] = g.y; spu[5][VT + l] = g.z;
     }
@@ -574,22 +624,25 @@ __global__ void __launch_bounds__(NT, MESH_TILED_MIN_BLOCKS) k_mesh_apply_tiled(
   __syncthreads();
   // B: own edges (displacement rows, S_i), their J_e p into the slots
   float q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  float S[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
+  float tq[3] = {0.f, 0.f, 0.f};
   if (own) {
-    float M[3][3];
-    rot3_dir(rot3(cs), pi[3], pi[4], pi[5], M);
+    float D[3][3], w[3];
+    angular_velocity(axes, pi[3], pi[4], pi[5], w);
+    quat_delta_matrix(qi, D);
     auto own_edge = [&](int k, int l) {
-      const float pj[3] = {spu[0][l], spu[1][l], spu[2][l]};
       const float v[3] = {ui[0] - spu[3][l], ui[1] - spu[4][l], ui[2] - spu[5][l]};
-      float t[3];
-      edge_jp(sw, M, pi, pj, v, t);
+      float t[3] = {pi[0] - spu[0][l], pi[1] - spu[1][l], pi[2] - spu[2][l]}, y[3];
+      mat_vec(D, v, y);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) y[a] += v[a];
+      sub_cross(t, w, y);
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
+        t[a] *= sw;
         q[a] = fmaf(sw, t[a], q[a]);
-#pragma unroll
-        for (int b = 0; b < 3; ++b) S[a][b] = fmaf(t[a], v[b], S[a][b]);
         st[a][k - ebase] = t[a];
       }
+      add_cross(tq, y, t);
     };
 #pragma unroll
     for (int t = 0; t < KB; ++t)
@@ -606,13 +659,16 @@ __global__ void __launch_bounds__(NT, MESH_TILED_MIN_BLOCKS) k_mesh_apply_tiled(
       float pj[6];
       mesh_direction<6>(pr, j, pl, update, beta, pin, pj);
       const GeoRec gj = load_geo(pr.grec, j);
-      float Mj[3][3], t[3];
-      rot3_dir(rot3(gj.cs), pj[3], pj[4], pj[5], Mj);
-      const float d[3] = {spu[0][dl], spu[1][dl], spu[2][dl]};
+      float wj[3], y[3];
+      angular_velocity(load_axes(pr, j), pj[3], pj[4], pj[5], wj);
       const float v[3] = {gj.U[0] - spu[3][dl], gj.U[1] - spu[4][dl], gj.U[2] - spu[5][dl]};
-      edge_jp(sw, Mj, pj, d, v, t);
+      float t[3] = {pj[0] - spu[0][dl], pj[1] - spu[1][dl], pj[2] - spu[2][dl]};
+      quat_delta(gj.q, v, y);
 #pragma unroll
-      for (int a = 0; a < 3; ++a) st[a][nout + r] = t[a];
+      for (int a = 0; a < 3; ++a) y[a] += v[a];
+      sub_cross(t, wj, y);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) st[a][nout + r] = sw * t[a];
     }
   }
   __syncthreads();
@@ -620,7 +676,7 @@ __global__ void __launch_bounds__(NT, MESH_TILED_MIN_BLOCKS) k_mesh_apply_tiled(
   F2 acc = f2_zero();
   if (own) {
     float ga[3];
-    rot3_contract(rot3(cs), S, ga);
+    axis_rows(axes, tq, ga);
 #pragma unroll
     for (int m = 0; m < 3; ++m) q[3 + m] = -sw * ga[m];
     auto in_edge = [&](int slot) {
@@ -722,93 +778,148 @@ __global__ void __launch_bounds__(NT) k_mesh_update(const MeshProb* __restrict__
 // ---------------------------------------------------------------------------
 // energies and the outer update
 // ---------------------------------------------------------------------------
-// Fit part: mode 0 -> part0 = E_fit(x); mode 1 -> part0 = E_fit(x + delta)
-// (the fit residual is linear, so the model value is the same).
+// Vertex pass of the energies on edge lists: what the gather reads of a
+// neighbour, its displacement, rest position and (mode 1) displacement step,
+// in one record.  (A voxel's neighbours lie next to it in the planes.)
 __global__ void __launch_bounds__(NT) k_mesh_energy_v(const MeshProb* __restrict__ probs,
-                                                      const Chunk* __restrict__ chunks,
-                                                      double* __restrict__ part, int mode) {
+                                                      const Chunk* __restrict__ chunks, int mode) {
   pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
-  Scalars* s = pr.s;
-  if (mode == 1 && s->done) return;
+  if (mode == 1 && pr.s->done) return;
   const long long pl = pr.Vp;
-  F2 e = f2_zero();
   for (int v = ch.begin + threadIdx.x; v < ch.end; v += NT) {
-    const int h = handle_of(pr, v);
-    if (h < 0) continue;
-    float ev = 0.f;
+    float x[3], U[3], d[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      float dv = pr.x[c * pl + v];
-      if (mode == 1) dv += pr.d[c * pl + v];
-      const float f = pr.s_f * (dv - pr.htgt[3 * h + c]);
-      ev += f * f;
+      x[c] = pr.x[c * pl + v];
+      U[c] = __ldg(pr.U + c * pl + v);
+      if (mode == 1) d[c] = pr.d[c * pl + v];
     }
-    f2_add(e, ev);
-  }
-  pdl_trigger();
-  if (publish_partials(part, blockIdx.x, e, f2_zero(), &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
-    double a, b;
-    gather_partials(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, a, b);
-    if (threadIdx.x == 0) s->part0 = a;
+    pr.vrec[3 * (size_t)v] = make_float4(x[0], x[1], x[2], U[0]);
+    pr.vrec[3 * (size_t)v + 1] = make_float4(U[1], U[2], d[0], d[1]);
+    if (mode == 1) pr.vrec[3 * (size_t)v + 2] = make_float4(d[2], 0.f, 0.f, 0.f);
   }
 }
 
-__global__ void __launch_bounds__(NT) k_mesh_energy_e(const MeshProb* __restrict__ probs,
-                                                      const Chunk* __restrict__ chunks,
-                                                      double* __restrict__ part, int mode,
-                                                      int hist_idx) {
+// Energy of every vertex's fit residual and out-edge residuals.  mode 0: at x;
+// mode 1: at x + delta, and the model value |F(x) + J(x) delta|^2 (the fit
+// residual is linear: one value serves both).  The rotations and the angular
+// velocity of delta are formed once per vertex, not per edge (edge-parallel
+// with sincosf at both ends: 166 us on the 128^3 volume).
+template <bool G3>
+__global__ void __launch_bounds__(NT) k_mesh_energy(const MeshProb* __restrict__ probs,
+                                                    const Chunk* __restrict__ chunks,
+                                                    double* __restrict__ part, int mode, int hist_idx) {
   pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
   Scalars* s = pr.s;
   if (mode == 1 && s->done) return;
   const long long pl = pr.Vp;
-  const float sw = pr.s_w;
   F2 e0 = f2_zero(), e1 = f2_zero();
-  for (int ei = ch.begin + threadIdx.x; ei < ch.end; ei += NT) {
-    const int a = pr.e0[ei], b = pr.e1[ei];
-    const float vx = pr.U[a] - pr.U[b];
-    const float vy = pr.U[pl + a] - pr.U[pl + b];
-    const float vz = pr.U[2 * pl + a] - pr.U[2 * pl + b];
-    const float dd0 = pr.x[a] - pr.x[b], dd1 = pr.x[pl + a] - pr.x[pl + b];
-    const float dd2 = pr.x[2 * pl + a] - pr.x[2 * pl + b];
-    const RotV R = rot_apply(pr.x[3 * pl + a], pr.x[4 * pl + a], pr.x[5 * pl + a], vx, vy, vz);
-    const float r0 = sw * (dd0 + (vx - R.rv[0]));
-    const float r1 = sw * (dd1 + (vy - R.rv[1]));
-    const float r2 = sw * (dd2 + (vz - R.rv[2]));
-    if (mode == 0) {
-      f2_add(e0, r0 * r0 + r1 * r1 + r2 * r2);
-    } else {
-      const float ea0 = pr.d[a] - pr.d[b], ea1 = pr.d[pl + a] - pr.d[pl + b];
-      const float ea2 = pr.d[2 * pl + a] - pr.d[2 * pl + b];
-      const float t3 = pr.d[3 * pl + a], t4 = pr.d[4 * pl + a], t5 = pr.d[5 * pl + a];
-      const RotV R2 = rot_apply(pr.x[3 * pl + a] + t3, pr.x[4 * pl + a] + t4, pr.x[5 * pl + a] + t5, vx, vy, vz);
-      const float u0 = sw * ((dd0 + ea0) + (vx - R2.rv[0]));
-      const float u1 = sw * ((dd1 + ea1) + (vy - R2.rv[1]));
-      const float u2 = sw * ((dd2 + ea2) + (vz - R2.rv[2]));
-      f2_add(e0, u0 * u0 + u1 * u1 + u2 * u2);
-      const float l0 = r0 + sw * ea0 - sw * (R.g[0][0] * t3 + R.g[1][0] * t4 + R.g[2][0] * t5);
-      const float l1 = r1 + sw * ea1 - sw * (R.g[0][1] * t3 + R.g[1][1] * t4 + R.g[2][1] * t5);
-      const float l2 = r2 + sw * ea2 - sw * (R.g[0][2] * t3 + R.g[1][2] * t4 + R.g[2][2] * t5);
-      f2_add(e1, l0 * l0 + l1 * l1 + l2 * l2);
+  for (int i = ch.begin + threadIdx.x; i < ch.end; i += NT) {
+    float xi[3], ui[3], di[3], w[3] = {0.f, 0.f, 0.f}, D[3][3], D2[3][3];
+    {
+      float a[3], q[4];
+      float4 axes;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        xi[c] = pr.x[c * pl + i];
+        ui[c] = __ldg(pr.U + c * pl + i);
+        a[c] = pr.x[(3 + c) * pl + i];
+      }
+      angles_to_quat(a, q, axes);
+      quat_delta_matrix(q, D);
+      if (mode == 1) {
+        float t[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          di[c] = pr.d[c * pl + i];
+          t[c] = pr.d[(3 + c) * pl + i];
+          a[c] += t[c];
+        }
+        angular_velocity(axes, t[0], t[1], t[2], w);
+        float4 unused;
+        angles_to_quat(a, q, unused);
+        quat_delta_matrix(q, D2);
+      }
     }
+    float se = 0.f, sm = 0.f, fit = 0.f;
+    const int h = handle_of(pr, i);
+    if (h >= 0) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        float dv = xi[c];
+        if (mode == 1) dv += di[c];
+        const float f = pr.s_f * (dv - pr.htgt[3 * h + c]);
+        fit = fmaf(f, f, fit);
+      }
+    }
+    auto edge = [&](int j) {
+      float d[3], v[3], dd[3];
+      if (G3) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          d[c] = xi[c] - pr.x[c * pl + j];
+          v[c] = ui[c] - __ldg(pr.U + c * pl + j);
+          if (mode == 1) dd[c] = di[c] - pr.d[c * pl + j];
+        }
+      } else {
+        const float4 ra = pr.vrec[3 * (size_t)j], rb = pr.vrec[3 * (size_t)j + 1];
+        d[0] = xi[0] - ra.x; d[1] = xi[1] - ra.y; d[2] = xi[2] - ra.z;
+        v[0] = ui[0] - ra.w; v[1] = ui[1] - rb.x; v[2] = ui[2] - rb.y;
+        if (mode == 1) {
+          dd[0] = di[0] - rb.z; dd[1] = di[1] - rb.w;
+          dd[2] = di[2] - pr.vrec[3 * (size_t)j + 2].x;
+        }
+      }
+      float y[3], r[3];
+      mat_vec(D, v, y);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) r[c] = d[c] - y[c];
+      if (mode == 0) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) se = fmaf(r[c], r[c], se);
+        return;
+      }
+      float y2[3];
+      mat_vec(D2, v, y2);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float u = (d[c] + dd[c]) - y2[c];
+        se = fmaf(u, u, se);
+        r[c] += dd[c];
+        y[c] += v[c];
+      }
+      sub_cross(r, w, y);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) sm = fmaf(r[c], r[c], sm);
+    };
+    if (G3) {
+      const Stencil3 st = stencil3(pr, i);
+#pragma unroll
+      for (int t = 0; t < 6; ++t)
+        if (st.ok[t]) edge(i + st.off[t]);
+    } else {
+      for (int k = pr.orow[i]; k < pr.orow[i + 1]; ++k) edge(pr.e1[k]);
+    }
+    f2_add(e0, fmaf(pr.w_reg, se, fit));
+    if (mode == 1) f2_add(e1, fmaf(pr.w_reg, sm, fit));
   }
   pdl_trigger();
-  if (publish_partials(part, blockIdx.x, e0, e1, &s->counter, pr.echunk_end - pr.echunk_begin)) {
+  if (publish_partials(part, blockIdx.x, e0, e1, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
     double a, b;
-    gather_partials(part, pr.echunk_begin, pr.echunk_end, &s->counter, a, b);
+    gather_partials(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, a, b);
     if (threadIdx.x == 0) {
       if (mode == 0) {
-        const double E = s->part0 + a;
-        s->E = E;
+        s->E = a;
         const int k = hist_idx >= 0 ? hist_idx : (hist_idx == -1 ? s->outer_done : -1);
-        if (pr.Ehist && k >= 0) pr.Ehist[k] = E;
-        if (!isfinite(E)) s->nonfinite = 1;
+        if (pr.Ehist && k >= 0) pr.Ehist[k] = a;
+        if (!isfinite(a)) s->nonfinite = 1;
       } else {
-        s->E_trial = s->part0 + a;
-        s->model = s->part0 + b;
+        s->E_trial = a;
+        s->model = b;
       }
     }
   }
@@ -857,10 +968,11 @@ void launch_mesh_apply(const MeshLaunch& L, const float* p_override, int par, in
     return;
   }
   launch_pdl(k_mesh_apply_v, L.nvchunks, NT, 0, L.stream, L.probs, L.vchunks, p_override, par, update);
+  const int pcur = update ? par + 1 : par;
   if (L.grid3)
-    launch_pdl(k_mesh_apply_pull<true>, L.nvchunks, NT, 0, L.stream, L.probs, L.vchunks, L.part);
+    launch_pdl(k_mesh_apply_pull<true>, L.nvchunks, NT, 0, L.stream, L.probs, L.vchunks, L.part, p_override, pcur);
   else
-    launch_pdl(k_mesh_apply_pull<false>, L.nvchunks, NT, 0, L.stream, L.probs, L.vchunks, L.part);
+    launch_pdl(k_mesh_apply_pull<false>, L.nvchunks, NT, 0, L.stream, L.probs, L.vchunks, L.part, p_override, pcur);
 }
 
 void launch_mesh_update(const MeshLaunch& L, int par) {
@@ -872,8 +984,11 @@ void launch_mesh_update(const MeshLaunch& L, int par) {
 void launch_mesh_energy(const MeshLaunch& L, int mode, int hist_idx) {
   if (L.dim == 2) return launch_wg_energy(L, mode, hist_idx);
   if (L.dim == 12) return launch_ed_energy(L, mode, hist_idx);
-  launch_pdl(k_mesh_energy_v, L.nvchunks, NT, 0, L.stream, L.probs, L.vchunks, L.part, mode);
-  launch_pdl(k_mesh_energy_e, L.nechunks, NT, 0, L.stream, L.probs, L.echunks, L.part, mode, hist_idx);
+  if (!L.grid3) launch_pdl(k_mesh_energy_v, L.nvchunks, NT, 0, L.stream, L.probs, L.vchunks, mode);
+  if (L.grid3)
+    launch_pdl(k_mesh_energy<true>, L.nvchunks, NT, 0, L.stream, L.probs, L.vchunks, L.part, mode, hist_idx);
+  else
+    launch_pdl(k_mesh_energy<false>, L.nvchunks, NT, 0, L.stream, L.probs, L.vchunks, L.part, mode, hist_idx);
 }
 
 void launch_mesh_step(const MeshLaunch& L, int cond) {

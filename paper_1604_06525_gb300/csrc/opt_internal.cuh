@@ -135,7 +135,8 @@ struct GridProb {
 
 // Graph problem (ARAP mesh).
 struct MeshProb {
-  int V, E, Vp, pad;
+  int V, E, Vp;
+  int sym;                      // every vertex's out- and in-edge lists are equal (edges given both ways)
   int gw, gh, gd, gpad;         // volumetric problems: voxel grid W x H x D (0 for graphs)
   int vchunk_begin, vchunk_end;
   int echunk_begin, echunk_end;
@@ -161,8 +162,8 @@ struct MeshProb {
   const int* itslot;            // E: shared-memory slot of each in-edge's J_e p (irow order)
   float *d, *r, *p, *q;         // 6 planes each
   float *m, *dc;                // 4 planes: displacement, ax, ay, az
-  float4* grec;                 // 3 float4 per vertex: U, cos / sin of the angles (PCGInit)
-  float4* vrec;                 // 2 float4 per vertex: x (PCGInit) or p (applyJTJ)
+  float4* grec;                 // geometry records, written by PCGInit (each energy's layout: its kernels' file)
+  float4* vrec;                 // vector records (x, p or the energies' data)
   const int* hbeg;              // per vertex tile: first handle
   const int* hpix;              // handle vertex, sorted
   const float* htgt;            // 3 per handle
