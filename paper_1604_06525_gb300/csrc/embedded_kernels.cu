@@ -108,9 +108,9 @@ __device__ __forceinline__ void col_constraints_t(const float* m, const float (&
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(NT) k_ed_init_v(const MeshProb* __restrict__ probs,
                                                   const Chunk* __restrict__ chunks) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   if (pr.s->done) return;
   const long long pl = pr.Vp;
   for (int v = ch.begin + threadIdx.x; v < ch.end; v += NT) {
@@ -133,9 +133,9 @@ __global__ void __launch_bounds__(NT, ED_INIT_MIN_BLOCKS) k_ed_init_pull(const M
                                                      const Chunk* __restrict__ chunks,
                                                      double* __restrict__ part, int k_outer, float dmin,
                                                      float dmax) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (s->done) return;
   const long long pl = pr.Vp;
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(NT, ED_INIT_MIN_BLOCKS) k_ed_init_pull(const M
     double rz, E;
     gather_partials(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, rz, E);
     if (threadIdx.x == 0) {
-      s->rz = rz;
+      set_rz(s, rz);
       s->E = E;
       if (pr.Ehist && k_outer >= 0) pr.Ehist[k_outer] = E;
       s->beta_f = 0.f;
@@ -254,9 +254,9 @@ __global__ void __launch_bounds__(NT, ED_INIT_MIN_BLOCKS) k_ed_init_pull(const M
 __global__ void __launch_bounds__(NT) k_ed_apply_v(const MeshProb* __restrict__ probs,
                                                    const Chunk* __restrict__ chunks,
                                                    const float* __restrict__ p_override, int par, int update) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;
   const long long pl = pr.Vp;
@@ -295,9 +295,9 @@ __global__ void __launch_bounds__(NT) k_ed_apply_v(const MeshProb* __restrict__ 
 __global__ void __launch_bounds__(NT) k_ed_apply_pull(const MeshProb* __restrict__ probs,
                                                       const Chunk* __restrict__ chunks,
                                                       double* __restrict__ part) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;
   const long long pl = pr.Vp;
@@ -360,19 +360,11 @@ __global__ void __launch_bounds__(NT) k_ed_apply_pull(const MeshProb* __restrict
     }
   }
   pdl_trigger();
-  if (publish_partials(part, blockIdx.x, acc, f2_zero(), &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
-    double pq, unused;
-    gather_partials(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, pq, unused);
-    if (threadIdx.x == 0) {
-      s->pq = pq;
-      if (pq > 0.0 && isfinite(pq)) {
-        s->alpha_f = (float)(s->rz / pq);
-      } else {
-        s->alpha_f = 0.f;
-        s->pcg_active = 0;
-        if (!isfinite(pq)) s->nonfinite = 1;
-      }
-    }
+  const F2 sums[1] = {acc};
+  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
+    F2 pq[1];
+    gather_pairs<1>(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, pq);
+    if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
 
@@ -388,9 +380,9 @@ __global__ void __launch_bounds__(NT) k_ed_apply_pull(const MeshProb* __restrict
 __global__ void __launch_bounds__(NT, ED_UPDATE_MIN_BLOCKS) k_ed_update(const MeshProb* __restrict__ probs,
                                                   const Chunk* __restrict__ chunks,
                                                   double* __restrict__ part, int par) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;
   const long long pl = pr.Vp;
@@ -433,16 +425,11 @@ __global__ void __launch_bounds__(NT, ED_UPDATE_MIN_BLOCKS) k_ed_update(const Me
     }
   }
   pdl_trigger();
-  if (publish_partials(part, blockIdx.x, acc, f2_zero(), &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
-    double rz, unused;
-    gather_partials(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, rz, unused);
-    if (threadIdx.x == 0) {
-      s->beta_f = (float)(rz / s->rz);
-      s->rz = rz;
-      s->pcg_iters += 1;
-      if (rz == 0.0 || !isfinite(rz)) s->pcg_active = 0;
-      if (!isfinite(rz)) s->nonfinite = 1;
-    }
+  const F2 sums[1] = {acc};
+  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
+    F2 rz[1];
+    gather_pairs<1>(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, rz);
+    if (threadIdx.x == 0) finish_beta(s, rz[0]);
   }
 }
 
@@ -455,9 +442,9 @@ __global__ void __launch_bounds__(NT, ED_UPDATE_MIN_BLOCKS) k_ed_update(const Me
 __global__ void __launch_bounds__(NT) k_ed_energy(const MeshProb* __restrict__ probs,
                                                   const Chunk* __restrict__ chunks,
                                                   double* __restrict__ part, int mode, int hist_idx) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (mode == 1 && s->done) return;
   const long long pl = pr.Vp;
@@ -542,9 +529,9 @@ __global__ void __launch_bounds__(NT) k_ed_energy(const MeshProb* __restrict__ p
 
 __global__ void __launch_bounds__(NT) k_ed_step(const MeshProb* __restrict__ probs,
                                                 const Chunk* __restrict__ chunks, int cond) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   if (cond && !pr.s->accept) return;
   if (!cond && pr.s->done) return;
   const long long pl = pr.Vp;

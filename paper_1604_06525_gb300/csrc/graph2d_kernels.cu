@@ -37,9 +37,9 @@ __device__ __forceinline__ float cc4(const float4& a, int k) {
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(NT) k_wg_init_v(const MeshProb* __restrict__ probs,
                                                   const Chunk* __restrict__ chunks) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   if (pr.s->done) return;
   const long long pl = pr.Vp;
   for (int v = ch.begin + threadIdx.x; v < ch.end; v += NT) {
@@ -59,9 +59,9 @@ __global__ void __launch_bounds__(NT) k_wg_init_pull(const MeshProb* __restrict_
                                                      const Chunk* __restrict__ chunks,
                                                      double* __restrict__ part, int k_outer, float dmin,
                                                      float dmax) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (s->done) return;
   const long long pl = pr.Vp;
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(NT) k_wg_init_pull(const MeshProb* __restrict_
     double rz, E;
     gather_partials(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, rz, E);
     if (threadIdx.x == 0) {
-      s->rz = rz;
+      set_rz(s, rz);
       s->E = E;
       if (pr.Ehist && k_outer >= 0) pr.Ehist[k_outer] = E;
       s->beta_f = 0.f;
@@ -142,9 +142,9 @@ __global__ void __launch_bounds__(NT) k_wg_init_pull(const MeshProb* __restrict_
 __global__ void __launch_bounds__(NT) k_wg_apply_v(const MeshProb* __restrict__ probs,
                                                    const Chunk* __restrict__ chunks,
                                                    const float* __restrict__ p_override, int par, int update) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;
   const long long pl = pr.Vp;
@@ -193,9 +193,9 @@ __global__ void __launch_bounds__(NT) k_wg_apply_v(const MeshProb* __restrict__ 
 __global__ void __launch_bounds__(NT) k_wg_apply_pull(const MeshProb* __restrict__ probs,
                                                       const Chunk* __restrict__ chunks,
                                                       double* __restrict__ part) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;
   const long long pl = pr.Vp;
@@ -238,19 +238,11 @@ __global__ void __launch_bounds__(NT) k_wg_apply_pull(const MeshProb* __restrict
     f2_add_prod(acc, pi.z, qt);
   }
   pdl_trigger();
-  if (publish_partials(part, blockIdx.x, acc, f2_zero(), &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
-    double pq, unused;
-    gather_partials(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, pq, unused);
-    if (threadIdx.x == 0) {
-      s->pq = pq;
-      if (pq > 0.0 && isfinite(pq)) {
-        s->alpha_f = (float)(s->rz / pq);
-      } else {
-        s->alpha_f = 0.f;
-        s->pcg_active = 0;
-        if (!isfinite(pq)) s->nonfinite = 1;
-      }
-    }
+  const F2 sums[1] = {acc};
+  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
+    F2 pq[1];
+    gather_pairs<1>(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, pq);
+    if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
 
@@ -259,9 +251,9 @@ __global__ void __launch_bounds__(NT) k_wg_apply_pull(const MeshProb* __restrict
 __global__ void __launch_bounds__(NT) k_wg_update(const MeshProb* __restrict__ probs,
                                                   const Chunk* __restrict__ chunks,
                                                   double* __restrict__ part, int par) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;
   const long long pl = pr.Vp;
@@ -296,16 +288,11 @@ __global__ void __launch_bounds__(NT) k_wg_update(const MeshProb* __restrict__ p
     }
   }
   pdl_trigger();
-  if (publish_partials(part, blockIdx.x, acc, f2_zero(), &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
-    double rz, unused;
-    gather_partials(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, rz, unused);
-    if (threadIdx.x == 0) {
-      s->beta_f = (float)(rz / s->rz);
-      s->rz = rz;
-      s->pcg_iters += 1;
-      if (rz == 0.0 || !isfinite(rz)) s->pcg_active = 0;
-      if (!isfinite(rz)) s->nonfinite = 1;
-    }
+  const F2 sums[1] = {acc};
+  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
+    F2 rz[1];
+    gather_pairs<1>(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, rz);
+    if (threadIdx.x == 0) finish_beta(s, rz[0]);
   }
 }
 
@@ -317,9 +304,9 @@ __global__ void __launch_bounds__(NT) k_wg_update(const MeshProb* __restrict__ p
 __global__ void __launch_bounds__(NT) k_wg_energy_v(const MeshProb* __restrict__ probs,
                                                     const Chunk* __restrict__ chunks,
                                                     double* __restrict__ part, int mode) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (mode == 1 && s->done) return;
   const long long pl = pr.Vp;
@@ -349,9 +336,9 @@ __global__ void __launch_bounds__(NT) k_wg_energy_v(const MeshProb* __restrict__
 __global__ void __launch_bounds__(NT) k_wg_energy_e(const MeshProb* __restrict__ probs,
                                                     const Chunk* __restrict__ chunks,
                                                     double* __restrict__ part, int mode, int hist_idx) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (mode == 1 && s->done) return;
   const long long pl = pr.Vp;
@@ -400,9 +387,9 @@ __global__ void __launch_bounds__(NT) k_wg_energy_e(const MeshProb* __restrict__
 
 __global__ void __launch_bounds__(NT) k_wg_step(const MeshProb* __restrict__ probs,
                                                 const Chunk* __restrict__ chunks, int cond) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   if (cond && !pr.s->accept) return;
   if (!cond && pr.s->done) return;
   const long long pl = pr.Vp;

@@ -218,9 +218,9 @@ __device__ __forceinline__ void for_neighbours(const MeshProb& pr, int i, Edge e
 // Vertex pass: the quaternion and axes of every vertex and both records.
 __global__ void __launch_bounds__(NT) k_mesh_init_v(const MeshProb* __restrict__ probs,
                                                     const Chunk* __restrict__ chunks) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   if (pr.s->done) return;
   const long long pl = pr.Vp;
   for (int v = ch.begin + threadIdx.x; v < ch.end; v += NT) {
@@ -253,9 +253,9 @@ __global__ void __launch_bounds__(NT, MESH_INIT_MIN_BLOCKS) k_mesh_init_pull(con
                                                        const Chunk* __restrict__ chunks,
                                                        double* __restrict__ part, int k_outer, float dmin,
                                                        float dmax) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (s->done) return;
   const long long pl = pr.Vp;
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(NT, MESH_INIT_MIN_BLOCKS) k_mesh_init_pull(con
     double rz, E;
     gather_partials(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, rz, E);
     if (threadIdx.x == 0) {
-      s->rz = rz;
+      set_rz(s, rz);
       s->E = E;
       if (pr.Ehist && k_outer >= 0) pr.Ehist[k_outer] = E;
       s->beta_f = 0.f;
@@ -372,9 +372,9 @@ __global__ void __launch_bounds__(NT) k_mesh_apply_v(const MeshProb* __restrict_
                                                      const Chunk* __restrict__ chunks,
                                                      const float* __restrict__ p_override, int par,
                                                      int update) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;
   const long long pl = pr.Vp;
@@ -434,9 +434,9 @@ __global__ void __launch_bounds__(NT, MESH_PULL_MIN_BLOCKS) k_mesh_apply_pull(co
                                                                              double* __restrict__ part,
                                                                              const float* __restrict__ p_override,
                                                                              int pcur) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;
   const long long pl = pr.Vp;
@@ -503,19 +503,11 @@ __global__ void __launch_bounds__(NT, MESH_PULL_MIN_BLOCKS) k_mesh_apply_pull(co
     }
   }
   pdl_trigger();
-  if (publish_partials(part, blockIdx.x, acc, f2_zero(), &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
-    double pq, unused;
-    gather_partials(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, pq, unused);
-    if (threadIdx.x == 0) {
-      s->pq = pq;
-      if (pq > 0.0 && isfinite(pq)) {
-        s->alpha_f = (float)(s->rz / pq);
-      } else {
-        s->alpha_f = 0.f;
-        s->pcg_active = 0;
-        if (!isfinite(pq)) s->nonfinite = 1;
-      }
-    }
+  const F2 sums[1] = {acc};
+  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
+    F2 pq[1];
+    gather_pairs<1>(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, pq);
+    if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
 
@@ -564,9 +556,9 @@ __device__ __forceinline__ void mesh_direction(const MeshProb& pr, int v, long l
 __global__ void __launch_bounds__(NT, MESH_TILED_MIN_BLOCKS) k_mesh_apply_tiled(
     const MeshProb* __restrict__ probs, const Chunk* __restrict__ tchunks, double* __restrict__ part,
     const float* __restrict__ p_override, int par, int update) {
-  pdl_begin();
   const Chunk ch = tchunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;
   __shared__ float spu[6][VT + MT_HALO];   // the tile's vertices, then its halo: p_d (3), U (3)
@@ -704,19 +696,11 @@ __global__ void __launch_bounds__(NT, MESH_TILED_MIN_BLOCKS) k_mesh_apply_tiled(
   }
   (void)ibase;
   pdl_trigger();
-  if (publish_partials(part, blockIdx.x, acc, f2_zero(), &s->counter, pr.tchunk_end - pr.tchunk_begin)) {
-    double pq, unused;
-    gather_partials(part, pr.tchunk_begin, pr.tchunk_end, &s->counter, pq, unused);
-    if (threadIdx.x == 0) {
-      s->pq = pq;
-      if (pq > 0.0 && isfinite(pq)) {
-        s->alpha_f = (float)(s->rz / pq);
-      } else {
-        s->alpha_f = 0.f;
-        s->pcg_active = 0;
-        if (!isfinite(pq)) s->nonfinite = 1;
-      }
-    }
+  const F2 sums[1] = {acc};
+  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.tchunk_end - pr.tchunk_begin)) {
+    F2 pq[1];
+    gather_pairs<1>(part, pr.tchunk_begin, pr.tchunk_end, &s->counter, pq);
+    if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
 
@@ -725,9 +709,9 @@ __global__ void __launch_bounds__(NT, MESH_TILED_MIN_BLOCKS) k_mesh_apply_tiled(
 __global__ void __launch_bounds__(NT) k_mesh_update(const MeshProb* __restrict__ probs,
                                                     const Chunk* __restrict__ chunks,
                                                     double* __restrict__ part, int par) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;
   const long long pl = pr.Vp;
@@ -762,16 +746,11 @@ __global__ void __launch_bounds__(NT) k_mesh_update(const MeshProb* __restrict__
     }
   }
   pdl_trigger();
-  if (publish_partials(part, blockIdx.x, f2x2_fold(acc), f2_zero(), &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
-    double rz, unused;
-    gather_partials(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, rz, unused);
-    if (threadIdx.x == 0) {
-      s->beta_f = (float)(rz / s->rz);
-      s->rz = rz;
-      s->pcg_iters += 1;
-      if (rz == 0.0 || !isfinite(rz)) s->pcg_active = 0;
-      if (!isfinite(rz)) s->nonfinite = 1;
-    }
+  const F2 sums[1] = {f2x2_fold(acc)};
+  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
+    F2 rz[1];
+    gather_pairs<1>(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, rz);
+    if (threadIdx.x == 0) finish_beta(s, rz[0]);
   }
 }
 
@@ -783,9 +762,9 @@ __global__ void __launch_bounds__(NT) k_mesh_update(const MeshProb* __restrict__
 // in one record.  (A voxel's neighbours lie next to it in the planes.)
 __global__ void __launch_bounds__(NT) k_mesh_energy_v(const MeshProb* __restrict__ probs,
                                                       const Chunk* __restrict__ chunks, int mode) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   if (mode == 1 && pr.s->done) return;
   const long long pl = pr.Vp;
   for (int v = ch.begin + threadIdx.x; v < ch.end; v += NT) {
@@ -811,9 +790,9 @@ template <bool G3>
 __global__ void __launch_bounds__(NT) k_mesh_energy(const MeshProb* __restrict__ probs,
                                                     const Chunk* __restrict__ chunks,
                                                     double* __restrict__ part, int mode, int hist_idx) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   Scalars* s = pr.s;
   if (mode == 1 && s->done) return;
   const long long pl = pr.Vp;
@@ -927,9 +906,9 @@ __global__ void __launch_bounds__(NT) k_mesh_energy(const MeshProb* __restrict__
 
 __global__ void __launch_bounds__(NT) k_mesh_step(const MeshProb* __restrict__ probs,
                                                   const Chunk* __restrict__ chunks, int cond) {
-  pdl_begin();
   const Chunk ch = chunks[blockIdx.x];
   const MeshProb pr = probs[ch.prob];
+  pdl_begin();
   if (cond && !pr.s->accept) return;
   if (!cond && pr.s->done) return;
   const long long pl = pr.Vp;

@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(NT) k_warp_init(const GridProb* __restrict__ p
     double rz, E;
     gather_partials(part, pr.chunk_begin, pr.chunk_end, &s->counter, rz, E);
     if (threadIdx.x == 0) {
-      s->rz = rz;
+      set_rz(s, rz);
       s->E = E;
       if (pr.Ehist && k_outer >= 0) pr.Ehist[k_outer] = E;
       s->beta_f = 0.f;
@@ -364,19 +364,11 @@ __global__ void __launch_bounds__(NT, 3) k_warp_apply(const GridProb* __restrict
       f2_add_prod(acc, pti, qt);
     }
   }
-  if (publish_partials(part, blockIdx.x, acc, f2_zero(), &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    double pq, unused;
-    gather_partials(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq, unused);
-    if (threadIdx.x == 0) {
-      s->pq = pq;
-      if (pq > 0.0 && isfinite(pq)) {
-        s->alpha_f = (float)(s->rz / pq);
-      } else {
-        s->alpha_f = 0.f;
-        s->pcg_active = 0;
-        if (!isfinite(pq)) s->nonfinite = 1;
-      }
-    }
+  const F2 sums[1] = {acc};
+  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
+    F2 pq[1];
+    gather_pairs<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq);
+    if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
 
@@ -919,19 +911,11 @@ __device__ __forceinline__ void apply_wide_body(WideSmem& sm, const Chunk& ch, c
     }
   }
   cp_async_wait_all();
-  if (publish_partials(part, blockIdx.x, f2x2_fold(acc), f2_zero(), &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    double pq, unused;
-    gather_partials(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq, unused);
-    if (threadIdx.x == 0) {
-      s->pq = pq;
-      if (pq > 0.0 && isfinite(pq)) {
-        s->alpha_f = (float)(s->rz / pq);
-      } else {
-        s->alpha_f = 0.f;
-        s->pcg_active = 0;
-        if (!isfinite(pq)) s->nonfinite = 1;
-      }
-    }
+  const F2 sums[1] = {f2x2_fold(acc)};
+  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
+    F2 pq[1];
+    gather_pairs<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq);
+    if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
 
@@ -1054,9 +1038,9 @@ __device__ __forceinline__ void fused_pending(const Chunk& ch, const GridProb& p
     }
   }
   const F2 none[4] = {f2_zero(), f2_zero(), f2_zero(), f2_zero()};
-  if (publish_partials4(part, blockIdx.x, none, &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    double unused[4];
-    gather_partials4(part, pr.chunk_begin, pr.chunk_end, &s->counter, unused);
+  if (publish_pairs<4>(part, blockIdx.x, none, &s->counter, pr.chunk_end - pr.chunk_begin)) {
+    F2 unused[4];
+    gather_pairs<4>(part, pr.chunk_begin, pr.chunk_end, &s->counter, unused);
     if (threadIdx.x == 0) s->alpha_f = 0.f;
   }
 }
@@ -1068,23 +1052,26 @@ __device__ __forceinline__ void fused_finish(const GridProb& pr, double* __restr
                                              const F2x2& acc_qz, const F2x2& acc_qw, const F2x2& acc_zr) {
   Scalars* s = pr.s;
   const F2 sums[4] = {f2x2_fold(acc_pq), f2x2_fold(acc_qz), f2x2_fold(acc_qw), f2x2_fold(acc_zr)};
-  if (publish_partials4(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    double v[4];
-    gather_partials4(part, pr.chunk_begin, pr.chunk_end, &s->counter, v);
+  if (publish_pairs<4>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
+    F2 v[4];
+    gather_pairs<4>(part, pr.chunk_begin, pr.chunk_end, &s->counter, v);
     if (threadIdx.x == 0) {
-      const double pq = v[0], qz = v[1], qw = v[2], rz = v[3];
-      s->pq = pq;
-      if (pq > 0.0 && isfinite(pq) && rz > 0.0 && isfinite(rz)) {
+      const F2 pq = v[0], rz = v[3];
+      s->pq = f2_to_double(pq);
+      if (pq.hi > 0.f && isfinite(pq.hi) && rz.hi > 0.f && isfinite(rz.hi)) {
         // alpha from the r.z of the stored z (as the two-pass form takes it);
-        // the recurrence only carries r.z one iteration ahead, to set beta
-        const float af = (float)(rz / pq);
-        const double a = (double)af;
-        const double rz_next = fma(a * a, qw, fma(-2.0 * a, qz, rz));
+        // the recurrence only carries r.z one iteration ahead, to set beta.  It
+        // cancels, so it is evaluated in float64.
+        const float af = f2_quot(rz, pq);
+        const double a = (double)af, rzd = f2_to_double(rz);
+        const double rz_next = fma(a * a, f2_to_double(v[2]), fma(-2.0 * a, f2_to_double(v[1]), rzd));
         s->alpha_f = af;
-        s->rz = rz;
+        s->rz = rzd;
+        s->rz_hi = rz.hi;
+        s->rz_lo = rz.lo;
         s->pcg_iters += 1;
         if (rz_next > 0.0 && isfinite(rz_next)) {
-          s->beta_f = (float)(rz_next / rz);
+          s->beta_f = f2_quot(f2_from_double(rz_next), rz);
         } else {
           s->pcg_active = 0;        // the step alpha p is still applied
           if (!isfinite(rz_next)) s->nonfinite = 1;
@@ -1092,7 +1079,7 @@ __device__ __forceinline__ void fused_finish(const GridProb& pr, double* __restr
       } else {
         s->alpha_f = 0.f;
         s->pcg_active = 0;
-        if (!isfinite(pq) || !isfinite(rz)) s->nonfinite = 1;
+        if (!isfinite(pq.hi) || !isfinite(rz.hi)) s->nonfinite = 1;
       }
     }
   }
@@ -1707,7 +1694,7 @@ __device__ __forceinline__ void k_warp_init_wide_body(InitSmem& sm, const Chunk&
     double rz, E;
     gather_partials(part, pr.chunk_begin, pr.chunk_end, &s->counter, rz, E);
     if (threadIdx.x == 0) {
-      s->rz = rz;
+      set_rz(s, rz);
       s->E = E;
       if (pr.Ehist && k_outer >= 0) pr.Ehist[k_outer] = E;
       s->beta_f = 0.f;
@@ -1938,7 +1925,7 @@ __global__ void __launch_bounds__(NT) k_poisson_init(const GridProb* __restrict_
     double rz, E;
     gather_partials(part, pr.chunk_begin, pr.chunk_end, &s->counter, rz, E);
     if (threadIdx.x == 0) {
-      s->rz = rz;
+      set_rz(s, rz);
       s->E = E;
       if (pr.Ehist && k_outer >= 0) pr.Ehist[k_outer] = E;
       s->beta_f = 0.f;
@@ -2068,19 +2055,11 @@ __global__ void __launch_bounds__(NT, 3) k_poisson_apply(const GridProb* __restr
       }
     }
   }
-  if (publish_partials(part, blockIdx.x, acc, f2_zero(), &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    double pq, unused;
-    gather_partials(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq, unused);
-    if (threadIdx.x == 0) {
-      s->pq = pq;
-      if (pq > 0.0 && isfinite(pq)) {
-        s->alpha_f = (float)(s->rz / pq);
-      } else {
-        s->alpha_f = 0.f;
-        s->pcg_active = 0;
-        if (!isfinite(pq)) s->nonfinite = 1;
-      }
-    }
+  const F2 sums[1] = {acc};
+  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
+    F2 pq[1];
+    gather_pairs<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq);
+    if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
 
@@ -2351,19 +2330,11 @@ __device__ __forceinline__ void k_poisson_apply_wide_body(PoisWideSmem& sm, cons
       pois_apply_quad<UPD>(sm.slot[b].raw, sm.slot[b].mk.v, pr, ty, lane, (long long)gy * pr.P + gx, use_beta, beta,
                            beta2, lam, pout, pl, acc);
   }
-  if (publish_partials(part, blockIdx.x, f2x2_fold(acc), f2_zero(), &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    double pq, unused;
-    gather_partials(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq, unused);
-    if (threadIdx.x == 0) {
-      s->pq = pq;
-      if (pq > 0.0 && isfinite(pq)) {
-        s->alpha_f = (float)(s->rz / pq);
-      } else {
-        s->alpha_f = 0.f;
-        s->pcg_active = 0;
-        if (!isfinite(pq)) s->nonfinite = 1;
-      }
-    }
+  const F2 sums[1] = {f2x2_fold(acc)};
+  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
+    F2 pq[1];
+    gather_pairs<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq);
+    if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
 
@@ -2519,7 +2490,7 @@ __device__ __forceinline__ void k_poisson_init_wide_body(PoisInitSmem& sm, const
     double rz, E;
     gather_partials(part, pr.chunk_begin, pr.chunk_end, &s->counter, rz, E);
     if (threadIdx.x == 0) {
-      s->rz = rz;
+      set_rz(s, rz);
       s->E = E;
       if (pr.Ehist && k_outer >= 0) pr.Ehist[k_outer] = E;
       s->beta_f = 0.f;
@@ -2910,17 +2881,11 @@ __device__ __forceinline__ void update_body(const Chunk& ch, const GridProb& pr,
       r4[c * pl4 + j] = rv[c];
     }
   }
-  if (publish_partials(part, blockIdx.x, f2x2_fold(acc), f2_zero(), &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    double rz, unused;
-    gather_partials(part, pr.chunk_begin, pr.chunk_end, &s->counter, rz, unused);
-    if (threadIdx.x == 0) {
-      const double beta = rz / s->rz;
-      s->beta_f = (float)beta;
-      s->rz = rz;
-      s->pcg_iters += 1;
-      if (rz == 0.0 || !isfinite(rz)) s->pcg_active = 0;
-      if (!isfinite(rz)) s->nonfinite = 1;
-    }
+  const F2 sums[1] = {f2x2_fold(acc)};
+  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
+    F2 rz[1];
+    gather_pairs<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, rz);
+    if (threadIdx.x == 0) finish_beta(s, rz[0]);
   }
 }
 

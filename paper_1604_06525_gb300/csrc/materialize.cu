@@ -130,19 +130,11 @@ __global__ void __launch_bounds__(NT) k_csr_jtt(int nT, const int* __restrict__ 
     q[u] = v;
     f2_add_prod(acc, pu, v);
   }
-  if (publish_partials(part, blockIdx.x, acc, f2_zero(), &s->counter, gridDim.x)) {
-    double pq, unused;
-    gather_partials(part, 0, gridDim.x, &s->counter, pq, unused);
-    if (threadIdx.x == 0) {
-      s->pq = pq;
-      if (pq > 0.0 && isfinite(pq)) {
-        s->alpha_f = (float)(s->rz / pq);
-      } else {
-        s->alpha_f = 0.f;
-        s->pcg_active = 0;
-        if (!isfinite(pq)) s->nonfinite = 1;
-      }
-    }
+  const F2 sums[1] = {acc};
+  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, gridDim.x)) {
+    F2 pq[1];
+    gather_pairs<1>(part, 0, gridDim.x, &s->counter, pq);
+    if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
 
@@ -199,19 +191,11 @@ __global__ void __launch_bounds__(NT) k_jtj_spmv(int nT, const int* __restrict__
     q[u] = v;
     f2_add_prod(acc, pu, v);
   }
-  if (publish_partials(part, blockIdx.x, acc, f2_zero(), &s->counter, gridDim.x)) {
-    double pq, unused;
-    gather_partials(part, 0, gridDim.x, &s->counter, pq, unused);
-    if (threadIdx.x == 0) {
-      s->pq = pq;
-      if (pq > 0.0 && isfinite(pq)) {
-        s->alpha_f = (float)(s->rz / pq);
-      } else {
-        s->alpha_f = 0.f;
-        s->pcg_active = 0;
-        if (!isfinite(pq)) s->nonfinite = 1;
-      }
-    }
+  const F2 sums[1] = {acc};
+  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, gridDim.x)) {
+    F2 pq[1];
+    gather_pairs<1>(part, 0, gridDim.x, &s->counter, pq);
+    if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
 

@@ -19,12 +19,12 @@
 // on: each thread accumulates its terms as a compensated float32 pair (every
 // product split exactly by one FMA, every addition made error-free by TwoSum:
 // Ogita, Rump & Oishi's Dot2, see F2 below), warps combine the pairs in a fixed
-// shuffle order, each warp's pair becomes a float64 hi + lo, and float64 takes
-// over from there (the float64 pipe of this part is narrow, so it is kept to
-// the last levels).  Each block writes its partial to a per-chunk slot, and the
-// last block of a problem to arrive (atomic counter) sums the problem's
-// partials in chunk order in float64, so the result does not depend on block
-// scheduling.
+// shuffle order; the sums behind alpha and beta stay pairs to the end (see
+// publish_pairs), energies go on in float64 (the float64 pipe of this part is
+// narrow, so it is kept to the last levels).  Each block writes its partial to a
+// per-chunk slot, and the last block of a problem to arrive (atomic counter)
+// sums the problem's partials in chunk order, so the result does not depend on
+// block scheduling.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -67,7 +67,7 @@ struct __align__(16) Scalars {
   float alpha_f;      // alpha = rz / pq, rounded once to float
   float beta_f;       // beta  = rz' / rz
   float lambda_f;
-  float pad0;
+  float rz_hi, rz_lo; // rz as an unevaluated float32 pair (PCG loops; set with rz)
   int pcg_active;     // 0 once PCG broke down (rz == 0 or pq <= 0)
   int pcg_iters;      // completed PCG iterations in the current solve
   int accept;         // LM: the last trial step was accepted
@@ -79,7 +79,6 @@ struct __align__(16) Scalars {
   unsigned int counter;   // last-block counter
   unsigned int timeout;   // a bounded wait for a tensor copy ran out (the solve reports OPT_ERR_TIMEOUT)
   unsigned int misaligned;  // a staging area could not take tensor copies (the solve reports OPT_ERR_CUDA)
-  unsigned int pad1;
   double alpha_d;     // float64 solver: alpha = rz / pq
   double beta_d;      // float64 solver: beta  = rz' / rz
 };
@@ -266,20 +265,32 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Sum of a and b over the block; the result is valid in thread 0.
+// Sum of a and b over the block; the result is valid in thread 0.  A float64
+// addition has a latency of 64 cycles here (a shuffle level 109), so the two
+// sums share the levels: after the first one the lower half warp carries a, the
+// upper half b.
+__device__ __forceinline__ double half_sums(double a, double b) {
+  const bool up = (threadIdx.x & 16) != 0;
+  double v = up ? b : a;
+  v += __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;                       // lanes 0..15: a, lanes 16..31: b
+}
 __device__ __forceinline__ void block_sum2(double& a, double& b) {
-  __shared__ double sa[NT / 32], sb[NT / 32];
-  a = warp_sum(a);
-  b = warp_sum(b);
+  __shared__ double sab[2][NT / 32];
+  const double v = half_sums(a, b);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   __syncthreads();
-  if (l == 0) { sa[w] = a; sb[w] = b; }
+  if ((l & 15) == 0) sab[l >> 4][w] = v;
   __syncthreads();
   if (w == 0) {
-    a = l < NT / 32 ? sa[l] : 0.0;
-    b = l < NT / 32 ? sb[l] : 0.0;
-    a = warp_sum(a);
-    b = warp_sum(b);
+    constexpr int NW = NT / 32;
+    double t = l < 2 * NW ? sab[l / NW][l % NW] : 0.0;
+#pragma unroll
+    for (int o = NW / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    a = t;
+    b = __shfl_down_sync(0xffffffffu, t, NW);
   }
 }
 
@@ -383,17 +394,21 @@ __device__ __forceinline__ F2 warp_sum_f2(F2 v) {
 // across the warps; the result is valid in thread 0.  Called once per kernel
 // (its shared slots are not reused).
 __device__ __forceinline__ void block_sum2f(F2 a, F2 b, double& ra, double& rb) {
-  __shared__ double sa[NT / 32], sb[NT / 32];
+  constexpr int NW = NT / 32;
+  __shared__ double sab[2][NW];
   a = warp_sum_f2(a);
   b = warp_sum_f2(b);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) { sa[w] = f2_to_double(a); sb[w] = f2_to_double(b); }
+  if (l == 0) { sab[0][w] = f2_to_double(a); sab[1][w] = f2_to_double(b); }
   __syncthreads();
   ra = 0.0;
   rb = 0.0;
-  if (threadIdx.x == 0) {
+  if (w == 0) {
+    double t = l < 2 * NW ? sab[l / NW][l % NW] : 0.0;
 #pragma unroll
-    for (int k = 0; k < NT / 32; ++k) { ra += sa[k]; rb += sb[k]; }
+    for (int o = NW / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    ra = t;
+    rb = __shfl_down_sync(0xffffffffu, t, NW);
   }
 }
 
@@ -431,63 +446,132 @@ __device__ __forceinline__ void gather_partials(const double* part, int cb, int 
   if (threadIdx.x == 0) *counter = 0u;
 }
 
-// Four partial sums per chunk (the single-reduction PCG iteration): as
-// publish_partials / gather_partials, with slots part[4 * chunk + 0..3] (the
-// grid problems' partial buffers hold four doubles per chunk).
-__device__ __forceinline__ bool publish_partials4(double* part, int chunk, const F2 (&f)[4],
-                                                  unsigned int* counter, unsigned int nchunks) {
-  __shared__ double s4[4][NT / 32];
+// ---------------------------------------------------------------------------
+// PCG scalars: dot products carried as pairs to the end
+// ---------------------------------------------------------------------------
+// The sums behind alpha and beta (p.q, r.z, ...) stay compensated pairs across
+// the warps and the blocks too.  alpha and beta are rounded to float32 once;
+// a pair (about 47 bits) carries them to that rounding as float64 does, and the
+// float64 tail it replaces was a serial chain of every launch: 64 cycles an
+// addition, 109 a shuffle level, 560 a division, about 3,000 cycles (1.5 us)
+// from the last block's partial sums to the published scalar against about 800
+// with pairs.  Energies and the LM decision stay in float64.
+__device__ __forceinline__ F2 f2_shfl_xor_add(F2 v, int o) {
+  F2 w;
+  w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
+  w.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
+  f2_add_f2(v, w);
+  return v;
+}
+__device__ __forceinline__ F2 f2_from_double(double d) {
+  const float hi = (float)d;
+  return F2{hi, isfinite(hi) ? (float)(d - (double)hi) : 0.f};
+}
+// a / b rounded to float32 (one correction step: the quotient of the leading
+// parts plus the remainder's; as the rounded float64 quotient unless that lies
+// within 2^-20 ulp of a rounding boundary)
+__device__ __forceinline__ float f2_quot(F2 a, F2 b) {
+  const float q = __fdiv_rn(a.hi, b.hi);
+  const float r = __fadd_rn(__fmaf_rn(-q, b.hi, a.hi), __fmaf_rn(-q, b.lo, a.lo));
+  const float c = __fadd_rn(q, __fdiv_rn(r, b.hi));
+  return isfinite(c) ? c : q;
+}
+
+// Stores this chunk's N partial pairs (N = 1: every other 8-byte slot of part, N =
+// 4: all) and reports whether this block is the last of its problem to do so.
+// Must be called by every thread of the block.
+template <int N>
+__device__ __forceinline__ bool publish_pairs(double* part, int chunk, const F2 (&f)[N], unsigned int* counter,
+                                              unsigned int nchunks) {
+  static_assert(NT == 256 && (N == 1 || N == 4), "one lane per warp and sum");
+  constexpr int NW = NT / 32, ST = N == 1 ? 2 : 4;
+  __shared__ F2 sw[N][NW];
   __shared__ int s_last;
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
+  for (int k = 0; k < N; ++k) {
     const F2 v = warp_sum_f2(f[k]);
-    if (l == 0) s4[k][w] = f2_to_double(v);
+    if (l == 0) sw[k][w] = v;
   }
   __syncthreads();
-  if (threadIdx.x < 4) {
-    double a = 0.0;
+  if (w == 0) {
+    F2 v = l / NW < N ? sw[l / NW][l % NW] : f2_zero();
 #pragma unroll
-    for (int j = 0; j < NT / 32; ++j) a += s4[threadIdx.x][j];
-    __stcg(&part[4 * chunk + threadIdx.x], a);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned int prev = atomicAdd(counter, 1u);
-    s_last = (prev == nchunks - 1);
+    for (int o = NW / 2; o > 0; o >>= 1) v = f2_shfl_xor_add(v, o);
+    if (l / NW < N && l % NW == 0)
+      __stcg(reinterpret_cast<float2*>(part) + (long long)ST * chunk + l / NW, make_float2(v.hi, v.lo));
+    __syncwarp();
+    if (l == 0) {
+      __threadfence();
+      const unsigned int prev = atomicAdd(counter, 1u);
+      s_last = (prev == nchunks - 1);
+    }
   }
   __syncthreads();
   return s_last != 0;
 }
 
-// In the last block: the four sums over chunks [cb, ce) in chunk order
-// (thread-strided, then a fixed tree); valid in thread 0; resets the counter.
-__device__ __forceinline__ void gather_partials4(const double* part, int cb, int ce, unsigned int* counter,
-                                                 double (&out)[4]) {
-  __shared__ double g4[4][NT / 32];
+// In the last block: the sums over chunks [cb, ce) (thread-strided in chunk
+// order, then a fixed tree); out is valid in thread 0; resets the counter.
+template <int N>
+__device__ __forceinline__ void gather_pairs(const double* part, int cb, int ce, unsigned int* counter, F2 (&out)[N]) {
+  constexpr int NW = NT / 32, ST = N == 1 ? 2 : 4;
+  __shared__ F2 g[N][NW];
   __threadfence();
-  double a[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll 2
-  for (int c = cb + (int)threadIdx.x; c < ce; c += NT) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) a[k] += __ldcg(&part[4 * c + k]);
+  const float2* p = reinterpret_cast<const float2*>(part);
+  const int k = threadIdx.x % N;
+  F2 v = f2_zero();
+#pragma unroll 4
+  for (int c = cb + (int)threadIdx.x / N; c < ce; c += NT / N) {
+    const float2 t = __ldcg(p + (long long)ST * c + k);
+    f2_add_f2(v, F2{t.x, t.y});
   }
+#pragma unroll
+  for (int o = 16; o >= N; o >>= 1) v = f2_shfl_xor_add(v, o);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    a[k] = warp_sum(a[k]);
-    if (l == 0) g4[k][w] = a[k];
-  }
+  if (l < N) g[l][w] = v;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (w == 0) {
+    F2 t = l / NW < N ? g[l / NW][l % NW] : f2_zero();
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      out[k] = 0.0;
-      for (int j = 0; j < NT / 32; ++j) out[k] += g4[k][j];
+    for (int o = NW / 2; o > 0; o >>= 1) t = f2_shfl_xor_add(t, o);
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      out[j].hi = __shfl_sync(0xffffffffu, t.hi, j * NW);
+      out[j].lo = __shfl_sync(0xffffffffu, t.lo, j * NW);
     }
-    *counter = 0u;
+    if (l == 0) *counter = 0u;
   }
+}
+
+// alpha from the sum p.q of the last block (thread 0); p.q <= 0 or not finite
+// ends the loop.
+__device__ __forceinline__ void finish_alpha(Scalars* s, F2 pq) {
+  s->pq = f2_to_double(pq);
+  if (pq.hi > 0.f && isfinite(pq.hi)) {
+    s->alpha_f = f2_quot(F2{s->rz_hi, s->rz_lo}, pq);
+  } else {
+    s->alpha_f = 0.f;
+    s->pcg_active = 0;
+    if (!isfinite(pq.hi)) s->nonfinite = 1;
+  }
+}
+// beta from the next r.z (thread 0 of the last block of a vector update)
+__device__ __forceinline__ void finish_beta(Scalars* s, F2 rz) {
+  s->beta_f = f2_quot(rz, F2{s->rz_hi, s->rz_lo});
+  s->rz = f2_to_double(rz);
+  s->rz_hi = rz.hi;
+  s->rz_lo = rz.lo;
+  s->pcg_iters += 1;
+  if (rz.hi == 0.f || !isfinite(rz.hi)) s->pcg_active = 0;
+  if (!isfinite(rz.hi)) s->nonfinite = 1;
+}
+// r.z of PCGInit
+__device__ __forceinline__ void set_rz(Scalars* s, double rz) {
+  const F2 t = f2_from_double(rz);
+  s->rz = rz;
+  s->rz_hi = t.hi;
+  s->rz_lo = t.lo;
 }
 
 __device__ __forceinline__ bool finite_d(double v) { return isfinite(v); }
