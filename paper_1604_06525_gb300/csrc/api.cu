@@ -353,12 +353,43 @@ bool use_fused(const opt_problem* pb, const opt_solve_params& p) {
          pb->hg.zb != nullptr;
 }
 
+// Plans the resident PCG loop of a GN (lm = 0) / LM solve and allocates its
+// slots and records once (outside any capture).
+opt_status resident_prepare(opt_problem* pb, int lm) {
+  if (pb->rplanned[lm]) return OPT_OK;
+  const bool grid = is_grid(pb);
+  ResidentPlan rp;
+  if (grid) {
+    const long long n = (long long)pb->ntiles * pb->hg.tw * TH;
+    // (records are indexed like the planes: a sparse mask on a huge image is left to the tiled kernels)
+    rp = n > (1 << 22) || pb->plane > (1 << 24) ? ResidentPlan{} : resident_plan(pb->kind, (int)n, pb->plane, lm, nullptr);
+  } else {
+    rp = resident_plan(pb->kind, pb->V, pb->plane, lm, pb->kind != K_VOLUME && pb->hm.sym ? pb->h_orow.data() : nullptr);
+  }
+  if (rp.blocks > 0) {
+    if (!pb->d_rsync) CKS(dalloc(pb, &pb->d_rsync, 1));
+    if (!pb->d_rrec) CKS(dalloc(pb, &pb->d_rrec, resident_records(pb->kind, pb->plane)));
+    CK(cudaStreamSynchronize(nullptr));
+  }
+  pb->rplan[lm] = rp;
+  pb->rplanned[lm] = true;
+  return OPT_OK;
+}
+
+// The resident loop serves the two-pass iteration (pcg_form 0, and form 1 on
+// problems without single-reduction buffers) of matrix-free solves.
+bool use_resident(const opt_problem* pb, const opt_solve_params& p, bool lm) {
+  return !p.materialized && p.inner > 0 && !use_fused(pb, p) && !use_persistent(pb, p) &&
+         pb->rplan[lm ? 1 : 0].blocks > 0;
+}
+
 opt_status enqueue_solve(opt_problem* pb, const opt_solve_params& p, bool lm, cudaStream_t st) {
   const float dmin = (float)p.diag_min, dmax = (float)p.diag_max;
   CKS(copy_planes_in(pb, pb->x, pb->user_x, pb->nx, st));
   k_reset<<<1, 32, 0, st>>>(pb->d_s, 1, lm ? p.lambda0 : 0.0);
   const bool fused = use_fused(pb, p) && p.inner > 0;
   const bool coop = !fused && use_persistent(pb, p);
+  const bool resident = use_resident(pb, p, lm);
   if (coop) CK(cudaMemsetAsync(pb->d_gbar, 0, sizeof(GridBarrier), st));
   for (int k = 0; k < p.outer; ++k) {
     // from the second outer iteration on, cos / sin of theta come from the
@@ -375,6 +406,10 @@ opt_status enqueue_solve(opt_problem* pb, const opt_solve_params& p, bool lm, cu
       // mid-count); its timeout flag accumulates over the solve
       CK(cudaMemsetAsync(&pb->d_gbar->count, 0, sizeof(unsigned int), st));
       CK(launch_grid_pcg_coop(grid_launch(pb, st), pb->d_gbar, 0, p.inner));
+    } else if (resident) {
+      const ResidentPlan& rp = pb->rplan[lm ? 1 : 0];
+      CK(is_grid(pb) ? launch_resident_grid(pb->kind, pb->dg, pb->d_tiles, pb->d_rsync, rp, pb->d_rrec, p.inner, st)
+                     : launch_resident_graph(pb->kind, pb->dm, pb->d_rsync, rp, pb->d_rrec, p.inner, st));
     } else {
       for (int i = 0; i < p.inner; ++i) {
         if (p.materialized) csr_apply(pb, st, i, p.materialized);
@@ -429,6 +464,7 @@ opt_status run_solve(opt_problem* pb, const opt_solve_params* prm_in, opt_report
   cudaStream_t st = (cudaStream_t)p.stream;
   CK(cudaStreamSynchronize(st));
   CKS(ensure_ehist(pb, p.outer + 1));
+  CKS(resident_prepare(pb, lm ? 1 : 0));
   set_flags(pb, lm ? 1 : 0, p.use_precond, pb->d_Ehist);
   CKS(upload_desc(pb, st));
   if (p.use_graph) {
@@ -485,7 +521,13 @@ opt_status run_solve(opt_problem* pb, const opt_solve_params* prm_in, opt_report
     CK(cudaMemcpy(&gb, pb->d_gbar, sizeof(gb), cudaMemcpyDeviceToHost));
     if (gb.timeout) return OPT_ERR_TIMEOUT;
   }
-  if (s.timeout) return OPT_ERR_TIMEOUT;
+  if (s.timeout) {
+    if (pb->d_rsync) {
+      // blocks gave up at different exchanges: back to a clean counter
+      CK(cudaMemset(pb->d_rsync, 0, sizeof(ResidentSync)));
+    }
+    return OPT_ERR_TIMEOUT;
+  }
   if (s.misaligned) return OPT_ERR_CUDA;
   if (s.nonfinite) return OPT_ERR_NUMERIC;
   return OPT_OK;
@@ -1068,6 +1110,7 @@ static opt_status create_graph_impl(const opt_graph_desc* d, int D, opt_problem*
   for (int k = 0; k < NXg; ++k) q->user_x[k] = ux[k];
   q->h_e0 = e0;
   q->h_e1 = e1;
+  q->h_orow = orow;
   q->h_hpix = hpix;
 
   MeshProb& g = q->hm;

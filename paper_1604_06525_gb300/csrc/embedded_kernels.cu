@@ -21,87 +21,12 @@
 // displacement rows (w_reg * degree + w_fit, planned) and one per matrix
 // entry.
 #include "opt_internal.cuh"
+#include "embedded_algebra.cuh"
 #include "opt_launch.h"
 
 namespace optgb {
 
 namespace {
-
-constexpr int NXE = 12;   // unknowns per vertex
-constexpr int NME = 10;   // distinct-diagonal planes
-constexpr int KBE = 6;    // neighbour indices fetched ahead per vertex (icosphere degree 5 / 6)
-
-// Visits the out-edge targets e1[o0 .. o1) (or in-edge sources) of a vertex:
-// the first KBE indices are loaded together before any neighbour record is
-// needed, the rest of a longer row one by one.
-template <typename F>
-__device__ __forceinline__ void for_neighbours(const int* __restrict__ idx, int o0, int o1, F&& f) {
-  int j[KBE];
-#pragma unroll
-  for (int t = 0; t < KBE; ++t) j[t] = o0 + t < o1 ? __ldg(idx + o0 + t) : 0;
-#pragma unroll
-  for (int t = 0; t < KBE; ++t)
-    if (o0 + t < o1) f(j[t]);
-  for (int k = o0 + KBE; k < o1; ++k) f(__ldg(idx + k));
-}
-
-__device__ __forceinline__ int mplane_e(int c) { return c < 3 ? 0 : c - 2; }
-
-__device__ __forceinline__ int handle_of_e(const MeshProb& pr, int v) {
-  const int t = v / VT;
-  for (int h = pr.hbeg[t]; h < pr.hbeg[t + 1]; ++h)
-    if (pr.hpix[h] == v) return h;
-  return -1;
-}
-
-__device__ __forceinline__ void load12(const float4* rec, int v, float (&o)[NXE]) {
-  const float4 a = rec[3 * v], b = rec[3 * v + 1], c = rec[3 * v + 2];
-  o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
-  o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
-  o[8] = c.x; o[9] = c.y; o[10] = c.z; o[11] = c.w;
-}
-__device__ __forceinline__ void store12(float4* rec, int v, const float (&o)[NXE]) {
-  rec[3 * v] = make_float4(o[0], o[1], o[2], o[3]);
-  rec[3 * v + 1] = make_float4(o[4], o[5], o[6], o[7]);
-  rec[3 * v + 2] = make_float4(o[8], o[9], o[10], o[11]);
-}
-
-// The six constraint values (c0.c1, c0.c2, c1.c2, c0.c0 - 1, c1.c1 - 1,
-// c2.c2 - 1) of the matrix m[9] (row-major), unscaled.
-__device__ __forceinline__ void col_constraints(const float* m, float (&f)[6]) {
-  float d01 = 0.f, d02 = 0.f, d12 = 0.f, d00 = 0.f, d11 = 0.f, d22 = 0.f;
-#pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    const float c0 = m[3 * r], c1 = m[3 * r + 1], c2 = m[3 * r + 2];
-    d01 += c0 * c1; d02 += c0 * c2; d12 += c1 * c2;
-    d00 += c0 * c0; d11 += c1 * c1; d22 += c2 * c2;
-  }
-  f[0] = d01; f[1] = d02; f[2] = d12; f[3] = d00 - 1.f; f[4] = d11 - 1.f; f[5] = d22 - 1.f;
-}
-
-// Linearised constraints J_rot t of a matrix direction t[9] at m[9], unscaled.
-__device__ __forceinline__ void col_constraints_lin(const float* m, const float* t, float (&f)[6]) {
-  float a01 = 0.f, a02 = 0.f, a12 = 0.f, a00 = 0.f, a11 = 0.f, a22 = 0.f;
-#pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    const float c0 = m[3 * r], c1 = m[3 * r + 1], c2 = m[3 * r + 2];
-    const float t0 = t[3 * r], t1 = t[3 * r + 1], t2 = t[3 * r + 2];
-    a01 += c1 * t0 + c0 * t1; a02 += c2 * t0 + c0 * t2; a12 += c2 * t1 + c1 * t2;
-    a00 += c0 * t0; a11 += c1 * t1; a22 += c2 * t2;
-  }
-  f[0] = a01; f[1] = a02; f[2] = a12; f[3] = 2.f * a00; f[4] = 2.f * a11; f[5] = 2.f * a22;
-}
-
-// out[9] += J_rot^T y for the six constraint values y (unscaled).
-__device__ __forceinline__ void col_constraints_t(const float* m, const float (&y)[6], float* out) {
-#pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    const float c0 = m[3 * r], c1 = m[3 * r + 1], c2 = m[3 * r + 2];
-    out[3 * r] += c1 * y[0] + c2 * y[1] + 2.f * c0 * y[3];
-    out[3 * r + 1] += c0 * y[0] + c2 * y[2] + 2.f * c1 * y[4];
-    out[3 * r + 2] += c0 * y[1] + c1 * y[2] + 2.f * c2 * y[5];
-  }
-}
 
 // ---------------------------------------------------------------------------
 // PCGInit
@@ -152,7 +77,7 @@ __global__ void __launch_bounds__(NT, ED_INIT_MIN_BLOCKS) k_ed_init_pull(const M
 #pragma unroll
     for (int k = 0; k < 9; ++k) dR[k] = 0.f;
     float e = 0.f;
-    const int h = handle_of_e(pr, i);
+    const int h = handle_of(pr, i);
     if (h >= 0) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -161,7 +86,7 @@ __global__ void __launch_bounds__(NT, ED_INIT_MIN_BLOCKS) k_ed_init_pull(const M
         e += f * f;
       }
     }
-    for_neighbours(pr.e1, pr.orow[i], pr.orow[i + 1], [&](int j) {
+    for_list(pr.e1, pr.orow[i], pr.orow[i + 1], [&](int j) {
       const float4 dj = pr.vrec[3 * j];
       const float4 uj = __ldg(pr.grec + j);
       const float wv[3] = {ui.x - uj.x, ui.y - uj.y, ui.z - uj.z};
@@ -181,7 +106,7 @@ __global__ void __launch_bounds__(NT, ED_INIT_MIN_BLOCKS) k_ed_init_pull(const M
         dR[c] += wc2; dR[3 + c] += wc2; dR[6 + c] += wc2;
       }
     });
-    for_neighbours(pr.isrc, pr.irow[i], pr.irow[i + 1], [&](int j) {
+    for_list(pr.isrc, pr.irow[i], pr.irow[i + 1], [&](int j) {
       float xj[NXE];
       load12(pr.vrec, j, xj);
       const float4 uj = __ldg(pr.grec + j);
@@ -301,57 +226,19 @@ __global__ void __launch_bounds__(NT) k_ed_apply_pull(const MeshProb* __restrict
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;
   const long long pl = pr.Vp;
-  const float wreg = pr.w_reg;
   const float lam = pr.lm ? s->lambda_f : 0.0f;
   F2 acc = f2_zero();
   for (int i = ch.begin + threadIdx.x; i < ch.end; i += NT) {
     float pi[NXE], q[NXE];
     load12(pr.vrec, i, pi);
     const float4 ui = __ldg(pr.grec + i);
+    float f[3] = {0.f, 0.f, 0.f}, g[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    ed_gather(pr, i, pr.e1, pr.orow[i], pr.orow[i + 1], pi, ui,
+              [&](int j, float (&pj)[NXE]) { load12(pr.vrec, j, pj); }, f, g);
+    ed_rows(pr, i, pi, f, g, handle_of(pr, i) >= 0, q);
+    if (pr.lm) {
 #pragma unroll
-    for (int c = 0; c < NXE; ++c) q[c] = pr.lm ? lam * pr.dc[mplane_e(c) * pl + i] * pi[c] : 0.f;
-    if (handle_of_e(pr, i) >= 0) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) q[c] += pr.w_fit * pi[c];
-    }
-    // (plain loops: prefetching the indices as PCGInit does costs this
-    // kernel occupancy -- 100 instead of 80 registers -- and was measured slower)
-    for (int k = pr.orow[i]; k < pr.orow[i + 1]; ++k) {
-      const int j = pr.e1[k];
-      const float4 pj = pr.vrec[3 * j];
-      const float4 uj = __ldg(pr.grec + j);
-      const float wv[3] = {ui.x - uj.x, ui.y - uj.y, ui.z - uj.z};
-      const float pd[3] = {pi[0] - pj.x, pi[1] - pj.y, pi[2] - pj.z};
-#pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        // J p / s_w of row r; J^T (J p) carries s_w^2 = w_reg
-        const float jp = pd[r] - (pi[3 + 3 * r] * wv[0] + pi[4 + 3 * r] * wv[1] + pi[5 + 3 * r] * wv[2]);
-        q[r] += wreg * jp;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) q[3 + 3 * r + c] -= wreg * wv[c] * jp;
-      }
-    }
-    for (int k = pr.irow[i]; k < pr.irow[i + 1]; ++k) {
-      const int j = pr.isrc[k];
-      float pj[NXE];
-      load12(pr.vrec, j, pj);
-      const float4 uj = __ldg(pr.grec + j);
-      const float wv[3] = {uj.x - ui.x, uj.y - ui.y, uj.z - ui.z};
-#pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        const float jp = (pj[r] - pi[r]) - (pj[3 + 3 * r] * wv[0] + pj[4 + 3 * r] * wv[1] + pj[5 + 3 * r] * wv[2]);
-        q[r] -= wreg * jp;
-      }
-    }
-    {
-      float m9[9];
-#pragma unroll
-      for (int k = 0; k < 9; ++k) m9[k] = pr.x[(3 + k) * pl + i];
-      float y[6];
-      col_constraints_lin(m9, pi + 3, y);
-#pragma unroll
-      for (int t = 0; t < 6; ++t) y[t] *= pr.w_rot;
-      col_constraints_t(m9, y, q + 3);
+      for (int c = 0; c < NXE; ++c) q[c] = fmaf(__fmul_rn(lam, pr.dc[mplane_e(c) * pl + i]), pi[c], q[c]);
     }
 #pragma unroll
     for (int c = 0; c < NXE; ++c) {
@@ -459,7 +346,7 @@ __global__ void __launch_bounds__(NT) k_ed_energy(const MeshProb* __restrict__ p
       di[c] = mode == 1 ? pr.d[c * pl + i] : 0.f;
     }
     const float ui[3] = {pr.U[i], pr.U[pl + i], pr.U[2 * pl + i]};
-    const int h = handle_of_e(pr, i);
+    const int h = handle_of(pr, i);
     if (h >= 0) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {

@@ -14,18 +14,12 @@
 // vertex for the geometry, grec[v] = (U_x, U_y, cos theta, sin theta), and
 // one for the 3-vector, vrec[v] = (x or p: dx, dy, theta, 0).
 #include "opt_internal.cuh"
+#include "graph2d_algebra.cuh"
 #include "opt_launch.h"
 
 namespace optgb {
 
 namespace {
-
-__device__ __forceinline__ int handle_of2(const MeshProb& pr, int v) {
-  const int t = v / VT;
-  for (int h = pr.hbeg[t]; h < pr.hbeg[t + 1]; ++h)
-    if (pr.hpix[h] == v) return h;
-  return -1;
-}
 
 __device__ __forceinline__ float4 ldg4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
 __device__ __forceinline__ float cc4(const float4& a, int k) {
@@ -72,7 +66,7 @@ __global__ void __launch_bounds__(NT) k_wg_init_pull(const MeshProb* __restrict_
     const float4 xi = pr.vrec[i];
     const float4 gi = __ldg(pr.grec + i);
     float g0 = 0.f, g1 = 0.f, gt = 0.f, dt = 0.f, e = 0.f;
-    const int h = handle_of2(pr, i);
+    const int h = handle_of(pr, i);
     if (h >= 0) {
       const float f0 = pr.s_f * (xi.x - pr.htgt[2 * h]), f1 = pr.s_f * (xi.y - pr.htgt[2 * h + 1]);
       g0 += pr.s_f * f0;
@@ -199,43 +193,23 @@ __global__ void __launch_bounds__(NT) k_wg_apply_pull(const MeshProb* __restrict
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;
   const long long pl = pr.Vp;
-  const float sw = pr.s_w;
   const float lam = pr.lm ? s->lambda_f : 0.0f;
   F2 acc = f2_zero();
   for (int i = ch.begin + threadIdx.x; i < ch.end; i += NT) {
     const float4 pi = pr.vrec[i];
     const float4 gi = __ldg(pr.grec + i);
-    float q0 = 0.f, q1 = 0.f, qt = 0.f;
+    float f[3] = {0.f, 0.f, 0.f}, q[3];
+    wg_gather(pr, i, pr.e1, pr.orow[i], pr.orow[i + 1], pi, gi, [&](int j) { return pr.vrec[j]; }, f);
+    const float p3[3] = {pi.x, pi.y, pi.z};
+    wg_rows(pr, f, p3, handle_of(pr, i) >= 0, q);
     if (pr.lm) {
-      const float dd = lam * pr.dc[i], dt = lam * pr.dc[pl + i];
-      q0 = dd * pi.x; q1 = dd * pi.y; qt = dt * pi.z;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) q[c] = fmaf(__fmul_rn(lam, pr.dc[(c == 2 ? pl : 0) + i]), p3[c], q[c]);
     }
-    if (handle_of2(pr, i) >= 0) { q0 += pr.w_fit * pi.x; q1 += pr.w_fit * pi.y; }
-    for (int k = pr.orow[i]; k < pr.orow[i + 1]; ++k) {
-      const int j = pr.e1[k];
-      const float4 pj = pr.vrec[j];
-      const float4 gj = __ldg(pr.grec + j);
-      const float vx = gi.x - gj.x, vy = gi.y - gj.y;
-      const float Gx = fmaf(gi.w, vx, gi.z * vy), Gy = fmaf(gi.w, vy, -gi.z * vx);
-      // J_e p / s_w = (p_a,d - p_b,d) + G p_a,t
-      const float j0 = fmaf(Gx, pi.z, pi.x - pj.x), j1 = fmaf(Gy, pi.z, pi.y - pj.y);
-      q0 += sw * sw * j0;
-      q1 += sw * sw * j1;
-      qt += sw * sw * (Gx * j0 + Gy * j1);
-    }
-    for (int k = pr.irow[i]; k < pr.irow[i + 1]; ++k) {
-      const int j = pr.isrc[k];
-      const float4 pj = pr.vrec[j];
-      const float4 gj = __ldg(pr.grec + j);
-      const float vx = gj.x - gi.x, vy = gj.y - gi.y;
-      const float Gx = fmaf(gj.w, vx, gj.z * vy), Gy = fmaf(gj.w, vy, -gj.z * vx);
-      q0 -= sw * sw * fmaf(Gx, pj.z, pj.x - pi.x);
-      q1 -= sw * sw * fmaf(Gy, pj.z, pj.y - pi.y);
-    }
-    pr.q[i] = q0; pr.q[pl + i] = q1; pr.q[2 * pl + i] = qt;
-    f2_add_prod(acc, pi.x, q0);
-    f2_add_prod(acc, pi.y, q1);
-    f2_add_prod(acc, pi.z, qt);
+    pr.q[i] = q[0]; pr.q[pl + i] = q[1]; pr.q[2 * pl + i] = q[2];
+    f2_add_prod(acc, pi.x, q[0]);
+    f2_add_prod(acc, pi.y, q[1]);
+    f2_add_prod(acc, pi.z, q[2]);
   }
   pdl_trigger();
   const F2 sums[1] = {acc};
@@ -312,7 +286,7 @@ __global__ void __launch_bounds__(NT) k_wg_energy_v(const MeshProb* __restrict__
   const long long pl = pr.Vp;
   F2 e = f2_zero();
   for (int v = ch.begin + threadIdx.x; v < ch.end; v += NT) {
-    const int h = handle_of2(pr, v);
+    const int h = handle_of(pr, v);
     if (h < 0) continue;
     float ev = 0.f;
 #pragma unroll

@@ -34,6 +34,7 @@
 #include <mutex>
 
 #include "opt_internal.cuh"
+#include "grid_algebra.cuh"
 #include "opt_launch.h"
 
 namespace optgb {
@@ -245,13 +246,13 @@ __device__ __forceinline__ void warp_cell_store(WarpApplyStage& st, int hy, int 
   float px = 0.f, py = 0.f, pt = 0.f, cs = 1.f, sn = 0.f;
   if (c.inb) {
     if (update) {
-      px = c.m0 * c.r0;
-      py = c.m0 * c.r1;
-      pt = c.m1 * c.r2;
+      px = __fmul_rn(c.m0, c.r0);
+      py = __fmul_rn(c.m0, c.r1);
+      pt = __fmul_rn(c.m1, c.r2);
       if (use_beta) {
-        px += beta * c.p0;
-        py += beta * c.p1;
-        pt += beta * c.p2;
+        px = __fmaf_rn(beta, c.p0, px);
+        py = __fmaf_rn(beta, c.p1, py);
+        pt = __fmaf_rn(beta, c.p2, pt);
       }
       if (i_owned >= 0) {
         const long long pl = pr.plane;
@@ -288,7 +289,7 @@ __global__ void __launch_bounds__(NT, 3) k_warp_apply(const GridProb* __restrict
   __shared__ WarpApplyStage st;
   const long long pl = pr.plane;
   const int P = pr.P, W = pr.W, H = pr.H;
-  const float sw = pr.s_w, wfit = pr.w_fit;
+  const float wreg = pr.w_reg, wfit = pr.w_fit;
   const float beta = s->beta_f;
   const int use_beta = beta != 0.0f;
   const float lam = pr.lm ? s->lambda_f : 0.0f;
@@ -322,40 +323,26 @@ __global__ void __launch_bounds__(NT, 3) k_warp_apply(const GridProb* __restrict
       const float pxi = st.a[ly][lx], pyi = st.b[ly][lx], pti = st.t[ly][lx];
       float qx = 0.f, qy = 0.f, qt = 0.f;
       if (st.v[ly][lx]) {
-        const float ci = st.cs[ly][lx], si = st.sn[ly][lx];
-        const float uxi = st.ux[ly][lx], uyi = st.uy[ly][lx];
+        auto pix = [&](int y, int x) {
+          return WarpPix{st.a[y][x], st.b[y][x], st.t[y][x], st.cs[y][x], st.sn[y][x], st.ux[y][x], st.uy[y][x]};
+        };
+        const WarpPix own = pix(ly, lx);
+        // left, right, above, below: the order of the 128-pixel-tile kernels
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const int nx = lx + dx4(k), ny = ly + dy4(k);
-          if (!st.v[ny][nx]) continue;
-          const float vx = uxi - st.ux[ny][nx], vy = uyi - st.uy[ny][nx];
-          const float pxj = st.a[ny][nx], pyj = st.b[ny][nx], ptj = st.t[ny][nx];
-          // own residual row: J p = s_w[(p_i - p_j) - R'(t_i) v p_t,i]
-          const float gx_ = -sw * (-si * vx - ci * vy);   // dr/dtheta_i
-          const float gy_ = -sw * (ci * vx - si * vy);
-          const float jpx = sw * (pxi - pxj) + gx_ * pti;
-          const float jpy = sw * (pyi - pyj) + gy_ * pti;
-          qx += sw * jpx;
-          qy += sw * jpy;
-          qt += gx_ * jpx + gy_ * jpy;
-          // incoming residual row (centre j, v' = -v): d/dd_i = -s_w I
-          const float cj = st.cs[ny][nx], sj = st.sn[ny][nx];
-          const float hx_ = -sw * (-sj * -vx - cj * -vy);
-          const float hy_ = -sw * (cj * -vx - sj * -vy);
-          const float kpx = sw * (pxj - pxi) + hx_ * ptj;
-          const float kpy = sw * (pyj - pyi) + hy_ * ptj;
-          qx -= sw * kpx;
-          qy -= sw * kpy;
+          const int nx = lx + (k == 0 ? -1 : (k == 1 ? 1 : 0)), ny = ly + (k == 2 ? -1 : (k == 3 ? 1 : 0));
+          if (st.v[ny][nx]) warp_pair(own, pix(ny, nx), qx, qy, qt);
         }
+        qx = __fmul_rn(wreg, qx); qy = __fmul_rn(wreg, qy); qt = __fmul_rn(wreg, qt);
         const int tid_ = tile_id(pr, tcur);
         for (int h = pr.hbeg[tid_]; h < pr.hbeg[tid_ + 1]; ++h) {
-          if (pr.hpix[h] == (int)i) { qx += wfit * pxi; qy += wfit * pyi; }
+          if (pr.hpix[h] == (int)i) { qx = __fmaf_rn(wfit, pxi, qx); qy = __fmaf_rn(wfit, pyi, qy); }
         }
         if (pr.lm) {
-          const float dd = pr.dc[i], dt = pr.dc[pl + i];
-          qx += lam * dd * pxi;
-          qy += lam * dd * pyi;
-          qt += lam * dt * pti;
+          const float dd = __fmul_rn(lam, pr.dc[i]), dt = __fmul_rn(lam, pr.dc[pl + i]);
+          qx = __fmaf_rn(dd, pxi, qx);
+          qy = __fmaf_rn(dd, pyi, qy);
+          qt = __fmaf_rn(dt, pti, qt);
         }
       }
       pr.q[i] = qx; pr.q[pl + i] = qy; pr.q[2 * pl + i] = qt;
@@ -1975,8 +1962,8 @@ __device__ __forceinline__ void pois_cell_store(PoisApplyStage& st, int hy, int 
   if (c.inb && c.f == 2) {   // fixed pixels carry no unknown: p = 0 there
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      pv[k] = update ? c.m * c.r[k] : c.p[k];
-      if (update && use_beta) pv[k] += beta * c.p[k];
+      pv[k] = update ? __fmul_rn(c.m, c.r[k]) : c.p[k];
+      if (update && use_beta) pv[k] = __fmaf_rn(beta, c.p[k], pv[k]);
     }
   }
   if (update && c.inb && i_owned >= 0) {
@@ -2033,19 +2020,17 @@ __global__ void __launch_bounds__(NT, 3) k_poisson_apply(const GridProb* __restr
       const int lx = tx + 1, ly = ty + 1;
       float q[4] = {0.f, 0.f, 0.f, 0.f};
       if (st.f[ly][lx] == 2) {
+        float S = 0.f;                               // diag(J^T J): 2 per free, 1 per fixed neighbour
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int nx = lx + dx4(k), ny = ly + dy4(k);
-          const unsigned char fj = st.f[ny][nx];
-          if (!fj) continue;
-          const float w = fj == 2 ? 2.0f : 1.0f;   // own + (free neighbour) incoming
+        for (int k = 0; k < 4; ++k) S += (float)st.f[ly + dy4(k)][lx + dx4(k)];
 #pragma unroll
-          for (int c = 0; c < 4; ++c) q[c] += w * (st.p[c][ly][lx] - st.p[c][ny][nx]);
-        }
+        for (int c = 0; c < 4; ++c)
+          q[c] = pois_row(S, st.p[c][ly][lx], st.p[c][ly][lx - 1], st.p[c][ly][lx + 1], st.p[c][ly - 1][lx],
+                          st.p[c][ly + 1][lx]);
         if (pr.lm) {
-          const float dd = lam * pr.dc[i];
+          const float dd = __fmul_rn(lam, pr.dc[i]);
 #pragma unroll
-          for (int c = 0; c < 4; ++c) q[c] += dd * st.p[c][ly][lx];
+          for (int c = 0; c < 4; ++c) q[c] = __fmaf_rn(dd, st.p[c][ly][lx], q[c]);
         }
       }
 #pragma unroll
@@ -2178,18 +2163,18 @@ __device__ __forceinline__ void pois_dir_quad(const PlaneT* raw, const unsigned 
 
 // applyJTJ stencil: with the directions zero off the free pixels, every
 // neighbour term w_j p_j is 2 p_j, so per pack and channel
-// S p_i - 2 (p_L + (p_R + (p_U + p_D))) (the same roundings as the weighted
-// sum: scaling by 2 is exact).  O / U / D swizzled, L / R as in the init.
+// S p_i - 2 (p_L + (p_R + (p_U + p_D))), the product and the difference rounded
+// once (scaling by 2 is exact).  O / U / D swizzled, L / R as in the init.
 __device__ __forceinline__ void pois_core_apply(const float4 (&O)[4], const float4 (&U)[4], const float4 (&D)[4],
                                                 const float (&L)[4], const float (&R)[4], float2 SA, float2 SB,
                                                 float2 (&outA)[4], float2 (&outB)[4]) {
-  const float2 two = make_float2(2.f, 2.f);
+  const float2 two = make_float2(-2.f, -2.f);
 #pragma unroll
   for (int ch = 0; ch < 4; ++ch) {
     const float2 nA = add2(make_float2(L[ch], O[ch].z), add2(hi2(O[ch]), add2(lo2(U[ch]), lo2(D[ch]))));
     const float2 nB = add2(lo2(O[ch]), add2(make_float2(O[ch].y, R[ch]), add2(hi2(U[ch]), hi2(D[ch]))));
-    outA[ch] = sub2(mul2(SA, lo2(O[ch])), mul2(two, nA));
-    outB[ch] = sub2(mul2(SB, hi2(O[ch])), mul2(two, nB));
+    outA[ch] = fma2(SA, lo2(O[ch]), mul2(two, nA));
+    outB[ch] = fma2(SB, hi2(O[ch]), mul2(two, nB));
   }
 }
 

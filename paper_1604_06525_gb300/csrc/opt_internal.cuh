@@ -257,6 +257,33 @@ __device__ __forceinline__ bool grid_sync(GridBarrier* gb, unsigned int expected
 }
 
 // ---------------------------------------------------------------------------
+// resident PCG loop (resident.cu)
+// ---------------------------------------------------------------------------
+constexpr int RES_MAX_BLOCKS = 160;
+constexpr int RES_LANES = 4;          // threads per vertex where a block has few of them
+constexpr int RES_CLUSTER = 16;       // blocks of the one-cluster form, at most
+// RES_D, RES_DC, RES_LIST: kept in shared memory; RES_Z: see Records (resident.cu)
+enum ResidentFlags : int { RES_D = 1, RES_DC = 2, RES_LIST = 4, RES_Z = 8 };
+// Exchange counter and slots of one problem (zeroed before the first launch, and
+// again after a timeout).
+struct ResidentSync {
+  unsigned int counter;         // arrivals, ever growing
+  unsigned int pad0[31];
+  unsigned int count;           // the counter's value between launches
+  unsigned int pad1[31];
+  unsigned long long slot[2][RES_MAX_BLOCKS];
+};
+struct ResidentPlan {
+  int n, per, blocks;           // units, units per block; blocks = 0: not available
+  int smem;                     // dynamic shared memory per block
+  int flags;
+  int cluster;                  // 1: one cluster, 0: cooperative launch over the device
+  int slots;                    // graphs: table entries for edges that leave a block (0: no table)
+  int lanes;                    // graphs: threads per vertex
+  long long plane;              // plane stride
+};
+
+// ---------------------------------------------------------------------------
 // reductions
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double warp_sum(double v) {

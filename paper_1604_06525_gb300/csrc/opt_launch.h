@@ -79,6 +79,16 @@ cudaError_t launch_staging_selftest(int complete, unsigned long long limit_ns, i
 cudaError_t launch_barrier_selftest(GridBarrier* gb, int nblocks, unsigned int expected, int rounds,
                                     unsigned long long limit_ns, cudaStream_t st);
 
+// resident.cu: the PCG loop of one outer iteration in one launch with the state
+// on chip.  orow (graphs; NULL for voxel grids): host copy of the CSR rows.
+// rec: resident_records() float4.
+ResidentPlan resident_plan(int kind, int n, long long plane, int lm, const int* orow);
+size_t resident_records(int kind, long long plane);
+cudaError_t launch_resident_grid(int kind, const GridProb* probs, const int* tiles, ResidentSync* sync,
+                                 const ResidentPlan& rp, float4* rec, int inner, cudaStream_t st);
+cudaError_t launch_resident_graph(int kind, const MeshProb* probs, ResidentSync* sync, const ResidentPlan& rp,
+                                  float4* rec, int inner, cudaStream_t st);
+
 // graph_kernels.cu
 void launch_mesh_init(const MeshLaunch& L, int k_outer, float dmin, float dmax);
 void launch_mesh_apply(const MeshLaunch& L, const float* p_override, int par, int update);

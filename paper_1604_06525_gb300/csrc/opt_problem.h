@@ -74,6 +74,7 @@ struct opt_problem {
   std::vector<unsigned char> h_mask;    // grid mask (empty = none)
   std::vector<int> h_hpix;              // grid handles (pitched index) / mesh handles (vertex)
   std::vector<int> h_e0, h_e1;          // sorted edges (internal vertex order)
+  std::vector<int> h_orow;              // their CSR rows
   int* d_perm = nullptr;                // graphs: internal vertex k is the caller's vertex d_perm[k]
   CsrJ csr;
   // common
@@ -97,6 +98,12 @@ struct opt_problem {
   // blocks that can be resident at once (0 = not available)
   optgb::GridBarrier* d_gbar = nullptr;
   int coop_cap = 0;
+  // resident PCG loop: plans of a GN and an LM solve (made at the first solve
+  // that may take it), exchange slots, direction records
+  optgb::ResidentPlan rplan[2] = {};
+  bool rplanned[2] = {false, false};
+  optgb::ResidentSync* d_rsync = nullptr;
+  float4* d_rrec = nullptr;
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t gexec = nullptr;
   std::vector<double> gkey;
@@ -118,12 +125,13 @@ struct opt_problem {
     swap(tile_w, o.tile_w); swap(has_grid_desc, o.has_grid_desc); swap(grid_desc, o.grid_desc);
     swap(h_tiles, o.h_tiles); swap(h_chunks, o.h_chunks); swap(h_vch, o.h_vch); swap(h_ech, o.h_ech);
     swap(h_tch, o.h_tch);
-    swap(h_mask, o.h_mask); swap(h_hpix, o.h_hpix); swap(h_e0, o.h_e0); swap(h_e1, o.h_e1);
+    swap(h_mask, o.h_mask); swap(h_hpix, o.h_hpix); swap(h_e0, o.h_e0); swap(h_e1, o.h_e1); swap(h_orow, o.h_orow);
     swap(d_perm, o.d_perm); swap(csr, o.csr);
     swap(d_part, o.d_part); swap(d_s, o.d_s); swap(d_Ehist, o.d_Ehist); swap(Ehist_cap, o.Ehist_cap);
     swap(user_x, o.user_x); swap(d_tmp, o.d_tmp); swap(d_jtf, o.d_jtf); swap(d_diag, o.d_diag);
     swap(x, o.x); swap(pbuf, o.pbuf); swap(dvec, o.dvec); swap(rvec, o.rvec); swap(qvec, o.qvec);
     swap(allocs, o.allocs); swap(pooled, o.pooled); swap(pcg_par, o.pcg_par);
+    swap(rplan, o.rplan); swap(rplanned, o.rplanned); swap(d_rsync, o.d_rsync); swap(d_rrec, o.d_rrec);
     swap(d_gbar, o.d_gbar); swap(coop_cap, o.coop_cap); swap(cap_stream, o.cap_stream);
     swap(gexec, o.gexec); swap(gkey, o.gkey); swap(ev0, o.ev0); swap(ev1, o.ev1);
   }
