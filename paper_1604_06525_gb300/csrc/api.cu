@@ -367,7 +367,10 @@ opt_status resident_prepare(opt_problem* pb, int lm) {
     rp = resident_plan(pb->kind, pb->V, pb->plane, lm, pb->kind != K_VOLUME && pb->hm.sym ? pb->h_orow.data() : nullptr);
   }
   if (rp.blocks > 0) {
-    if (!pb->d_rsync) CKS(dalloc(pb, &pb->d_rsync, 1));
+    if (!pb->d_rsync) {
+      CKS(dalloc(pb, &pb->d_rsync, 1));
+      CK(cudaMemsetAsync(pb->d_rsync->slot, 0xff, sizeof(pb->d_rsync->slot), nullptr));
+    }
     if (!pb->d_rrec) CKS(dalloc(pb, &pb->d_rrec, resident_records(pb->kind, pb->plane)));
     CK(cudaStreamSynchronize(nullptr));
   }
@@ -523,8 +526,9 @@ opt_status run_solve(opt_problem* pb, const opt_solve_params* prm_in, opt_report
   }
   if (s.timeout) {
     if (pb->d_rsync) {
-      // blocks gave up at different exchanges: back to a clean counter
+      // blocks gave up at different exchanges: back to empty slots
       CK(cudaMemset(pb->d_rsync, 0, sizeof(ResidentSync)));
+      CK(cudaMemset(pb->d_rsync->slot, 0xff, sizeof(pb->d_rsync->slot)));
     }
     return OPT_ERR_TIMEOUT;
   }

@@ -264,14 +264,15 @@ constexpr int RES_LANES = 4;          // threads per vertex where a block has fe
 constexpr int RES_CLUSTER = 16;       // blocks of the one-cluster form, at most
 // RES_D, RES_DC, RES_LIST: kept in shared memory; RES_Z: see Records (resident.cu)
 enum ResidentFlags : int { RES_D = 1, RES_DC = 2, RES_LIST = 4, RES_Z = 8 };
-// Exchange counter and slots of one problem (zeroed before the first launch, and
-// again after a timeout).
+// Exchange slots of one problem; the host fills slot with ones (empty) and the
+// rest with zeros before the first launch, and again after a timeout.
 struct ResidentSync {
-  unsigned int counter;         // arrivals, ever growing
+  unsigned int counter;         // arrivals at meetings, ever growing
   unsigned int pad0[31];
-  unsigned int count;           // the counter's value between launches
-  unsigned int pad1[31];
-  unsigned long long slot[2][RES_MAX_BLOCKS];
+  unsigned int meetings;        // the counter's value between launches
+  unsigned int sums;            // sums done so far (modulo the three sets)
+  unsigned int pad1[30];
+  unsigned long long slot[3][RES_MAX_BLOCKS][16];   // a cache line each
 };
 struct ResidentPlan {
   int n, per, blocks;           // units, units per block; blocks = 0: not available

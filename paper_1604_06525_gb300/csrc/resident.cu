@@ -20,11 +20,11 @@
 //    shared memory, one hardware cluster barrier, about 500 cycles (1,100 with a
 //    sum);
 //  * the whole device, one block per SM (cooperative launch): every block stores
-//    its sum in a slot, adds itself to a counter, polls the counter and then
-//    reads all slots, about 3,500 cycles.  (Polling the slots themselves queues up
-//    on their cache lines: 9,000 cycles with 152 blocks and packed slots, 2,900 with
-//    a line per slot, against 1,500 for one word that only grows; fences add
-//    800-1,300 to either.)
+//    its sum in a slot of its own cache line and polls the slots of all others
+//    (2,500 cycles, 4,200 with the fences that order records).  Slots packed in
+//    shared lines cost 9,000: a line that blocks of both dies write is slow to read
+//    from the far die (4,500-6,400 cycles against 1,100).  Meetings without a
+//    sum poll one counter (1,500; 2,400 with fences).
 //
 // The arithmetic is that of the per-launch kernels, in the same roundings and
 // the same order (grid_algebra.cuh, mesh_algebra.cuh, ...); the dot products are
@@ -32,11 +32,14 @@
 // alpha and beta are the same and with them every iterate.  (Only the mesh
 // energies' records with RES_Z carry w = w(z) + beta w(p_old) in place of w(p).)
 //
-// Slots are used in turn by parity: a block stores its sum of exchange k + 2
-// only after exchange k + 1, which all blocks reach after reading those of k.
-// The counter goes on from launch to launch (sync->count holds its value).
-// Every wait is bounded (1 s); a block that gives up flags s->timeout and
-// returns, the others run into their own limit, and the host clears the counter.
+// Slots: three sets, used in turn.  A slot holds kEmpty until its block stores the
+// sum of an exchange; a block that has finished sum k empties its slot of sum k
+// - 1 (every block has read it: all have arrived at k), which is next used at k +
+// 2; by then the emptying is visible to whoever waits, since the store of sum k + 1
+// lies in between.  The counts go on from launch to launch (sync->sums,
+// sync->meetings).  Every wait is bounded (1 s); a block that gives up flags
+// s->timeout and returns, the others run into their own limit, and the host
+// resets the slots.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -54,11 +57,20 @@ namespace {
 constexpr int RT = 512;               // threads per block, one block per SM
 constexpr int RW = RT / 32;
 constexpr int CELL = 256;             // grids: 32 x 8 pixels
+constexpr unsigned long long kEmpty = ~0ull;
 
 __device__ __forceinline__ unsigned ld_relaxed(const unsigned* p) {
   unsigned v;
   asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
+}
+__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 __device__ __forceinline__ void red_add(unsigned* p, unsigned v) {
   asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
@@ -80,95 +92,119 @@ __device__ __forceinline__ void st_cluster(unsigned long long* local, unsigned r
   asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
 }
 __device__ __forceinline__ unsigned long long pack(F2 a) {
-  return (unsigned long long)__float_as_uint(a.hi) | ((unsigned long long)__float_as_uint(a.lo) << 32);
+  const unsigned long long b =
+      (unsigned long long)__float_as_uint(a.hi) | ((unsigned long long)__float_as_uint(a.lo) << 32);
+  return b == kEmpty ? b - 1 : b;     // a NaN either way
 }
 __device__ __forceinline__ F2 unpack(unsigned long long b) {
   return F2{__uint_as_float((unsigned)b), __uint_as_float((unsigned)(b >> 32))};
 }
 
+// A wait's time limit: called now and then while waiting.
+__device__ __forceinline__ bool waited_too_long(int spin, unsigned long long& t0) {
+  if ((spin & 255) != 255) return false;
+  const unsigned long long now = global_ns();
+  if (t0 == 0) t0 = now;
+  return now - t0 > kBarrierLimitNs;
+}
+
+// What a launch knows of the device-wide exchanges: those done so far, by kind.
+struct Meet {
+  ResidentSync* sy;
+  unsigned base, meetings, sums;
+};
+
 // Meeting of all blocks: what any thread wrote to global memory before is
-// visible to every thread of every block after.  SUM: the total of every
-// thread's pair, the same in every thread of every block.  k: exchanges of this
-// launch so far; base: the counter at its start.  Returns false if a block did
+// visible to every thread of every block after.  Returns false if a block did
 // not arrive in time.
-template <bool CL, bool SUM>
-__device__ __forceinline__ bool exchange(ResidentSync* sy, unsigned base, unsigned& k, F2 acc, F2& total) {
+template <bool CL>
+__device__ __forceinline__ bool meet(Meet& M) {
+  if (CL) {
+    cluster_meet();
+    return true;
+  }
+  __shared__ int s_ok;
+  __syncthreads();
+  M.meetings += 1;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    red_add(&M.sy->counter, 1u);
+    const unsigned want = M.base + M.meetings * gridDim.x;
+    unsigned long long t0 = 0;
+    int ok = 1;
+    for (int spin = 0; ok && (int)(ld_relaxed(&M.sy->counter) - want) < 0; ++spin) ok = !waited_too_long(spin, t0);
+    __threadfence();
+    s_ok = ok;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
+// The same with the total of every thread's pair, equal in every thread of
+// every block.  FENCE: global writes are ordered too (a cluster's barrier always
+// does).
+template <bool CL, bool FENCE>
+__device__ __forceinline__ bool meet_sum(Meet& M, F2 acc, F2& total) {
   __shared__ unsigned long long sw[RW];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (SUM) {
-    acc = warp_sum_f2(acc);
-    if (l == 0) sw[w] = pack(acc);
-  }
+  acc = warp_sum_f2(acc);
+  if (l == 0) sw[w] = pack(acc);
+  __syncthreads();
   auto block_total = [&] {
-    F2 v = f2_zero();
-    if (SUM) {
-      v = unpack(sw[l % RW]);
+    F2 v = unpack(sw[l % RW]);
 #pragma unroll
-      for (int o = RW / 2; o > 0; o >>= 1) v = f2_shfl_xor_add(v, o);
-    }
+    for (int o = RW / 2; o > 0; o >>= 1) v = f2_shfl_xor_add(v, o);
     return v;
   };
+  const unsigned k = M.sums;
+  M.sums += 1;
   if (CL) {
     __shared__ unsigned long long part[2][RES_CLUSTER];
     const unsigned n = gridDim.x;
-    if (SUM) {
-      __syncthreads();
-      if (w == 0) {
-        const F2 v = block_total();
-        if (l < n) st_cluster(&part[k & 1][cluster_rank()], l, pack(v));
-        __syncwarp();
-      }
+    if (w == 0) {
+      const F2 v = block_total();
+      if (l < n) st_cluster(&part[k & 1][cluster_rank()], l, pack(v));
+      __syncwarp();
     }
     cluster_meet();
-    if (SUM) {
-      total = l % RES_CLUSTER < n ? unpack(part[k & 1][l % RES_CLUSTER]) : f2_zero();
+    total = l % RES_CLUSTER < n ? unpack(part[k & 1][l % RES_CLUSTER]) : f2_zero();
 #pragma unroll
-      for (int o = RES_CLUSTER / 2; o > 0; o >>= 1) total = f2_shfl_xor_add(total, o);
-    }
-    k += 1;
+    for (int o = RES_CLUSTER / 2; o > 0; o >>= 1) total = f2_shfl_xor_add(total, o);
     return true;
   } else {
-    __shared__ unsigned long long s_total;
-    __shared__ int s_ok;
-    __syncthreads();
+    constexpr int NP = RES_MAX_BLOCKS / 32;      // polling warps, one slot a thread
+    __shared__ unsigned long long sg[NP];
+    __shared__ int s_ok[NP];
+    auto slot = [&](unsigned set, int b) { return &M.sy->slot[set % 3][b][0]; };
     if (w == 0) {
-      F2 v = block_total();
-      unsigned long long* slot = sy->slot[k & 1];
+      const F2 v = block_total();
+      if (FENCE) __threadfence();
+      if (l == 0) st_relaxed(slot(k, blockIdx.x), pack(v));
+    }
+    if (w < NP) {
+      const bool on = threadIdx.x < gridDim.x;
+      const unsigned long long* p = slot(k, on ? threadIdx.x : 0);
+      unsigned long long b, t0 = 0;
       int ok = 1;
+      for (int spin = 0; (b = ld_relaxed(p)) == kEmpty && ok; ++spin) ok = !waited_too_long(spin, t0);
+      if (FENCE) __threadfence();
+      ok = __all_sync(0xffffffffu, ok);
+      const F2 v = warp_sum_f2(on ? unpack(b) : f2_zero());
       if (l == 0) {
-        if (SUM) __stcg(slot + blockIdx.x, pack(v));
-        __threadfence();
-        red_add(&sy->counter, 1u);
-        const unsigned want = base + (k + 1) * gridDim.x;
-        unsigned long long t0 = 0;
-        for (int spin = 0; (int)(ld_relaxed(&sy->counter) - want) < 0; ++spin) {
-          if ((spin & 255) == 255) {
-            const unsigned long long now = global_ns();
-            if (t0 == 0) t0 = now;
-            if (now - t0 > kBarrierLimitNs) { ok = 0; break; }
-          }
-        }
-        __threadfence();
-        s_ok = ok;
-      }
-      __syncwarp();
-      if (SUM) {
-        constexpr int NP = RES_MAX_BLOCKS / 32;
-        unsigned long long b[NP];
-#pragma unroll
-        for (int t = 0; t < NP; ++t) b[t] = l + 32 * t < gridDim.x ? __ldcg(slot + l + 32 * t) : 0ull;
-        v = unpack(b[0]);
-#pragma unroll
-        for (int t = 1; t < NP; ++t) f2_add_f2(v, unpack(b[t]));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v = f2_shfl_xor_add(v, o);
-        if (l == 0) s_total = pack(v);
+        sg[w] = pack(v);
+        s_ok[w] = ok;
       }
     }
-    k += 1;
     __syncthreads();
-    if (SUM) total = unpack(s_total);
-    return s_ok != 0;
+    if (threadIdx.x == 0) st_relaxed(slot(k + 2, blockIdx.x), kEmpty);
+    total = unpack(sg[0]);
+    int ok = s_ok[0];
+#pragma unroll
+    for (int t = 1; t < NP; ++t) {
+      f2_add_f2(total, unpack(sg[t]));
+      ok &= s_ok[t];
+    }
+    return ok != 0;
   }
 }
 
@@ -647,8 +683,7 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
   if (CL) pdl_begin();
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;      // the same for every block: none has passed an exchange
-  const unsigned base = CL ? 0u : sync->count;
-  unsigned met_no = 0;
+  Meet M{sync, CL ? 0u : sync->meetings, 0u, CL ? 0u : sync->sums};
   const int tid = threadIdx.x;
   const int u0 = blockIdx.x * rp.per, cnt = min(rp.per, rp.n - u0), cap = rp.per;
   const long long pl = rp.plane;
@@ -807,7 +842,7 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
   F2 rz = F2{s->rz_hi, s->rz_lo}, pq = f2_zero();   // the same values in every thread
   int iters = 0, nonfinite = 0, active = 1;
   float alpha = 0.f, beta = 0.f;
-  bool met = exchange<CL, false>(sync, base, met_no, f2_zero(), pq);
+  bool met = meet<CL>(M);
   for (int it = 0; met && it < inner; ++it) {
     const Records R = {recp[zrec && it > 0 ? (it - 1) & 1 : 0], recz, beta, zrec && it > 0};
     if (it > 0) {
@@ -822,7 +857,7 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
         }
         put_p(j, p, recp[zrec ? it & 1 : 0]);
       }
-      if (!zrec && !(met = exchange<CL, false>(sync, base, met_no, f2_zero(), pq))) break;
+      if (!zrec && !(met = meet<CL>(M))) break;
     }
     // q = (J^T J + lambda D) p, p.q -> alpha
     F2 acc = f2_zero();
@@ -899,7 +934,7 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
         }
       }
     }
-    if (!(met = exchange<CL, true>(sync, base, met_no, acc, pq))) break;
+    if (!(met = meet_sum<CL, false>(M, acc, pq))) break;
     if (!(pq.hi > 0.f && isfinite(pq.hi))) {  // breakdown
       alpha = 0.f;
       active = 0;
@@ -923,7 +958,8 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
       if (zrec) put_z(j, z);
     }
     F2 rz2 = f2_zero();
-    if (!(met = exchange<CL, true>(sync, base, met_no, acc, rz2))) break;
+    met = zrec ? meet_sum<CL, true>(M, acc, rz2) : meet_sum<CL, false>(M, acc, rz2);
+    if (!met) break;
     iters += 1;
     beta = f2_quot(rz2, rz);
     rz = rz2;
@@ -955,7 +991,10 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
     s->pcg_iters += iters;
     if (!active) s->pcg_active = 0;
     if (nonfinite) s->nonfinite = 1;
-    if (!CL) sync->count = base + met_no * gridDim.x;
+    if (!CL) {
+      sync->meetings = M.base + M.meetings * gridDim.x;
+      sync->sums = M.sums % 3u;
+    }
   }
 }
 
