@@ -591,8 +591,7 @@ __device__ __forceinline__ void graph_sums(const GraphCtx& c, int j, bool ok, co
 #pragma unroll
   for (int k = 0; k < NT_; ++k) t[k] = 0.f;
   const int lane = threadIdx.x % LANES;
-  auto nbr = [&](int e, bool out, bool in, float (&v)[NT_]) {
-    float d[K::ND], g[K::NS];
+  auto fetch = [&](int e, float (&d)[K::ND], float (&g)[K::NS]) {
     if (c.staged) {
 #pragma unroll
       for (int k = 0; k < K::ND; ++k) d[k] = c.dyn[k * c.tab + e];
@@ -602,14 +601,39 @@ __device__ __forceinline__ void graph_sums(const GraphCtx& c, int j, bool ok, co
       K::unpack_rec(R, e, d);
       K::geometry(pr, e, g);
     }
+  };
+  auto nbr = [&](int e, bool out, bool in, float (&v)[NT_]) {
+    float d[K::ND], g[K::NS];
+    fetch(e, d, g);
     K::terms(pr, o, d, g, out, in, v);
   };
   if (K::G3) {
     const Stencil3 st = stencil3(pr, c.u0 + (ok ? j : 0));
+    if (LANES == 1) {
+      const int i = c.u0 + j;
+#pragma unroll
+      for (int r = 0; r < 6; r += 2) {
+        float d1[K::ND], g1[K::NS], d2[K::ND], g2[K::NS], v[NT_];
+        const bool on1 = ok && st.ok[r], on2 = ok && st.ok[r + 1];
+        if (on1) fetch(i + st.off[r], d1, g1);
+        if (on2) fetch(i + st.off[r + 1], d2, g2);
+        if (on1) {
+          K::terms(pr, o, d1, g1, true, true, v);
+#pragma unroll
+          for (int n = 0; n < NT_; ++n) t[n] += v[n];
+        }
+        if (on2) {
+          K::terms(pr, o, d2, g2, true, true, v);
+#pragma unroll
+          for (int n = 0; n < NT_; ++n) t[n] += v[n];
+        }
+      }
+      return;
+    }
 #pragma unroll
     for (int r = 0; r < 6; r += LANES) {
       float v[NT_];
-      // the thread's neighbour of this round (LANES = 1: compile-time)
+      // the thread's neighbour of this round
       int off = 0;
       bool has = false;
 #pragma unroll
@@ -618,10 +642,10 @@ __device__ __forceinline__ void graph_sums(const GraphCtx& c, int j, bool ok, co
       if (has) nbr(c.u0 + j + off, true, true, v);
 #pragma unroll
       for (int s = 0; s < LANES; ++s) {
-        const bool from = LANES == 1 ? has : __shfl_sync(0xffffffffu, (int)has, s, LANES) != 0;
+        const bool from = __shfl_sync(0xffffffffu, (int)has, s, LANES) != 0;
 #pragma unroll
         for (int k = 0; k < NT_; ++k) {
-          const float a = LANES == 1 ? v[k] : __shfl_sync(0xffffffffu, has ? v[k] : 0.f, s, LANES);
+          const float a = __shfl_sync(0xffffffffu, has ? v[k] : 0.f, s, LANES);
           if (from) t[k] += a;
         }
       }
@@ -631,11 +655,21 @@ __device__ __forceinline__ void graph_sums(const GraphCtx& c, int j, bool ok, co
   const int o0 = ok ? c.row[j] : 0, deg = ok ? c.row[j + 1] - o0 : 0;
   const bool sym = pr.sym != 0;
   if (LANES == 1) {
-    for (int k = 0; k < deg; ++k) {
-      float v[NT_];
-      nbr(c.lst[o0 + k], true, sym, v);
+    // two neighbours at a time: their records are in flight together
+    for (int k = 0; k < deg; k += 2) {
+      float d1[K::ND], g1[K::NS], d2[K::ND], g2[K::NS], v[NT_];
+      const bool two = k + 1 < deg;
+      const int e1 = c.lst[o0 + k], e2 = two ? c.lst[o0 + k + 1] : e1;
+      fetch(e1, d1, g1);
+      if (two) fetch(e2, d2, g2);
+      K::terms(pr, o, d1, g1, true, sym, v);
 #pragma unroll
       for (int n = 0; n < NT_; ++n) t[n] += v[n];
+      if (two) {
+        K::terms(pr, o, d2, g2, true, sym, v);
+#pragma unroll
+        for (int n = 0; n < NT_; ++n) t[n] += v[n];
+      }
     }
     if (!sym && ok) {
       for (int k = pr.irow[c.u0 + j]; k < pr.irow[c.u0 + j + 1]; ++k) {
@@ -863,8 +897,11 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
     F2 acc = f2_zero();
     auto finish_rows = [&](int j, const float (&p)[NX], float (&q)[NX]) {
       if (lm) {
+        float c[NM];                          // (all loads before the stores)
 #pragma unroll
-        for (int k = 0; k < NX; ++k) q[k] = __fmaf_rn(__fmul_rn(lam, sc[K::mp(k) * cs + j]), p[k], q[k]);
+        for (int k = 0; k < NM; ++k) c[k] = __fmul_rn(lam, sc[k * cs + j]);
+#pragma unroll
+        for (int k = 0; k < NX; ++k) q[k] = __fmaf_rn(c[K::mp(k)], p[k], q[k]);
       }
 #pragma unroll
       for (int k = 0; k < NX; ++k) {
@@ -946,10 +983,13 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
     acc = f2_zero();
     for (int j = tid; j < cnt; j += RT) {
       if (skip(j)) continue;
-      float z[NX];
+      float z[NX], d[NX];                     // (all loads of delta before its stores)
+#pragma unroll
+      for (int k = 0; k < NX; ++k) d[k] = sd[k * ds + j];
+#pragma unroll
+      for (int k = 0; k < NX; ++k) sd[k * ds + j] = __fmaf_rn(alpha, p_at(k, j), d[k]);
 #pragma unroll
       for (int k = 0; k < NX; ++k) {
-        sd[k * ds + j] = __fmaf_rn(alpha, p_at(k, j), sd[k * ds + j]);
         const float r = __fmaf_rn(-alpha, sq[k * cap + j], sr[k * cap + j]);
         sr[k * cap + j] = r;
         z[k] = __fmul_rn(sm[K::mp(k) * cap + j], r);
@@ -1130,8 +1170,11 @@ size_t resident_records(int kind, long long plane) {
 #ifndef RES_CLUSTER_UNITS
 #define RES_CLUSTER_UNITS 8192
 #endif
+#ifndef RES_LANE_UNITS
+#define RES_LANE_UNITS 256
+#endif
 #ifndef RES_Z_UNITS
-#define RES_Z_UNITS 100000
+#define RES_Z_UNITS 32768
 #endif
 // Blocks, shared memory and what it holds for a problem of n units (pixels of
 // the active tiles in cells of 256, or vertices); blocks = 0 if the state does
@@ -1162,15 +1205,15 @@ ResidentPlan resident_plan(int kind, int n, long long plane, int lm, const int* 
       return true;
     };
     if (words > room) return false;
-    rp.lanes = !grid && per * RES_LANES <= 2 * RT ? RES_LANES : 1;
+    rp.lanes = !grid && per <= RES_LANE_UNITS ? RES_LANES : 1;
     if (orow) {
       int most = 0;
       for (int b = 0; b < rp.blocks; ++b)
         most = std::max(most, orow[std::min(n, (b + 1) * rp.per)] - orow[b * rp.per]);
-      // the lists, and the table: entries for about as many edges as leave a
-      // compact patch of that many vertices (all of them where the patch is small)
-      const long long slots =
-          std::min<long long>(most, (long long)(30.0 * std::sqrt((double)per)) + 64);
+      // the lists, and the table: entries for as many edges as leave a run of
+      // that many vertices in locality order (measured at most 14 sqrt(per) on
+      // sheets and 22 on icospheres; a block where more leave reads records)
+      const long long slots = std::min<long long>(most, (long long)(24.0 * std::sqrt((double)per)) + 32);
       if (take(per + 1 + most + slots * (s.ND + 1) + s.NS * (per + slots), RES_LIST)) rp.slots = (int)slots;
       else take(per + 1 + most, RES_LIST);
     }
