@@ -14,10 +14,16 @@
 // only twice the bytes.  The float64 kernels are therefore bound by float64
 // arithmetic, not by memory, and are written for the fewest float64
 // operations rather than for the fewest bytes:
-//  * the Jacobian entries that depend on x and are not constants -- the angle
-//    columns (warp: R'(theta_i) v per residual; mesh: dR/dA_m (U_a - U_b) per
-//    directed edge) -- are evaluated once per outer iteration by PCGInit and
-//    read by every applyJTJ of the PCG solve (the rest of J is +-s_w);
+//  * what of the Jacobian depends on x -- the angle columns -- is evaluated
+//    once per outer iteration by PCGInit and read by every applyJTJ of the PCG
+//    solve (the rest of J is +-s_w): the warp keeps R'(theta_i) v per residual,
+//    the mesh y = R(A_a) (U_a - U_b) per directed edge: dR/dA_m v = beta_m x y with
+//    the axes beta_m of the Euler angles (see graph_kernels.cu), so an edge's J p
+//    is (p_a - p_b) - w_a x y with one angular velocity w_a = sum_m p_m beta_m per
+//    vertex, and its angle rows are one torque y x (J p) per vertex.  27 operations
+//    per neighbour where both directions of an edge exist (visited once) in place
+//    of 45 with the three derivative columns of either end; level 7 (163,842
+//    vertices): applyJTJ 120 -> 76 us, PCGInit 263 -> 176 us, energies 209 -> 131 us;
 //  * the direction update p = M^-1 r + beta p is its own streaming pass, so
 //    applyJTJ reads p at the neighbours instead of re-forming it;
 //  * the own and the incoming residual of a stencil pair are folded into one
@@ -36,6 +42,7 @@
 #include <vector>
 
 #include "opt_gb300.h"
+#include "meet.cuh"
 #include "opt_internal.cuh"
 #include "opt_problem.h"
 
@@ -66,8 +73,11 @@ struct P64 {
   double *d, *r, *q, *m, *dc;   // nx planes each
   double* p;                    // PCG direction (nx planes)
   double* cs;                   // cos / sin planes of the angles (warp 2, mesh 6)
-  double* G;                    // angle columns of J at x: warp 8 planes of n (R'(theta) v per
-                                // direction, x / y), mesh 9 planes of ne (dR/dA_m w, m-major)
+  double* G;                    // warp: angle columns of J at x, 8 planes of n (R'(theta) v per
+                                // direction, x / y); mesh: y = R(A_a) (U_a - U_b) of each directed
+                                // edge, 4 doubles an edge (one 32-byte sector; the last unused)
+  double* rec;                  // mesh: direction records, 6 doubles a vertex (p_d, w)
+  int sym;                      // mesh: out- and in-edge lists are equal (edges given both ways)
   const double* pin;            // apply hook: caller direction (NULL in a solve)
   double* jtf_out;              // hook outputs (nx planes each) or NULL
   double* diag_out;
@@ -76,14 +86,25 @@ struct P64 {
   double* Ehist;
 };
 
-constexpr int kBlocksPerSM64 = 4;
+// Resident blocks per SM, all at once: the float64 pipe issues one warp
+// instruction in about 15 cycles per SM, so a few warps keep it busy, and what
+// counts is that every SM gets the same number of elements.
+#ifndef F64_BLOCKS_PER_SM
+#define F64_BLOCKS_PER_SM 2
+#endif
+constexpr int kBlocksPerSM64 = F64_BLOCKS_PER_SM;
 
 // grid direction k: +x, -x, +y, -y
 __device__ __forceinline__ int ddx(int k) { return k == 0 ? 1 : (k == 1 ? -1 : 0); }
 __device__ __forceinline__ int ddy(int k) { return k == 2 ? 1 : (k == 3 ? -1 : 0); }
 
-#define FOR_ELEMENTS(P, i) \
-  for (long long i = (long long)blockIdx.x * NT + threadIdx.x; i < (P).n; i += (long long)gridDim.x * NT)
+// The block's elements: equal contiguous runs (grid-strided, 163,842 vertices on
+// 608 blocks gave 32 of them twice the work of the others).
+__device__ __forceinline__ long long run_begin(long long n, unsigned b) { return (n * b / gridDim.x) & ~7ll; }
+#define FOR_ELEMENTS(P, i)                                                                                    \
+  for (long long i = run_begin((P).n, blockIdx.x) + threadIdx.x,                                              \
+                 i##_end = blockIdx.x + 1 == gridDim.x ? (P).n : run_begin((P).n, blockIdx.x + 1);            \
+       i < i##_end; i += NT)
 
 // Block sums of a and b published to this block's slot; true in every thread
 // of the last block to arrive.
@@ -202,7 +223,7 @@ __global__ void k64_lm_decide(Scalars* s, double eta, double lmin, double lmax, 
 
 // cos / sin of the rotation angles at x (warp: theta; mesh: ax, ay, az),
 // once per outer iteration (Sec. 4.2: evalJ's values depend only on x).
-__global__ void __launch_bounds__(NT) k64_rot(P64 P) {
+__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_rot(P64 P) {
   const int na = P.kind == F64_WARP ? 1 : 3;
   const int a0 = P.kind == F64_WARP ? 2 : 3;
   FOR_ELEMENTS(P, i) {
@@ -215,10 +236,41 @@ __global__ void __launch_bounds__(NT) k64_rot(P64 P) {
   }
 }
 
+// Mesh: cos / sin of a_y and a_z of a vertex (what its axes need), the angular
+// velocity of angles p[3..5], and the direction record.
+struct Axes64 {
+  double cb, sb, cc, sc;
+};
+__device__ __forceinline__ Axes64 axes_at(const P64& P, long long v) {
+  const long long n = P.n;
+  return Axes64{P.cs[2 * n + v], P.cs[3 * n + v], P.cs[4 * n + v], P.cs[5 * n + v]};
+}
+__device__ __forceinline__ void angular_velocity64(const Axes64& a, double pa, double pb, double pc, double (&w)[3]) {
+  const double h = pa * a.cb;
+  w[0] = fma(a.cc, h, -a.sc * pb);
+  w[1] = fma(a.sc, h, a.cc * pb);
+  w[2] = fma(-a.sb, pa, pc);
+}
+// (beta_x . t, beta_y . t, beta_z . t)
+__device__ __forceinline__ void axis_rows64(const Axes64& a, const double (&t)[3], double (&o)[3]) {
+  const double t1 = fma(a.cc, t[0], a.sc * t[1]);
+  o[0] = fma(a.cb, t1, -a.sb * t[2]);
+  o[1] = fma(a.cc, t[1], -a.sc * t[0]);
+  o[2] = t[2];
+}
+__device__ __forceinline__ void mesh_record(const P64& P, long long v, const double (&p)[6]) {
+  double w[3];
+  angular_velocity64(axes_at(P, v), p[3], p[4], p[5], w);
+  double2* r = reinterpret_cast<double2*>(P.rec + 6 * v);
+  r[0] = make_double2(p[0], p[1]);
+  r[1] = make_double2(p[2], w[0]);
+  r[2] = make_double2(w[1], w[2]);
+}
+
 // Direction update (Sec. 4.1 PCGStep): p = z + beta p, z = M^-1 r (every
 // PCG iteration after the first; PCGInit writes the first direction).
 template <int NX>
-__global__ void __launch_bounds__(NT) k64_direction(P64 P) {
+__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_direction(P64 P) {
   const Scalars* s = P.s;
   if (s->done || !s->pcg_active) return;
   const double beta = s->beta_d;
@@ -234,14 +286,29 @@ __global__ void __launch_bounds__(NT) k64_direction(P64 P) {
       rv[c] = rr[c * P.n + i];
     }
 #pragma unroll
-    for (int c = 0; c < NX; ++c) pp[c * P.n + i] = fma(beta, pv[c], mv[c] * rv[c]);
+    for (int c = 0; c < NX; ++c) {
+      pv[c] = fma(beta, pv[c], mv[c] * rv[c]);
+      pp[c * P.n + i] = pv[c];
+    }
+    if constexpr (NX == 6) mesh_record(P, i, pv);
+  }
+}
+
+// The mesh's direction records from a given p (apply hook).
+__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_mesh_records(P64 P) {
+  const double* __restrict__ pp = P.pin ? P.pin : P.p;
+  FOR_ELEMENTS(P, i) {
+    double pv[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) pv[c] = pp[c * P.n + i];
+    mesh_record(P, i, pv);
   }
 }
 
 // PCG vector update (Sec. 4.1 PCGStep): delta += alpha p, r -= alpha q,
 // z = M^-1 r, r.z -> beta = r.z / r.z_old.
 template <int NX>
-__global__ void __launch_bounds__(NT) k64_update(P64 P) {
+__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_update(P64 P) {
   Scalars* s = P.s;
   if (s->done || !s->pcg_active) return;
   const double alpha = s->alpha_d;
@@ -285,7 +352,7 @@ __global__ void __launch_bounds__(NT) k64_update(P64 P) {
 }
 
 // x += delta (cond 0: unless the solve is done; cond 1: only if LM accepted).
-__global__ void __launch_bounds__(NT) k64_step(P64 P, int cond) {
+__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_step(P64 P, int cond) {
   const Scalars* s = P.s;
   if (cond ? !s->accept : s->done) return;
   FOR_ELEMENTS(P, i) {
@@ -298,7 +365,7 @@ __global__ void __launch_bounds__(NT) k64_step(P64 P, int cond) {
 // Residual (k, d) for valid k, k+d: s_w ((O_k - O_{k+d}) - R(theta_k) v),
 // v = U_k - U_{k+d}; handle h: s_f (O_h - C_h) = s_f ((dx, dy)_h - target).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(NT) k64_warp_init(P64 P, int k_outer, double dmin, double dmax) {
+__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_warp_init(P64 P, int k_outer, double dmin, double dmax) {
   Scalars* s = P.s;
   if (s->done) return;
   const double lam = P.lm ? s->lambda : 0.0;
@@ -364,20 +431,18 @@ __global__ void __launch_bounds__(NT) k64_warp_init(P64 P, int k_outer, double d
 // (both pixels valid); with dp = p_i - p_j (x, y), a = dp - R'_i v pt_i the
 // own row's J p / s_w and b = -dp - R'_j (-v) pt_j the incoming one's:
 //   q_O += w (a - b) = w (a + dp + R'_j(-v) pt_j),   q_t -= w R'_i v . a.
-__global__ void __launch_bounds__(NT) k64_warp_apply(P64 P) {
-  Scalars* s = P.s;
-  if (s->done || !s->pcg_active) return;
-  const double lam = P.lm ? s->lambda : 0.0;
-  const double* __restrict__ pp = P.pin ? P.pin : P.p;
-  const long long n = P.n;
-  const double w = P.w_reg;
-  double pq = 0.0;
-  FOR_ELEMENTS(P, i) {
+struct Warp64 {
+  static constexpr int NX = 3;
+  static __device__ __forceinline__ void rows(const P64& P, long long i, const double* pp, double lam,
+                                              const double (&pv)[NX], double (&q)[NX]) {
+    const long long n = P.n;
+    const double w = P.w_reg;
     // rows without residuals (excluded pixels) carry only the damping term
-    const double pxi = pp[i], pyi = pp[n + i], pti = pp[2 * n + i];
+    const double pxi = pv[0], pyi = pv[1], pti = pv[2];
     double ax_ = 0.0, ay_ = 0.0, at_ = 0.0;
     if (elem_valid(P, i)) {
       const int gx = (int)(i % P.W), gy = (int)(i / P.W);
+#pragma unroll
       for (int k = 0; k < 4; ++k) {
         const int nx_ = gx + ddx(k), ny_ = gy + ddy(k);
         if (nx_ < 0 || nx_ >= P.W || ny_ < 0 || ny_ >= P.H) continue;
@@ -394,26 +459,22 @@ __global__ void __launch_bounds__(NT) k64_warp_apply(P64 P) {
         ay_ += fma(qpy, ptj, ay + dy);
       }
     }
-    double qx = w * ax_, qy = w * ay_, qt = -w * at_;
+    q[0] = w * ax_;
+    q[1] = w * ay_;
+    q[2] = -w * at_;
     if (P.hslot[i] >= 0) {
-      qx = fma(P.w_fit, pxi, qx);
-      qy = fma(P.w_fit, pyi, qy);
+      q[0] = fma(P.w_fit, pxi, q[0]);
+      q[1] = fma(P.w_fit, pyi, q[1]);
     }
     if (lam != 0.0) {
-      qx += lam * P.dc[i] * pxi;
-      qy += lam * P.dc[n + i] * pyi;
-      qt += lam * P.dc[2 * n + i] * pti;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) q[c] = fma(lam * P.dc[c * n + i], pv[c], q[c]);
     }
-    P.q[i] = qx;
-    P.q[n + i] = qy;
-    P.q[2 * n + i] = qt;
-    pq += pxi * qx + pyi * qy + pti * qt;
   }
-  apply_finish(P, pq);
-}
+};
 
 // E(x) (mode 0) or E(x + delta) and |F(x) + J(x) delta|^2 (mode 1).
-__global__ void __launch_bounds__(NT) k64_warp_energy(P64 P, int mode, int hist_idx) {
+__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_warp_energy(P64 P, int mode, int hist_idx) {
   Scalars* s = P.s;
   if (mode == 1 && s->done) return;
   const long long n = P.n;
@@ -469,7 +530,7 @@ __global__ void __launch_bounds__(NT) k64_warp_energy(P64 P, int mode, int hist_
 // neighbour k+d in the image: residual (X_k - X_{k+d}) - (T_k - T_{k+d});
 // fixed pixels' X are constants.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(NT) k64_poisson_init(P64 P, int k_outer, double dmin, double dmax) {
+__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_poisson_init(P64 P, int k_outer, double dmin, double dmax) {
   Scalars* s = P.s;
   if (s->done) return;
   const double lam = P.lm ? s->lambda : 0.0;
@@ -501,20 +562,17 @@ __global__ void __launch_bounds__(NT) k64_poisson_init(P64 P, int k_outer, doubl
   init_finish(P, rz, E, k_outer);
 }
 
-__global__ void __launch_bounds__(NT) k64_poisson_apply(P64 P) {
-  Scalars* s = P.s;
-  if (s->done || !s->pcg_active) return;
-  const double lam = P.lm ? s->lambda : 0.0;
-  const double* __restrict__ pp = P.pin ? P.pin : P.p;
-  const long long n = P.n;
-  double pq = 0.0;
-  FOR_ELEMENTS(P, i) {
+struct Poisson64 {
+  static constexpr int NX = 4;
+  static __device__ __forceinline__ void rows(const P64& P, long long i, const double* pp, double lam,
+                                              const double (&pv)[NX], double (&q)[NX]) {
+    const long long n = P.n;
     // fixed pixels carry only the damping term (their p is 0 in a solve)
-    double pv[4], qv[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-    for (int c = 0; c < 4; ++c) pv[c] = pp[c * n + i];
+    for (int c = 0; c < 4; ++c) q[c] = 0.0;
     if (elem_valid(P, i)) {
       const int gx = (int)(i % P.W), gy = (int)(i / P.W);
+#pragma unroll
       for (int k = 0; k < 4; ++k) {
         const int nx_ = gx + ddx(k), ny_ = gy + ddy(k);
         if (nx_ < 0 || nx_ >= P.W || ny_ < 0 || ny_ >= P.H) continue;
@@ -524,20 +582,17 @@ __global__ void __launch_bounds__(NT) k64_poisson_apply(P64 P) {
         const bool fj = elem_valid(P, j);
         const double f = fj ? 2.0 : 1.0;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) qv[c] = fma(f, pv[c] - (fj ? pp[c * n + j] : 0.0), qv[c]);
+        for (int c = 0; c < 4; ++c) q[c] = fma(f, pv[c] - (fj ? pp[c * n + j] : 0.0), q[c]);
       }
     }
+    if (lam != 0.0) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      if (lam != 0.0) qv[c] += lam * P.dc[c * n + i] * pv[c];
-      P.q[c * n + i] = qv[c];
-      pq += pv[c] * qv[c];
+      for (int c = 0; c < 4; ++c) q[c] = fma(lam * P.dc[c * n + i], pv[c], q[c]);
     }
   }
-  apply_finish(P, pq);
-}
+};
 
-__global__ void __launch_bounds__(NT) k64_poisson_energy(P64 P, int mode, int hist_idx) {
+__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_poisson_energy(P64 P, int mode, int hist_idx) {
   Scalars* s = P.s;
   if (mode == 1 && s->done) return;
   const long long n = P.n;
@@ -573,163 +628,474 @@ __global__ void __launch_bounds__(NT) k64_poisson_energy(P64 P, int mode, int hi
 // Vertex-centric gather: a vertex sums its out-edges' rows (own residuals)
 // and its in-edges' rows (far-end residuals), so no atomics are needed.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ RotVT<double> rot_at(const P64& P, long long v, double wx, double wy, double wz) {
-  const long long n = P.n;
-  return rot_apply_cs<double>(P.cs[v], P.cs[n + v], P.cs[2 * n + v], P.cs[3 * n + v], P.cs[4 * n + v],
-                              P.cs[5 * n + v], wx, wy, wz);
+// R = Rz(az) Ry(ay) Rx(ax) from the angles' cos / sin
+__device__ __forceinline__ void rot_matrix64(const double (&cs)[6], double (&R)[3][3]) {
+  const double ca = cs[0], sa = cs[1], cb = cs[2], sb = cs[3], cc = cs[4], sc = cs[5];
+  const double a1 = sa * sb, a2 = ca * sb;
+  R[0][0] = cb * cc; R[0][1] = fma(a1, cc, -ca * sc); R[0][2] = fma(a2, cc, sa * sc);
+  R[1][0] = cb * sc; R[1][1] = fma(a1, sc, ca * cc);  R[1][2] = fma(a2, sc, -sa * cc);
+  R[2][0] = -sb;     R[2][1] = sa * cb;               R[2][2] = ca * cb;
+}
+__device__ __forceinline__ void mat_vec64(const double (&R)[3][3], const double (&v)[3], double (&o)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) o[i] = fma(R[i][0], v[0], fma(R[i][1], v[1], R[i][2] * v[2]));
+}
+// o += a x b
+__device__ __forceinline__ void add_cross64(double (&o)[3], const double (&a)[3], const double (&b)[3]) {
+  o[0] = fma(a[1], b[2], fma(-a[2], b[1], o[0]));
+  o[1] = fma(a[2], b[0], fma(-a[0], b[2], o[1]));
+  o[2] = fma(a[0], b[1], fma(-a[1], b[0], o[2]));
+}
+// o -= a x b
+__device__ __forceinline__ void sub_cross64(double (&o)[3], const double (&a)[3], const double (&b)[3]) {
+  o[0] = fma(-a[1], b[2], fma(a[2], b[1], o[0]));
+  o[1] = fma(-a[2], b[0], fma(a[0], b[2], o[1]));
+  o[2] = fma(-a[0], b[1], fma(a[1], b[0], o[2]));
+}
+__device__ __forceinline__ void load_y(const P64& P, long long e, double (&y)[3]) {
+  const double2* g = reinterpret_cast<const double2*>(P.G + 4 * e);
+  const double2 a = g[0];
+  y[0] = a.x; y[1] = a.y;
+  y[2] = P.G[4 * e + 2];
 }
 
-__global__ void __launch_bounds__(NT) k64_mesh_init(P64 P, int k_outer, double dmin, double dmax) {
-  Scalars* s = P.s;
-  if (s->done) return;
-  const double lam = P.lm ? s->lambda : 0.0;
+// y of every directed edge at x, by the edge's own vertex (ahead of PCGInit,
+// which reads it at both ends).
+__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_mesh_edges(P64 P) {
+  if (P.s->done) return;
   const long long n = P.n;
-  const double sw = P.s_w, w = P.w_reg;
-  double rz = 0.0, E = 0.0;
   FOR_ELEMENTS(P, v) {
-    double g[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, dg[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    const double xv[3] = {P.x[v], P.x[n + v], P.x[2 * n + v]};
+    double cs[6], R[3][3];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) cs[k] = P.cs[k * n + v];
+    rot_matrix64(cs, R);
     const double uv[3] = {P.c[v], P.c[n + v], P.c[2 * n + v]};
     for (int e = P.orow[v]; e < P.orow[v + 1]; ++e) {
       const int b = P.oe1[e];
       const double wv[3] = {uv[0] - P.c[b], uv[1] - P.c[n + b], uv[2] - P.c[2 * n + b]};
-      const RotVT<double> R = rot_at(P, v, wv[0], wv[1], wv[2]);
-      for (int m = 0; m < 3; ++m)
-        for (int c = 0; c < 3; ++c) P.G[(3 * m + c) * P.ne + e] = R.g[m][c];
-      double f[3];
-      for (int c = 0; c < 3; ++c) f[c] = sw * ((xv[c] - P.x[c * n + b]) + wv[c] - R.rv[c]);
-      E += f[0] * f[0] + f[1] * f[1] + f[2] * f[2];
-      for (int c = 0; c < 3; ++c) {
-        g[c] += sw * f[c];
-        dg[c] += w;
-      }
-      for (int m = 0; m < 3; ++m) {
-        g[3 + m] -= sw * (R.g[m][0] * f[0] + R.g[m][1] * f[1] + R.g[m][2] * f[2]);
-        dg[3 + m] += w * (R.g[m][0] * R.g[m][0] + R.g[m][1] * R.g[m][1] + R.g[m][2] * R.g[m][2]);
-      }
+      double y[3];
+      mat_vec64(R, wv, y);
+      double2* g = reinterpret_cast<double2*>(P.G + 4 * (long long)e);
+      g[0] = make_double2(y[0], y[1]);
+      g[1] = make_double2(y[2], 0.0);
     }
-    for (int e = P.irow[v]; e < P.irow[v + 1]; ++e) {
-      const int a = P.isrc[e];
-      const double wv[3] = {P.c[a] - uv[0], P.c[n + a] - uv[1], P.c[2 * n + a] - uv[2]};
-      const RotVT<double> R = rot_at(P, a, wv[0], wv[1], wv[2]);
+  }
+}
+
+__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_mesh_init(P64 P, int k_outer, double dmin, double dmax) {
+  Scalars* s = P.s;
+  if (s->done) return;
+  const double lam = P.lm ? s->lambda : 0.0;
+  const long long n = P.n;
+  const double w = P.w_reg;
+  double rz = 0.0, E = 0.0;
+  FOR_ELEMENTS(P, v) {
+    double f[3] = {0.0, 0.0, 0.0}, tq[3] = {0.0, 0.0, 0.0}, da[3] = {0.0, 0.0, 0.0}, es = 0.0;
+    const double xv[3] = {P.x[v], P.x[n + v], P.x[2 * n + v]};
+    const double uv[3] = {P.c[v], P.c[n + v], P.c[2 * n + v]};
+    const Axes64 ax = axes_at(P, v);
+    const int o0 = P.orow[v], o1 = P.orow[v + 1];
+    for (int e = o0; e < o1; ++e) {
+      const int b = P.oe1[e];
+      double y[3], r[3];
+      load_y(P, e, y);
+#pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const double f = sw * ((P.x[c * n + a] - xv[c]) + wv[c] - R.rv[c]);
-        g[c] -= sw * f;
-        dg[c] += w;
+        r[c] = (xv[c] - P.x[c * n + b]) + (uv[c] - P.c[c * n + b]) - y[c];
+        f[c] += r[c];
+        es = fma(r[c], r[c], es);
       }
+      add_cross64(tq, y, r);
+      // |beta_m x y|^2 in the frame (e1, e2, e3) = (Rz e_x, Rz e_y, e_z)
+      const double y1 = fma(ax.cc, y[0], ax.sc * y[1]), y2 = fma(ax.cc, y[1], -ax.sc * y[0]);
+      const double t = fma(ax.sb, y1, ax.cb * y[2]);
+      da[0] = fma(t, t, fma(y2, y2, da[0]));
+      da[1] = fma(y1, y1, fma(y[2], y[2], da[1]));
+      da[2] = fma(y1, y1, fma(y2, y2, da[2]));
     }
+    const int i0 = P.irow[v], i1 = P.irow[v + 1];
+    for (int k = i0; k < i1; ++k) {
+      const int a = P.isrc[k];
+      double y[3];
+      load_y(P, P.ieid[k], y);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) f[c] -= (P.x[c * n + a] - xv[c]) + (P.c[c * n + a] - uv[c]) - y[c];
+    }
+    double ga[3];
+    axis_rows64(ax, tq, ga);
+    const double deg = w * (double)((o1 - o0) + (i1 - i0));
+    double g[6] = {w * f[0], w * f[1], w * f[2], -w * ga[0], -w * ga[1], -w * ga[2]};
+    double dg[6] = {deg, deg, deg, w * da[0], w * da[1], w * da[2]};
+    E += w * es;
     const int h = P.hslot[v];
     if (h >= 0) {
       for (int c = 0; c < 3; ++c) {
-        const double f = P.s_f * (xv[c] - P.htgt[3 * h + c]);
-        E += f * f;
-        g[c] += P.s_f * f;
+        const double fh = P.s_f * (xv[c] - P.htgt[3 * h + c]);
+        E += fh * fh;
+        g[c] += P.s_f * fh;
         dg[c] += P.w_fit;
       }
     }
     rz += init_store<6>(P, v, g, dg, lam, dmin, dmax);
+    const double p0[6] = {P.p[v], P.p[n + v], P.p[2 * n + v], P.p[3 * n + v], P.p[4 * n + v], P.p[5 * n + v]};
+    mesh_record(P, v, p0);
   }
   init_finish(P, rz, E, k_outer);
 }
 
-// q = (J^T J + lambda D) p with every edge's angle columns g_m = dR/dA_m w
-// (w = U_a - U_b) from PCGInit: J_e p / s_w = (pd_a - pd_b) - sum_m g_m pA_m(a);
-// own edges add w J_e p / s_w to q_d and -w g_m . (J_e p / s_w) to q_A, in-edges
-// subtract w J_e p / s_w from q_d.
-__global__ void __launch_bounds__(NT) k64_mesh_apply(P64 P) {
-  Scalars* s = P.s;
-  if (s->done || !s->pcg_active) return;
-  const double lam = P.lm ? s->lambda : 0.0;
-  const double* __restrict__ pp = P.pin ? P.pin : P.p;
-  const long long n = P.n, ne = P.ne;
-  const double w = P.w_reg;
-  double pq = 0.0;
-  FOR_ELEMENTS(P, v) {
-    double pv[6], qd[3] = {0.0, 0.0, 0.0}, qa[3] = {0.0, 0.0, 0.0};
+// q = (J^T J + lambda D) p with y of every edge from PCGInit and the direction
+// records: J_e p / s_w = (pd_a - pd_b) - w_a x y; own edges add w J_e p / s_w to q_d
+// and the torque rows to q_A, in-edges subtract w J_e p / s_w from q_d.
+struct Mesh64 {
+  static constexpr int NX = 6;
+  static __device__ __forceinline__ void rows(const P64& P, long long v, const double*, double lam,
+                                              const double (&pv)[NX], double (&qv)[NX]) {
+    const double* rec = P.rec;
+    const long long n = P.n;
+    const double w = P.w_reg;
+    double wv[3], qd[3] = {0.0, 0.0, 0.0}, tq[3] = {0.0, 0.0, 0.0};
+    const Axes64 ax = axes_at(P, v);
+    angular_velocity64(ax, pv[3], pv[4], pv[5], wv);
+    auto own_edge = [&](const double (&d)[3], const double (&y)[3]) {
+      double t[3] = {d[0], d[1], d[2]};
+      sub_cross64(t, wv, y);
 #pragma unroll
-    for (int c = 0; c < 6; ++c) pv[c] = pp[c * n + v];
-    for (int e = P.orow[v]; e < P.orow[v + 1]; ++e) {
-      const int b = P.oe1[e];
-      double g[9];
+      for (int c = 0; c < 3; ++c) qd[c] += t[c];
+      add_cross64(tq, y, t);
+    };
+    // minus J_e p / s_w of (j, v): (pd_v - pd_j) + w_j x y_e
+    auto in_edge = [&](const double (&d)[3], const double (&wj)[3], const double (&y)[3]) {
+      double t[3] = {d[0], d[1], d[2]};
+      add_cross64(t, wj, y);
 #pragma unroll
-      for (int k = 0; k < 9; ++k) g[k] = P.G[k * ne + e];
-      double jp[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const double t = fma(g[c], pv[3], fma(g[3 + c], pv[4], g[6 + c] * pv[5]));
-        jp[c] = (pv[c] - pp[c * n + b]) - t;
-        qd[c] += jp[c];
+      for (int c = 0; c < 3; ++c) qd[c] += t[c];
+    };
+    auto load = [&](int j, double (&d)[3], double (&wj)[3]) {
+      const double2* r = reinterpret_cast<const double2*>(rec + 6 * (long long)j);
+      const double2 a = r[0], b = r[1], c = r[2];
+      d[0] = pv[0] - a.x; d[1] = pv[1] - a.y; d[2] = pv[2] - b.x;
+      wj[0] = b.y; wj[1] = c.x; wj[2] = c.y;
+    };
+    const int o0 = P.orow[v], o1 = P.orow[v + 1];
+    double d[3], wj[3], y[3];
+    if (P.sym) {
+      for (int e = o0; e < o1; ++e) {
+        const int ei = P.ieid[e];
+        double yi[3];
+        load(P.oe1[e], d, wj);
+        load_y(P, e, y);
+        load_y(P, ei, yi);
+        own_edge(d, y);
+        in_edge(d, wj, yi);
       }
-#pragma unroll
-      for (int m = 0; m < 3; ++m) qa[m] = fma(g[3 * m], jp[0], fma(g[3 * m + 1], jp[1], fma(g[3 * m + 2], jp[2], qa[m])));
-    }
-    for (int k = P.irow[v]; k < P.irow[v + 1]; ++k) {
-      const int a = P.isrc[k], e = P.ieid[k];
-      const double pa3 = pp[3 * n + a], pa4 = pp[4 * n + a], pa5 = pp[5 * n + a];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const double t = fma(P.G[c * ne + e], pa3, fma(P.G[(3 + c) * ne + e], pa4, P.G[(6 + c) * ne + e] * pa5));
-        qd[c] -= (pp[c * n + a] - pv[c]) - t;
+    } else {
+      for (int e = o0; e < o1; ++e) {
+        load(P.oe1[e], d, wj);
+        load_y(P, e, y);
+        own_edge(d, y);
+      }
+      for (int k = P.irow[v]; k < P.irow[v + 1]; ++k) {
+        load(P.isrc[k], d, wj);
+        load_y(P, P.ieid[k], y);
+        in_edge(d, wj, y);
       }
     }
-    double qv[6] = {w * qd[0], w * qd[1], w * qd[2], -w * qa[0], -w * qa[1], -w * qa[2]};
+    double qa[3];
+    axis_rows64(ax, tq, qa);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      qv[c] = w * qd[c];
+      qv[3 + c] = -w * qa[c];
+    }
     if (P.hslot[v] >= 0)
 #pragma unroll
       for (int c = 0; c < 3; ++c) qv[c] = fma(P.w_fit, pv[c], qv[c]);
     if (lam != 0.0)
 #pragma unroll
-      for (int c = 0; c < 6; ++c) qv[c] += lam * P.dc[c * n + v] * pv[c];
+      for (int c = 0; c < 6; ++c) qv[c] = fma(lam * P.dc[c * n + v], pv[c], qv[c]);
+  }
+};
+
+// applyJTJ as a launch of its own: q, and p.q -> alpha.
+template <class K>
+__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_apply(P64 P) {
+  Scalars* s = P.s;
+  if (s->done || !s->pcg_active) return;
+  const double lam = P.lm ? s->lambda : 0.0;
+  const double* pp = P.pin ? P.pin : P.p;
+  double pq = 0.0;
+  FOR_ELEMENTS(P, i) {
+    double pv[K::NX], q[K::NX];
 #pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      P.q[c * n + v] = qv[c];
-      pq += pv[c] * qv[c];
+    for (int c = 0; c < K::NX; ++c) pv[c] = pp[c * P.n + i];
+    K::rows(P, i, pp, lam, pv, q);
+#pragma unroll
+    for (int c = 0; c < K::NX; ++c) {
+      P.q[c * P.n + i] = q[c];
+      pq = fma(pv[c], q[c], pq);
     }
   }
   apply_finish(P, pq);
 }
 
-__global__ void __launch_bounds__(NT) k64_mesh_energy(P64 P, int mode, int hist_idx) {
+// ---------------------------------------------------------------------------
+// resident PCG loop
+// ---------------------------------------------------------------------------
+// All PCG iterations of an outer iteration in one cooperative launch, one block
+// per SM, as resident.cu does for float32: a block keeps r, q, delta and M^-1 of its
+// run of elements in shared memory; p (the mesh: its records) goes through
+// global memory.  It replaces three launches an iteration and the traffic of the
+// direction and update passes.  Sums stay float64: per thread, per warp and block by
+// shuffles, then across blocks in block order from the slots.
+__device__ __forceinline__ double block_sum64(double v, int cnt, double* sw) {
+  // (a warp without elements has nothing to add; a shuffle level costs it 15
+  // issue cycles of the float64 pipe)
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  if (w * 32 < cnt) v = warp_sum(v);
+  if (l == 0) sw[w] = w * 32 < cnt ? v : 0.0;
+  __syncthreads();
+  if (w == 0) {
+    v = l < RW ? sw[l] : 0.0;
+#pragma unroll
+    for (int o = RW / 2; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  }
+  return v;                            // thread 0
+}
+
+// Slot of a block in the set of sum k.  Three sets, used in turn: a slot holds
+// kEmpty until its block stores the sum; a block that has finished sum k empties its
+// slot of sum k - 1 (every block has read it: all have arrived at k), which is next
+// used at k + 2, and the fence before its store of sum k + 1 orders the emptying
+// before whatever a block that waits for k + 2 has seen.
+constexpr unsigned long long kEmpty = ~0ull;
+__device__ __forceinline__ unsigned long long* sum_slot(const Meet& M, unsigned k, int b) {
+  return &M.sy->slot[k % 3][b][0];
+}
+
+// The sum over all threads of all blocks in thread 0 of every block (the same
+// bits); orders global writes like a meeting.
+__device__ __forceinline__ bool meet_sum64(Meet& M, double acc, int cnt, double& total) {
+  __shared__ double sw[RW];
+  constexpr int NP = RES_MAX_BLOCKS / 32;
+  __shared__ double sg[NP];
+  __shared__ int s_ok[NP];
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const double v = block_sum64(acc, cnt, sw);
+  const unsigned k = M.sums;
+  M.sums += 1;
+  if (threadIdx.x == 0) {
+    // a NaN total keeps one bit pattern, so that no sum looks like an empty slot
+    const unsigned long long b = v != v ? 0x7ff8000000000000ull : (unsigned long long)__double_as_longlong(v);
+    __threadfence();
+    st_relaxed(sum_slot(M, k, blockIdx.x), b);
+  }
+  if (w < NP) {
+    const bool on = threadIdx.x < gridDim.x;
+    const unsigned long long* p = sum_slot(M, k, on ? threadIdx.x : 0);
+    unsigned long long b, t0 = 0;
+    int ok = 1;
+    for (int spin = 0; (b = ld_relaxed(p)) == kEmpty && ok; ++spin) ok = !waited_too_long(spin, t0);
+    __threadfence();
+    ok = __all_sync(0xffffffffu, ok);
+    double t = on ? __longlong_as_double((long long)b) : 0.0;
+    if (w * 32 < gridDim.x) t = warp_sum(t);
+    if (l == 0) {
+      sg[w] = t;
+      s_ok[w] = ok;
+    }
+  }
+  __syncthreads();
+  int ok = s_ok[0];
+#pragma unroll
+  for (int t = 1; t < NP; ++t) ok &= s_ok[t];
+  if (threadIdx.x == 0) {
+    st_relaxed(sum_slot(M, k + 2, blockIdx.x), kEmpty);
+    total = sg[0];
+#pragma unroll
+    for (int t = 1; t < NP; ++t) total += sg[t];
+  }
+  return ok != 0;
+}
+
+template <class K>
+__global__ void __launch_bounds__(RT, 1) k64_pcg_loop(P64 P, ResidentSync* sync, int per, int inner) {
+  constexpr int NX = K::NX;
+  extern __shared__ double sh64[];
+  Scalars* s = P.s;
+  if (s->done || !s->pcg_active) return;       // the same for every block: none has met another
+  Meet M{sync, sync->meetings, 0u, sync->sums};
+  const double lam = P.lm ? s->lambda : 0.0;
+  const int tid = threadIdx.x;
+  const long long n = P.n, lo = (long long)blockIdx.x * per;
+  const int cnt = (int)min((long long)per, n - lo);
+  double* const sr = sh64;
+  double* const sq = sr + NX * per;
+  double* const sd = sq + NX * per;
+  double* const sm = sd + NX * per;
+  for (int j = tid; j < cnt; j += RT) {
+#pragma unroll
+    for (int c = 0; c < NX; ++c) {
+      sr[c * per + j] = P.r[c * n + lo + j];
+      sm[c * per + j] = P.m[c * n + lo + j];
+      sd[c * per + j] = 0.0;
+    }
+  }
+  __shared__ double s_step;
+  __shared__ int s_go;
+  double rz = s->rz, pq = 0.0;                 // thread 0
+  int iters = 0, nonfinite = 0, active = 1;
+  bool met = true;
+  for (int it = 0; it < inner; ++it) {
+    if (it > 0) {
+      const double beta = s_step;
+      for (int j = tid; j < cnt; j += RT) {
+        double p[NX];
+#pragma unroll
+        for (int c = 0; c < NX; ++c) p[c] = P.p[c * n + lo + j];
+#pragma unroll
+        for (int c = 0; c < NX; ++c) {
+          p[c] = fma(beta, p[c], sm[c * per + j] * sr[c * per + j]);
+          P.p[c * n + lo + j] = p[c];
+        }
+        if constexpr (NX == 6) mesh_record(P, lo + j, p);
+      }
+      if (!(met = meet_device(M))) break;
+    }
+    double acc = 0.0;
+    for (int j = tid; j < cnt; j += RT) {
+      double p[NX], q[NX];
+#pragma unroll
+      for (int c = 0; c < NX; ++c) p[c] = P.p[c * n + lo + j];
+      K::rows(P, lo + j, P.p, lam, p, q);
+#pragma unroll
+      for (int c = 0; c < NX; ++c) {
+        sq[c * per + j] = q[c];
+        acc = fma(p[c], q[c], acc);
+      }
+    }
+    if (!(met = meet_sum64(M, acc, cnt, pq))) break;
+    if (tid == 0) {
+      s_go = pq > 0.0 && isfinite(pq);
+      s_step = s_go ? rz / pq : 0.0;
+    }
+    __syncthreads();
+    const double alpha = s_step;
+    if (!s_go) {                               // breakdown
+      active = 0;
+      if (tid == 0 && !isfinite(pq)) nonfinite = 1;
+      break;
+    }
+    acc = 0.0;
+    for (int j = tid; j < cnt; j += RT) {
+      double p[NX];
+#pragma unroll
+      for (int c = 0; c < NX; ++c) p[c] = P.p[c * n + lo + j];
+#pragma unroll
+      for (int c = 0; c < NX; ++c) {
+        sd[c * per + j] = fma(alpha, p[c], sd[c * per + j]);
+        const double r = fma(-alpha, sq[c * per + j], sr[c * per + j]);
+        sr[c * per + j] = r;
+        acc += r * sm[c * per + j] * r;
+      }
+    }
+    double rz2 = 0.0;
+    if (!(met = meet_sum64(M, acc, cnt, rz2))) break;
+    iters += 1;
+    if (tid == 0) {
+      s_step = rz2 / rz;
+      s_go = rz2 != 0.0 && isfinite(rz2);
+      if (!isfinite(rz2)) nonfinite = 1;
+      rz = rz2;
+    }
+    __syncthreads();
+    if (!s_go) {
+      active = 0;
+      break;
+    }
+  }
+  if (!met) {
+    if (tid == 0) s->timeout = 1;
+    return;
+  }
+  for (int j = tid; j < cnt; j += RT) {
+#pragma unroll
+    for (int c = 0; c < NX; ++c) P.d[c * n + lo + j] = sd[c * per + j];
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    s->rz = rz;
+    s->pq = pq;
+    s->pcg_iters += iters;
+    if (!active) s->pcg_active = 0;
+    if (nonfinite) s->nonfinite = 1;
+    sync->meetings = M.base + M.meetings * gridDim.x;
+    sync->sums = M.sums % 3u;
+  }
+}
+
+// E(x) (mode 0), or E(x + delta) and |F(x) + J(x) delta|^2 (mode 1: cos / sin at
+// x are those of this outer iteration's PCGInit).
+__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_mesh_energy(P64 P, int mode, int hist_idx) {
   Scalars* s = P.s;
   if (mode == 1 && s->done) return;
   const long long n = P.n;
-  const double sw = P.s_w;
   double e0 = 0.0, e1 = 0.0;
   FOR_ELEMENTS(P, v) {
-    double cs[6], cs2[6], ev[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int a = 0; a < 3; ++a) sincos(P.x[(3 + a) * n + v], &cs[2 * a + 1], &cs[2 * a]);
+    double cs[6], R[3][3], R2[3][3], wd[3] = {0.0, 0.0, 0.0}, ev[3] = {0.0, 0.0, 0.0};
     if (mode == 1) {
-      for (int c = 0; c < 6; ++c) ev[c] = P.d[c * n + v];
-      for (int a = 0; a < 3; ++a) sincos(P.x[(3 + a) * n + v] + ev[3 + a], &cs2[2 * a + 1], &cs2[2 * a]);
+      double cs2[6], ea[3];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) cs[k] = P.cs[k * n + v];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        ev[c] = P.d[c * n + v];
+        ea[c] = P.d[(3 + c) * n + v];
+        sincos(P.x[(3 + c) * n + v] + ea[c], &cs2[2 * c + 1], &cs2[2 * c]);
+      }
+      rot_matrix64(cs2, R2);
+      angular_velocity64(Axes64{cs[2], cs[3], cs[4], cs[5]}, ea[0], ea[1], ea[2], wd);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) sincos(P.x[(3 + c) * n + v], &cs[2 * c + 1], &cs[2 * c]);
     }
+    rot_matrix64(cs, R);
     const double xv[3] = {P.x[v], P.x[n + v], P.x[2 * n + v]};
     const double uv[3] = {P.c[v], P.c[n + v], P.c[2 * n + v]};
+    double se = 0.0, sl = 0.0;
     for (int e = P.orow[v]; e < P.orow[v + 1]; ++e) {
       const int b = P.oe1[e];
-      const double wv[3] = {uv[0] - P.c[b], uv[1] - P.c[n + b], uv[2] - P.c[2 * n + b]};
-      const RotVT<double> R =
-          rot_apply_cs<double>(cs[0], cs[1], cs[2], cs[3], cs[4], cs[5], wv[0], wv[1], wv[2]);
-      double f[3];
-      for (int c = 0; c < 3; ++c) f[c] = sw * ((xv[c] - P.x[c * n + b]) + wv[c] - R.rv[c]);
+      double wv[3], y[3], f[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) wv[c] = uv[c] - P.c[c * n + b];
+      mat_vec64(R, wv, y);
       if (mode == 0) {
-        e0 += f[0] * f[0] + f[1] * f[1] + f[2] * f[2];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          f[c] = (xv[c] - P.x[c * n + b]) + wv[c] - y[c];
+          se = fma(f[c], f[c], se);
+        }
         continue;
       }
-      const RotVT<double> R2 =
-          rot_apply_cs<double>(cs2[0], cs2[1], cs2[2], cs2[3], cs2[4], cs2[5], wv[0], wv[1], wv[2]);
+      double y2[3], l[3];
+      mat_vec64(R2, wv, y2);
+#pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const double ed = ev[c] - P.d[c * n + b];
-        const double t = sw * ((xv[c] - P.x[c * n + b] + ed) + wv[c] - R2.rv[c]);
-        const double l = f[c] + sw * (ed - (R.g[0][c] * ev[3] + R.g[1][c] * ev[4] + R.g[2][c] * ev[5]));
-        e0 += t * t;
-        e1 += l * l;
+        const double ed = ev[c] - P.d[c * n + b], dx = xv[c] - P.x[c * n + b];
+        const double t = (dx + ed) + wv[c] - y2[c];
+        se = fma(t, t, se);
+        l[c] = (dx + wv[c] - y[c]) + ed;
       }
+      sub_cross64(l, wd, y);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) sl = fma(l[c], l[c], sl);
     }
+    e0 = fma(P.w_reg, se, e0);
+    e1 = fma(P.w_reg, sl, e1);
     const int h = P.hslot[v];
     if (h >= 0) {
       for (int c = 0; c < 3; ++c) {
         const double f = P.s_f * (xv[c] + ev[c] - P.htgt[3 * h + c]);
-        e0 += f * f;
-        e1 += f * f;
+        e0 = fma(f, f, e0);
+        e1 = fma(f, f, e1);
       }
     }
   }
@@ -739,7 +1105,7 @@ __global__ void __launch_bounds__(NT) k64_mesh_energy(P64 P, int mode, int hist_
 // Float64 multiply-add throughput probe: 8 independent dependency chains per
 // thread, enough blocks to fill every SM; the result is consumed so the
 // chains are not removed.
-__global__ void __launch_bounds__(NT) k64_fma_probe(double* out, int iters, double a, double b) {
+__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_fma_probe(double* out, int iters, double a, double b) {
   double v[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) v[k] = 1e-3 * (threadIdx.x + k);
@@ -767,6 +1133,8 @@ struct opt_problem_f64 {
   double* d_Ehist = nullptr;
   int Ehist_cap = 0;
   double* d_pin = nullptr;      // apply hook: caller p copied here (nx planes)
+  ResidentSync* d_rsync = nullptr;   // resident PCG loop (NULL: launches per phase)
+  int loop_blocks = 0, loop_per = 0, loop_smem = 0;
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t gexec = nullptr;
   std::vector<double> gkey;
@@ -870,6 +1238,47 @@ opt_status plan_common(opt_problem_f64* pb, const std::vector<double>& consts, c
   return OPT_OK;
 }
 
+const void* loop_kernel(int kind) {
+  return kind == F64_WARP ? (const void*)k64_pcg_loop<Warp64>
+                          : kind == F64_POISSON ? (const void*)k64_pcg_loop<Poisson64>
+                                                : (const void*)k64_pcg_loop<Mesh64>;
+}
+
+// Plans the resident PCG loop where a block's share of r, q, delta and M^-1 fits
+// in shared memory (warp 360k pixels, Poisson 270k, mesh 180k vertices).
+opt_status plan_loop(opt_problem_f64* pb) {
+  int dev = 0, coop = 0, optin = 0, per_sm = 0;
+  CK64(cudaGetDevice(&dev));
+  CK64(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+  CK64(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  const void* k = loop_kernel(pb->kind);
+  cudaFuncAttributes fa;
+  CK64(cudaFuncGetAttributes(&fa, k));
+  const int room = optin - (int)fa.sharedSizeBytes;
+  const int sms = std::min(pb->sms, RES_MAX_BLOCKS);
+  const long long share = std::max<long long>(64, (pb->hp.n + sms - 1) / sms);
+  const long long per = (share + 31) / 32 * 32, bytes = per * 4 * pb->nx * (long long)sizeof(double);
+  if (!coop || bytes > room) return OPT_OK;
+  CK64(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, room));
+  CK64(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, RT, (size_t)bytes));
+  if (per_sm < 1) return OPT_OK;
+  pb->loop_per = (int)per;
+  pb->loop_blocks = (int)((pb->hp.n + per - 1) / per);
+  pb->loop_smem = (int)bytes;
+  CKS64(alloc64(pb, &pb->d_rsync, 1));
+  CK64(cudaMemset(pb->d_rsync, 0, sizeof(ResidentSync)));
+  CK64(cudaMemset(pb->d_rsync->slot, 0xff, sizeof(pb->d_rsync->slot)));
+  return OPT_OK;
+}
+
+opt_status launch_loop(opt_problem_f64* pb, const P64& P, cudaStream_t st, int inner) {
+  P64 arg = P;
+  void* args[] = {&arg, &pb->d_rsync, &pb->loop_per, &inner};
+  CK64(cudaLaunchCooperativeKernel(loop_kernel(pb->kind), dim3(pb->loop_blocks), dim3(RT), args,
+                                   (size_t)pb->loop_smem, st));
+  return OPT_OK;
+}
+
 // Handle slots: OPT_ERR_INVALID_ARG on an index outside [0, n) or a repeat.
 opt_status handle_slots(const int32_t* d_idx, int nh, long long n, std::vector<int>& hslot, std::vector<int>& hidx) {
   hslot.assign((size_t)n, -1);
@@ -893,7 +1302,10 @@ void k_rot(opt_problem_f64* pb, cudaStream_t st) {
 void k_init(opt_problem_f64* pb, const P64& P, cudaStream_t st, int k, double dmin, double dmax) {
   if (pb->kind == F64_WARP) k64_warp_init<<<pb->nblk, NT, 0, st>>>(P, k, dmin, dmax);
   else if (pb->kind == F64_POISSON) k64_poisson_init<<<pb->nblk, NT, 0, st>>>(P, k, dmin, dmax);
-  else k64_mesh_init<<<pb->nblk, NT, 0, st>>>(P, k, dmin, dmax);
+  else {
+    k64_mesh_edges<<<pb->nblk, NT, 0, st>>>(P);
+    k64_mesh_init<<<pb->nblk, NT, 0, st>>>(P, k, dmin, dmax);
+  }
 }
 // applyJTJ of PCG iteration i: the direction update (from the second
 // iteration on; PCGInit writes the first direction), then q = A p
@@ -903,9 +1315,10 @@ void k_apply(opt_problem_f64* pb, const P64& P, cudaStream_t st, int i) {
     else if (pb->kind == F64_POISSON) k64_direction<4><<<pb->nblk, NT, 0, st>>>(P);
     else k64_direction<6><<<pb->nblk, NT, 0, st>>>(P);
   }
-  if (pb->kind == F64_WARP) k64_warp_apply<<<pb->nblk, NT, 0, st>>>(P);
-  else if (pb->kind == F64_POISSON) k64_poisson_apply<<<pb->nblk, NT, 0, st>>>(P);
-  else k64_mesh_apply<<<pb->nblk, NT, 0, st>>>(P);
+  if (pb->kind == F64_MESH && P.pin) k64_mesh_records<<<pb->nblk, NT, 0, st>>>(P);
+  if (pb->kind == F64_WARP) k64_apply<Warp64><<<pb->nblk, NT, 0, st>>>(P);
+  else if (pb->kind == F64_POISSON) k64_apply<Poisson64><<<pb->nblk, NT, 0, st>>>(P);
+  else k64_apply<Mesh64><<<pb->nblk, NT, 0, st>>>(P);
 }
 void k_update(opt_problem_f64* pb, const P64& P, cudaStream_t st) {
   if (pb->kind == F64_WARP) k64_update<3><<<pb->nblk, NT, 0, st>>>(P);
@@ -952,9 +1365,13 @@ opt_status enqueue_solve64(opt_problem_f64* pb, const opt_solve_params& p, bool 
   for (int k = 0; k < p.outer; ++k) {
     k_rot(pb, st);
     k_init(pb, P, st, k, p.diag_min, p.diag_max);
-    for (int i = 0; i < p.inner; ++i) {
-      k_apply(pb, P, st, i);
-      k_update(pb, P, st);
+    if (pb->d_rsync && p.inner > 0) {
+      CKS64(launch_loop(pb, P, st, p.inner));
+    } else {
+      for (int i = 0; i < p.inner; ++i) {
+        k_apply(pb, P, st, i);
+        k_update(pb, P, st);
+      }
     }
     if (!lm) {
       k64_step<<<pb->nblk, NT, 0, st>>>(P, 0);
@@ -1037,6 +1454,12 @@ opt_status run_solve64(opt_problem_f64* pb, const opt_solve_params* prm_in, opt_
     CK64(cudaEventElapsedTime(&ms, pb->ev0, pb->ev1));
     rep->ms = ms;
   }
+  if (s.timeout) {
+    // blocks gave up at different meetings: back to empty slots
+    CK64(cudaMemset(pb->d_rsync, 0, sizeof(ResidentSync)));
+    CK64(cudaMemset(pb->d_rsync->slot, 0xff, sizeof(pb->d_rsync->slot)));
+    return OPT_ERR_TIMEOUT;
+  }
   if (s.nonfinite) return OPT_ERR_NUMERIC;
   return OPT_OK;
 }
@@ -1065,6 +1488,7 @@ opt_status hook_init64(opt_problem_f64* pb, double lambda, double* jtf, double* 
 }
 
 opt_status finish_create64(std::unique_ptr<opt_problem_f64>& pb, opt_problem_f64** out) {
+  CKS64(plan_loop(pb.get()));
   CK64(cudaDeviceSynchronize());
   *out = pb.release();
   return OPT_OK;
@@ -1205,7 +1629,9 @@ opt_status opt_problem_create_graph_f64(const opt_graph_desc_f64* d, const opt_s
   CKS64(upload64(pb.get(), &c2, irow));
   CKS64(upload64(pb.get(), &d2, isrc));
   CKS64(upload64(pb.get(), &e2, ieid));
-  CKS64(alloc64(pb.get(), &P.G, 9 * (size_t)E));            // dR/dA_m w per directed edge
+  CKS64(alloc64(pb.get(), &P.G, 4 * (size_t)E));
+  CKS64(alloc64(pb.get(), &P.rec, 6 * (size_t)V));
+  P.sym = orow == irow && oe1 == isrc;
   P.orow = a;
   P.oe1 = b;
   P.irow = c2;

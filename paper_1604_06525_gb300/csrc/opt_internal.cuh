@@ -270,7 +270,7 @@ struct ResidentSync {
   unsigned int counter;         // arrivals at meetings, ever growing
   unsigned int pad0[31];
   unsigned int meetings;        // the counter's value between launches
-  unsigned int sums;            // sums done so far (modulo the three sets)
+  unsigned int sums;            // sums done so far (modulo the sets / tags of the loop that uses them)
   unsigned int pad1[30];
   unsigned long long slot[3][RES_MAX_BLOCKS][16];   // a cache line each
 };
@@ -669,13 +669,11 @@ __device__ __forceinline__ float minv_entry(float dg, float lam, float dmin, flo
 // ARAP mesh rotation (Fig. 25 Rotate3D, read as Rz(az) Ry(ay) Rx(ax))
 // ---------------------------------------------------------------------------
 // Rotation R = Rz(c) Ry(b) Rx(a) applied to v, and its three angle
-// derivatives applied to v (float32 kernels: RotV; float64 solver: RotVT<double>).
-template <typename T>
-struct RotVT {
-  T rv[3];
-  T g[3][3];        // g[m] = dR/dA_m v
+// derivatives applied to v (the materialized Jacobian).
+struct RotV {
+  float rv[3];
+  float g[3][3];    // g[m] = dR/dA_m v
 };
-using RotV = RotVT<float>;
 
 __device__ __forceinline__ RotV rot_apply(float ax, float ay, float az, float vx, float vy, float vz) {
   float sa, ca, sb, cb, sc, cc;
@@ -706,30 +704,6 @@ __device__ __forceinline__ RotV rot_apply(float ax, float ay, float az, float vx
   o.g[2][0] = -sc * y0 - cc * y1;
   o.g[2][1] = cc * y0 - sc * y1;
   o.g[2][2] = 0.f;
-  return o;
-}
-
-// Same as rot_apply with the angles' cos / sin given.
-template <typename T>
-__device__ __forceinline__ RotVT<T> rot_apply_cs(T ca, T sa, T cb, T sb, T cc, T sc, T vx, T vy, T vz) {
-  const T w0 = vx, w1 = ca * vy - sa * vz, w2 = sa * vy + ca * vz;
-  const T wd1 = -sa * vy - ca * vz, wd2 = ca * vy - sa * vz;
-  const T y0 = cb * w0 + sb * w2, y1 = w1, y2 = -sb * w0 + cb * w2;
-  const T yb0 = -sb * w0 + cb * w2, yb2 = -cb * w0 - sb * w2;
-  const T ya0 = sb * wd2, ya1 = wd1, ya2 = cb * wd2;
-  RotVT<T> o;
-  o.rv[0] = cc * y0 - sc * y1;
-  o.rv[1] = sc * y0 + cc * y1;
-  o.rv[2] = y2;
-  o.g[0][0] = cc * ya0 - sc * ya1;
-  o.g[0][1] = sc * ya0 + cc * ya1;
-  o.g[0][2] = ya2;
-  o.g[1][0] = cc * yb0;
-  o.g[1][1] = sc * yb0;
-  o.g[1][2] = yb2;
-  o.g[2][0] = -sc * y0 - cc * y1;
-  o.g[2][1] = cc * y0 - sc * y1;
-  o.g[2][2] = T(0);
   return o;
 }
 

@@ -32,14 +32,13 @@
 // alpha and beta are the same and with them every iterate.  (Only the mesh
 // energies' records with RES_Z carry w = w(z) + beta w(p_old) in place of w(p).)
 //
-// Slots: three sets, used in turn.  A slot holds kEmpty until its block stores the
-// sum of an exchange; a block that has finished sum k empties its slot of sum k
-// - 1 (every block has read it: all have arrived at k), which is next used at k +
-// 2; by then the emptying is visible to whoever waits, since the store of sum k + 1
-// lies in between.  The counts go on from launch to launch (sync->sums,
-// sync->meetings).  Every wait is bounded (1 s); a block that gives up flags
-// s->timeout and returns, the others run into their own limit, and the host
-// resets the slots.
+// Slots: two sets, used in turn; the two lowest bits of a stored pair's low part
+// (2^-46 of the sum) say which sum it belongs to, so a slot needs no emptying and a
+// stale one is never taken for the next: a block stores sum k + 2 only after sum k
+// + 1, which every block reaches after reading those of k.  The counts go on from
+// launch to launch (sync->sums, sync->meetings).  Every wait is bounded (1 s); a
+// block that gives up flags s->timeout and returns, the others run into their own
+// limit, and the host resets the slots.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -48,33 +47,15 @@
 #include "graph2d_algebra.cuh"
 #include "grid_algebra.cuh"
 #include "mesh_algebra.cuh"
+#include "meet.cuh"
 #include "opt_launch.h"
 
 namespace optgb {
 
 namespace {
 
-constexpr int RT = 512;               // threads per block, one block per SM
-constexpr int RW = RT / 32;
 constexpr int CELL = 256;             // grids: 32 x 8 pixels
-constexpr unsigned long long kEmpty = ~0ull;
 
-__device__ __forceinline__ unsigned ld_relaxed(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ void red_add(unsigned* p, unsigned v) {
-  asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 __device__ __forceinline__ unsigned cluster_rank() {
   unsigned r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -92,27 +73,11 @@ __device__ __forceinline__ void st_cluster(unsigned long long* local, unsigned r
   asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
 }
 __device__ __forceinline__ unsigned long long pack(F2 a) {
-  const unsigned long long b =
-      (unsigned long long)__float_as_uint(a.hi) | ((unsigned long long)__float_as_uint(a.lo) << 32);
-  return b == kEmpty ? b - 1 : b;     // a NaN either way
+  return (unsigned long long)__float_as_uint(a.hi) | ((unsigned long long)__float_as_uint(a.lo) << 32);
 }
 __device__ __forceinline__ F2 unpack(unsigned long long b) {
   return F2{__uint_as_float((unsigned)b), __uint_as_float((unsigned)(b >> 32))};
 }
-
-// A wait's time limit: called now and then while waiting.
-__device__ __forceinline__ bool waited_too_long(int spin, unsigned long long& t0) {
-  if ((spin & 255) != 255) return false;
-  const unsigned long long now = global_ns();
-  if (t0 == 0) t0 = now;
-  return now - t0 > kBarrierLimitNs;
-}
-
-// What a launch knows of the device-wide exchanges: those done so far, by kind.
-struct Meet {
-  ResidentSync* sy;
-  unsigned base, meetings, sums;
-};
 
 // Meeting of all blocks: what any thread wrote to global memory before is
 // visible to every thread of every block after.  Returns false if a block did
@@ -123,21 +88,7 @@ __device__ __forceinline__ bool meet(Meet& M) {
     cluster_meet();
     return true;
   }
-  __shared__ int s_ok;
-  __syncthreads();
-  M.meetings += 1;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    red_add(&M.sy->counter, 1u);
-    const unsigned want = M.base + M.meetings * gridDim.x;
-    unsigned long long t0 = 0;
-    int ok = 1;
-    for (int spin = 0; ok && (int)(ld_relaxed(&M.sy->counter) - want) < 0; ++spin) ok = !waited_too_long(spin, t0);
-    __threadfence();
-    s_ok = ok;
-  }
-  __syncthreads();
-  return s_ok != 0;
+  return meet_device(M);
 }
 
 // The same with the total of every thread's pair, equal in every thread of
@@ -156,8 +107,8 @@ __device__ __forceinline__ bool meet_sum(Meet& M, F2 acc, F2& total) {
     for (int o = RW / 2; o > 0; o >>= 1) v = f2_shfl_xor_add(v, o);
     return v;
   };
-  const unsigned k = M.sums;
   M.sums += 1;
+  const unsigned k = M.sums;
   if (CL) {
     __shared__ unsigned long long part[2][RES_CLUSTER];
     const unsigned n = gridDim.x;
@@ -175,28 +126,28 @@ __device__ __forceinline__ bool meet_sum(Meet& M, F2 acc, F2& total) {
     constexpr int NP = RES_MAX_BLOCKS / 32;      // polling warps, one slot a thread
     __shared__ unsigned long long sg[NP];
     __shared__ int s_ok[NP];
-    auto slot = [&](unsigned set, int b) { return &M.sy->slot[set % 3][b][0]; };
     if (w == 0) {
       const F2 v = block_total();
       if (FENCE) __threadfence();
-      if (l == 0) st_relaxed(slot(k, blockIdx.x), pack(v));
+      if (l == 0)
+        st_relaxed(&M.sy->slot[k & 1][blockIdx.x][0],
+                   (pack(v) & ~(3ull << 32)) | ((unsigned long long)(k & 3) << 32));
     }
     if (w < NP) {
       const bool on = threadIdx.x < gridDim.x;
-      const unsigned long long* p = slot(k, on ? threadIdx.x : 0);
+      const unsigned long long* p = &M.sy->slot[k & 1][on ? threadIdx.x : 0][0];
       unsigned long long b, t0 = 0;
       int ok = 1;
-      for (int spin = 0; (b = ld_relaxed(p)) == kEmpty && ok; ++spin) ok = !waited_too_long(spin, t0);
+      for (int spin = 0; (((b = ld_relaxed(p)) >> 32) & 3) != (k & 3) && ok; ++spin) ok = !waited_too_long(spin, t0);
       if (FENCE) __threadfence();
       ok = __all_sync(0xffffffffu, ok);
-      const F2 v = warp_sum_f2(on ? unpack(b) : f2_zero());
+      const F2 v = warp_sum_f2(on ? unpack(b & ~(3ull << 32)) : f2_zero());
       if (l == 0) {
         sg[w] = pack(v);
         s_ok[w] = ok;
       }
     }
     __syncthreads();
-    if (threadIdx.x == 0) st_relaxed(slot(k + 2, blockIdx.x), kEmpty);
     total = unpack(sg[0]);
     int ok = s_ok[0];
 #pragma unroll
@@ -1033,7 +984,7 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
     if (nonfinite) s->nonfinite = 1;
     if (!CL) {
       sync->meetings = M.base + M.meetings * gridDim.x;
-      sync->sums = M.sums % 3u;
+      sync->sums = M.sums & 3u;
     }
   }
 }
