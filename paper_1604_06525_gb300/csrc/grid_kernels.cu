@@ -55,16 +55,13 @@ __device__ __forceinline__ int tile_id(const GridProb& pr, int tc) {
 // ARAP image warping
 // ---------------------------------------------------------------------------
 struct WarpStage {
-  float a[HH][HW];     // dx  (init / energy) or p.x (apply)
-  float b[HH][HW];     // dy  or p.y
-  float t[HH][HW];     // theta (energy) or p.theta (apply)
+  float a[HH][HW];     // dx (init) or p.x (apply)
+  float b[HH][HW];     // dy or p.y
+  float t[HH][HW];     // p.theta (apply)
   float cs[HH][HW];    // cos theta
   float sn[HH][HW];    // sin theta
   float ux[HH][HW];
   float uy[HH][HW];
-  float ea[HH][HW];    // energy trial: delta x / delta y / delta theta
-  float eb[HH][HW];
-  float et[HH][HW];
   unsigned char v[HH][HW];
 };
 
@@ -1710,103 +1707,16 @@ __global__ void __launch_bounds__(NT, WARP_INIT_WIDE_MINB) k_warp_init_wide(cons
   if (tma_ready(pr, &sm)) k_warp_init_wide_body<MASK, CSN>(sm, ch, pr, tiles, part, k_outer, dmin, dmax);
 }
 
-// E(x) (mode 0) or E(x + delta) and |F(x) + J(x) delta|^2 (mode 1).
-__global__ void __launch_bounds__(NT) k_warp_energy(const GridProb* __restrict__ probs,
-                                                    const Chunk* __restrict__ chunks,
-                                                    const int* __restrict__ tiles,
-                                                    double* __restrict__ part, int mode,
-                                                    int hist_idx) {
-  const Chunk ch = chunks[blockIdx.x];
-  const GridProb pr = probs[ch.prob];
-  pdl_begin();
+// End of an energy kernel: the last block of the problem stores the sums.
+template <int MODE>
+__device__ __forceinline__ void energy_finish(const GridProb& pr, double* __restrict__ part, F2 acc0, F2 acc1,
+                                              int hist_idx) {
   Scalars* s = pr.s;
-  if (mode == 1 && s->done) return;
-  __shared__ WarpStage st;
-  const long long pl = pr.plane;
-  const int P = pr.P, W = pr.W, H = pr.H;
-  const float sw = pr.s_w, sf = pr.s_f;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  F2 acc0 = f2_zero(), acc1 = f2_zero();
-  const int nsub = pr.tw / TW;
-  for (int ts = ch.begin * nsub; ts < ch.end * nsub; ++ts) {
-    const int tc = tiles[ts / nsub];
-    const int x0 = tile_x0(tc, pr.tw) + TW * (ts % nsub), y0 = tile_y0(tc);
-    for (int hc = threadIdx.x; hc < HW * HH; hc += NT) {
-      const int hy = hc / HW, hx = hc - hy * HW;
-      const int gx = x0 - 1 + hx, gy = y0 - 1 + hy;
-      float dx = 0.f, dy = 0.f, th = 0.f, ux = 0.f, uy = 0.f, ex = 0.f, ey = 0.f, et = 0.f;
-      unsigned char v = 0;
-      if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
-        const long long i = (long long)gy * P + gx;
-        dx = pr.x[i]; dy = pr.x[pl + i]; th = pr.x[2 * pl + i];
-        ux = pr.c[i]; uy = pr.c[pl + i];
-        if (mode == 1) { ex = pr.d[i]; ey = pr.d[pl + i]; et = pr.d[2 * pl + i]; }
-        v = pr.mask ? (pr.mask[i] == 0) : 1;
-      }
-      float sn, cs;
-      sincosf(th, &sn, &cs);
-      st.a[hy][hx] = dx; st.b[hy][hx] = dy; st.t[hy][hx] = th;
-      st.cs[hy][hx] = cs; st.sn[hy][hx] = sn;
-      st.ux[hy][hx] = ux; st.uy[hy][hx] = uy;
-      st.ea[hy][hx] = ex; st.eb[hy][hx] = ey; st.et[hy][hx] = et;
-      st.v[hy][hx] = v;
-    }
-    __syncthreads();
-    const int gx = x0 + tx, gy = y0 + ty;
-    if (gx < W && gy < H && st.v[ty + 1][tx + 1]) {
-      const int lx = tx + 1, ly = ty + 1;
-      const long long i = (long long)gy * P + gx;
-      const float dxi = st.a[ly][lx], dyi = st.b[ly][lx];
-      const float ci = st.cs[ly][lx], si = st.sn[ly][lx];
-      const float uxi = st.ux[ly][lx], uyi = st.uy[ly][lx];
-      const float exi = st.ea[ly][lx], eyi = st.eb[ly][lx], eti = st.et[ly][lx];
-      float c2 = 0.f, s2 = 0.f;
-      if (mode == 1) sincosf(st.t[ly][lx] + eti, &s2, &c2);
-      float e0 = 0.f, e1 = 0.f;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int nx = lx + dx4(k), ny = ly + dy4(k);
-        if (!st.v[ny][nx]) continue;
-        const float vx = uxi - st.ux[ny][nx], vy = uyi - st.uy[ny][nx];
-        const float ddx = dxi - st.a[ny][nx], ddy = dyi - st.b[ny][nx];
-        const float rx = sw * (ddx + (vx - (ci * vx - si * vy)));
-        const float ry = sw * (ddy + (vy - (si * vx + ci * vy)));
-        if (mode == 0) {
-          e0 += rx * rx + ry * ry;
-        } else {
-          const float edx = exi - st.ea[ny][nx], edy = eyi - st.eb[ny][nx];
-          const float tx_ = sw * ((ddx + edx) + (vx - (c2 * vx - s2 * vy)));
-          const float ty_ = sw * ((ddy + edy) + (vy - (s2 * vx + c2 * vy)));
-          e0 += tx_ * tx_ + ty_ * ty_;
-          const float lx_ = rx + sw * edx + (-sw * (-si * vx - ci * vy)) * eti;
-          const float ly_ = ry + sw * edy + (-sw * (ci * vx - si * vy)) * eti;
-          e1 += lx_ * lx_ + ly_ * ly_;
-        }
-      }
-      const int tid = tile_id(pr, tc);
-      for (int h = pr.hbeg[tid]; h < pr.hbeg[tid + 1]; ++h) {
-        if (pr.hpix[h] == (int)i) {
-          const float fx = sf * (dxi - pr.htgt[2 * h]);
-          const float fy = sf * (dyi - pr.htgt[2 * h + 1]);
-          if (mode == 0) {
-            e0 += fx * fx + fy * fy;
-          } else {
-            const float gx2 = fx + sf * exi, gy2 = fy + sf * eyi;   // linear in d: trial == model
-            e0 += gx2 * gx2 + gy2 * gy2;
-            e1 += gx2 * gx2 + gy2 * gy2;
-          }
-        }
-      }
-      f2_add(acc0, e0);
-      f2_add(acc1, e1);
-    }
-    __syncthreads();
-  }
   if (publish_partials(part, blockIdx.x, acc0, acc1, &s->counter, pr.chunk_end - pr.chunk_begin)) {
     double a, b;
     gather_partials(part, pr.chunk_begin, pr.chunk_end, &s->counter, a, b);
     if (threadIdx.x == 0) {
-      if (mode == 0) {
+      if (MODE == 0) {
         s->E = a;
         const int k = hist_idx >= 0 ? hist_idx : (hist_idx == -1 ? s->outer_done : -1);
         if (pr.Ehist && k >= 0) pr.Ehist[k] = a;
@@ -1819,13 +1729,160 @@ __global__ void __launch_bounds__(NT) k_warp_energy(const GridProb* __restrict__
   }
 }
 
+// E(x) (MODE 0) or E(x + delta) and |F(x) + J(x) delta|^2 (MODE 1).  A quad of
+// four pixels per thread straight from the planes: a residual needs of its far
+// end only displacement, rest position and delta, so cos / sin are evaluated once
+// per pixel and nothing is staged (staging tiles with the angles of their halo:
+// 4096^2 462 -> TBD us, 1411 x 1003 LM 51 -> TBD us).
+struct EnergyRow {
+  float4 x, y, ux, uy, ex, ey;
+  unsigned v;                     // bit k: pixel k exists and is not excluded
+};
+template <int MODE>
+__device__ __forceinline__ void energy_row(const GridProb& pr, long long i, int gx, EnergyRow& r) {
+  const long long pl = pr.plane;
+  r.x = *reinterpret_cast<const float4*>(pr.x + i);
+  r.y = *reinterpret_cast<const float4*>(pr.x + pl + i);
+  r.ux = ld4(pr.c + i);
+  r.uy = ld4(pr.c + pl + i);
+  if (MODE == 1) {
+    r.ex = *reinterpret_cast<const float4*>(pr.d + i);
+    r.ey = *reinterpret_cast<const float4*>(pr.d + pl + i);
+  }
+  const unsigned m = pr.mask ? *reinterpret_cast<const unsigned*>(pr.mask + i) : 0u;
+  r.v = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (gx + k < pr.W && ((m >> (8 * k)) & 0xffu) == 0u) r.v |= 1u << k;
+}
+// the pixel at i (a quad's left / right neighbour)
+struct EnergyPix {
+  float x, y, ux, uy, ex, ey;
+};
+template <int MODE>
+__device__ __forceinline__ bool energy_side(const GridProb& pr, long long i, bool in, EnergyPix& p) {
+  p = EnergyPix{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  if (!in || (pr.mask && pr.mask[i] != 0)) return false;
+  const long long pl = pr.plane;
+  p.x = pr.x[i];
+  p.y = pr.x[pl + i];
+  p.ux = __ldg(pr.c + i);
+  p.uy = __ldg(pr.c + pl + i);
+  if (MODE == 1) {
+    p.ex = pr.d[i];
+    p.ey = pr.d[pl + i];
+  }
+  return true;
+}
+template <int MODE>
+__global__ void __launch_bounds__(NT, 2) k_warp_energy(const GridProb* __restrict__ probs,
+                                                       const Chunk* __restrict__ chunks,
+                                                       const int* __restrict__ tiles,
+                                                       double* __restrict__ part, int hist_idx) {
+  const Chunk ch = chunks[blockIdx.x];
+  const GridProb pr = probs[ch.prob];
+  pdl_begin();
+  Scalars* s = pr.s;
+  if (MODE == 1 && s->done) return;
+  const long long pl = pr.plane;
+  const int P = pr.P, H = pr.H;
+  const float sw = pr.s_w, sf = pr.s_f;
+  F2 acc0 = f2_zero(), acc1 = f2_zero();
+  const int qrow = pr.tw / 4, qpt = qrow * TH;
+  const int nq = (ch.end - ch.begin) * qpt;
+  for (int u = threadIdx.x; u < nq; u += NT) {
+    const int tc = tiles[ch.begin + u / qpt];
+    const int q = u % qpt;
+    const int gx = tile_x0(tc, pr.tw) + 4 * (q % qrow), gy = tile_y0(tc) + q / qrow;
+    if (gy >= H || gx >= pr.W) continue;
+    const long long i = (long long)gy * P + gx;
+    EnergyRow o, up, dn;
+    energy_row<MODE>(pr, i, gx, o);
+    up.v = dn.v = 0;
+    if (gy > 0) energy_row<MODE>(pr, i - P, gx, up);
+    if (gy + 1 < H) energy_row<MODE>(pr, i + P, gx, dn);
+    EnergyPix lf, rt;
+    const bool has_l = energy_side<MODE>(pr, i - 1, gx > 0, lf);
+    const bool has_r = energy_side<MODE>(pr, i + 4, gx + 4 < pr.W, rt);
+    const float4 th = *reinterpret_cast<const float4*>(pr.x + 2 * pl + i);
+    const float4 et = MODE == 1 ? *reinterpret_cast<const float4*>(pr.d + 2 * pl + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    float e0[4] = {0.f, 0.f, 0.f, 0.f}, e1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (!((o.v >> k) & 1u)) continue;
+      float ci, si, c2 = 0.f, s2 = 0.f;
+      sincosf(cmp(th, k), &si, &ci);
+      const float eti = cmp(et, k);
+      if (MODE == 1) sincosf(cmp(th, k) + eti, &s2, &c2);
+      const float dxi = cmp(o.x, k), dyi = cmp(o.y, k), uxi = cmp(o.ux, k), uyi = cmp(o.uy, k);
+      const float exi = MODE == 1 ? cmp(o.ex, k) : 0.f, eyi = MODE == 1 ? cmp(o.ey, k) : 0.f;
+      auto edge = [&](float xj, float yj, float uxj, float uyj, float exj, float eyj) {
+        const float vx = uxi - uxj, vy = uyi - uyj;
+        const float ddx = dxi - xj, ddy = dyi - yj;
+        const float rx = sw * (ddx + (vx - (ci * vx - si * vy)));
+        const float ry = sw * (ddy + (vy - (si * vx + ci * vy)));
+        if (MODE == 0) {
+          e0[k] += rx * rx + ry * ry;
+        } else {
+          const float edx = exi - exj, edy = eyi - eyj;
+          const float tx = sw * ((ddx + edx) + (vx - (c2 * vx - s2 * vy)));
+          const float ty = sw * ((ddy + edy) + (vy - (s2 * vx + c2 * vy)));
+          e0[k] += tx * tx + ty * ty;
+          const float lx = rx + sw * edx + (-sw * (-si * vx - ci * vy)) * eti;
+          const float ly = ry + sw * edy + (-sw * (ci * vx - si * vy)) * eti;
+          e1[k] += lx * lx + ly * ly;
+        }
+      };
+      auto row = [&](const EnergyRow& r, int j) {
+        edge(cmp(r.x, j), cmp(r.y, j), cmp(r.ux, j), cmp(r.uy, j), MODE == 1 ? cmp(r.ex, j) : 0.f,
+             MODE == 1 ? cmp(r.ey, j) : 0.f);
+      };
+      if (k < 3) {
+        if ((o.v >> (k + 1)) & 1u) row(o, k < 3 ? k + 1 : 3);
+      } else if (has_r) {
+        edge(rt.x, rt.y, rt.ux, rt.uy, rt.ex, rt.ey);
+      }
+      if (k > 0) {
+        if ((o.v >> (k - 1)) & 1u) row(o, k > 0 ? k - 1 : 0);
+      } else if (has_l) {
+        edge(lf.x, lf.y, lf.ux, lf.uy, lf.ex, lf.ey);
+      }
+      if ((dn.v >> k) & 1u) row(dn, k);
+      if ((up.v >> k) & 1u) row(up, k);
+    }
+    const int tid = tile_id(pr, tc);
+    for (int h = pr.hbeg[tid]; h < pr.hbeg[tid + 1]; ++h) {
+      const long long kk = pr.hpix[h] - i;
+      if (kk < 0 || kk >= 4) continue;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (k != kk || !((o.v >> k) & 1u)) continue;
+        const float fx = sf * (cmp(o.x, k) - pr.htgt[2 * h]);
+        const float fy = sf * (cmp(o.y, k) - pr.htgt[2 * h + 1]);
+        if (MODE == 0) {
+          e0[k] += fx * fx + fy * fy;
+        } else {
+          const float gx2 = fx + sf * cmp(o.ex, k), gy2 = fy + sf * cmp(o.ey, k);   // linear in d: trial == model
+          e0[k] += gx2 * gx2 + gy2 * gy2;
+          e1[k] += gx2 * gx2 + gy2 * gy2;
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      f2_add(acc0, e0[k]);
+      if (MODE == 1) f2_add(acc1, e1[k]);
+    }
+  }
+  energy_finish<MODE>(pr, part, acc0, acc1, hist_idx);
+}
+
 // ---------------------------------------------------------------------------
 // Poisson image editing (4 channels, constant J)
 // ---------------------------------------------------------------------------
 struct PoissonStage {
-  float x[4][HH][HW];   // X (init / energy) or p (apply)
-  float g[4][HH][HW];   // guidance T (init / energy)
-  float e[4][HH][HW];   // delta (energy, mode 1)
+  float x[4][HH][HW];   // X
+  float g[4][HH][HW];   // guidance T
   unsigned char f[HH][HW];   // 0 = outside, 1 = fixed, 2 = free
 };
 
@@ -2724,80 +2781,91 @@ __global__ void k_pois_sdeg(int W, int H, int P, const uint8_t* __restrict__ mas
   }
 }
 
-__global__ void __launch_bounds__(NT) k_poisson_energy(const GridProb* __restrict__ probs,
-                                                       const Chunk* __restrict__ chunks,
-                                                       const int* __restrict__ tiles,
-                                                       double* __restrict__ part, int mode,
-                                                       int hist_idx) {
+// Poisson energies (the residual is linear: trial value and model agree), a quad
+// of pixels per thread straight from the planes (1024^2: 27 -> 16 us).
+template <int MODE>
+__global__ void __launch_bounds__(NT, 2) k_poisson_energy(const GridProb* __restrict__ probs,
+                                                          const Chunk* __restrict__ chunks,
+                                                          const int* __restrict__ tiles,
+                                                          double* __restrict__ part, int hist_idx) {
   const Chunk ch = chunks[blockIdx.x];
   const GridProb pr = probs[ch.prob];
   pdl_begin();
   Scalars* s = pr.s;
-  if (mode == 1 && s->done) return;
-  __shared__ PoissonStage st;
+  if (MODE == 1 && s->done) return;
   const long long pl = pr.plane;
   const int P = pr.P, W = pr.W, H = pr.H;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  F2 acc0 = f2_zero(), acc1 = f2_zero();
-  const int nsub = pr.tw / TW;
-  for (int ts = ch.begin * nsub; ts < ch.end * nsub; ++ts) {
-    const int tc = tiles[ts / nsub];
-    const int x0 = tile_x0(tc, pr.tw) + TW * (ts % nsub), y0 = tile_y0(tc);
-    for (int hc = threadIdx.x; hc < HW * HH; hc += NT) {
-      const int hy = hc / HW, hx = hc - hy * HW;
-      const int gx = x0 - 1 + hx, gy = y0 - 1 + hy;
-      unsigned char f = 0;
-      float xv[4] = {0.f, 0.f, 0.f, 0.f}, gv[4] = {0.f, 0.f, 0.f, 0.f}, ev[4] = {0.f, 0.f, 0.f, 0.f};
-      if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
-        const long long i = (long long)gy * P + gx;
-        f = poisson_flag(pr, i);
+  F2 acc = f2_zero();
+  const int qrow = pr.tw / 4, qpt = qrow * TH;
+  const int nq = (ch.end - ch.begin) * qpt;
+  for (int u = threadIdx.x; u < nq; u += NT) {
+    const int tc = tiles[ch.begin + u / qpt];
+    const int q = u % qpt;
+    const int gx = tile_x0(tc, pr.tw) + 4 * (q % qrow), gy = tile_y0(tc) + q / qrow;
+    if (gy >= H || gx >= W) continue;
+    const long long i = (long long)gy * P + gx;
+    const unsigned m = pr.mask ? *reinterpret_cast<const unsigned*>(pr.mask + i) : 0u;
+    unsigned v = 0, in = 0;         // bit k: pixel k is free / lies in the image
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          xv[c] = pr.x[c * pl + i];
-          gv[c] = pr.c[c * pl + i];
-          if (mode == 1 && f == 2) ev[c] = pr.d[c * pl + i];
-        }
+    for (int k = 0; k < 4; ++k)
+      if (gx + k < W) {
+        in |= 1u << k;
+        if (((m >> (8 * k)) & 0xffu) == 0u) v |= 1u << k;
       }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) { st.x[c][hy][hx] = xv[c]; st.g[c][hy][hx] = gv[c]; st.e[c][hy][hx] = ev[c]; }
-      st.f[hy][hx] = f;
+    if (!v) continue;
+    const bool hu = gy > 0, hd = gy + 1 < H, hl = gx > 0, hr = gx + 4 < W;
+    // a fixed pixel has no delta, whatever its slot holds
+    unsigned mu = 0, md = 0;
+    bool ml = false, mr = false;
+    if (MODE == 1 && pr.mask) {
+      if (hu) mu = *reinterpret_cast<const unsigned*>(pr.mask + i - P);
+      if (hd) md = *reinterpret_cast<const unsigned*>(pr.mask + i + P);
+      ml = hl && pr.mask[i - 1] != 0;
+      mr = hr && pr.mask[i + 4] != 0;
     }
-    __syncthreads();
-    const int gx = x0 + tx, gy = y0 + ty;
-    if (gx < W && gy < H && st.f[ty + 1][tx + 1] == 2) {
-      const int lx = tx + 1, ly = ty + 1;
-      float e0 = 0.f;
+    auto moved = [](const float4& d, unsigned fixed, int k) { return (fixed >> (8 * k)) & 0xffu ? 0.f : cmp(d, k); };
+    float e[4] = {0.f, 0.f, 0.f, 0.f};
+    // Y = X - T (+ delta): the residual of a pair is the difference of its Y
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float* __restrict__ x = pr.x + c * pl;
+      const float* __restrict__ t = pr.c + c * pl;
+      const float* __restrict__ d = pr.d + c * pl;
+      auto quad = [&](long long k, float4& X, float4& T, float4& D) {
+        X = *reinterpret_cast<const float4*>(x + k);
+        T = ld4(t + k);
+        D = MODE == 1 ? *reinterpret_cast<const float4*>(d + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+      };
+      float4 ox, ot, od, ux, ut, ud, bx, bt, bd;
+      quad(i, ox, ot, od);
+      quad(hu ? i - P : i, ux, ut, ud);
+      quad(hd ? i + P : i, bx, bt, bd);
+      const long long l = hl ? i - 1 : i, r = hr ? i + 4 : i + 3;
+      const float lx = x[l], lt = __ldg(t + l), ld_ = MODE == 1 && !ml ? d[l] : 0.f;
+      const float rx = x[r], rt = __ldg(t + r), rd = MODE == 1 && !mr ? d[r] : 0.f;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const int nx = lx + dx4(k), ny = ly + dy4(k);
-        if (!st.f[ny][nx]) continue;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          float r = (st.x[c][ly][lx] - st.x[c][ny][nx]) - (st.g[c][ly][lx] - st.g[c][ny][nx]);
-          if (mode == 1) r += st.e[c][ly][lx] - st.e[c][ny][nx];   // linear: trial == model
-          e0 += r * r;
+        if (!((v >> k) & 1u)) continue;
+        auto pair = [&](float xj, float tj, float dj) {
+          float f = (cmp(ox, k) - xj) - (cmp(ot, k) - tj);
+          if (MODE == 1) f += cmp(od, k) - dj;
+          e[k] = fmaf(f, f, e[k]);
+        };
+        if (k < 3) {
+          if ((in >> (k + 1)) & 1u) pair(cmp(ox, k + 1), cmp(ot, k + 1), moved(od, m, k + 1));
+        } else if (hr) {
+          pair(rx, rt, rd);
         }
-      }
-      f2_add(acc0, e0);
-      f2_add(acc1, e0);
-    }
-    __syncthreads();
-  }
-  if (publish_partials(part, blockIdx.x, acc0, acc1, &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    double a, b;
-    gather_partials(part, pr.chunk_begin, pr.chunk_end, &s->counter, a, b);
-    if (threadIdx.x == 0) {
-      if (mode == 0) {
-        s->E = a;
-        const int k = hist_idx >= 0 ? hist_idx : (hist_idx == -1 ? s->outer_done : -1);
-        if (pr.Ehist && k >= 0) pr.Ehist[k] = a;
-        if (!isfinite(a)) s->nonfinite = 1;
-      } else {
-        s->E_trial = a;
-        s->model = b;
+        if (k > 0) pair(cmp(ox, k - 1), cmp(ot, k - 1), moved(od, m, k - 1));
+        else if (hl) pair(lx, lt, ld_);
+        if (hd) pair(cmp(bx, k), cmp(bt, k), moved(bd, md, k));
+        if (hu) pair(cmp(ux, k), cmp(ut, k), moved(ud, mu, k));
       }
     }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) f2_add(acc, e[k]);
   }
+  energy_finish<MODE>(pr, part, acc, acc, hist_idx);
 }
 
 // ---------------------------------------------------------------------------
@@ -3111,10 +3179,9 @@ void launch_grid_csn(const GridLaunch& L) {
 }
 
 void launch_grid_energy(int kind, const GridLaunch& L, int mode, int hist_idx) {
-  if (kind == K_WARP)
-    launch_pdl(k_warp_energy, L.nchunks, NT, 0, L.stream, L.probs, L.chunks, L.tiles, L.part, mode, hist_idx);
-  else
-    launch_pdl(k_poisson_energy, L.nchunks, NT, 0, L.stream, L.probs, L.chunks, L.tiles, L.part, mode, hist_idx);
+  auto k = kind == K_WARP ? (mode ? k_warp_energy<1> : k_warp_energy<0>)
+                          : (mode ? k_poisson_energy<1> : k_poisson_energy<0>);
+  launch_pdl(k, L.nchunks, NT, 0, L.stream, L.probs, L.chunks, L.tiles, L.part, hist_idx);
 }
 
 void launch_pois_sdeg(int W, int H, int P, const uint8_t* mask, uint8_t* out, cudaStream_t st) {
