@@ -400,8 +400,9 @@ opt_status opt_batch_create(opt_problem* const* probs, int32_t n, opt_batch** ou
 /* Frees the batch (not its problems).  NULL is accepted. */
 opt_status opt_batch_destroy(opt_batch* batch);
 
-/* Work granularity: tiles_per_chunk consecutive 32x8 tiles of one problem per
- * block (0 = each problem's own default, about 8 blocks per SM per problem). */
+/* Work granularity: tiles_per_chunk consecutive tiles of one problem per block
+ * (0, the default: each problem's own default split, or coarser, so that the
+ * blocks of a launch are on the device at once). */
 opt_status opt_batch_set_chunking(opt_batch* batch, int32_t tiles_per_chunk);
 
 /* Autotuner: times one outer iteration (<= 4 PCG iterations) of the batch for

@@ -141,7 +141,7 @@ struct opt_batch {
   std::vector<GridGroup> grids;
   MeshGroup graphs[4];               // [0]: ARAP meshes, [1]: warps on graphs, [2]: volumes,
                                      // [3]: embedded deformation
-  int tiles_per_chunk = 0;          // 0 = per-problem default
+  int tiles_per_chunk = 0;          // 0 = default
   std::vector<void*> table_allocs;  // rebuilt with the chunking
   std::vector<void*> allocs;        // fixed for the batch's life
   Scalars** d_stab = nullptr;
@@ -173,8 +173,35 @@ namespace {
 
 bool is_grid_kind(int k) { return k == K_WARP || k == K_POISSON; }
 
+// Tiles per chunk of a group of grids: the fewest for which all chunks of the
+// group are on the device at once, two blocks per SM (the residency of the
+// wide-tile kernels).  A member's own split is for the device to itself -- one
+// tile per block up to 304 tiles -- and in a group every such block pays the
+// descriptor, the partial sums and its share of another wave: 96 warps of 32^2 to
+// 512^2, GN 3 x 10: 9.1 ms with the members' own splits, 6.5 ms so; at most 4 or 6
+// tiles per chunk 6.8 and 6.7 ms, two or four waves of smaller chunks 7.0 and 6.9 ms.
+// With so many members that one wave would take chunks half as large again as a
+// block's even share, a quarter of that share: the device then evens itself out.
+int one_wave_tiles(const std::vector<int>& ntiles, int blocks) {
+  const auto chunks = [&](int per) {
+    long long c = 0;
+    for (int t : ntiles) c += (t + per - 1) / per;
+    return c;
+  };
+  int lo = 1, hi = 1;
+  for (int t : ntiles) hi = std::max(hi, t);
+  while (lo < hi) {
+    const int mid = (lo + hi) / 2;
+    if (chunks(mid) <= blocks) hi = mid;
+    else lo = mid + 1;
+  }
+  long long total = 0;
+  for (int t : ntiles) total += t;
+  return 2ll * lo * blocks <= 3 * total || lo == 1 ? lo : std::max<int>(1, (int)(total / (4ll * blocks)));
+}
+
 // (Re)builds the combined work tables with `tpc` tiles per chunk (0 = each
-// member's own chunking).
+// member's own chunking, or one_wave_tiles() of its group where that is coarser).
 opt_status build_tables(opt_batch* b, int tpc) {
   cudaDeviceSynchronize();
   for (void* p : b->table_allocs) cudaFree(p);
@@ -187,7 +214,9 @@ opt_status build_tables(opt_batch* b, int tpc) {
   for (GridGroup& g : b->grids) {
     std::vector<GridProb> gp;
     std::vector<Chunk> chunks;
-    std::vector<int> tiles;
+    std::vector<int> tiles, nt;
+    for (int i : g.members) nt.push_back(b->probs[i]->ntiles);
+    const int wave = one_wave_tiles(nt, 2 * b->probs[0]->sms);
     for (size_t mi = 0; mi < g.members.size(); ++mi) {
       opt_problem* pb = b->probs[g.members[mi]];
       const std::vector<int>& t = pb->h_tiles;
@@ -197,6 +226,11 @@ opt_status build_tables(opt_batch* b, int tpc) {
       if (tpc > 0) {
         for (int s = 0; s < pb->ntiles; s += tpc)
           chunks.push_back(Chunk{(int)mi, base + s, base + std::min(s + tpc, pb->ntiles), 0});
+      } else if ((pb->ntiles + wave - 1) / wave < (int)pb->h_chunks.size()) {
+        const int n = (pb->ntiles + wave - 1) / wave;   // sizes differ by at most one tile
+        for (int k = 0; k < n; ++k)
+          chunks.push_back(Chunk{(int)mi, base + (int)((long long)pb->ntiles * k / n),
+                                 base + (int)((long long)pb->ntiles * (k + 1) / n), 0});
       } else {
         // the member's own split: identical reductions to its solo solve
         for (Chunk c : pb->h_chunks) chunks.push_back(Chunk{(int)mi, base + c.begin, base + c.end, 0});
