@@ -40,6 +40,8 @@ opt_status optgb::cuda_fail(cudaError_t e, const char* what) {
   return e == cudaErrorMemoryAllocation ? OPT_ERR_OOM : OPT_ERR_CUDA;
 }
 
+void optgb::set_last_error(const std::string& text) { g_err = text; }
+
 namespace {
 
 #define CK(call)                                         \

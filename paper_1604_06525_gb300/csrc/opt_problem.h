@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <utility>
+#include <string>
 #include <vector>
 
 #include "opt_gb300.h"
@@ -153,6 +154,8 @@ struct opt_batch;
 namespace optgb {
 // api.cu: records a failed CUDA call for opt_last_error (OOM or CUDA status)
 opt_status cuda_fail(cudaError_t e, const char* what);
+// api.cu: the calling thread's opt_last_error text
+void set_last_error(const std::string& text);
 // batch.cu (serving engine interface)
 // What a server round leaves of each member after its LM decision: the
 // energy at the start of the round, the trial energy, the decision and the
