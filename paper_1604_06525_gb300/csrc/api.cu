@@ -276,7 +276,7 @@ void dense_planes(const opt_problem* pb, const float* base, float** out, int n) 
 
 GridLaunch grid_launch(const opt_problem* pb, cudaStream_t st) {
   return GridLaunch{pb->dg, pb->d_chunks, pb->d_tiles, pb->d_part, pb->nchunks, st, pb->hg.tw,
-                    pb->hg.mask != nullptr};
+                    pb->hg.mask != nullptr, pb->hg.lattice};
 }
 MeshLaunch mesh_launch(const opt_problem* pb, cudaStream_t st) {
   return MeshLaunch{pb->dm, pb->d_vchunks, pb->d_echunks, pb->d_part, pb->nvchunks,
@@ -861,6 +861,14 @@ opt_status opt_problem_create_grid(const opt_grid_desc* d, const opt_solve_param
   for (int k = 0; k < nc; ++k)
     CK(cudaMemcpy2D(c + k * pl, (size_t)P * 4, d->consts[k], (size_t)W * 4, (size_t)W * 4, H,
                     cudaMemcpyDeviceToDevice));
+  int broken = 1;
+  if (warp && tw == 128) {
+    int* dbroken = nullptr;
+    CKS(dalloc(q, &dbroken, 1));
+    launch_warp_lattice(W, H, P, c, (long long)pl, dbroken, nullptr);
+    CK(cudaGetLastError());
+    CK(cudaMemcpy(&broken, dbroken, sizeof(int), cudaMemcpyDeviceToHost));
+  }
   CKS(dalloc(q, &dhbeg, hbeg.size()));
   CKS(upload(dhbeg, hbeg));
   CKS(dalloc(q, &dhpix, hpix.size()));
@@ -905,6 +913,7 @@ opt_status opt_problem_create_grid(const opt_grid_desc* d, const opt_solve_param
   g.zpack = zof(q->rvec) | zof(m) << 6 | zof(q->pbuf) << 12 | (csn ? zof(csn) : 0) << 18 | zof(c) << 24;
   g.zb = zb;
   g.wb = wb;
+  g.lattice = !broken;
   g.zpack2 = zb ? (zof(zb) | zof(wb) << 6) : 0;
   if (tw == 128) CKS(make_grid_tmaps(q, slab, nfp, warp ? dmask : dsdeg));
   g.d = q->dvec; g.r = q->rvec; g.p = q->pbuf; g.q = q->qvec; g.m = m; g.dc = dc;

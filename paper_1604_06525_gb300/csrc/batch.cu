@@ -114,6 +114,7 @@ struct GridGroup {
   int kind = 0;
   int tw = 32;
   int masked = 0;
+  int lattice = 0;                     // every member has GridProb::lattice
   std::vector<int> members;            // indices into opt_batch::probs
   GridProb* d_probs = nullptr;
   Chunk* d_chunks = nullptr;
@@ -224,6 +225,8 @@ opt_status build_tables(opt_batch* b, int tpc) {
     std::vector<Chunk> chunks;
     std::vector<int> tiles, nt;
     for (int i : g.members) nt.push_back(b->probs[i]->ntiles);
+    g.lattice = 1;
+    for (int i : g.members) g.lattice = g.lattice && b->probs[i]->hg.lattice;
     const int wave = one_wave_tiles(nt, 2 * b->probs[0]->sms);
     for (size_t mi = 0; mi < g.members.size(); ++mi) {
       opt_problem* pb = b->probs[g.members[mi]];
@@ -298,7 +301,7 @@ opt_status build_tables(opt_batch* b, int tpc) {
 }
 
 GridLaunch gl(const GridGroup& g, cudaStream_t st) {
-  return GridLaunch{g.d_probs, g.d_chunks, g.d_tiles, g.d_part, g.nchunks, st, g.tw, g.masked};
+  return GridLaunch{g.d_probs, g.d_chunks, g.d_tiles, g.d_part, g.nchunks, st, g.tw, g.masked, g.lattice};
 }
 MeshLaunch ml(const MeshGroup& g, cudaStream_t st) {
   return MeshLaunch{g.d_probs, g.d_vch, g.d_ech, g.d_part, g.nv, g.ne, st, g.dim, g.grid3, g.d_tch, g.nt};

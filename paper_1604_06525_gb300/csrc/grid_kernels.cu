@@ -32,6 +32,7 @@
 // Poisson algebra (per channel): r_{k,d} = (X_k - X_{k+d}) - (T_k - T_{k+d});
 //   the residual of a free neighbour towards k is exactly -r_{k,d}.
 #include <mutex>
+#include <type_traits>
 
 #include "opt_internal.cuh"
 #include "grid_algebra.cuh"
@@ -627,7 +628,7 @@ __device__ __forceinline__ void sts4(float* p, const float4& v) { *reinterpret_c
 // Phase 2 for one staged quad: direction, copied geometry and validity (1 / 0),
 // stored in the staged order 0 2 1 3 so that pixels {0, 2} and {1, 3} form the
 // two float2 packs of the stencil.
-template <bool MASK>
+template <bool MASK, bool LAT>
 __device__ __forceinline__ void wide_stage_quad(WideSmem& sm, int row, int lane, const GridProb& pr, int gx, int gy,
                                                 int update, int use_beta, float2 beta2) {
   const int c = 4 + 4 * lane;
@@ -650,7 +651,7 @@ __device__ __forceinline__ void wide_stage_quad(WideSmem& sm, int row, int lane,
   sts4(&sm.stg[1][row][c], swz4(b));
   sts4(&sm.stg[2][row][c], swz4(t));
 #pragma unroll
-  for (int k = 0; k < 4; ++k) sts4(&sm.stg[3 + k][row][c], swz4(R(8 + k)));
+  for (int k = 0; k < (LAT ? 2 : 4); ++k) sts4(&sm.stg[3 + k][row][c], swz4(R(8 + k)));
   float vk[4] = {0.f, 0.f, 0.f, 0.f};
   if (gy >= 0 && gy < pr.H) {
     const unsigned int m4 = MASK ? *reinterpret_cast<const unsigned int*>(&sm.mk.v[row][16 + 4 * lane]) : 0u;
@@ -683,12 +684,37 @@ __device__ __forceinline__ void pair2(const Own2& o, float2 pxj, float2 pyj, flo
   at = fma2(mj, fma2(gix, tx, mul2(giy, ty)), at);
 }
 
+// The same pairs on a unit lattice (GridProb::lattice), where v is (+-1, 0) or
+// (0, +-1): |G| is (s, c) for horizontal and (c, s) for vertical neighbours, and a
+// component whose G is negative is formed with every sign turned and subtracted
+// in the end.  Rounding to nearest is symmetric, so the bits are those of pair2.
+enum { DIR_L, DIR_R, DIR_U, DIR_D };
+template <int D>
+using Dir = std::integral_constant<int, D>;
+template <bool LAT, int DIR>
+__device__ __forceinline__ void warp_pair2(const Own2& o, float2 pxj, float2 pyj, float2 ptj, float2 cj, float2 sj,
+                                           float2 uxj, float2 uyj, float2 mj, float2& ax, float2& ay, float2& at) {
+  if (!LAT) {
+    pair2(o, pxj, pyj, ptj, cj, sj, uxj, uyj, mj, ax, ay, at);
+    return;
+  }
+  constexpr bool HOR = DIR == DIR_L || DIR == DIR_R;
+  constexpr bool XN = DIR == DIR_R || DIR == DIR_D, YN = DIR == DIR_L || DIR == DIR_D;
+  const float2 a = XN ? sub2(pxj, o.px) : sub2(o.px, pxj), b = YN ? sub2(pyj, o.py) : sub2(o.py, pyj);
+  const float2 gix = HOR ? o.s : o.c, giy = HOR ? o.c : o.s, gjx = HOR ? sj : cj, gjy = HOR ? cj : sj;
+  const float2 tx = fma2(gix, o.pt, a), ty = fma2(giy, o.pt, b);
+  const float2 nm = mul2(mj, make_float2(-1.f, -1.f));
+  ax = fma2(XN ? nm : mj, add2(tx, fma2(gjx, ptj, a)), ax);
+  ay = fma2(YN ? nm : mj, add2(ty, fma2(gjy, ptj, b)), ay);
+  at = fma2(mj, fma2(gix, tx, mul2(giy, ty)), at);
+}
+
 // One applyJTJ pass of the block's chunk (shared by the per-step kernel and
 // the persistent PCG kernel).
 // The raw planes of the PCG path arrive by tensor copies (sm.bar, whose next
 // phase has parity `phase`; the caller initialised it), a caller's p by
 // cp.async.
-template <bool MASK, bool TMA>
+template <bool MASK, bool TMA, bool LAT>
 __device__ __forceinline__ void apply_wide_body(WideSmem& sm, const Chunk& ch, const GridProb& pr,
                                                 const int* __restrict__ tiles, double* __restrict__ part,
                                                 const float* __restrict__ p_in_override, int par, int update,
@@ -733,7 +759,7 @@ __device__ __forceinline__ void apply_wide_body(WideSmem& sm, const Chunk& ch, c
   };
   auto issue = [&](int tcx) {
     if (tma) {
-      if (tid == 0) tile_tma<NRAW>(sm.raw, &sm.mk, plane, MASK, pr, tile_x0(tcx, W4), tile_y0(tcx), &sm.bar);
+      if (tid == 0) tile_tma<LAT ? NRAW - 2 : NRAW>(sm.raw, &sm.mk, plane, MASK, pr, tile_x0(tcx, W4), tile_y0(tcx), &sm.bar);
     } else {
       wide_issue<MASK>(sm, pp, pr, tile_x0(tcx, W4), tile_y0(tcx), tid);
     }
@@ -759,10 +785,10 @@ __device__ __forceinline__ void apply_wide_body(WideSmem& sm, const Chunk& ch, c
       return;
     }
     // phase 2: staged direction, geometry and validity
-    wide_stage_quad<MASK>(sm, ty + 1, lane, pr, gx, gy, update, use_beta, beta2);
+    wide_stage_quad<MASK, LAT>(sm, ty + 1, lane, pr, gx, gy, update, use_beta, beta2);
     if (tid < 64) {
       const int row = tid < 32 ? 0 : HH - 1;
-      wide_stage_quad<MASK>(sm, row, lane, pr, gx, y0 - 1 + row, update, use_beta, beta2);
+      wide_stage_quad<MASK, LAT>(sm, row, lane, pr, gx, y0 - 1 + row, update, use_beta, beta2);
     } else if (tid < 64 + 2 * TH) {
       const int h = tid - 64;
       const int row = 1 + (h % TH), side = h / TH;
@@ -782,7 +808,7 @@ __device__ __forceinline__ void apply_wide_body(WideSmem& sm, const Chunk& ch, c
       }
       sm.stg[0][row][col] = a; sm.stg[1][row][col] = b; sm.stg[2][row][col] = c;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) sm.stg[3 + k][row][col] = sm.raw[8 + k].v[row][col];
+      for (int k = 0; k < (LAT ? 2 : 4); ++k) sm.stg[3 + k][row][col] = sm.raw[8 + k].v[row][col];
       const int hy = y0 + row - 1, hx = side ? x0 + W4 : x0 - 1;
       const bool ok = hy < pr.H && hx >= 0 && hx < pr.W;
       sm.stg[7][row][col] = (ok && (!MASK || halo_mask(sm.mk.v, row, side) == 0)) ? 1.f : 0.f;
@@ -803,7 +829,9 @@ __device__ __forceinline__ void apply_wide_body(WideSmem& sm, const Chunk& ch, c
       const int c = 4 + 4 * lane;
       float4 O[NSTG];
 #pragma unroll
-      for (int k = 0; k < NSTG; ++k) O[k] = lds4(&sm.stg[k][ty + 1][c]);
+      for (int k = 0; k < NSTG; ++k)
+        if (!LAT || k < 5 || k == 7) O[k] = lds4(&sm.stg[k][ty + 1][c]);
+        else O[k] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (update) {
         *reinterpret_cast<float4*>(pout + i) = swz4(O[0]);
         *reinterpret_cast<float4*>(pout + pl + i) = swz4(O[1]);
@@ -818,38 +846,49 @@ __device__ __forceinline__ void apply_wide_body(WideSmem& sm, const Chunk& ch, c
         float L[NSTG], R[NSTG];
 #pragma unroll
         for (int k = 0; k < NSTG; ++k) {
+          if (LAT && (k == 5 || k == 6)) { L[k] = R[k] = 0.f; continue; }
           L[k] = __shfl_up_sync(0xffffffffu, O[k].w, 1);
           R[k] = __shfl_down_sync(0xffffffffu, O[k].x, 1);
         }
         if (lane == 0) {
 #pragma unroll
-          for (int k = 0; k < NSTG; ++k) L[k] = sm.stg[k][ty + 1][3];
+          for (int k = 0; k < NSTG; ++k)
+            if (!LAT || k < 5 || k == 7) L[k] = sm.stg[k][ty + 1][3];
         }
         if (lane == 31) {
 #pragma unroll
-          for (int k = 0; k < NSTG; ++k) R[k] = sm.stg[k][ty + 1][4 + W4];
+          for (int k = 0; k < NSTG; ++k)
+            if (!LAT || k < 5 || k == 7) R[k] = sm.stg[k][ty + 1][4 + W4];
         }
         // A: left neighbours {-1, 1}, right neighbours {1, 3} = B
-        pair2(oa, make_float2(L[0], O[0].z), make_float2(L[1], O[1].z), make_float2(L[2], O[2].z),
+        warp_pair2<LAT, DIR_L>(oa, make_float2(L[0], O[0].z), make_float2(L[1], O[1].z), make_float2(L[2], O[2].z),
               make_float2(L[3], O[3].z), make_float2(L[4], O[4].z), make_float2(L[5], O[5].z),
               make_float2(L[6], O[6].z), make_float2(L[7], O[7].z), axA, ayA, atA);
-        pair2(oa, ob.px, ob.py, ob.pt, ob.c, ob.s, ob.ux, ob.uy, hi2(O[7]), axA, ayA, atA);
+        warp_pair2<LAT, DIR_R>(oa, ob.px, ob.py, ob.pt, ob.c, ob.s, ob.ux, ob.uy, hi2(O[7]), axA, ayA, atA);
         // B: left neighbours {0, 2} = A, right neighbours {2, 4}
-        pair2(ob, oa.px, oa.py, oa.pt, oa.c, oa.s, oa.ux, oa.uy, lo2(O[7]), axB, ayB, atB);
-        pair2(ob, make_float2(O[0].y, R[0]), make_float2(O[1].y, R[1]), make_float2(O[2].y, R[2]),
+        warp_pair2<LAT, DIR_L>(ob, oa.px, oa.py, oa.pt, oa.c, oa.s, oa.ux, oa.uy, lo2(O[7]), axB, ayB, atB);
+        warp_pair2<LAT, DIR_R>(ob, make_float2(O[0].y, R[0]), make_float2(O[1].y, R[1]), make_float2(O[2].y, R[2]),
               make_float2(O[3].y, R[3]), make_float2(O[4].y, R[4]), make_float2(O[5].y, R[5]),
               make_float2(O[6].y, R[6]), make_float2(O[7].y, R[7]), axB, ayB, atB);
       }
-#pragma unroll 1
-      for (int dr = 0; dr < 2; ++dr) {        // rows above and below
+      auto row = [&](auto dir, int y) {         // rows above and below
         float4 U[NSTG];
-        const int row = dr ? ty + 2 : ty;
 #pragma unroll
-        for (int k = 0; k < NSTG; ++k) U[k] = lds4(&sm.stg[k][row][c]);
-        pair2(oa, lo2(U[0]), lo2(U[1]), lo2(U[2]), lo2(U[3]), lo2(U[4]), lo2(U[5]), lo2(U[6]), lo2(U[7]), axA,
-              ayA, atA);
-        pair2(ob, hi2(U[0]), hi2(U[1]), hi2(U[2]), hi2(U[3]), hi2(U[4]), hi2(U[5]), hi2(U[6]), hi2(U[7]), axB,
-              ayB, atB);
+        for (int k = 0; k < NSTG; ++k)
+          if (!LAT || k < 5 || k == 7) U[k] = lds4(&sm.stg[k][y][c]);
+          else U[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        constexpr int D = decltype(dir)::value;
+        warp_pair2<LAT, D>(oa, lo2(U[0]), lo2(U[1]), lo2(U[2]), lo2(U[3]), lo2(U[4]), lo2(U[5]), lo2(U[6]), lo2(U[7]),
+                           axA, ayA, atA);
+        warp_pair2<LAT, D>(ob, hi2(U[0]), hi2(U[1]), hi2(U[2]), hi2(U[3]), hi2(U[4]), hi2(U[5]), hi2(U[6]), hi2(U[7]),
+                           axB, ayB, atB);
+      };
+      if (LAT) {
+        row(Dir<DIR_U>{}, ty);
+        row(Dir<DIR_D>{}, ty + 2);
+      } else {
+#pragma unroll 1
+        for (int dr = 0; dr < 2; ++dr) row(Dir<DIR_U>{}, ty + 2 * dr);
       }
       // scale by w and the own validity, back to plain pixel order
       const float2 wa = mul2(w2, lo2(O[7])), wb = mul2(w2, hi2(O[7]));
@@ -903,7 +942,7 @@ __device__ __forceinline__ void apply_wide_body(WideSmem& sm, const Chunk& ch, c
   }
 }
 
-template <bool MASK>
+template <bool MASK, bool LAT>
 __global__ void __launch_bounds__(NT, 2) k_warp_apply_wide(const GridProb* __restrict__ probs,
                                                            const Chunk* __restrict__ chunks,
                                                            const int* __restrict__ tiles,
@@ -920,9 +959,9 @@ __global__ void __launch_bounds__(NT, 2) k_warp_apply_wide(const GridProb* __res
   unsigned phase = 0;
   // the PCG path stages by tensor copies, a caller's p (the J^T J p hook) by cp.async
   if (update && !p_in_override && wide_tma(pr, &sm))
-    apply_wide_body<MASK, true>(sm, ch, pr, tiles, part, p_in_override, par, update, phase);
+    apply_wide_body<MASK, true, LAT>(sm, ch, pr, tiles, part, p_in_override, par, update, phase);
   else
-    apply_wide_body<MASK, false>(sm, ch, pr, tiles, part, p_in_override, par, update, phase);
+    apply_wide_body<MASK, false, LAT>(sm, ch, pr, tiles, part, p_in_override, par, update, phase);
 }
 
 // cos / sin of the new theta quad into the cos / sin planes (wide warps: the
@@ -1071,9 +1110,10 @@ __device__ __forceinline__ void fused_finish(const GridProb& pr, double* __restr
 
 // One single-reduction PCG iteration `it` of the block's chunk (staged by
 // tensor copies, like the wide apply).
-template <bool MASK>
+template <bool MASK, bool LAT>
 __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, const GridProb& pr,
                                                 const int* __restrict__ tiles, double* __restrict__ part, int it) {
+  constexpr int NS = LAT ? NSTG_F - 2 : NSTG_F;   // a unit lattice needs no UrShape
   Scalars* s = pr.s;
   if (s->done) return;
   const int first = it == 0;
@@ -1107,7 +1147,7 @@ __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, 
     }
   };
   auto issue = [&](int tcx, int slot) {
-    if (tid == 0) tile_tma<NRAW_F>(sm.raw, &sm.mk[slot], plane, MASK, pr, tile_x0(tcx, W4), tile_y0(tcx), &sm.bar);
+    if (tid == 0) tile_tma<LAT ? NRAW_F - 2 : NRAW_F>(sm.raw, &sm.mk[slot], plane, MASK, pr, tile_x0(tcx, W4), tile_y0(tcx), &sm.bar);
   };
   // direction and z of one quad of staged row `row` (column c); ownrow:
   // also the z / delta stores of the thread's own pixels
@@ -1131,7 +1171,7 @@ __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, 
     sts4(&sm.stg[1][row][c], swz4(py));
     sts4(&sm.stg[2][row][c], swz4(pt));
 #pragma unroll
-    for (int k = 0; k < 4; ++k) sts4(&sm.stg[3 + k][row][c], swz4(R(9 + k)));
+    for (int k = 3; k < NS; ++k) sts4(&sm.stg[k][row][c], swz4(R(6 + k)));
     if (own && gy < pr.H) {
       *reinterpret_cast<float4*>(zout + i) = zx;
       *reinterpret_cast<float4*>(zout + pl + i) = zy;
@@ -1187,7 +1227,7 @@ __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, 
       }
       sm.stg[0][row][col] = zx; sm.stg[1][row][col] = zy; sm.stg[2][row][col] = zt;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) sm.stg[3 + k][row][col] = R(9 + k);
+      for (int k = 3; k < NS; ++k) sm.stg[k][row][col] = R(6 + k);
     }
     __syncthreads();
     // the raw buffer is free: start the next tile's copies
@@ -1203,7 +1243,9 @@ __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, 
       const int c = 4 + 4 * lane;
       float4 O[NSTG_F];
 #pragma unroll
-      for (int k = 0; k < NSTG_F; ++k) O[k] = lds4(&sm.stg[k][ty + 1][c]);
+      for (int k = 0; k < NS; ++k) O[k] = lds4(&sm.stg[k][ty + 1][c]);
+#pragma unroll
+      for (int k = NS; k < NSTG_F; ++k) O[k] = make_float4(0.f, 0.f, 0.f, 0.f);
       *reinterpret_cast<float4*>(pout + i) = swz4(O[0]);
       *reinterpret_cast<float4*>(pout + pl + i) = swz4(O[1]);
       *reinterpret_cast<float4*>(pout + 2 * pl + i) = swz4(O[2]);
@@ -1243,36 +1285,47 @@ __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, 
       {
         float L[NSTG_F], R[NSTG_F];
 #pragma unroll
-        for (int k = 0; k < NSTG_F; ++k) {
+        for (int k = NS; k < NSTG_F; ++k) L[k] = R[k] = 0.f;
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
           L[k] = __shfl_up_sync(0xffffffffu, O[k].w, 1);
           R[k] = __shfl_down_sync(0xffffffffu, O[k].x, 1);
         }
         if (lane == 0) {
 #pragma unroll
-          for (int k = 0; k < NSTG_F; ++k) L[k] = sm.stg[k][ty + 1][3];
+          for (int k = 0; k < NS; ++k) L[k] = sm.stg[k][ty + 1][3];
         }
         if (lane == 31) {
 #pragma unroll
-          for (int k = 0; k < NSTG_F; ++k) R[k] = sm.stg[k][ty + 1][4 + W4];
+          for (int k = 0; k < NS; ++k) R[k] = sm.stg[k][ty + 1][4 + W4];
         }
-        pair2(oa, make_float2(L[0], O[0].z), make_float2(L[1], O[1].z), make_float2(L[2], O[2].z),
+        warp_pair2<LAT, DIR_L>(oa, make_float2(L[0], O[0].z), make_float2(L[1], O[1].z), make_float2(L[2], O[2].z),
               make_float2(L[3], O[3].z), make_float2(L[4], O[4].z), make_float2(L[5], O[5].z),
               make_float2(L[6], O[6].z), lA, axA, ayA, atA);
-        pair2(oa, ob.px, ob.py, ob.pt, ob.c, ob.s, ob.ux, ob.uy, rA, axA, ayA, atA);
-        pair2(ob, oa.px, oa.py, oa.pt, oa.c, oa.s, oa.ux, oa.uy, vA, axB, ayB, atB);
-        pair2(ob, make_float2(O[0].y, R[0]), make_float2(O[1].y, R[1]), make_float2(O[2].y, R[2]),
+        warp_pair2<LAT, DIR_R>(oa, ob.px, ob.py, ob.pt, ob.c, ob.s, ob.ux, ob.uy, rA, axA, ayA, atA);
+        warp_pair2<LAT, DIR_L>(ob, oa.px, oa.py, oa.pt, oa.c, oa.s, oa.ux, oa.uy, vA, axB, ayB, atB);
+        warp_pair2<LAT, DIR_R>(ob, make_float2(O[0].y, R[0]), make_float2(O[1].y, R[1]), make_float2(O[2].y, R[2]),
               make_float2(O[3].y, R[3]), make_float2(O[4].y, R[4]), make_float2(O[5].y, R[5]),
               make_float2(O[6].y, R[6]), rB, axB, ayB, atB);
       }
-#pragma unroll 1
-      for (int dr = 0; dr < 2; ++dr) {        // rows above and below
+      auto row = [&](auto dir, int y, const float2& mA, const float2& mB) {   // rows above and below
         float4 U[NSTG_F];
-        const int row = dr ? ty + 2 : ty;
 #pragma unroll
-        for (int k = 0; k < NSTG_F; ++k) U[k] = lds4(&sm.stg[k][row][c]);
-        const float2 mA = dr ? dn2A : up2A, mB = dr ? dn2B : up2B;
-        pair2(oa, lo2(U[0]), lo2(U[1]), lo2(U[2]), lo2(U[3]), lo2(U[4]), lo2(U[5]), lo2(U[6]), mA, axA, ayA, atA);
-        pair2(ob, hi2(U[0]), hi2(U[1]), hi2(U[2]), hi2(U[3]), hi2(U[4]), hi2(U[5]), hi2(U[6]), mB, axB, ayB, atB);
+        for (int k = 0; k < NS; ++k) U[k] = lds4(&sm.stg[k][y][c]);
+#pragma unroll
+        for (int k = NS; k < NSTG_F; ++k) U[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        constexpr int D = decltype(dir)::value;
+        warp_pair2<LAT, D>(oa, lo2(U[0]), lo2(U[1]), lo2(U[2]), lo2(U[3]), lo2(U[4]), lo2(U[5]), lo2(U[6]), mA, axA,
+                           ayA, atA);
+        warp_pair2<LAT, D>(ob, hi2(U[0]), hi2(U[1]), hi2(U[2]), hi2(U[3]), hi2(U[4]), hi2(U[5]), hi2(U[6]), mB, axB,
+                           ayB, atB);
+      };
+      if (LAT) {
+        row(Dir<DIR_U>{}, ty, up2A, up2B);
+        row(Dir<DIR_D>{}, ty + 2, dn2A, dn2B);
+      } else {
+#pragma unroll 1
+        for (int dr = 0; dr < 2; ++dr) row(Dir<DIR_U>{}, ty + 2 * dr, dr ? dn2A : up2A, dr ? dn2B : up2B);
       }
       const float2 wa = mul2(w2, vA), wb = mul2(w2, vB);
       axA = mul2(wa, axA); ayA = mul2(wa, ayA); atA = mul2(wa, atA);
@@ -1337,7 +1390,7 @@ __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, 
   fused_finish(pr, part, acc_pq, acc_qz, acc_qw, acc_zr);
 }
 
-template <bool MASK>
+template <bool MASK, bool LAT>
 __global__ void __launch_bounds__(NT, 2) k_warp_fused_wide(const GridProb* __restrict__ probs,
                                                            const Chunk* __restrict__ chunks,
                                                            const int* __restrict__ tiles,
@@ -1349,7 +1402,7 @@ __global__ void __launch_bounds__(NT, 2) k_warp_fused_wide(const GridProb* __res
   pdl_begin();
   if (threadIdx.x == 0) mbar_init(&sm.bar);
   __syncthreads();
-  if (tma_ready(pr, &sm)) fused_wide_body<MASK>(sm, ch, pr, tiles, part, it);
+  if (tma_ready(pr, &sm)) fused_wide_body<MASK, LAT>(sm, ch, pr, tiles, part, it);
 }
 
 // After the last single-reduction iteration: delta += alpha p for the step
@@ -2976,9 +3029,9 @@ __global__ void __launch_bounds__(NT, 2) k_warp_pcg_coop(const GridProb* __restr
   const bool tma = wide_tma(pr, &sm);
   for (int it = 0; it < n_inner; ++it) {
     if (tma)
-      apply_wide_body<MASK, true>(sm, ch, pr, tiles, part, nullptr, par0 + it, 1, phase);
+      apply_wide_body<MASK, true, false>(sm, ch, pr, tiles, part, nullptr, par0 + it, 1, phase);
     else
-      apply_wide_body<MASK, false>(sm, ch, pr, tiles, part, nullptr, par0 + it, 1, phase);
+      apply_wide_body<MASK, false, false>(sm, ch, pr, tiles, part, nullptr, par0 + it, 1, phase);
     if (!grid_sync(gb, gridDim.x)) return;
     update_body<3>(ch, pr, tiles, part, par0 + it);
     if (it + 1 < n_inner && !grid_sync(gb, gridDim.x)) return;
@@ -3055,13 +3108,15 @@ cudaError_t grid_kernels_prepare() {
   static std::once_flag once;
   std::call_once(once, [] {
     const int bytes = (int)sizeof(WideSmem);
-    cudaError_t e = cudaFuncSetAttribute(k_warp_apply_wide<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_warp_apply_wide<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_warp_apply_wide<true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_warp_apply_wide<false>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    cudaError_t e = cudaSuccess;
+    const auto staged = [&](auto* k, int smem) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    };
+    staged(k_warp_apply_wide<true, true>, bytes);
+    staged(k_warp_apply_wide<true, false>, bytes);
+    staged(k_warp_apply_wide<false, true>, bytes);
+    staged(k_warp_apply_wide<false, false>, bytes);
     const int ibytes = (int)sizeof(InitSmem);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_warp_init_wide<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ibytes);
@@ -3088,14 +3143,10 @@ cudaError_t grid_kernels_prepare() {
       e = cudaFuncSetAttribute(k_poisson_init_wide, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)sizeof(PoisInitSmem));
     const int fbytes = (int)sizeof(FusedSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_warp_fused_wide<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fbytes);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_warp_fused_wide<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fbytes);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_warp_fused_wide<true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_warp_fused_wide<false>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    staged(k_warp_fused_wide<true, true>, fbytes);
+    staged(k_warp_fused_wide<true, false>, fbytes);
+    staged(k_warp_fused_wide<false, true>, fbytes);
+    staged(k_warp_fused_wide<false, false>, fbytes);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_poisson_fused_wide, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)sizeof(PoisFusedSmem));
@@ -3128,12 +3179,12 @@ void launch_grid_init(int kind, const GridLaunch& L, int k_outer, float dmin, fl
 }
 
 void launch_grid_apply(int kind, const GridLaunch& L, const float* p_override, int par, int update) {
-  if (kind == K_WARP && L.tw == 128 && L.masked)
-    launch_pdl(k_warp_apply_wide<true>, L.nchunks, NT, sizeof(WideSmem), L.stream, L.probs, L.chunks, L.tiles, L.part,
-                                                                         p_override, par, update);
-  else if (kind == K_WARP && L.tw == 128)
-    launch_pdl(k_warp_apply_wide<false>, L.nchunks, NT, sizeof(WideSmem), L.stream, L.probs, L.chunks, L.tiles, L.part,
-                                                                          p_override, par, update);
+  if (kind == K_WARP && L.tw == 128) {
+    auto k = L.masked ? (L.lattice ? k_warp_apply_wide<true, true> : k_warp_apply_wide<true, false>)
+                      : (L.lattice ? k_warp_apply_wide<false, true> : k_warp_apply_wide<false, false>);
+    launch_pdl(k, L.nchunks, NT, sizeof(WideSmem), L.stream, L.probs, L.chunks, L.tiles, L.part, p_override, par,
+               update);
+  }
   else if (kind == K_WARP)
     launch_pdl(k_warp_apply, L.nchunks, NT, 0, L.stream, L.probs, L.chunks, L.tiles, L.part, p_override, par, update);
   else
@@ -3159,12 +3210,11 @@ void launch_grid_fused(int kind, const GridLaunch& L, int it) {
   if (kind == K_POISSON)
     launch_pdl(k_poisson_fused_wide, L.nchunks, NT, sizeof(PoisFusedSmem), L.stream, L.probs, L.chunks, L.tiles,
                L.part, it);
-  else if (L.masked)
-    launch_pdl(k_warp_fused_wide<true>, L.nchunks, NT, sizeof(FusedSmem), L.stream, L.probs, L.chunks, L.tiles,
-               L.part, it);
-  else
-    launch_pdl(k_warp_fused_wide<false>, L.nchunks, NT, sizeof(FusedSmem), L.stream, L.probs, L.chunks, L.tiles,
-               L.part, it);
+  else {
+    auto k = L.masked ? (L.lattice ? k_warp_fused_wide<true, true> : k_warp_fused_wide<true, false>)
+                      : (L.lattice ? k_warp_fused_wide<false, true> : k_warp_fused_wide<false, false>);
+    launch_pdl(k, L.nchunks, NT, sizeof(FusedSmem), L.stream, L.probs, L.chunks, L.tiles, L.part, it);
+  }
 }
 
 void launch_grid_fused_fin(int kind, const GridLaunch& L, int par, int step, int csn_out) {
@@ -3182,6 +3232,23 @@ void launch_grid_energy(int kind, const GridLaunch& L, int mode, int hist_idx) {
   auto k = kind == K_WARP ? (mode ? k_warp_energy<1> : k_warp_energy<0>)
                           : (mode ? k_poisson_energy<1> : k_poisson_energy<0>);
   launch_pdl(k, L.nchunks, NT, 0, L.stream, L.probs, L.chunks, L.tiles, L.part, hist_idx);
+}
+
+// Sets *broken unless UrShape is the pixel lattice up to an offset: every
+// difference the stencil takes of it is exactly 1 or 0.
+__global__ void __launch_bounds__(NT) k_warp_lattice(int W, int H, int P, const float* __restrict__ ux,
+                                                     const float* __restrict__ uy, int* __restrict__ broken) {
+  bool ok = true;
+  for (int y = blockIdx.x; y < H; y += gridDim.x)
+    for (int x = threadIdx.x; x < W; x += NT) {
+      const long long i = (long long)y * P + x;
+      if (x + 1 < W) ok = ok && ux[i + 1] - ux[i] == 1.f && uy[i + 1] == uy[i];
+      if (y + 1 < H) ok = ok && uy[i + P] - uy[i] == 1.f && ux[i + P] == ux[i];
+    }
+  if (!ok) *broken = 1;
+}
+void launch_warp_lattice(int W, int H, int P, const float* u, long long plane, int* broken, cudaStream_t st) {
+  k_warp_lattice<<<std::min(H, 1024), NT, 0, st>>>(W, H, P, u, u + plane, broken);
 }
 
 void launch_pois_sdeg(int W, int H, int P, const uint8_t* mask, uint8_t* out, cudaStream_t st) {

@@ -120,6 +120,9 @@ struct GridProb {
   // (zpack2 = z_z | z_w << 6)
   float *zb, *wb;
   int zpack2;
+  // warp: UrShape is the pixel lattice up to an offset (checked when the problem
+  // is planned), so the 128-pixel-tile kernels need not read it
+  int lattice;
   float *d, *r, *p, *q;         // PCG vectors
   float *m, *dc;                // M^-1 and LM diagonal (distinct-diagonal planes)
   float* csn;                   // warp, tw = 128: cos / sin of theta (2 planes, written by PCGInit)

@@ -14,6 +14,7 @@ struct GridLaunch {
   cudaStream_t stream;
   int tw;        // tile width of every problem in the launch (32 or 128)
   int masked;    // every problem in the launch has a mask (wide warp kernel variant)
+  int lattice;   // every problem in the launch has GridProb::lattice (wide warp kernel variant)
 };
 
 struct MeshLaunch {
@@ -69,6 +70,8 @@ void launch_grid_csn(const GridLaunch& L);
 // Poisson, tile width 128: the degree plane the wide kernels read (S_i + 1 on
 // free pixels, 0 elsewhere; pitched like the mask, P x H bytes)
 void launch_pois_sdeg(int W, int H, int P, const uint8_t* mask, uint8_t* out, cudaStream_t st);
+// sets *broken (device) unless the two planes at u are the pixel lattice up to an offset
+void launch_warp_lattice(int W, int H, int P, const float* u, long long plane, int* broken, cudaStream_t st);
 // Persistent PCG loop (wide warp tiles only): the largest chunk count whose
 // blocks are all resident at once (0 if unknown), and the cooperative launch
 // of n_inner PCG iterations (applyJTJ + update) starting at parity par0.
