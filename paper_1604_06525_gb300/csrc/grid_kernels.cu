@@ -407,6 +407,10 @@ __device__ __forceinline__ float cmp(const float4& a, int k) {
   return k == 0 ? a.x : (k == 1 ? a.y : (k == 2 ? a.z : a.w));
 }
 
+__device__ __forceinline__ float& cmp_ref(float4& a, int k) {
+  return k == 0 ? a.x : (k == 1 ? a.y : (k == 2 ? a.z : a.w));
+}
+
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool valid) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
   const int n = valid ? 16 : 0;   // 0: the 16 destination bytes are zero-filled
@@ -684,7 +688,8 @@ __device__ __forceinline__ void pair2(const Own2& o, float2 pxj, float2 pyj, flo
   at = fma2(mj, fma2(gix, tx, mul2(giy, ty)), at);
 }
 
-// The same pairs on a unit lattice (GridProb::lattice), where v is (+-1, 0) or
+// The same pairs on a unit lattice (GridProb::lattice; masked 1411 x 1003 applyJTJ
+// 31.7 -> 27.7 us), where v is (+-1, 0) or
 // (0, +-1): |G| is (s, c) for horizontal and (c, s) for vertical neighbours, and a
 // component whose G is negative is formed with every sign turned and subtracted
 // in the end.  Rounding to nearest is symmetric, so the bits are those of pair2.
@@ -1004,7 +1009,13 @@ __device__ __forceinline__ void store_csn(const GridProb& pr, long long i, const
 // = z_0); the last iteration's update is applied by k_grid_fused_fin (for
 // Gauss-Newton together with the outer update x += delta).
 // Per pixel: read z, w, p (halos), cos / sin, UrShape, M^-1, delta; write z,
-// w, p, delta: 120 B against 152 B for the two-pass form.
+// w, p, delta: 120 B against 152 B for the two-pass form.  On a unit lattice
+// (GridProb::lattice) UrShape is not read, z of the own pixels waits for the inner
+// products in the staging planes that leaves free instead of being read back, and
+// without a mask a Gauss-Newton solve knows M^-1 of interior pixels (four pairs of
+// |G| = 1, with or without a handle): 104 B.  Memory bounds it at 4096^2 (357 us an
+// iteration, 331 without UrShape, 312 so: 5.6 TB/s), the chain from the copies to the
+// sums with 16 warps an SM at 1024^2 (30.4, 28.7, 27.1 us).
 // Breakdown (p.q <= 0 or r.z = 0, or a recurrence r.z <= 0) stops the loop
 // as in the two-pass form; a step whose alpha is known is still applied.
 // ---------------------------------------------------------------------------
@@ -1113,6 +1124,7 @@ __device__ __forceinline__ void fused_finish(const GridProb& pr, double* __restr
 template <bool MASK, bool LAT>
 __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, const GridProb& pr,
                                                 const int* __restrict__ tiles, double* __restrict__ part, int it) {
+  constexpr bool CONSTM = LAT && !MASK;
   constexpr int NS = LAT ? NSTG_F - 2 : NSTG_F;   // a unit lattice needs no UrShape
   Scalars* s = pr.s;
   if (s->done) return;
@@ -1149,6 +1161,17 @@ __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, 
   auto issue = [&](int tcx, int slot) {
     if (tid == 0) tile_tma<LAT ? NRAW_F - 2 : NRAW_F>(sm.raw, &sm.mk[slot], plane, MASK, pr, tile_x0(tcx, W4), tile_y0(tcx), &sm.bar);
   };
+  // a unit lattice leaves four staging planes free: three keep z of the own pixels
+  auto zown = [&](int k) { return k < 2 ? sm.stg[NSTG_F - 2 + k] : sm.raw[NRAW_F - 1].v; };
+  // interior pixels of a unit lattice: M^-1 of a pixel without and with a handle
+  // and of its angle, as PCGInit forms them
+  float mi = 0.f, mh = 0.f, mt = 0.f;
+  if (CONSTM) {
+    const float dd = __fmul_rn(__fadd_rn(pr.w_reg, pr.w_reg), 4.f);
+    mi = minv_entry(dd, 0.f, 0.f, 0.f, pr.use_precond, nullptr);
+    mh = minv_entry(__fadd_rn(dd, wfit), 0.f, 0.f, 0.f, pr.use_precond, nullptr);
+    mt = minv_entry(__fmul_rn(pr.w_reg, 4.f), 0.f, 0.f, 0.f, pr.use_precond, nullptr);
+  }
   // direction and z of one quad of staged row `row` (column c); ownrow:
   // also the z / delta stores of the thread's own pixels
   // delta of the thread's own pixels, loaded before the staging wait
@@ -1173,6 +1196,11 @@ __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, 
 #pragma unroll
     for (int k = 3; k < NS; ++k) sts4(&sm.stg[k][row][c], swz4(R(6 + k)));
     if (own && gy < pr.H) {
+      if (LAT) {                              // for phase 3 of the same thread
+        sts4(&zown(0)[row][c], zx);
+        sts4(&zown(1)[row][c], zy);
+        sts4(&zown(2)[row][c], zt);
+      }
       *reinterpret_cast<float4*>(zout + i) = zx;
       *reinterpret_cast<float4*>(zout + pl + i) = zy;
       *reinterpret_cast<float4*>(zout + 2 * pl + i) = zt;
@@ -1241,6 +1269,12 @@ __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, 
     }
     if (gy < pr.H) {                          // warp-uniform: one warp per row
       const int c = 4 + 4 * lane;
+      const bool inner = CONSTM && !pr.lm && gx > 0 && gx + 4 < pr.W && gy > 0 && gy + 1 < pr.H;
+      float4 m0 = make_float4(mi, mi, mi, mi), m1 = make_float4(mt, mt, mt, mt);
+      if (LAT && !inner) {
+        m0 = ld4(pr.m + i);
+        m1 = ld4(pr.m + pl + i);
+      }
       float4 O[NSTG_F];
 #pragma unroll
       for (int k = 0; k < NS; ++k) O[k] = lds4(&sm.stg[k][ty + 1][c]);
@@ -1343,6 +1377,7 @@ __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, 
             if (kk == k && vf[kk] != 0.f) {
               qx[kk] = __fmaf_rn(wfit, cmp(opx, kk), qx[kk]);
               qy[kk] = __fmaf_rn(wfit, cmp(opy, kk), qy[kk]);
+              if (CONSTM && inner) cmp_ref(m0, kk) = mh;
             }
         }
       }
@@ -1358,7 +1393,10 @@ __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, 
       }
       // w = M^-1 q and the three inner products; z of the own pixels comes
       // back from the stores of phase 2 (this thread's own writes)
-      const float4 m0 = ld4(pr.m + i), m1 = ld4(pr.m + pl + i);
+      if (!LAT) {
+        m0 = ld4(pr.m + i);
+        m1 = ld4(pr.m + pl + i);
+      }
       const float4 qxv = make_float4(qx[0], qx[1], qx[2], qx[3]);
       const float4 qyv = make_float4(qy[0], qy[1], qy[2], qy[3]);
       const float4 qtv = make_float4(qt[0], qt[1], qt[2], qt[3]);
@@ -1366,9 +1404,9 @@ __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, 
       *reinterpret_cast<float4*>(wout + i) = wx;
       *reinterpret_cast<float4*>(wout + pl + i) = wy;
       *reinterpret_cast<float4*>(wout + 2 * pl + i) = wt;
-      const float4 zxv = *reinterpret_cast<const float4*>(zout + i);
-      const float4 zyv = *reinterpret_cast<const float4*>(zout + pl + i);
-      const float4 ztv = *reinterpret_cast<const float4*>(zout + 2 * pl + i);
+      const float4 zxv = LAT ? lds4(&zown(0)[ty + 1][c]) : *reinterpret_cast<const float4*>(zout + i);
+      const float4 zyv = LAT ? lds4(&zown(1)[ty + 1][c]) : *reinterpret_cast<const float4*>(zout + pl + i);
+      const float4 ztv = LAT ? lds4(&zown(2)[ty + 1][c]) : *reinterpret_cast<const float4*>(zout + 2 * pl + i);
       f2x2_add_prod(acc_pq, lo2(opx), lo2(qxv)); f2x2_add_prod(acc_pq, hi2(opx), hi2(qxv));
       f2x2_add_prod(acc_pq, lo2(opy), lo2(qyv)); f2x2_add_prod(acc_pq, hi2(opy), hi2(qyv));
       f2x2_add_prod(acc_pq, lo2(opt), lo2(qtv)); f2x2_add_prod(acc_pq, hi2(opt), hi2(qtv));
@@ -1518,7 +1556,7 @@ struct AccI2 {
 // G_k = (s_k v_x + c_k v_y, s_k v_y - c_k v_x), the rotation residual part is
 // e_k = v - R(theta_k) v = (v_x + G_k,y, v_y - G_k,x), own residual / s_w
 // o = a + e_i:
-//   J^T F_d += o + (a + e_j),  J^T F_t += G_i . o,  diag_t += |G_i|^2,
+//   J^T F_d += o + (a + e_j),  J^T F_t += G_i . o,  diag_t += |G_i|^2 = |v|^2,
 //   E += |o|^2,  np += 1 (diag_d = 2 w np).
 __device__ __forceinline__ void init_pair2(const OwnI2& o, float2 dxj, float2 dyj, float2 cj, float2 sj, float2 uxj,
                                            float2 uyj, float2 mj, AccI2& A) {
@@ -1531,7 +1569,7 @@ __device__ __forceinline__ void init_pair2(const OwnI2& o, float2 dxj, float2 dy
   A.gx = fma2(mj, fx, A.gx);
   A.gy = fma2(mj, fy, A.gy);
   A.gt = fma2(mj, fma2(gix, ox, mul2(giy, oy)), A.gt);
-  A.dt = fma2(mj, fma2(gix, gix, mul2(giy, giy)), A.dt);
+  A.dt = fma2(mj, fma2(vx, vx, mul2(vy, vy)), A.dt);
   A.e = fma2(mj, fma2(ox, ox, mul2(oy, oy)), A.e);
   A.np = add2(A.np, mj);
 }
