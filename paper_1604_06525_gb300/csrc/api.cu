@@ -220,50 +220,92 @@ opt_status common_setup(opt_problem* pb) {
   return OPT_OK;
 }
 
-// Graph problems keep their vertices in a locality order (internal vertex k
-// is the caller's vertex perm[k]); these move one plane between the orders.
-__global__ void k_gather_vertices(float* __restrict__ dst, const float* __restrict__ src, const int* __restrict__ perm,
-                                  int V) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < V) dst[k] = src[perm[k]];
+// Caller planes (dense, caller order) <-> internal planes (pitched rows for grids;
+// graph problems keep their vertices in a locality order, internal vertex k is the
+// caller's perm[k]): all planes in one launch, and on the way in of a solve its
+// scalars reset as well.  A launch for each plane (graphs) or a copy node for each
+// (grids), after a launch for the scalars, took longer than the planes of a small
+// problem: with x += delta of a Gauss-Newton solve moved into the resident loop,
+// 64^2 warp GN 4 x 10 306 -> 295 us, level-5 mesh LM 3 x 10 415 -> 403 us, 4096^2
+// warp GN 2 x 15 11.00 -> 10.61 ms (the copy nodes ran at a fraction of the bandwidth).
+enum class PlaneDir { In, Out };
+struct PlaneSet {
+  float* user[12];
+  float* own;                   // internal plane 0
+  long long plane;
+  int n, W, H, P;               // graphs: W = vertices, H = 1
+  const int* perm;              // graphs
+  int vec;                      // grids: quads of every user row are 16-byte aligned
+};
+
+template <bool IN>
+__global__ void __launch_bounds__(256) k_move_planes(const __grid_constant__ PlaneSet ps, Scalars* reset,
+                                                     double lambda0) {
+  if (IN && reset && blockIdx.x == 0 && threadIdx.x == 0) scalars_reset(reset, lambda0);
+  const long long t0 = blockIdx.x * 256ll + threadIdx.x, step = gridDim.x * 256ll;
+  auto move = [&](float* own, float* user) {
+    if (IN) *own = *user;
+    else *user = *own;
+  };
+  if (ps.perm) {
+    for (long long k = t0; k < ps.W; k += step) {
+      const int v = ps.perm[k];
+      for (int c = 0; c < ps.n; ++c) move(ps.own + c * ps.plane + k, ps.user[c] + v);
+    }
+  } else if (ps.vec) {
+    const int qpr = ps.W / 4;
+    const long long nq = (long long)qpr * ps.H;
+    for (long long k = t0; k < nq; k += step) {
+      const int y = (int)(k / qpr), x = 4 * (int)(k - (long long)y * qpr);
+      for (int c = 0; c < ps.n; ++c) {
+        float4* own = reinterpret_cast<float4*>(ps.own + c * ps.plane + (long long)y * ps.P + x);
+        float4* user = reinterpret_cast<float4*>(ps.user[c] + (long long)y * ps.W + x);
+        if (IN) *own = *user;
+        else *user = *own;
+      }
+    }
+  } else {
+    const long long np = (long long)ps.W * ps.H;
+    for (long long k = t0; k < np; k += step) {
+      const int y = (int)(k / ps.W), x = (int)(k - (long long)y * ps.W);
+      for (int c = 0; c < ps.n; ++c) move(ps.own + c * ps.plane + (long long)y * ps.P + x, ps.user[c] + k);
+    }
+  }
 }
-__global__ void k_scatter_vertices(float* __restrict__ dst, const float* __restrict__ src,
-                                   const int* __restrict__ perm, int V) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < V) dst[perm[k]] = src[k];
+
+opt_status copy_planes(const opt_problem* pb, PlaneDir dir, float* own, float* const* user, int n, cudaStream_t st,
+                       Scalars* reset = nullptr, double lambda0 = 0.0) {
+  PlaneSet ps = {};
+  const bool grid = is_grid(pb);
+  ps.own = own;
+  ps.plane = pb->plane;
+  ps.n = n;
+  ps.W = grid ? pb->W : pb->V;
+  ps.H = grid ? pb->H : 1;
+  ps.P = grid ? pb->P : pb->V;
+  ps.perm = grid ? nullptr : pb->d_perm;
+  ps.vec = grid && pb->W % 4 == 0 && reinterpret_cast<uintptr_t>(own) % 16 == 0;
+  for (int c = 0; c < n; ++c) {
+    ps.user[c] = user[c];
+    ps.vec = ps.vec && reinterpret_cast<uintptr_t>(user[c]) % 16 == 0;
+  }
+  const long long units = (long long)ps.W * ps.H / (ps.vec ? 4 : 1);
+  const unsigned blocks = (unsigned)std::max(1ll, std::min((units + 255) / 256, 16ll * pb->sms));
+  if (dir == PlaneDir::In) k_move_planes<true><<<blocks, 256, 0, st>>>(ps, reset, lambda0);
+  else k_move_planes<false><<<blocks, 256, 0, st>>>(ps, nullptr, 0.0);
+  CK(cudaGetLastError());
+  return OPT_OK;
 }
 
 }  // namespace
 
 namespace optgb {
 
-// copy between caller dense planes (caller order) and internal planes
-// (pitched rows for grids, locality order for graphs)
-opt_status copy_planes_in(const opt_problem* pb, float* internal, float* const* user, int n,
-                          cudaStream_t st) {
-  for (int c = 0; c < n; ++c) {
-    if (is_grid(pb)) {
-      CK(cudaMemcpy2DAsync(internal + c * pb->plane, (size_t)pb->P * 4, user[c], (size_t)pb->W * 4,
-                           (size_t)pb->W * 4, pb->H, cudaMemcpyDeviceToDevice, st));
-    } else {
-      k_gather_vertices<<<(pb->V + 255) / 256, 256, 0, st>>>(internal + c * pb->plane, user[c], pb->d_perm, pb->V);
-      CK(cudaGetLastError());
-    }
-  }
-  return OPT_OK;
+opt_status copy_planes_in(const opt_problem* pb, float* internal, float* const* user, int n, cudaStream_t st) {
+  return copy_planes(pb, PlaneDir::In, internal, user, n, st);
 }
-opt_status copy_planes_out(const opt_problem* pb, float* const* user, const float* internal, int n,
-                           cudaStream_t st) {
-  for (int c = 0; c < n; ++c) {
-    if (is_grid(pb)) {
-      CK(cudaMemcpy2DAsync(user[c], (size_t)pb->W * 4, internal + c * pb->plane, (size_t)pb->P * 4,
-                           (size_t)pb->W * 4, pb->H, cudaMemcpyDeviceToDevice, st));
-    } else {
-      k_scatter_vertices<<<(pb->V + 255) / 256, 256, 0, st>>>(user[c], internal + c * pb->plane, pb->d_perm, pb->V);
-      CK(cudaGetLastError());
-    }
-  }
-  return OPT_OK;
+opt_status copy_planes_out(const opt_problem* pb, float* const* user, const float* internal, int n, cudaStream_t st) {
+  return copy_planes(pb, PlaneDir::Out, const_cast<float*>(internal), user, n, st);
 }
 
 }  // namespace optgb
@@ -395,8 +437,7 @@ bool use_resident(const opt_problem* pb, const opt_solve_params& p, bool lm) {
 
 opt_status enqueue_solve(opt_problem* pb, const opt_solve_params& p, bool lm, cudaStream_t st) {
   const float dmin = (float)p.diag_min, dmax = (float)p.diag_max;
-  CKS(copy_planes_in(pb, pb->x, pb->user_x, pb->nx, st));
-  k_reset<<<1, 32, 0, st>>>(pb->d_s, 1, lm ? p.lambda0 : 0.0);
+  CKS(copy_planes(pb, PlaneDir::In, pb->x, pb->user_x, pb->nx, st, pb->d_s, lm ? p.lambda0 : 0.0));
   const bool fused = use_fused(pb, p) && p.inner > 0;
   const bool coop = !fused && use_persistent(pb, p);
   const bool resident = use_resident(pb, p, lm);
@@ -418,8 +459,9 @@ opt_status enqueue_solve(opt_problem* pb, const opt_solve_params& p, bool lm, cu
       CK(launch_grid_pcg_coop(grid_launch(pb, st), pb->d_gbar, 0, p.inner));
     } else if (resident) {
       const ResidentPlan& rp = pb->rplan[lm ? 1 : 0];
-      CK(is_grid(pb) ? launch_resident_grid(pb->kind, pb->dg, pb->d_tiles, pb->d_rsync, rp, pb->d_rrec, p.inner, st)
-                     : launch_resident_graph(pb->kind, pb->dm, pb->d_rsync, rp, pb->d_rrec, p.inner, st));
+      CK(is_grid(pb) ? launch_resident_grid(pb->kind, pb->dg, pb->d_tiles, pb->d_rsync, rp, pb->d_rrec, p.inner,
+                                            lm ? 0 : 1, csn_next, st)
+                     : launch_resident_graph(pb->kind, pb->dm, pb->d_rsync, rp, pb->d_rrec, p.inner, lm ? 0 : 1, st));
     } else {
       for (int i = 0; i < p.inner; ++i) {
         if (p.materialized) csr_apply(pb, st, i, p.materialized);
@@ -428,7 +470,7 @@ opt_status enqueue_solve(opt_problem* pb, const opt_solve_params& p, bool lm, cu
       }
     }
     if (!lm) {
-      if (!fused) st_step(pb, st, 0, csn_next);
+      if (!fused && !resident) st_step(pb, st, 0, csn_next);
     } else {
       st_energy(pb, st, 1, -2);
       k_lm_decide<<<1, 32, 0, st>>>(pb->d_s, 1, p.eta, p.lambda_min, p.lambda_max, p.rel_tol);

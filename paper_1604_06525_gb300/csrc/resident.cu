@@ -661,7 +661,8 @@ struct Lanes {
 template <class K, bool CL>
 __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* __restrict__ probs,
                                                         const int* __restrict__ tiles, ResidentSync* sync,
-                                                        const ResidentPlan rp, float4* rec, int inner) {
+                                                        const ResidentPlan rp, float4* rec, int inner, int step,
+                                                        int csn_out) {
   constexpr int NX = K::NX, NM = K::NM;
   extern __shared__ float sh[];
   const typename K::Prob pr = probs[0];
@@ -964,12 +965,29 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
     if (tid == 0) s->timeout = 1;
     return;
   }
-  if (rp.flags & RES_D) {
+  if ((rp.flags & RES_D) || step) {
     for (int j = tid; j < cnt; j += RT) {
       if (skip(j)) continue;
       const long long i = K::index(ctx, j);
+      float d[NX], x[NX];
 #pragma unroll
-      for (int k = 0; k < NX; ++k) pr.d[k * pl + i] = sd[k * ds + j];
+      for (int k = 0; k < NX; ++k) {
+        d[k] = sd[k * ds + j];
+        if (step) x[k] = pr.x[k * pl + i];
+      }
+#pragma unroll
+      for (int k = 0; k < NX; ++k) {
+        if (rp.flags & RES_D) pr.d[k * pl + i] = d[k];
+        if (step) pr.x[k * pl + i] = x[k] = __fadd_rn(x[k], d[k]);
+      }
+      if constexpr (!K::GRAPH) {
+        if (NX == 3 && step && csn_out && pr.csn) {
+          float sn, cn;
+          sincosf(x[2], &sn, &cn);
+          pr.csn[i] = cn;
+          pr.csn[pl + i] = sn;
+        }
+      }
     }
   }
   if (blockIdx.x == 0 && tid == 0) {
@@ -991,7 +1009,7 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
 
 template <class K, bool CL>
 cudaError_t launch(const typename K::Prob* probs, const int* tiles, ResidentSync* sync, const ResidentPlan& rp,
-                   float4* rec, int inner, cudaStream_t st) {
+                   float4* rec, int inner, int step, int csn_out, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(rp.blocks);
   cfg.blockDim = dim3(RT);
@@ -1011,13 +1029,13 @@ cudaError_t launch(const typename K::Prob* probs, const int* tiles, ResidentSync
   }
   cfg.attrs = attr;
   cfg.numAttrs = CL ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, k_pcg_resident<K, CL>, probs, tiles, sync, rp, rec, inner);
+  return cudaLaunchKernelEx(&cfg, k_pcg_resident<K, CL>, probs, tiles, sync, rp, rec, inner, step, csn_out);
 }
 template <class K>
 cudaError_t launch(const typename K::Prob* probs, const int* tiles, ResidentSync* sync, const ResidentPlan& rp,
-                   float4* rec, int inner, cudaStream_t st) {
-  return rp.cluster ? launch<K, true>(probs, tiles, sync, rp, rec, inner, st)
-                    : launch<K, false>(probs, tiles, sync, rp, rec, inner, st);
+                   float4* rec, int inner, int step, int csn_out, cudaStream_t st) {
+  return rp.cluster ? launch<K, true>(probs, tiles, sync, rp, rec, inner, step, csn_out, st)
+                    : launch<K, false>(probs, tiles, sync, rp, rec, inner, step, csn_out, st);
 }
 
 struct DeviceLimits {
@@ -1184,18 +1202,19 @@ ResidentPlan resident_plan(int kind, int n, long long plane, int lm, const int* 
 }
 
 cudaError_t launch_resident_grid(int kind, const GridProb* probs, const int* tiles, ResidentSync* sync,
-                                 const ResidentPlan& rp, float4* rec, int inner, cudaStream_t st) {
-  return kind == K_WARP ? launch<WarpKind>(probs, tiles, sync, rp, rec, inner, st)
-                        : launch<PoissonKind>(probs, tiles, sync, rp, rec, inner, st);
+                                 const ResidentPlan& rp, float4* rec, int inner, int step, int csn_out,
+                                 cudaStream_t st) {
+  return kind == K_WARP ? launch<WarpKind>(probs, tiles, sync, rp, rec, inner, step, csn_out, st)
+                        : launch<PoissonKind>(probs, tiles, sync, rp, rec, inner, step, 0, st);
 }
 
 cudaError_t launch_resident_graph(int kind, const MeshProb* probs, ResidentSync* sync, const ResidentPlan& rp,
-                                  float4* rec, int inner, cudaStream_t st) {
+                                  float4* rec, int inner, int step, cudaStream_t st) {
   switch (kind) {
-    case K_VOLUME: return launch<MeshKind<true>>(probs, nullptr, sync, rp, rec, inner, st);
-    case K_WARPG: return launch<WarpGraphKind>(probs, nullptr, sync, rp, rec, inner, st);
-    case K_EMBED: return launch<EmbeddedKind>(probs, nullptr, sync, rp, rec, inner, st);
-    default: return launch<MeshKind<false>>(probs, nullptr, sync, rp, rec, inner, st);
+    case K_VOLUME: return launch<MeshKind<true>>(probs, nullptr, sync, rp, rec, inner, step, 0, st);
+    case K_WARPG: return launch<WarpGraphKind>(probs, nullptr, sync, rp, rec, inner, step, 0, st);
+    case K_EMBED: return launch<EmbeddedKind>(probs, nullptr, sync, rp, rec, inner, step, 0, st);
+    default: return launch<MeshKind<false>>(probs, nullptr, sync, rp, rec, inner, step, 0, st);
   }
 }
 
