@@ -117,6 +117,7 @@ struct GridGroup {
   int lattice = 0;                     // every member has GridProb::lattice
   std::vector<int> members;            // indices into opt_batch::probs
   GridProb* d_probs = nullptr;
+  std::vector<GridProb> h_probs;       // as on the device
   Chunk* d_chunks = nullptr;
   int* d_tiles = nullptr;
   double* d_part = nullptr;
@@ -128,6 +129,7 @@ struct MeshGroup {
   int grid3 = 0;                       // volumetric problems (7-point stencil)
   std::vector<int> members;
   MeshProb* d_probs = nullptr;
+  std::vector<MeshProb> h_probs;       // as on the device
   Chunk* d_vch = nullptr;
   Chunk* d_ech = nullptr;
   Chunk* d_tch = nullptr;              // tile chunks of the tiled ARAP-mesh apply (NULL: some member untiled)
@@ -147,6 +149,7 @@ struct opt_batch {
   std::vector<void*> allocs;        // fixed for the batch's life
   Scalars** d_stab = nullptr;
   double** d_htab = nullptr;
+  std::vector<double*> h_htab;      // as on the device (none yet: nullptr)
   PlaneCopy* d_copy_in = nullptr;
   PlaneCopy* d_copy_out = nullptr;
   int ncopy = 0, max_plane = 0;
@@ -256,6 +259,7 @@ opt_status build_tables(opt_batch* b, int tpc) {
     if ((s = bupload(b->table_allocs, &g.d_tiles, tiles)) != OPT_OK) return s;
     if ((s = balloc(b->table_allocs, &g.d_part, 4 * chunks.size())) != OPT_OK) return s;   // up to 4 partials
     g.nchunks = (int)chunks.size();
+    g.h_probs = gp;
   }
   for (MeshGroup& g : b->graphs) {
     if (g.members.empty()) continue;
@@ -295,6 +299,7 @@ opt_status build_tables(opt_batch* b, int tpc) {
     g.nv = (int)vch.size();
     g.ne = (int)ech.size();
     g.nt = tiled ? (int)tch.size() : 0;
+    g.h_probs = mp;
   }
   b->tiles_per_chunk = tpc;
   return OPT_OK;
@@ -308,7 +313,7 @@ MeshLaunch ml(const MeshGroup& g, cudaStream_t st) {
 }
 
 // Uploads the members' descriptors with the solve's flags (outside any capture).
-opt_status refresh_descriptors(opt_batch* b, int lm, int use_precond, int outer) {
+opt_status refresh_descriptors(opt_batch* b, int lm, int use_precond, int outer, cudaStream_t st) {
   for (opt_problem* pb : b->probs) {
     if (pb->Ehist_cap < outer + 1) {
       double* e = nullptr;
@@ -326,37 +331,36 @@ opt_status refresh_descriptors(opt_batch* b, int lm, int use_precond, int outer)
       }
     }
   }
-  for (GridGroup& g : b->grids) {
-    std::vector<GridProb> gp(g.members.size());
-    BCK(cudaMemcpy(gp.data(), g.d_probs, gp.size() * sizeof(GridProb), cudaMemcpyDeviceToHost));
-    for (size_t i = 0; i < gp.size(); ++i) {
-      opt_problem* pb = b->probs[g.members[i]];
-      gp[i].lm = lm;
-      gp[i].use_precond = use_precond;
-      gp[i].Ehist = pb->d_Ehist;
-      gp[i].jtf_out = nullptr;
-      gp[i].diag_out = nullptr;
+  bool waited = false;
+  // copies host -> device only what differs from what is there, after the stream's work
+  const auto put = [&](void* dev, void* there, const void* want, size_t bytes) -> opt_status {
+    if (!std::memcmp(there, want, bytes)) return OPT_OK;
+    if (!waited) BCK(cudaStreamSynchronize(st));
+    waited = true;
+    BCK(cudaMemcpy(dev, want, bytes, cudaMemcpyHostToDevice));
+    std::memcpy(there, want, bytes);
+    return OPT_OK;
+  };
+  const auto refresh = [&](auto& g) -> opt_status {
+    auto want = g.h_probs;
+    for (size_t i = 0; i < want.size(); ++i) {
+      want[i].lm = lm;
+      want[i].use_precond = use_precond;
+      want[i].Ehist = b->probs[g.members[i]]->d_Ehist;
+      want[i].jtf_out = nullptr;
+      want[i].diag_out = nullptr;
     }
-    BCK(cudaMemcpy(g.d_probs, gp.data(), gp.size() * sizeof(GridProb), cudaMemcpyHostToDevice));
-  }
-  for (MeshGroup& g : b->graphs) {
-    if (g.members.empty()) continue;
-    std::vector<MeshProb> mp(g.members.size());
-    BCK(cudaMemcpy(mp.data(), g.d_probs, mp.size() * sizeof(MeshProb), cudaMemcpyDeviceToHost));
-    for (size_t i = 0; i < mp.size(); ++i) {
-      opt_problem* pb = b->probs[g.members[i]];
-      mp[i].lm = lm;
-      mp[i].use_precond = use_precond;
-      mp[i].Ehist = pb->d_Ehist;
-      mp[i].jtf_out = nullptr;
-      mp[i].diag_out = nullptr;
-    }
-    BCK(cudaMemcpy(g.d_probs, mp.data(), mp.size() * sizeof(MeshProb), cudaMemcpyHostToDevice));
-  }
+    return put(g.d_probs, g.h_probs.data(), want.data(), want.size() * sizeof(want[0]));
+  };
+  opt_status s;
+  for (GridGroup& g : b->grids)
+    if ((s = refresh(g)) != OPT_OK) return s;
+  for (MeshGroup& g : b->graphs)
+    if (!g.members.empty() && (s = refresh(g)) != OPT_OK) return s;
   std::vector<double*> ht;
   for (opt_problem* pb : b->probs) ht.push_back(pb->d_Ehist);
-  BCK(cudaMemcpy(b->d_htab, ht.data(), ht.size() * sizeof(double*), cudaMemcpyHostToDevice));
-  return OPT_OK;
+  b->h_htab.resize(ht.size(), nullptr);
+  return put(b->d_htab, b->h_htab.data(), ht.data(), ht.size() * sizeof(double*));
 }
 
 void enqueue_copies(opt_batch* b, const PlaneCopy* tab, cudaStream_t st) {
@@ -478,13 +482,17 @@ opt_status batch_solve(opt_batch* b, const opt_solve_params* prm_in, opt_report*
   if (lm && (!(p.lambda0 >= 0.0) || !(p.lambda_min <= p.lambda_max) || !(p.diag_min <= p.diag_max)))
     return OPT_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)p.stream;
-  BCK(cudaStreamSynchronize(st));
-  opt_status s = refresh_descriptors(b, lm ? 1 : 0, p.use_precond, p.outer);
+  opt_status s = refresh_descriptors(b, lm ? 1 : 0, p.use_precond, p.outer, st);
   if (s != OPT_OK) return s;
   const int n = (int)b->probs.size();
   const int hlen = p.outer + 1;
   if (b->hcap < hlen) {
-    if ((s = balloc(b->allocs, &b->d_hout, (size_t)n * hlen)) != OPT_OK) return s;
+    // the members' scalars and histories next to each other: one copy fetches them
+    BCK(cudaStreamSynchronize(st));
+    char* r = nullptr;
+    if ((s = balloc(b->allocs, &r, n * (sizeof(Scalars) + hlen * sizeof(double)))) != OPT_OK) return s;
+    b->d_sout = reinterpret_cast<Scalars*>(r);
+    b->d_hout = reinterpret_cast<double*>(b->d_sout + n);
     b->hcap = hlen;
   }
   const std::vector<double> key = {double(p.outer), double(p.inner), double(lm), double(p.use_precond), p.lambda0,
@@ -522,14 +530,16 @@ opt_status batch_solve(opt_batch* b, const opt_solve_params* prm_in, opt_report*
   }
   k_gather_results<<<n, 128, 0, st>>>(b->d_stab, b->d_htab, n, hlen, b->d_sout, b->d_hout);
   BCK(cudaGetLastError());
+  std::vector<char> res(n * (sizeof(Scalars) + hlen * sizeof(double)));
+  BCK(cudaMemcpyAsync(res.data(), b->d_sout, res.size(), cudaMemcpyDeviceToHost, st));
   BCK(cudaStreamSynchronize(st));
   float ms = 0.f;
   BCK(cudaEventElapsedTime(&ms, b->ev0, b->ev1));
   if (ms_out) *ms_out = ms;
   std::vector<Scalars> sv(n);
   std::vector<double> hv((size_t)n * hlen);
-  BCK(cudaMemcpy(sv.data(), b->d_sout, n * sizeof(Scalars), cudaMemcpyDeviceToHost));
-  BCK(cudaMemcpy(hv.data(), b->d_hout, hv.size() * sizeof(double), cudaMemcpyDeviceToHost));
+  std::memcpy(sv.data(), res.data(), n * sizeof(Scalars));
+  std::memcpy(hv.data(), res.data() + n * sizeof(Scalars), hv.size() * sizeof(double));
   bool nonfinite = false, timeout = false, misaligned = false;
   for (int i = 0; i < n; ++i) {
     const Scalars& t = sv[i];
@@ -697,8 +707,8 @@ opt_status opt_batch_autotune(opt_batch* b, const opt_solve_params* params, int3
 // ---------------------------------------------------------------------------
 namespace optgb {
 
-opt_status batch_prepare_round(opt_batch* b, const opt_solve_params& p) {
-  return refresh_descriptors(b, 1, p.use_precond, 1);
+opt_status batch_prepare_round(opt_batch* b, const opt_solve_params& p, cudaStream_t st) {
+  return refresh_descriptors(b, 1, p.use_precond, 1, st);
 }
 
 opt_status batch_reserve_rounds(opt_batch* b, int rounds) {

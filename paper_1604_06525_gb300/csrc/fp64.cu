@@ -1132,6 +1132,7 @@ struct opt_problem_f64 {
   Scalars* d_s = nullptr;
   double* d_Ehist = nullptr;
   int Ehist_cap = 0;
+  Scalars* d_res = nullptr;      // the last solve's scalars and energies (SolveResult)
   double* d_pin = nullptr;      // apply hook: caller p copied here (nx planes)
   ResidentSync* d_rsync = nullptr;   // resident PCG loop (NULL: launches per phase)
   int loop_blocks = 0, loop_per = 0, loop_smem = 0;
@@ -1331,13 +1332,36 @@ void k_energy(opt_problem_f64* pb, const P64& P, cudaStream_t st, int mode, int 
   else k64_mesh_energy<<<pb->nblk, NT, 0, st>>>(P, mode, hist);
 }
 
-opt_status copy_x(opt_problem_f64* pb, bool in, cudaStream_t st) {
-  const size_t bytes = (size_t)pb->hp.n * sizeof(double);
-  for (int c = 0; c < pb->nx; ++c) {
-    double* dev = pb->hp.x + (size_t)c * pb->hp.n;
-    if (in) CK64(cudaMemcpyAsync(dev, pb->user_x[c], bytes, cudaMemcpyDeviceToDevice, st));
-    else CK64(cudaMemcpyAsync(pb->user_x[c], dev, bytes, cudaMemcpyDeviceToDevice, st));
-  }
+// All unknown planes in one launch: on the way in of a solve with its scalars reset, on
+// the way out with its result gathered.
+struct Planes64 {
+  double* user[6];
+  double* own;
+  long long n;
+  int planes;
+};
+template <bool IN>
+__global__ void __launch_bounds__(NT) k64_move_planes(const __grid_constant__ Planes64 ps, Scalars* reset,
+                                                      double lambda0, const SolveResult res) {
+  if (!IN) gather_result(res);
+  if (IN && reset && blockIdx.x == 0 && threadIdx.x == 0) scalars_reset(reset, lambda0);
+  for (long long k = blockIdx.x * (long long)NT + threadIdx.x; k < ps.n; k += (long long)gridDim.x * NT)
+    for (int c = 0; c < ps.planes; ++c) {
+      if (IN) ps.own[c * ps.n + k] = ps.user[c][k];
+      else ps.user[c][k] = ps.own[c * ps.n + k];
+    }
+}
+opt_status copy_x(opt_problem_f64* pb, bool in, cudaStream_t st, Scalars* reset = nullptr, double lambda0 = 0.0,
+                  const SolveResult& res = SolveResult{}) {
+  Planes64 ps = {};
+  for (int c = 0; c < pb->nx; ++c) ps.user[c] = pb->user_x[c];
+  ps.own = pb->hp.x;
+  ps.n = pb->hp.n;
+  ps.planes = pb->nx;
+  const unsigned blocks = (unsigned)std::max(1ll, std::min((ps.n + NT - 1) / NT, 8ll * pb->nblk));
+  if (in) k64_move_planes<true><<<blocks, NT, 0, st>>>(ps, reset, lambda0, res);
+  else k64_move_planes<false><<<blocks, NT, 0, st>>>(ps, nullptr, 0.0, res);
+  CK64(cudaGetLastError());
   return OPT_OK;
 }
 
@@ -1360,8 +1384,7 @@ opt_status enqueue_solve64(opt_problem_f64* pb, const opt_solve_params& p, bool 
   P.use_precond = p.use_precond;
   P.Ehist = pb->d_Ehist;
   pb->hp = P;
-  CKS64(copy_x(pb, true, st));
-  k64_reset<<<1, 1, 0, st>>>(pb->d_s, lm ? p.lambda0 : 0.0);
+  CKS64(copy_x(pb, true, st, pb->d_s, lm ? p.lambda0 : 0.0));
   for (int k = 0; k < p.outer; ++k) {
     k_rot(pb, st);
     k_init(pb, P, st, k, p.diag_min, p.diag_max);
@@ -1382,7 +1405,7 @@ opt_status enqueue_solve64(opt_problem_f64* pb, const opt_solve_params& p, bool 
     }
   }
   k_energy(pb, P, st, 0, lm ? -1 : p.outer);
-  CKS64(copy_x(pb, false, st));
+  CKS64(copy_x(pb, false, st, nullptr, 0.0, SolveResult{pb->d_s, pb->d_Ehist, p.outer + 1, pb->d_res}));
   CK64(cudaGetLastError());
   return OPT_OK;
 }
@@ -1394,14 +1417,18 @@ opt_status run_solve64(opt_problem_f64* pb, const opt_solve_params* prm_in, opt_
   else opt_solve_params_default(&p);
   CKS64(check_params64(p, lm));
   cudaStream_t st = (cudaStream_t)p.stream;
-  CK64(cudaStreamSynchronize(st));
   if (pb->Ehist_cap < p.outer + 1) {
+    CK64(cudaStreamSynchronize(st));
     if (pb->gexec) {
       cudaGraphExecDestroy(pb->gexec);
       pb->gexec = nullptr;
       pb->gkey.clear();
     }
     CKS64(alloc64(pb, &pb->d_Ehist, (size_t)p.outer + 1));
+    char* r = nullptr;
+    CKS64(alloc64(pb, &r, sizeof(Scalars) + (size_t)(p.outer + 1) * sizeof(double)));
+    pb->d_res = reinterpret_cast<Scalars*>(r);
+    CK64(cudaStreamSynchronize(nullptr));
     pb->Ehist_cap = p.outer + 1;
   }
   if (p.use_graph) {
@@ -1435,12 +1462,14 @@ opt_status run_solve64(opt_problem_f64* pb, const opt_solve_params* prm_in, opt_
     CKS64(enqueue_solve64(pb, p, lm, st));
     CK64(cudaEventRecord(pb->ev1, st));
   }
-  CK64(cudaEventSynchronize(pb->ev1));
+  std::vector<char> res(sizeof(Scalars) + (size_t)(p.outer + 1) * sizeof(double));
+  CK64(cudaMemcpyAsync(res.data(), pb->d_res, res.size(), cudaMemcpyDeviceToHost, st));
+  CK64(cudaStreamSynchronize(st));
   Scalars s;
-  CK64(cudaMemcpy(&s, pb->d_s, sizeof(Scalars), cudaMemcpyDeviceToHost));
+  std::memcpy(&s, res.data(), sizeof(Scalars));
   const int outer_done = lm ? s.outer_done : p.outer;
-  std::vector<double> eh;
-  CKS64(download64(eh, pb->d_Ehist, (size_t)outer_done + 1));
+  std::vector<double> eh((size_t)outer_done + 1);
+  std::memcpy(eh.data(), res.data() + sizeof(Scalars), eh.size() * sizeof(double));
   if (rep) {
     rep->outer_done = outer_done;
     rep->pcg_done = s.pcg_iters;

@@ -83,6 +83,21 @@ struct __align__(16) Scalars {
   double beta_d;      // float64 solver: beta  = rz' / rz
 };
 
+// What a solve reports, gathered by its last launch: *s and the first n energies, next
+// to each other, so that one copy fetches them.
+struct SolveResult {
+  const Scalars* s;
+  const double* E;
+  int n;
+  Scalars* out;                 // followed by n doubles
+};
+__device__ __forceinline__ void gather_result(const SolveResult& r) {
+  if (r.out == nullptr || blockIdx.x != 0) return;
+  if (threadIdx.x == 0) *r.out = *r.s;
+  double* e = reinterpret_cast<double*>(r.out + 1);
+  for (int k = threadIdx.x; k < r.n; k += blockDim.x) e[k] = r.E[k];
+}
+
 struct Chunk {
   int prob;           // problem index
   int begin, end;     // tile (grid) / vertex / edge range

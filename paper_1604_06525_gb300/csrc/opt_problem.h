@@ -83,6 +83,12 @@ struct opt_problem {
   optgb::Scalars* d_s = nullptr;
   double* d_Ehist = nullptr;
   int Ehist_cap = 0;
+  optgb::Scalars* d_res = nullptr;      // the last solve's scalars and energies (SolveResult)
+  int res_cap = 0;                      // energies it has room for
+  // the descriptor on the device, as last uploaded
+  optgb::GridProb sent_hg{};
+  optgb::MeshProb sent_hm{};
+  bool sent = false;
   float* user_x[12] = {};
   float* d_tmp = nullptr;     // nx planes: caller p (apply hook)
   float* d_jtf = nullptr;     // nx planes: J^T F (hook)
@@ -129,6 +135,8 @@ struct opt_problem {
     swap(h_mask, o.h_mask); swap(h_hpix, o.h_hpix); swap(h_e0, o.h_e0); swap(h_e1, o.h_e1); swap(h_orow, o.h_orow);
     swap(d_perm, o.d_perm); swap(csr, o.csr);
     swap(d_part, o.d_part); swap(d_s, o.d_s); swap(d_Ehist, o.d_Ehist); swap(Ehist_cap, o.Ehist_cap);
+    swap(d_res, o.d_res); swap(res_cap, o.res_cap);
+    swap(sent_hg, o.sent_hg); swap(sent_hm, o.sent_hm); swap(sent, o.sent);
     swap(user_x, o.user_x); swap(d_tmp, o.d_tmp); swap(d_jtf, o.d_jtf); swap(d_diag, o.d_diag);
     swap(x, o.x); swap(pbuf, o.pbuf); swap(dvec, o.dvec); swap(rvec, o.rvec); swap(qvec, o.qvec);
     swap(allocs, o.allocs); swap(pooled, o.pooled); swap(pcg_par, o.pcg_par);
@@ -164,7 +172,7 @@ struct RoundRec {
   double E, E_trial;
   int accept, outer_done;
 };
-opt_status batch_prepare_round(opt_batch* b, const opt_solve_params& p);
+opt_status batch_prepare_round(opt_batch* b, const opt_solve_params& p, cudaStream_t st);
 // Room for `rounds` rounds of records (one RoundRec per member and round).
 opt_status batch_reserve_rounds(opt_batch* b, int rounds);
 // One LM outer iteration of every member; the records of round `round` (of

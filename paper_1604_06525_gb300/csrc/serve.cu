@@ -320,7 +320,7 @@ opt_status opt_server_step(opt_server* s, int32_t* n_active, int32_t* n_queued) 
       opt_status st = s->inject;
       s->inject = OPT_OK;
       if (st == OPT_OK) st = opt_batch_create(ps.data(), (int)ps.size(), &s->batch);
-      if (st == OPT_OK) st = batch_prepare_round(s->batch, s->prm);
+      if (st == OPT_OK) st = batch_prepare_round(s->batch, s->prm, s->st);
       if (st != OPT_OK) return counts(fail_active(s, st));
       s->dirty = false;
     }

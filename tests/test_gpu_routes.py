@@ -148,3 +148,38 @@ def test_requests_planned_together_fail_alone():
         alone.close()
     torch.cuda.synchronize()
     srv.close()
+
+
+@pytest.mark.parametrize("kind", ["warp", "mesh", "mesh64"])
+def test_repeated_solves_equal_fresh_ones(kind):
+    """Nothing of a call (its method, preconditioner, history length, a product in
+    between) stays in the next one's descriptor, graph or results."""
+    from paper_1604_06525_gb300 import api
+    prob = make(("warp", 150, 40, 1)) if kind == "warp" else make(("mesh", 3, 1.0))
+    cls = api.ProblemF64 if kind.endswith("64") else api.Problem
+    calls = [("gn", 2, 5, {}), ("lm", 3, 4, {}), ("lm", 3, 4, {}), ("gn", 5, 3, {"use_precond": 0}), ("gn", 2, 5, {}),
+             ("lm", 2, 6, {"use_graph": 0}), ("lm", 6, 2, {})]
+    g = cls(prob)
+    x0 = g.x.clone()
+    batch_members = [] if kind.endswith("64") else [api.Problem(prob), api.Problem(prob)]
+    batch = api.Batch(batch_members) if batch_members else None
+    for method, outer, inner, kw in calls:
+        fresh = cls(prob)
+        want = getattr(fresh, "solve_" + method)(outer, inner, **kw)
+        g.x.copy_(x0)
+        got = getattr(g, "solve_" + method)(outer, inner, **kw)
+        assert got["E_history"] == want["E_history"] and got["pcg_done"] == want["pcg_done"]
+        np.testing.assert_array_equal(g.x.cpu().numpy(), fresh.x.cpu().numpy())
+        fresh.close()
+        g.eval_jtf()
+        if batch:
+            for m in batch_members:
+                m.x.copy_(x0)
+            reports, _ = getattr(batch, "solve_" + method)(outer, inner, **kw)
+            for r in reports:
+                assert len(r["E_history"]) == len(want["E_history"])
+                for s, t in zip(r["E_history"], want["E_history"]):
+                    assert abs(s - t) <= 1e-5 * max(abs(t), 1e-3 * abs(want["E_history"][0]))
+    if batch:
+        batch.close()
+    g.close()
