@@ -419,7 +419,7 @@ opt_status resident_prepare(opt_problem* pb, int lm) {
   const bool grid = is_grid(pb);
   ResidentPlan rp;
   if (grid) {
-    const long long n = (long long)pb->ntiles * pb->hg.tw * TH;
+    const long long n = (long long)pb->h_cells.size() * TW * TH;
     // (records are indexed like the planes: a sparse mask on a huge image is left to the tiled kernels)
     rp = n > (1 << 22) || pb->plane > (1 << 24) ? ResidentPlan{} : resident_plan(pb->kind, (int)n, pb->plane, lm, nullptr);
   } else {
@@ -429,6 +429,10 @@ opt_status resident_prepare(opt_problem* pb, int lm) {
     if (!pb->d_rsync) {
       CKS(dalloc(pb, &pb->d_rsync, 1));
       CK(cudaMemsetAsync(pb->d_rsync->slot, 0xff, sizeof(pb->d_rsync->slot), nullptr));
+    }
+    if (grid && !pb->d_cells) {
+      CKS(dalloc(pb, &pb->d_cells, pb->h_cells.size()));
+      CKS(upload(pb->d_cells, pb->h_cells));
     }
     if (!pb->d_rrec) CKS(dalloc(pb, &pb->d_rrec, resident_records(pb->kind, pb->plane)));
     CK(cudaStreamSynchronize(nullptr));
@@ -469,7 +473,7 @@ opt_status enqueue_solve(opt_problem* pb, const opt_solve_params& p, bool lm, cu
       CK(launch_grid_pcg_coop(grid_launch(pb, st), pb->d_gbar, 0, p.inner));
     } else if (resident) {
       const ResidentPlan& rp = pb->rplan[lm ? 1 : 0];
-      CK(is_grid(pb) ? launch_resident_grid(pb->kind, pb->dg, pb->d_tiles, pb->d_rsync, rp, pb->d_rrec, p.inner,
+      CK(is_grid(pb) ? launch_resident_grid(pb->kind, pb->dg, pb->d_cells, pb->d_rsync, rp, pb->d_rrec, p.inner,
                                             lm ? 0 : 1, csn_next, st)
                      : launch_resident_graph(pb->kind, pb->dm, pb->d_rsync, rp, pb->d_rrec, p.inner, lm ? 0 : 1, st));
     } else {
@@ -841,16 +845,20 @@ opt_status opt_problem_create_grid(const opt_grid_desc* d, const opt_solve_param
 
   // active tiles: at least one unmasked (warp) / free (Poisson) pixel
   const int ntx = (W + tw - 1) / tw, nty = (H + TH - 1) / TH;
-  std::vector<int> tiles;
+  std::vector<int> tiles, cells;
   for (int ty = 0; ty < nty; ++ty)
     for (int tx = 0; tx < ntx; ++tx) {
-      bool act = mask.empty();
-      for (int y = ty * TH; !act && y < std::min(H, ty * TH + TH); ++y)
-        for (int x = tx * tw; x < std::min(W, tx * tw + tw); ++x)
-          if (mask[(size_t)y * W + x] == 0) { act = true; break; }
-      if (act) tiles.push_back((ty << 16) | tx);
+      const size_t before = cells.size();
+      for (int cx = tx * tw; cx < std::min(W, tx * tw + tw); cx += TW) {
+        bool act = mask.empty();
+        for (int y = ty * TH; !act && y < std::min(H, ty * TH + TH); ++y)
+          act = std::memchr(&mask[(size_t)y * W + cx], 0, (size_t)std::min(W - cx, TW)) != nullptr;
+        if (act) cells.push_back((ty << 16) | (cx / TW));
+      }
+      if (cells.size() > before) tiles.push_back((ty << 16) | tx);
     }
   if (tiles.empty()) tiles.push_back(0);
+  if (cells.empty()) cells.push_back(0);
   std::vector<Chunk> chunks = make_chunks_balanced((int)tiles.size(), pb->sms * kDefaultBlocksPerSM, 0);
 
   // handles sorted by tile
@@ -948,6 +956,7 @@ opt_status opt_problem_create_grid(const opt_grid_desc* d, const opt_solve_param
   CKS(dalloc(q, &q->d_tiles, tiles.size()));
   CKS(upload(q->d_tiles, tiles));
   q->h_tiles = tiles;
+  q->h_cells = cells;
   q->ntiles = (int)tiles.size();
   CKS(dalloc(q, &q->d_chunks, chunks.size()));
   CKS(upload(q->d_chunks, chunks));

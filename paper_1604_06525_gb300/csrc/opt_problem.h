@@ -70,6 +70,8 @@ struct opt_problem {
   opt_grid_desc grid_desc{};            //   tile width (its arrays are the caller's and outlive the problem)
   // host mirrors of the work tables (batches build their combined tables from these)
   std::vector<int> h_tiles;
+  std::vector<int> h_cells;             // 32 x 8 pixel cells holding an unmasked / free pixel
+  int* d_cells = nullptr;               // on the device where the resident loop may run
   std::vector<optgb::Chunk> h_chunks, h_vch, h_ech, h_tch;
   // host copies kept for building the materialized Jacobian
   std::vector<unsigned char> h_mask;    // grid mask (empty = none)
@@ -130,7 +132,7 @@ struct opt_problem {
     swap(nvchunks, o.nvchunks); swap(nechunks, o.nechunks); swap(d_tchunks, o.d_tchunks);
     swap(ntchunks, o.ntchunks); swap(tileable, o.tileable); swap(apply_form, o.apply_form); swap(chunking, o.chunking);
     swap(tile_w, o.tile_w); swap(has_grid_desc, o.has_grid_desc); swap(grid_desc, o.grid_desc);
-    swap(h_tiles, o.h_tiles); swap(h_chunks, o.h_chunks); swap(h_vch, o.h_vch); swap(h_ech, o.h_ech);
+    swap(h_tiles, o.h_tiles); swap(h_cells, o.h_cells); swap(d_cells, o.d_cells); swap(h_chunks, o.h_chunks); swap(h_vch, o.h_vch); swap(h_ech, o.h_ech);
     swap(h_tch, o.h_tch);
     swap(h_mask, o.h_mask); swap(h_hpix, o.h_hpix); swap(h_e0, o.h_e0); swap(h_e1, o.h_e1); swap(h_orow, o.h_orow);
     swap(d_perm, o.d_perm); swap(csr, o.csr);

@@ -54,7 +54,12 @@ namespace optgb {
 
 namespace {
 
-constexpr int CELL = 256;             // grids: 32 x 8 pixels
+// Grids: 32 x 8 pixels.  The loop runs over the cells that hold an unknown, not over
+// the tiles of the launches: of the 128-pixel tiles that a region to edit touches up to
+// half the pixels are fixed, which took shared memory and passes, and now and then the
+// loop did not fit (1024^2 Poisson, 30 % free, GN 2 x 20: 0.50 ms, or 0.80 ms in
+// launches, by where the region lies; 0.47 ms over the cells).
+constexpr int CELL = 256;
 
 __device__ __forceinline__ unsigned cluster_rank() {
   unsigned r;
@@ -200,7 +205,7 @@ __device__ __forceinline__ float4 load_rec(const Records& R, long long k) {
 // --- grids -----------------------------------------------------------------
 struct GridCtx {
   const GridProb& pr;
-  const int* tiles;
+  const int* cells;
   float2* csn;          // warp: cos / sin of theta, index y * P + x
   int* idx;             // shared: plane index of each unit
   int* flg;             // shared: neighbour flags of each unit
@@ -213,11 +218,9 @@ struct GridUnits {
   static constexpr int NR = 1;
   static __device__ __forceinline__ bool locate(const GridCtx& c, int u, int& x, int& y) {
     const GridProb& pr = c.pr;
-    const int cell = u / CELL, t = u % CELL;
-    const int per = pr.tw / TW;
-    const int tc = c.tiles[cell / per];
-    x = (tc & 0xffff) * pr.tw + (cell % per) * TW + (t & 31);
-    y = (tc >> 16) * TH + (t >> 5);
+    const int cc = c.cells[u / CELL], t = u % CELL;
+    x = (cc & 0xffff) * TW + (t & 31);
+    y = (cc >> 16) * TH + (t >> 5);
     return x < pr.W && y < pr.H;
   }
   static __device__ __forceinline__ int index(const GridCtx& c, int j) { return c.idx[j]; }
@@ -660,7 +663,7 @@ struct Lanes {
 
 template <class K, bool CL>
 __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* __restrict__ probs,
-                                                        const int* __restrict__ tiles, ResidentSync* sync,
+                                                        const int* __restrict__ cells, ResidentSync* sync,
                                                         const ResidentPlan rp, float4* rec, int inner, int step,
                                                         int csn_out) {
   constexpr int NX = K::NX, NM = K::NM;
@@ -747,7 +750,7 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
     } else {
       sp = take(NX * cap);
       idx = reinterpret_cast<int*>(take(cap));
-      return GridCtx{pr, tiles, reinterpret_cast<float2*>(rec + 3 * pl), idx, flg};
+      return GridCtx{pr, cells, reinterpret_cast<float2*>(rec + 3 * pl), idx, flg};
     }
   }();
   // the vertices behind the entries of edges that leave the block
@@ -1008,7 +1011,7 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
 }
 
 template <class K, bool CL>
-cudaError_t launch(const typename K::Prob* probs, const int* tiles, ResidentSync* sync, const ResidentPlan& rp,
+cudaError_t launch(const typename K::Prob* probs, const int* cells, ResidentSync* sync, const ResidentPlan& rp,
                    float4* rec, int inner, int step, int csn_out, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(rp.blocks);
@@ -1029,13 +1032,13 @@ cudaError_t launch(const typename K::Prob* probs, const int* tiles, ResidentSync
   }
   cfg.attrs = attr;
   cfg.numAttrs = CL ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, k_pcg_resident<K, CL>, probs, tiles, sync, rp, rec, inner, step, csn_out);
+  return cudaLaunchKernelEx(&cfg, k_pcg_resident<K, CL>, probs, cells, sync, rp, rec, inner, step, csn_out);
 }
 template <class K>
-cudaError_t launch(const typename K::Prob* probs, const int* tiles, ResidentSync* sync, const ResidentPlan& rp,
+cudaError_t launch(const typename K::Prob* probs, const int* cells, ResidentSync* sync, const ResidentPlan& rp,
                    float4* rec, int inner, int step, int csn_out, cudaStream_t st) {
-  return rp.cluster ? launch<K, true>(probs, tiles, sync, rp, rec, inner, step, csn_out, st)
-                    : launch<K, false>(probs, tiles, sync, rp, rec, inner, step, csn_out, st);
+  return rp.cluster ? launch<K, true>(probs, cells, sync, rp, rec, inner, step, csn_out, st)
+                    : launch<K, false>(probs, cells, sync, rp, rec, inner, step, csn_out, st);
 }
 
 struct DeviceLimits {
@@ -1146,7 +1149,7 @@ size_t resident_records(int kind, long long plane) {
 #define RES_Z_UNITS 32768
 #endif
 // Blocks, shared memory and what it holds for a problem of n units (pixels of
-// the active tiles in cells of 256, or vertices); blocks = 0 if the state does
+// the listed cells, or vertices); blocks = 0 if the state does
 // not fit.  orow: the CSR rows of a graph whose edges are given both ways (else
 // NULL).
 ResidentPlan resident_plan(int kind, int n, long long plane, int lm, const int* orow) {
@@ -1201,11 +1204,11 @@ ResidentPlan resident_plan(int kind, int n, long long plane, int lm, const int* 
   return rp;
 }
 
-cudaError_t launch_resident_grid(int kind, const GridProb* probs, const int* tiles, ResidentSync* sync,
+cudaError_t launch_resident_grid(int kind, const GridProb* probs, const int* cells, ResidentSync* sync,
                                  const ResidentPlan& rp, float4* rec, int inner, int step, int csn_out,
                                  cudaStream_t st) {
-  return kind == K_WARP ? launch<WarpKind>(probs, tiles, sync, rp, rec, inner, step, csn_out, st)
-                        : launch<PoissonKind>(probs, tiles, sync, rp, rec, inner, step, 0, st);
+  return kind == K_WARP ? launch<WarpKind>(probs, cells, sync, rp, rec, inner, step, csn_out, st)
+                        : launch<PoissonKind>(probs, cells, sync, rp, rec, inner, step, 0, st);
 }
 
 cudaError_t launch_resident_graph(int kind, const MeshProb* probs, ResidentSync* sync, const ResidentPlan& rp,

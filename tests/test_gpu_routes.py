@@ -42,6 +42,14 @@ def make(case):
         return synth.warp_problem(W, H, max(1, W * H // 300), seed=W + H, max_disp=2.0, mask=mask)
     if kind == "poisson":
         return synth.poisson_problem(a[0], a[1], seed=a[0])
+    if kind in ("cutout", "patch"):        # whole cells and tiles without an unknown
+        W, H = a
+        mask = np.ones((H, W), np.uint8)
+        mask[H // 3:H // 3 + 11, 5:W - 3] = 0
+        mask[:, W // 2] = 0
+        if kind == "patch":
+            return synth.poisson_problem(W, H, seed=4, mask=mask)
+        return synth.warp_problem(W, H, 9, seed=6, max_disp=2.0, mask=mask)
     if kind == "graph":
         return synth.warp_graph_from_grid(make(("warp", *a)))
     if kind == "volume":
@@ -56,6 +64,7 @@ def make(case):
 # device; ragged tiles and runs, odd quads, masks, one-way edges
 CASES = [("warp", 1, 1, 0), ("warp", 37, 5, 0), ("warp", 64, 64, 1), ("warp", 127, 65, 0), ("warp", 300, 57, 1),
          ("warp", 411, 303, 0), ("poisson", 37, 29), ("poisson", 130, 63), ("poisson", 500, 333),
+         ("cutout", 200, 90), ("cutout", 37, 61), ("patch", 301, 77), ("patch", 40, 200),
          ("graph", 33, 17, 1), ("graph", 111, 99, 0), ("volume", 5, 4, 3), ("volume", 31, 21, 13),
          ("embedded", 1), ("embedded", 4), ("mesh", 0, 1.0), ("mesh", 3, 0.6), ("mesh", 5, 1.0), ("mesh", 6, 0.7)]
 
