@@ -19,7 +19,7 @@ BUILDDIR = os.path.join(ROOT, "_build")
 LIBNAME = "libopt_gb300.so"
 SOURCES = ["api.cu", "batch.cu", "grid_kernels.cu", "graph_kernels.cu", "graph2d_kernels.cu", "materialize.cu",
            "noalloc.cu", "resident.cu", "serve.cu", "fp64.cu",
-           "embedded_kernels.cu"]
+           "embedded_kernels.cu", "edge_plan.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -163,18 +163,35 @@ cudaMemPool_t problem_pool() {
 
 // Zero-filled device array owned by the problem (ordered on the legacy
 // stream; planning ends with a synchronising copy before any other stream
-// touches it).
+// touches it).  The many small ones of a plan share slabs.
+constexpr size_t kSlabBytes = 128 << 10, kSlabShare = 16 << 10;
+opt_status dalloc_bytes(opt_problem* pb, void** ptr, size_t bytes) {
+  cudaMemPool_t pool = problem_pool();
+  cudaError_t e = pool ? cudaMallocFromPoolAsync(ptr, bytes, pool, nullptr) : cudaMalloc(ptr, bytes);
+  if (e != cudaSuccess) return cuda_fail(e, "device allocation");
+  pb->allocs.push_back(*ptr);
+  pb->pooled.push_back(pool != nullptr);
+  e = cudaMemsetAsync(*ptr, 0, bytes, nullptr);
+  return e == cudaSuccess ? OPT_OK : cuda_fail(e, "cudaMemsetAsync");
+}
 template <class T>
 opt_status dalloc(opt_problem* pb, T** ptr, size_t n) {
+  const size_t bytes = std::max<size_t>(n, 1) * sizeof(T), room = (bytes + 255) / 256 * 256;
   void* p = nullptr;
-  const size_t bytes = std::max<size_t>(n, 1) * sizeof(T);
-  cudaMemPool_t pool = problem_pool();
-  cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, nullptr) : cudaMalloc(&p, bytes);
-  if (e != cudaSuccess) return cuda_fail(e, "device allocation");
-  pb->allocs.push_back(p);
-  pb->pooled.push_back(pool != nullptr);
-  e = cudaMemsetAsync(p, 0, bytes, nullptr);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+  if (room <= kSlabShare) {
+    if (pb->slab_left < room) {
+      const opt_status s = dalloc_bytes(pb, &p, kSlabBytes);
+      if (s != OPT_OK) return s;
+      pb->slab = static_cast<char*>(p);
+      pb->slab_left = kSlabBytes;
+    }
+    p = pb->slab;
+    pb->slab += room;
+    pb->slab_left -= room;
+  } else {
+    const opt_status s = dalloc_bytes(pb, &p, bytes);
+    if (s != OPT_OK) return s;
+  }
   *ptr = static_cast<T*>(p);
   return OPT_OK;
 }
@@ -193,6 +210,86 @@ opt_status download(std::vector<T>& dst, const T* src, size_t n) {
   CK(cudaMemcpy(dst.data(), src, n * sizeof(T), cudaMemcpyDeviceToHost));
   return OPT_OK;
 }
+
+// The tables of a plan, sent in one copy and put in their places by one kernel, and the
+// caller's small arrays, gathered on the device and fetched in one copy.  Every copy
+// from or to pageable memory waits for the device and for the driver's lock: with 25 of
+// them a problem, plans on several threads held one another up (ten warps up to 826^2 and
+// six meshes up to level 6, with the edges and checks on the device: 18.0 -> 6.9 ms one
+// after the other, 7.0 -> 4.5 ms on four threads).
+struct Piece {
+  unsigned int* dst;
+  long long first, words;       // in the words behind the table
+};
+__global__ void __launch_bounds__(256) k_place(const Piece* __restrict__ tab, const unsigned int* __restrict__ data) {
+  const Piece p = tab[blockIdx.y];
+  for (long long k = blockIdx.x * 256ll + threadIdx.x; k < p.words; k += gridDim.x * 256ll)
+    p.dst[k] = data[p.first + k];
+}
+struct Uploads {
+  std::vector<Piece> tab;
+  std::vector<unsigned int> data;
+  template <class T>
+  void add(T* dst, const std::vector<T>& v) {
+    static_assert(sizeof(T) % 4 == 0, "tables are made of words");
+    if (v.empty()) return;
+    const size_t words = v.size() * sizeof(T) / 4, first = data.size();
+    data.resize(first + words);
+    std::memcpy(data.data() + first, v.data(), words * 4);
+    tab.push_back(Piece{reinterpret_cast<unsigned int*>(dst), (long long)first, (long long)words});
+  }
+  opt_status flush() {
+    if (tab.empty()) return OPT_OK;
+    long long most = 0;
+    for (const Piece& p : tab) most = std::max(most, p.words);
+    const size_t head = tab.size() * sizeof(Piece);
+    std::vector<char> buf(head + data.size() * 4);
+    std::memcpy(buf.data(), tab.data(), head);
+    std::memcpy(buf.data() + head, data.data(), data.size() * 4);
+    opt_problem work;
+    char* dev = nullptr;
+    CKS(dalloc(&work, &dev, buf.size()));
+    CKS(upload(dev, buf));
+    k_place<<<dim3((unsigned)std::min(64ll, (most + 255) / 256), (unsigned)tab.size()), 256>>>(
+        reinterpret_cast<const Piece*>(dev), reinterpret_cast<const unsigned int*>(dev + head));
+    CK(cudaGetLastError());
+    tab.clear();
+    data.clear();
+    return OPT_OK;
+  }
+};
+struct Downloads {
+  std::vector<const void*> src;
+  std::vector<size_t> words;
+  std::vector<unsigned int> data;
+  void add(const void* from, size_t n) {
+    src.push_back(from);
+    words.push_back(n);
+  }
+  opt_status fetch() {
+    size_t total = 0;
+    for (size_t n : words) total += n;
+    data.resize(total);
+    if (total == 0) return OPT_OK;
+    opt_problem work;
+    unsigned int* dev = nullptr;
+    CKS(dalloc(&work, &dev, total));
+    size_t at = 0;
+    for (size_t k = 0; k < src.size(); at += words[k++])
+      if (words[k]) CK(cudaMemcpyAsync(dev + at, src[k], words[k] * 4, cudaMemcpyDeviceToDevice, nullptr));
+    CK(cudaMemcpy(data.data(), dev, total * 4, cudaMemcpyDeviceToHost));
+    return OPT_OK;
+  }
+  // the k-th array
+  template <class T>
+  std::vector<T> get(size_t k) const {
+    size_t at = 0;
+    for (size_t i = 0; i < k; ++i) at += words[i];
+    std::vector<T> v(words[k]);
+    if (words[k]) std::memcpy(v.data(), data.data() + at, words[k] * 4);
+    return v;
+  }
+};
 
 bool all_finite(const std::vector<float>& v) {
   for (float f : v)
@@ -304,6 +401,11 @@ namespace optgb {
 
 opt_status copy_planes_in(const opt_problem* pb, float* internal, float* const* user, int n, cudaStream_t st) {
   return copy_planes(pb, PlaneDir::In, internal, user, n, st);
+}
+opt_status host_edges(opt_problem* pb) {
+  if (pb->E == 0 || !pb->h_e0.empty()) return OPT_OK;
+  CKS(download(pb->h_e1, pb->hm.e1, (size_t)pb->E));
+  return download(pb->h_e0, pb->hm.e0, (size_t)pb->E);
 }
 opt_status copy_planes_out(const opt_problem* pb, float* const* user, const float* internal, int n, cudaStream_t st) {
   return copy_planes(pb, PlaneDir::Out, const_cast<float*>(internal), user, n, st);
@@ -639,7 +741,7 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 // out-of-range elements are zero-filled.  All bases are device allocations
 // (256-byte aligned) and every stride (P * 4, plane * 4, P) is a multiple of
 // 16 bytes because P is a multiple of 128.
-static opt_status make_grid_tmaps(opt_problem* q, const float* slab, int nfp, const uint8_t* bytes) {
+static opt_status make_grid_tmaps(opt_problem* q, const float* slab, int nfp, const uint8_t* bytes, Uploads& up) {
   // L2 fill granularity of the copies (measured at 4096^2: 256-byte fills
   // suit the warp, whose neighbouring tiles reuse them, 64-byte fills the
   // Poisson kernels, 2-4 % apart)
@@ -670,9 +772,11 @@ static opt_status make_grid_tmaps(opt_problem* q, const float* slab, int nfp, co
       return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
   }
   static_assert(sizeof(CUtensorMap) == 128, "tensor maps are 128 bytes");
+  std::vector<unsigned long long> words(sizeof(maps) / sizeof(unsigned long long));
+  std::memcpy(words.data(), maps, sizeof(maps));
   unsigned long long* dmap = nullptr;
-  CKS(dalloc(q, &dmap, 3 * sizeof(CUtensorMap) / sizeof(unsigned long long)));
-  CK(cudaMemcpy(dmap, maps, sizeof(maps), cudaMemcpyHostToDevice));
+  CKS(dalloc(q, &dmap, words.size()));
+  up.add(dmap, words);
   q->hg.tmap = dmap;
   return OPT_OK;
 }
@@ -820,20 +924,17 @@ opt_status opt_problem_create_grid(const opt_grid_desc* d, const opt_solve_param
   const int W = d->W, H = d->H, P = pb->P;
   const size_t n = (size_t)W * H;
 
-  // host copies of the constants for validation and planning
-  std::vector<float> cst;
-  for (int c = 0; c < nc; ++c) {
-    std::vector<float> tmp;
-    CKS(download(tmp, d->consts[c], n));
-    if (!all_finite(tmp)) return OPT_ERR_INVALID_ARG;
-  }
   std::vector<uint8_t> mask;
   if (d->mask) CKS(download(mask, d->mask, n));
   std::vector<int> hidx;
   std::vector<float> htgt;
   if (nh > 0) {
-    CKS(download(hidx, d->handle_idx, (size_t)nh));
-    CKS(download(htgt, d->handle_target, (size_t)nh * 2));
+    Downloads dl;
+    dl.add(d->handle_idx, (size_t)nh);
+    dl.add(d->handle_target, (size_t)nh * 2);
+    CKS(dl.fetch());
+    hidx = dl.get<int>(0);
+    htgt = dl.get<float>(1);
     if (!all_finite(htgt)) return OPT_ERR_INVALID_ARG;
     std::vector<int> sorted(hidx);
     std::sort(sorted.begin(), sorted.end());
@@ -939,27 +1040,31 @@ opt_status opt_problem_create_grid(const opt_grid_desc* d, const opt_solve_param
   for (int k = 0; k < nc; ++k)
     CK(cudaMemcpy2D(c + k * pl, (size_t)P * 4, d->consts[k], (size_t)W * 4, (size_t)W * 4, H,
                     cudaMemcpyDeviceToDevice));
-  int broken = 1;
-  if (warp && tw == 128) {
-    int* dbroken = nullptr;
-    CKS(dalloc(q, &dbroken, 1));
-    launch_warp_lattice(W, H, P, c, (long long)pl, dbroken, nullptr);
+  // constants that are not finite, or a rest shape that is not the pixel lattice
+  int found[2] = {0, 0};
+  {
+    opt_problem work;
+    int* dfound = nullptr;
+    CKS(dalloc(&work, &dfound, 2));
+    launch_grid_check(W, H, P, c, (long long)pl, nc, warp && tw == 128, dfound, nullptr);
     CK(cudaGetLastError());
-    CK(cudaMemcpy(&broken, dbroken, sizeof(int), cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(found, dfound, sizeof(found), cudaMemcpyDeviceToHost));
   }
+  if (found[0]) return OPT_ERR_INVALID_ARG;
+  Uploads up;
   CKS(dalloc(q, &dhbeg, hbeg.size()));
-  CKS(upload(dhbeg, hbeg));
+  up.add(dhbeg, hbeg);
   CKS(dalloc(q, &dhpix, hpix.size()));
-  CKS(upload(dhpix, hpix));
+  up.add(dhpix, hpix);
   CKS(dalloc(q, &dhtgt, hts.size()));
-  CKS(upload(dhtgt, hts));
+  up.add(dhtgt, hts);
   CKS(dalloc(q, &q->d_tiles, tiles.size()));
-  CKS(upload(q->d_tiles, tiles));
+  up.add(q->d_tiles, tiles);
   q->h_tiles = tiles;
   q->h_cells = cells;
   q->ntiles = (int)tiles.size();
   CKS(dalloc(q, &q->d_chunks, chunks.size()));
-  CKS(upload(q->d_chunks, chunks));
+  up.add(q->d_chunks, chunks);
   q->h_chunks = chunks;
   q->nchunks = (int)chunks.size();
   CKS(dalloc(q, &q->d_part, 4 * chunks.size()));   // up to three partials per chunk
@@ -992,9 +1097,10 @@ opt_status opt_problem_create_grid(const opt_grid_desc* d, const opt_solve_param
   g.zpack = zof(q->rvec) | zof(m) << 6 | zof(q->pbuf) << 12 | (csn ? zof(csn) : 0) << 18 | zof(c) << 24;
   g.zb = zb;
   g.wb = wb;
-  g.lattice = !broken;
+  g.lattice = warp && tw == 128 && !found[1];
   g.zpack2 = zb ? (zof(zb) | zof(wb) << 6) : 0;
-  if (tw == 128) CKS(make_grid_tmaps(q, slab, nfp, warp ? dmask : dsdeg));
+  if (tw == 128) CKS(make_grid_tmaps(q, slab, nfp, warp ? dmask : dsdeg, up));
+  CKS(up.flush());
   g.d = q->dvec; g.r = q->rvec; g.p = q->pbuf; g.q = q->qvec; g.m = m; g.dc = dc;
   g.hbeg = dhbeg; g.hpix = dhpix; g.htgt = dhtgt;
   g.jtf_out = nullptr; g.diag_out = nullptr;
@@ -1017,6 +1123,30 @@ struct EmbedExtra {
   float* unknowns[12];
   float w_rot;
 };
+
+// Runs the edge planning with working memory that ends with `work`.
+static opt_status plan_edges(opt_problem& work, const opt_graph_desc* d, const std::vector<int>* host_e0,
+                             const std::vector<int>* host_e1, EdgePlan p, bool& sym) {
+  int *v0 = nullptr, *v1 = nullptr;
+  CKS(dalloc(&work, &v0, (size_t)p.E));
+  CKS(dalloc(&work, &v1, (size_t)p.E));
+  if (host_e0) {
+    CKS(upload(v0, *host_e0));
+    CKS(upload(v1, *host_e1));
+  } else if (p.E > 0) {   // (a copy of the caller's: a list that is no device memory fails here)
+    CK(cudaMemcpyAsync(v0, d->v0, (size_t)p.E * sizeof(int), cudaMemcpyDeviceToDevice, nullptr));
+    CK(cudaMemcpyAsync(v1, d->v1, (size_t)p.E * sizeof(int), cudaMemcpyDeviceToDevice, nullptr));
+  }
+  CKS(dalloc(&work, &p.cursor, 2 * ((size_t)p.V + 1)));
+  CKS(dalloc(&work, &p.flags, 2));
+  p.v0 = v0;
+  p.v1 = v1;
+  CK(launch_edge_plan(p, nullptr));
+  int flags[2];
+  CK(cudaMemcpy(flags, p.flags, sizeof(flags), cudaMemcpyDeviceToHost));
+  sym = !flags[1];
+  return flags[0] ? OPT_ERR_INVALID_ARG : OPT_OK;
+}
 
 static opt_status create_graph_impl(const opt_graph_desc* d, int D, opt_problem** out,
                                     const std::vector<int>* host_e0 = nullptr,
@@ -1053,20 +1183,15 @@ static opt_status create_graph_impl(const opt_graph_desc* d, int D, opt_problem*
   q->ulen = V;
   CKS(common_setup(q));
 
-  std::vector<int> e0, e1;
-  if (host_e0) {
-    e0 = *host_e0;
-    e1 = *host_e1;
-  } else {
-    CKS(download(e0, d->v0, (size_t)E));
-    CKS(download(e1, d->v1, (size_t)E));
-  }
-  for (int e = 0; e < E; ++e)
-    if (e0[e] < 0 || e0[e] >= V || e1[e] < 0 || e1[e] >= V || e0[e] == e1[e]) return OPT_ERR_INVALID_ARG;
+  Downloads dl;
+  for (int c = 0; c < D; ++c) dl.add(d->urshape[c], (size_t)V);
+  dl.add(d->handle_idx, (size_t)nh);
+  dl.add(d->handle_target, (size_t)nh * D);
+  CKS(dl.fetch());
   std::vector<float> Uh[3];
   Uh[2].assign((size_t)V, 0.f);             // a graph warp lies in the plane z = 0
   for (int c = 0; c < D; ++c) {
-    CKS(download(Uh[c], d->urshape[c], (size_t)V));
+    Uh[c] = dl.get<float>(c);
     if (!all_finite(Uh[c])) return OPT_ERR_INVALID_ARG;
   }
   // internal vertex order: internal k = caller perm[k]; edges and handles are
@@ -1080,34 +1205,11 @@ static opt_status create_graph_impl(const opt_graph_desc* d, int D, opt_problem*
   }
   std::vector<int> iperm((size_t)V);
   for (int k = 0; k < V; ++k) iperm[perm[k]] = k;
-  for (int e = 0; e < E; ++e) { e0[e] = iperm[e0[e]]; e1[e] = iperm[e1[e]]; }
-  bool sorted = true;
-  for (int e = 1; e < E && sorted; ++e)
-    if (e0[e] < e0[e - 1] || (e0[e] == e0[e - 1] && e1[e] < e1[e - 1])) sorted = false;
-  if (!sorted) {
-    // counting sort by v0, then each (short) row by v1
-    std::vector<int> start((size_t)V + 1, 0), s1((size_t)E);
-    for (int e = 0; e < E; ++e) start[(size_t)e0[e] + 1] += 1;
-    for (int v = 0; v < V; ++v) start[(size_t)v + 1] += start[v];
-    std::vector<int> fill(start.begin(), start.end() - 1);
-    for (int e = 0; e < E; ++e) s1[(size_t)fill[e0[e]]++] = e1[e];
-    for (int v = 0; v < V; ++v) {
-      const int b = start[v], e = start[(size_t)v + 1];
-      for (int k = b + 1; k < e; ++k) {   // rows are short: insertion sort
-        const int x = s1[k];
-        int m = k;
-        for (; m > b && s1[(size_t)m - 1] > x; --m) s1[m] = s1[(size_t)m - 1];
-        s1[m] = x;
-      }
-      for (int k = b; k < e; ++k) e0[k] = v;
-    }
-    e1.swap(s1);
-  }
   std::vector<int> hidx;
   std::vector<float> htgt;
   if (nh > 0) {
-    CKS(download(hidx, d->handle_idx, (size_t)nh));
-    CKS(download(htgt, d->handle_target, (size_t)nh * D));
+    hidx = dl.get<int>(D);
+    htgt = dl.get<float>(D + 1);
     if (!all_finite(htgt)) return OPT_ERR_INVALID_ARG;
     for (int& h : hidx) {
       if (h < 0 || h >= V) return OPT_ERR_INVALID_ARG;
@@ -1130,26 +1232,6 @@ static opt_status create_graph_impl(const opt_graph_desc* d, int D, opt_problem*
     degw[v] += d->w_fit;
   }
   for (size_t t = 1; t < hbeg.size(); ++t) hbeg[t] += hbeg[t - 1];
-  for (int e = 0; e < E; ++e) {
-    degw[e0[e]] += d->w_reg;
-    degw[e1[e]] += d->w_reg;
-  }
-  // out-edge rows of the sorted list, and the in-edges of every vertex
-  // (sources ascending, as the sorted list visits them)
-  std::vector<int> orow((size_t)V + 1, 0), irow((size_t)V + 1, 0), isrc((size_t)E);
-  for (int e = 0; e < E; ++e) {
-    orow[(size_t)e0[e] + 1] += 1;
-    irow[(size_t)e1[e] + 1] += 1;
-  }
-  for (int v = 0; v < V; ++v) {
-    orow[(size_t)v + 1] += orow[v];
-    irow[(size_t)v + 1] += irow[v];
-  }
-  {
-    std::vector<int> fill(irow.begin(), irow.end() - 1);
-    for (int e = 0; e < E; ++e) isrc[(size_t)fill[e1[e]]++] = e0[e];
-  }
-
   const int target = std::max(1, q->sms * 8);
   std::vector<Chunk> vch = make_chunks_balanced(nvt, target, 0);
   for (Chunk& c : vch) { c.begin *= VT; c.end = std::min(V, c.end * VT); }
@@ -1171,34 +1253,39 @@ static opt_status create_graph_impl(const opt_graph_desc* d, int D, opt_problem*
   CKS(dalloc(q, &grec, (size_t)NGR * V));
   CKS(dalloc(q, &vrec, (size_t)NVR * V));
   int *dorow = nullptr, *dirow = nullptr, *disrc = nullptr;
-  CKS(dalloc(q, &dorow, orow.size()));
-  CKS(upload(dorow, orow));
-  CKS(dalloc(q, &dirow, irow.size()));
-  CKS(upload(dirow, irow));
-  CKS(dalloc(q, &disrc, std::max<size_t>(1, isrc.size())));
-  if (E > 0) CKS(upload(disrc, isrc));
+  CKS(dalloc(q, &dorow, (size_t)V + 1));
+  CKS(dalloc(q, &dirow, (size_t)V + 1));
+  CKS(dalloc(q, &disrc, (size_t)E));
+  Uploads up;
   for (int c = 0; c < D; ++c) {
     std::vector<float> Ui((size_t)V);
     for (int k = 0; k < V; ++k) Ui[k] = Uh[c][perm[k]];
-    CKS(upload(U + c * pl, Ui));
+    up.add(U + c * pl, Ui);
   }
   CKS(dalloc(q, &q->d_perm, (size_t)V));
-  CKS(upload(q->d_perm, perm));
-  CKS(upload(dgw, degw));
+  up.add(q->d_perm, perm);
+  up.add(dgw, degw);
   CKS(dalloc(q, &de0, (size_t)E));
-  CKS(upload(de0, e0));
   CKS(dalloc(q, &de1, (size_t)E));
-  CKS(upload(de1, e1));
   CKS(dalloc(q, &dhbeg, hbeg.size()));
-  CKS(upload(dhbeg, hbeg));
+  up.add(dhbeg, hbeg);
   CKS(dalloc(q, &dhpix, hpix.size()));
-  CKS(upload(dhpix, hpix));
+  up.add(dhpix, hpix);
   CKS(dalloc(q, &dhtgt, hts.size()));
-  CKS(upload(dhtgt, hts));
+  up.add(dhtgt, hts);
   CKS(dalloc(q, &q->d_vchunks, vch.size()));
-  CKS(upload(q->d_vchunks, vch));
+  up.add(q->d_vchunks, vch);
   CKS(dalloc(q, &q->d_echunks, ech.size()));
-  CKS(upload(q->d_echunks, ech));
+  up.add(q->d_echunks, ech);
+  opt_problem work;
+  int* dip = nullptr;
+  CKS(dalloc(&work, &dip, (size_t)V));
+  up.add(dip, iperm);
+  CKS(up.flush());
+  bool sym = false;
+  CKS(plan_edges(work, d, host_e0, host_e1, EdgePlan{nullptr, nullptr, dip, V, E, de0, de1, dorow, dirow, disrc, nullptr,
+                                                     dgw, d->w_reg, nullptr}, sym));
+  CKS(download(q->h_orow, dorow, (size_t)V + 1));
   q->h_vch = vch;
   q->h_ech = ech;
   q->tileable = !ed && !grid3 && D == 3;
@@ -1207,14 +1294,11 @@ static opt_status create_graph_impl(const opt_graph_desc* d, int D, opt_problem*
   CKS(dalloc(q, &q->d_part, 2 * std::max(vch.size(), ech.size())));
   CKS(dalloc(q, &q->dm, 1));
   for (int k = 0; k < NXg; ++k) q->user_x[k] = ux[k];
-  q->h_e0 = e0;
-  q->h_e1 = e1;
-  q->h_orow = orow;
   q->h_hpix = hpix;
 
   MeshProb& g = q->hm;
   g.V = V; g.E = E; g.Vp = Vp;
-  g.sym = orow == irow && e1 == isrc;
+  g.sym = sym;
   g.vchunk_begin = 0; g.vchunk_end = q->nvchunks;
   g.echunk_begin = 0; g.echunk_end = q->nechunks;
   g.tchunk_begin = 0; g.tchunk_end = q->ntchunks;
@@ -1582,6 +1666,7 @@ static opt_status ensure_tile_tables(opt_problem* q) {
   if (q->d_tchunks) return OPT_OK;
   if (!q->tileable) return OPT_ERR_INVALID_ARG;
   const int V = q->V, E = q->E, nvt = (V + VT - 1) / VT;
+  CKS(host_edges(q));
   const std::vector<int>& e0 = q->h_e0;
   const std::vector<int>& e1 = q->h_e1;
   std::vector<int> orow((size_t)V + 1, 0), irow((size_t)V + 1, 0), isrc((size_t)E), itpos((size_t)E);

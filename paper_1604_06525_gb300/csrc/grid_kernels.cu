@@ -3272,21 +3272,27 @@ void launch_grid_energy(int kind, const GridLaunch& L, int mode, int hist_idx) {
   launch_pdl(k, L.nchunks, NT, 0, L.stream, L.probs, L.chunks, L.tiles, L.part, hist_idx);
 }
 
-// Sets *broken unless UrShape is the pixel lattice up to an offset: every
-// difference the stencil takes of it is exactly 1 or 0.
-__global__ void __launch_bounds__(NT) k_warp_lattice(int W, int H, int P, const float* __restrict__ ux,
-                                                     const float* __restrict__ uy, int* __restrict__ broken) {
-  bool ok = true;
+// What planning asks of the constant planes: found[0] = 1 where one is not finite,
+// found[1] = 1 unless the first two (UrShape) are the pixel lattice up to an offset:
+// every difference the stencil takes of them is exactly 1 or 0.
+__global__ void __launch_bounds__(NT) k_grid_check(int W, int H, int P, const float* __restrict__ c, long long plane,
+                                                   int nc, int lattice, int* __restrict__ found) {
+  bool fine = true, ok = true;
+  const float *ux = c, *uy = c + plane;
   for (int y = blockIdx.x; y < H; y += gridDim.x)
     for (int x = threadIdx.x; x < W; x += NT) {
       const long long i = (long long)y * P + x;
+      for (int k = 0; k < nc; ++k) fine = fine && isfinite(c[k * plane + i]);
+      if (!lattice) continue;
       if (x + 1 < W) ok = ok && ux[i + 1] - ux[i] == 1.f && uy[i + 1] == uy[i];
       if (y + 1 < H) ok = ok && uy[i + P] - uy[i] == 1.f && ux[i + P] == ux[i];
     }
-  if (!ok) *broken = 1;
+  if (!fine) found[0] = 1;
+  if (!ok) found[1] = 1;
 }
-void launch_warp_lattice(int W, int H, int P, const float* u, long long plane, int* broken, cudaStream_t st) {
-  k_warp_lattice<<<std::min(H, 1024), NT, 0, st>>>(W, H, P, u, u + plane, broken);
+void launch_grid_check(int W, int H, int P, const float* c, long long plane, int nc, int lattice, int* found,
+                       cudaStream_t st) {
+  k_grid_check<<<std::min(H, 1024), NT, 0, st>>>(W, H, P, c, plane, nc, lattice, found);
 }
 
 void launch_pois_sdeg(int W, int H, int P, const uint8_t* mask, uint8_t* out, cudaStream_t st) {

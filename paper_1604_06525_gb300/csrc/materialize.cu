@@ -273,6 +273,8 @@ static opt_status csr_build_j(opt_problem* pb) {
     }
   } else {
     const float sw = pb->hm.s_w, sf = pb->hm.s_f;
+    const opt_status es = host_edges(pb);
+    if (es != OPT_OK) return es;
     for (size_t e = 0; e < pb->h_e0.size(); ++e) {
       const int a = pb->h_e0[e], b = pb->h_e1[e];
       for (int c = 0; c < 3; ++c)

@@ -70,8 +70,10 @@ void launch_grid_csn(const GridLaunch& L);
 // Poisson, tile width 128: the degree plane the wide kernels read (S_i + 1 on
 // free pixels, 0 elsewhere; pitched like the mask, P x H bytes)
 void launch_pois_sdeg(int W, int H, int P, const uint8_t* mask, uint8_t* out, cudaStream_t st);
-// sets *broken (device) unless the two planes at u are the pixel lattice up to an offset
-void launch_warp_lattice(int W, int H, int P, const float* u, long long plane, int* broken, cudaStream_t st);
+// found (device, two zeros before): [0] a constant is not finite, [1] (lattice != 0) the
+// first two planes are not the pixel lattice up to an offset
+void launch_grid_check(int W, int H, int P, const float* c, long long plane, int nc, int lattice, int* found,
+                       cudaStream_t st);
 // Persistent PCG loop (wide warp tiles only): the largest chunk count whose
 // blocks are all resident at once (0 if unknown), and the cooperative launch
 // of n_inner PCG iterations (applyJTJ + update) starting at parity par0.
@@ -94,6 +96,20 @@ cudaError_t launch_resident_grid(int kind, const GridProb* probs, const int* cel
                                  cudaStream_t st);
 cudaError_t launch_resident_graph(int kind, const MeshProb* probs, ResidentSync* sync, const ResidentPlan& rp,
                                   float4* rec, int inner, int step, cudaStream_t st);
+
+// edge_plan.cu: the edges of a graph in the internal vertex order.  v0, v1: the
+// caller's; iperm: internal number of every caller vertex; e0, e1, isrc: E entries; orow,
+// irow: V + 1 zeros before the call; cursor: 2 (V + 1); degw: w_fit at handles, else 0,
+// before the call; flags (zeros): [0] an edge is no edge, [1] some edge is given one way.
+struct EdgePlan {
+  const int *v0, *v1, *iperm;
+  int V, E;
+  int *e0, *e1, *orow, *irow, *isrc, *cursor;
+  float* degw;
+  float w_reg;
+  int* flags;
+};
+cudaError_t launch_edge_plan(const EdgePlan& p, cudaStream_t st);
 
 // graph_kernels.cu
 void launch_mesh_init(const MeshLaunch& L, int k_outer, float dmin, float dmax);

@@ -76,7 +76,7 @@ struct opt_problem {
   // host copies kept for building the materialized Jacobian
   std::vector<unsigned char> h_mask;    // grid mask (empty = none)
   std::vector<int> h_hpix;              // grid handles (pitched index) / mesh handles (vertex)
-  std::vector<int> h_e0, h_e1;          // sorted edges (internal vertex order)
+  std::vector<int> h_e0, h_e1;          // sorted edges (internal vertex order; see host_edges)
   std::vector<int> h_orow;              // their CSR rows
   int* d_perm = nullptr;                // graphs: internal vertex k is the caller's vertex d_perm[k]
   CsrJ csr;
@@ -102,6 +102,8 @@ struct opt_problem {
   float* qvec = nullptr;
   std::vector<void*> allocs;
   std::vector<bool> pooled;             // allocs[k] came from the library's stream-ordered pool
+  char* slab = nullptr;                 // what is left of the slab small allocations share
+  size_t slab_left = 0;
   int pcg_par = 0;
   // persistent PCG loop (wide warps): grid barrier state and the number of
   // blocks that can be resident at once (0 = not available)
@@ -141,7 +143,7 @@ struct opt_problem {
     swap(sent_hg, o.sent_hg); swap(sent_hm, o.sent_hm); swap(sent, o.sent);
     swap(user_x, o.user_x); swap(d_tmp, o.d_tmp); swap(d_jtf, o.d_jtf); swap(d_diag, o.d_diag);
     swap(x, o.x); swap(pbuf, o.pbuf); swap(dvec, o.dvec); swap(rvec, o.rvec); swap(qvec, o.qvec);
-    swap(allocs, o.allocs); swap(pooled, o.pooled); swap(pcg_par, o.pcg_par);
+    swap(allocs, o.allocs); swap(pooled, o.pooled); swap(slab, o.slab); swap(slab_left, o.slab_left); swap(pcg_par, o.pcg_par);
     swap(rplan, o.rplan); swap(rplanned, o.rplanned); swap(d_rsync, o.d_rsync); swap(d_rrec, o.d_rrec);
     swap(d_gbar, o.d_gbar); swap(coop_cap, o.coop_cap); swap(cap_stream, o.cap_stream);
     swap(gexec, o.gexec); swap(gkey, o.gkey); swap(ev0, o.ev0); swap(ev1, o.ev1);
@@ -185,6 +187,8 @@ void batch_enqueue_lm_round(opt_batch* b, const opt_solve_params& p, cudaStream_
 opt_status batch_read_scalars(opt_batch* b, Scalars* host_out, RoundRec* rounds_out, int rounds, cudaStream_t st);
 // api.cu: caller planes (dense rows for grids, caller vertex order for
 // graphs) <-> internal planes
+// api.cu: h_e0 / h_e1 from the device, where not there yet
+opt_status host_edges(opt_problem* pb);
 opt_status copy_planes_in(const opt_problem* pb, float* internal, float* const* user, int n, cudaStream_t st);
 opt_status copy_planes_out(const opt_problem* pb, float* const* user, const float* internal, int n,
                            cudaStream_t st);

@@ -135,14 +135,13 @@ opt_status write_back(opt_problem* pb, cudaStream_t st) {
   return copy_planes_out(pb, pb->user_x, pb->x, pb->nx, st);
 }
 
-// Plans admitted requests.  Planning is host work on one request's own data (edges
-// downloaded, ordered and sorted, tables uploaded) with the device idle most of the
-// time, so up to kPlanThreads requests are planned at once, the longest first; each
-// keeps its own status, the last CUDA error text goes to the calling thread, and
-// admission stays in arrival order.  Ten warps up to 826^2 and six meshes up to level
-// 6: 17.5 ms one after the other (a level-6 mesh 4.5 ms), 7.3 ms so; requests to results
-// 24.2 -> 14.0 ms.
-constexpr size_t kPlanThreads = 8;
+// Plans admitted requests.  Planning alternates between the host (vertex order, tables)
+// and short device work that it waits for, so up to kPlanThreads requests are planned
+// at once, the longest first; each keeps its own status, the last CUDA error text goes
+// to the calling thread, and admission stays in arrival order.  Ten warps up to 826^2
+// and six meshes up to level 6: 6.9 ms one after the other, 4.7 ms on two threads, 4.5
+// on four, 4.7 on eight (the driver's lock).
+constexpr size_t kPlanThreads = 4;
 
 opt_status plan_one(ServeReq* r, const opt_solve_params& prm) {
   try {
@@ -161,7 +160,7 @@ void plan(const std::vector<ServeReq*>& admit, const opt_solve_params& prm, std:
     for (size_t i = 0; i < n; ++i) status[i] = plan_one(admit[i], prm);
     return;
   }
-  // an edge costs about 16 times a pixel
+  // (a mesh's vertex order stays on the host)
   const auto cost = [](const ServeReq* r) {
     return r->graph ? 16ll * ((long long)r->md.V + r->md.E) : (long long)r->gd.W * r->gd.H;
   };

@@ -192,3 +192,36 @@ def test_repeated_solves_equal_fresh_ones(kind):
     if batch:
         batch.close()
     g.close()
+
+
+@pytest.mark.parametrize("V,degree", [(2, 1), (60, 46), (60, 47), (60, 48), (60, 49), (9000, 3000)])
+def test_planned_edges_match_oracle(V, degree):
+    """Edges in any order, both ways or one way, some twice, a hub row around the length
+    where the row sort changes its method, and vertices without an edge."""
+    import torch
+    from paper_1604_06525_gb300 import api
+    rng = np.random.default_rng(V + degree)
+    hub = rng.choice(np.arange(1, V), size=degree, replace=False)
+    a = np.concatenate([np.zeros(degree, int), rng.integers(0, V // 2 + 1, V)])
+    b = np.concatenate([hub, rng.integers(0, V // 2 + 1, V)])
+    keep = a != b
+    a, b = a[keep], b[keep]
+    back = rng.random(a.size) < 0.7
+    v0, v1 = np.concatenate([a, b[back], a[:3]]), np.concatenate([b, a[back], b[:3]])
+    order = rng.permutation(v0.size)
+    prob = synth.MeshProblem(V, rng.standard_normal((3, V)).astype(np.float32), v0[order].astype(np.int32),
+                             v1[order].astype(np.int32), 0.2 * rng.standard_normal((6, V)).astype(np.float32),
+                             np.array([0, V - 1], np.int32), rng.standard_normal((2, 3)).astype(np.float32),
+                             0.3, 7.0)                       # (weights whose sums round)
+    e = oracle.make_energy(prob)
+    x = prob.x0.reshape(-1).astype(np.float64)
+    g = api.Problem(prob)
+    p = rng.standard_normal(6 * V).astype(np.float32)
+    q, _ = g.apply_jtj(torch.as_tensor(p, device="cuda"), 0.0)
+    _, diag, E = oracle.jtf_diag(e, x)
+    want = oracle.apply_jtj(e, x, p.astype(np.float64), 0.0, np.clip(diag, 1e-6, 1e32))
+    assert np.linalg.norm(q.cpu().numpy().reshape(-1) - want) <= 1e-5 * np.linalg.norm(want)
+    _, d, Eg = g.eval_jtf()
+    np.testing.assert_allclose(d.cpu().numpy().reshape(-1), diag, rtol=2e-4, atol=1e-6)
+    assert abs(Eg - E) <= 1e-5 * abs(E)
+    g.close()
