@@ -186,14 +186,19 @@ typedef struct {
     int32_t persistent;       /* 1 = run each outer iteration's PCG loop as one cooperative
                                  launch with grid-wide barriers when the problem is a wide-tile
                                  warp, matrix-free, and all its blocks fit on the device at once;
-                                 0 (default) = one launch per PCG kernel, measured faster on
-                                 GB300 (a barrier costs more than a kernel boundary with
-                                 programmatic dependent launch).  Same arithmetic either way.  A
+                                 0 (default) = on chip where the state fits (pcg_form 0), else
+                                 one launch per PCG kernel, measured faster on GB300 (a barrier
+                                 costs more than a kernel boundary with programmatic dependent
+                                 launch).  Same arithmetic either way.  A
                                  barrier wait is bounded (1 s): OPT_ERR_TIMEOUT. */
     void* stream;             /* cudaStream_t; NULL = legacy default stream */
     int32_t pcg_form;         /* 0 (default) = the two-pass Jacobi-PCG iteration of Sec. 4.1
                                  (applyJTJ with p.q, then the vector update with r.z: two
-                                 grid-wide reductions, two launches per iteration).
+                                 reductions per iteration).  A solve of one problem whose state
+                                 fits on chip runs all iterations of an outer iteration in one
+                                 launch (one thread-block cluster, or one block per SM), else
+                                 two launches per iteration, as batches do; the same arithmetic.
+                                 A wait inside the launch is bounded (1 s): OPT_ERR_TIMEOUT.
                                  1 = single-reduction iteration, taken by matrix-free solves of
                                  OPT_ARAP_WARP_2D and OPT_POISSON_2D grids planned with 128-pixel
                                  tiles (other problems run form 0): it carries z = M^-1 r and
@@ -367,7 +372,7 @@ opt_status opt_problem_info(const opt_problem* prob, int64_t* n_unknowns, int32_
  * default), apply_form = how an ARAP mesh forms J^T J p (1: one block per
  * vertex tile with the tile's halo staged in shared memory, every residual of
  * the tile evaluated once; 0: the two-pass vertex gather; -1: not an ARAP mesh
- * with tile tables).  opt_problem_autotune chooses all three: the form and
+ * with tile tables; a solve whose loop runs on chip uses neither).  opt_problem_autotune chooses all three: the form and
  * granularity of a mesh, the granularity and tile width of a grid (the other
  * width is planned afresh from the creation descriptor, whose arrays must
  * still be valid, and kept if faster).  Results agree across configurations
