@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(NT) k_mesh_energy(const MeshProb* __restrict__
         quat_delta_matrix(q, D2);
       }
     }
-    float se = 0.f, sm = 0.f, fit = 0.f;
+    float fit = 0.f;
     const int h = handle_of(pr, i);
     if (h >= 0) {
 #pragma unroll
@@ -672,9 +672,11 @@ __global__ void __launch_bounds__(NT) k_mesh_energy(const MeshProb* __restrict__
       mat_vec(D, v, y);
 #pragma unroll
       for (int c = 0; c < 3; ++c) r[c] = d[c] - y[c];
+      float se = 0.f, sm = 0.f;
       if (mode == 0) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) se = fmaf(r[c], r[c], se);
+        f2_add_prod(e0, pr.w_reg, se);
         return;
       }
       float y2[3];
@@ -689,6 +691,8 @@ __global__ void __launch_bounds__(NT) k_mesh_energy(const MeshProb* __restrict__
       sub_cross(r, w, y);
 #pragma unroll
       for (int c = 0; c < 3; ++c) sm = fmaf(r[c], r[c], sm);
+      f2_add_prod(e0, pr.w_reg, se);
+      f2_add_prod(e1, pr.w_reg, sm);
     };
     if (G3) {
       const Stencil3 st = stencil3(pr, i);
@@ -698,8 +702,10 @@ __global__ void __launch_bounds__(NT) k_mesh_energy(const MeshProb* __restrict__
     } else {
       for (int k = pr.orow[i]; k < pr.orow[i + 1]; ++k) edge(pr.e1[k]);
     }
-    f2_add(e0, fmaf(pr.w_reg, se, fit));
-    if (mode == 1) f2_add(e1, fmaf(pr.w_reg, sm, fit));
+    if (h >= 0) {
+      f2_add(e0, fit);
+      if (mode == 1) f2_add(e1, fit);
+    }
   }
   pdl_trigger();
   if (publish_partials(part, blockIdx.x, e0, e1, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
