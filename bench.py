@@ -42,13 +42,13 @@ METRIC = "PCG iters/s and % HBM roofline; batched solves/s and p99 latency vs pl
 UNIT = "PCG iters/s"
 W_BENCH, H_BENCH, HANDLES, OUTER, INNER = 1024, 1024, 64, 20, 20
 # algorithmic bytes per pixel (float32 planes, each touched once per launch)
-BYTES_APPLY_WARP = 72      # read r 12, M^-1 8, p_old 12, cos/sin 8, UrShape 8; write p 12, q 12
+BYTES_APPLY_WARP = 64      # read r 12, M^-1 8, p_old 12, cos/sin 8 (a pixel lattice: no UrShape); write p 12, q 12
 BYTES_UPDATE_WARP = 80     # read delta 12, p 12, r 12, q 12, M^-1 8; write delta 12, r 12
 BYTES_INIT_WARP = 56       # as a solve runs it from the second outer iteration on (cos / sin of theta written by
 #                            the previous outer update): read dx, dy 8, cos/sin 8, UrShape 8; write r 12, M^-1 8,
 #                            delta 12 (GN)
 # single-reduction PCG iteration (pcg_form = 1), one launch per PCG iteration
-BYTES_FUSED_WARP = 120     # read z 12, w 12, p_old 12, cos/sin 8, UrShape 8, M^-1 8, delta 12;
+BYTES_FUSED_WARP = 104     # read z 12, w 12, p_old 12, cos/sin 8, delta 12 (a lattice under GN: no UrShape, M^-1 formed);
 #                            write z 12, w 12, p 12, delta 12
 BYTES_FIN_WARP = 36        # the last iteration's step: read delta 12, p 12; write delta 12
 PCG_FORM = 1               # the headline's PCG iteration: 1 single-reduction, 0 two-pass
@@ -1009,7 +1009,8 @@ def run_ours(args):
     fused = PCG_FORM == 1 and head_cfg["tile_w"] == 128
     # per outer iteration: PCGInit, the PCG launches, and the outer update (the
     # single-reduction form applies its last step and x += delta in one pass)
-    launches_per_step = 2 + OUTER * ((2 + INNER) if fused else (2 + 2 * INNER))
+    # (and the planes in, the final energy and the planes out)
+    launches_per_step = 3 + OUTER * ((2 + INNER) if fused else (2 + 2 * INNER))
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
