@@ -88,11 +88,10 @@ struct P64 {
 
 // Resident blocks per SM, all at once: the float64 pipe issues one warp
 // instruction in about 15 cycles per SM, so a few warps keep it busy, and what
-// counts is that every SM gets the same number of elements.
-#ifndef F64_BLOCKS_PER_SM
-#define F64_BLOCKS_PER_SM 2
-#endif
-constexpr int kBlocksPerSM64 = F64_BLOCKS_PER_SM;
+// counts is that every SM gets the same number of elements.  A warp's rows wait more for
+// memory: with three blocks instead of two 1024^2 GN 1 x 20 takes 3.93 ms instead of
+// 4.26, while Poisson 900^2 takes 2.05 instead of 1.99 and a level-8 mesh 8.3 instead of 8.1.
+__host__ __device__ constexpr int blocks64(int nx) { return nx == 3 ? 3 : 2; }
 
 // grid direction k: +x, -x, +y, -y
 __device__ __forceinline__ int ddx(int k) { return k == 0 ? 1 : (k == 1 ? -1 : 0); }
@@ -223,7 +222,7 @@ __global__ void k64_lm_decide(Scalars* s, double eta, double lmin, double lmax, 
 
 // cos / sin of the rotation angles at x (warp: theta; mesh: ax, ay, az),
 // once per outer iteration (Sec. 4.2: evalJ's values depend only on x).
-__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_rot(P64 P) {
+__global__ void __launch_bounds__(NT, blocks64(3)) k64_rot(P64 P) {
   const int na = P.kind == F64_WARP ? 1 : 3;
   const int a0 = P.kind == F64_WARP ? 2 : 3;
   FOR_ELEMENTS(P, i) {
@@ -270,7 +269,7 @@ __device__ __forceinline__ void mesh_record(const P64& P, long long v, const dou
 // Direction update (Sec. 4.1 PCGStep): p = z + beta p, z = M^-1 r (every
 // PCG iteration after the first; PCGInit writes the first direction).
 template <int NX>
-__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_direction(P64 P) {
+__global__ void __launch_bounds__(NT, blocks64(NX)) k64_direction(P64 P) {
   const Scalars* s = P.s;
   if (s->done || !s->pcg_active) return;
   const double beta = s->beta_d;
@@ -295,7 +294,7 @@ __global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_direction(P64 P) {
 }
 
 // The mesh's direction records from a given p (apply hook).
-__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_mesh_records(P64 P) {
+__global__ void __launch_bounds__(NT, blocks64(6)) k64_mesh_records(P64 P) {
   const double* __restrict__ pp = P.pin ? P.pin : P.p;
   FOR_ELEMENTS(P, i) {
     double pv[6];
@@ -308,7 +307,7 @@ __global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_mesh_records(P64 P)
 // PCG vector update (Sec. 4.1 PCGStep): delta += alpha p, r -= alpha q,
 // z = M^-1 r, r.z -> beta = r.z / r.z_old.
 template <int NX>
-__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_update(P64 P) {
+__global__ void __launch_bounds__(NT, blocks64(NX)) k64_update(P64 P) {
   Scalars* s = P.s;
   if (s->done || !s->pcg_active) return;
   const double alpha = s->alpha_d;
@@ -352,7 +351,7 @@ __global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_update(P64 P) {
 }
 
 // x += delta (cond 0: unless the solve is done; cond 1: only if LM accepted).
-__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_step(P64 P, int cond) {
+__global__ void __launch_bounds__(NT, blocks64(3)) k64_step(P64 P, int cond) {
   const Scalars* s = P.s;
   if (cond ? !s->accept : s->done) return;
   FOR_ELEMENTS(P, i) {
@@ -365,7 +364,7 @@ __global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_step(P64 P, int con
 // Residual (k, d) for valid k, k+d: s_w ((O_k - O_{k+d}) - R(theta_k) v),
 // v = U_k - U_{k+d}; handle h: s_f (O_h - C_h) = s_f ((dx, dy)_h - target).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_warp_init(P64 P, int k_outer, double dmin, double dmax) {
+__global__ void __launch_bounds__(NT, blocks64(3)) k64_warp_init(P64 P, int k_outer, double dmin, double dmax) {
   Scalars* s = P.s;
   if (s->done) return;
   const double lam = P.lm ? s->lambda : 0.0;
@@ -474,7 +473,7 @@ struct Warp64 {
 };
 
 // E(x) (mode 0) or E(x + delta) and |F(x) + J(x) delta|^2 (mode 1).
-__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_warp_energy(P64 P, int mode, int hist_idx) {
+__global__ void __launch_bounds__(NT, blocks64(3)) k64_warp_energy(P64 P, int mode, int hist_idx) {
   Scalars* s = P.s;
   if (mode == 1 && s->done) return;
   const long long n = P.n;
@@ -530,7 +529,7 @@ __global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_warp_energy(P64 P, 
 // neighbour k+d in the image: residual (X_k - X_{k+d}) - (T_k - T_{k+d});
 // fixed pixels' X are constants.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_poisson_init(P64 P, int k_outer, double dmin, double dmax) {
+__global__ void __launch_bounds__(NT, blocks64(4)) k64_poisson_init(P64 P, int k_outer, double dmin, double dmax) {
   Scalars* s = P.s;
   if (s->done) return;
   const double lam = P.lm ? s->lambda : 0.0;
@@ -592,7 +591,7 @@ struct Poisson64 {
   }
 };
 
-__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_poisson_energy(P64 P, int mode, int hist_idx) {
+__global__ void __launch_bounds__(NT, blocks64(4)) k64_poisson_energy(P64 P, int mode, int hist_idx) {
   Scalars* s = P.s;
   if (mode == 1 && s->done) return;
   const long long n = P.n;
@@ -661,7 +660,7 @@ __device__ __forceinline__ void load_y(const P64& P, long long e, double (&y)[3]
 
 // y of every directed edge at x, by the edge's own vertex (ahead of PCGInit,
 // which reads it at both ends).
-__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_mesh_edges(P64 P) {
+__global__ void __launch_bounds__(NT, blocks64(6)) k64_mesh_edges(P64 P) {
   if (P.s->done) return;
   const long long n = P.n;
   FOR_ELEMENTS(P, v) {
@@ -682,7 +681,7 @@ __global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_mesh_edges(P64 P) {
   }
 }
 
-__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_mesh_init(P64 P, int k_outer, double dmin, double dmax) {
+__global__ void __launch_bounds__(NT, blocks64(6)) k64_mesh_init(P64 P, int k_outer, double dmin, double dmax) {
   Scalars* s = P.s;
   if (s->done) return;
   const double lam = P.lm ? s->lambda : 0.0;
@@ -818,7 +817,7 @@ struct Mesh64 {
 
 // applyJTJ as a launch of its own: q, and p.q -> alpha.
 template <class K>
-__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_apply(P64 P) {
+__global__ void __launch_bounds__(NT, blocks64(K::NX)) k64_apply(P64 P) {
   Scalars* s = P.s;
   if (s->done || !s->pcg_active) return;
   const double lam = P.lm ? s->lambda : 0.0;
@@ -1034,7 +1033,7 @@ __global__ void __launch_bounds__(RT, 1) k64_pcg_loop(P64 P, ResidentSync* sync,
 
 // E(x) (mode 0), or E(x + delta) and |F(x) + J(x) delta|^2 (mode 1: cos / sin at
 // x are those of this outer iteration's PCGInit).
-__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_mesh_energy(P64 P, int mode, int hist_idx) {
+__global__ void __launch_bounds__(NT, blocks64(6)) k64_mesh_energy(P64 P, int mode, int hist_idx) {
   Scalars* s = P.s;
   if (mode == 1 && s->done) return;
   const long long n = P.n;
@@ -1105,7 +1104,7 @@ __global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_mesh_energy(P64 P, 
 // Float64 multiply-add throughput probe: 8 independent dependency chains per
 // thread, enough blocks to fill every SM; the result is consumed so the
 // chains are not removed.
-__global__ void __launch_bounds__(NT, F64_BLOCKS_PER_SM) k64_fma_probe(double* out, int iters, double a, double b) {
+__global__ void __launch_bounds__(NT, blocks64(3)) k64_fma_probe(double* out, int iters, double a, double b) {
   double v[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) v[k] = 1e-3 * (threadIdx.x + k);
@@ -1203,7 +1202,7 @@ opt_status plan_common(opt_problem_f64* pb, const std::vector<double>& consts, c
   CK64(cudaGetDevice(&dev));
   CK64(cudaDeviceGetAttribute(&pb->sms, cudaDevAttrMultiProcessorCount, dev));
   const long long full = (P.n + NT - 1) / NT;
-  pb->nblk = (int)std::max<long long>(1, std::min<long long>(full, (long long)kBlocksPerSM64 * pb->sms));
+  pb->nblk = (int)std::max<long long>(1, std::min<long long>(full, (long long)blocks64(pb->nx) * pb->sms));
   P.w_reg = w_reg;
   P.w_fit = w_fit;
   P.s_w = std::sqrt(w_reg);
