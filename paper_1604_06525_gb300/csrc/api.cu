@@ -330,7 +330,7 @@ struct PlaneSet {
   float* user[12];
   float* own;                   // internal plane 0
   long long plane;
-  int n, W, H, P;               // graphs: W = vertices, H = 1
+  int n, W, H, P;               // graphs: W = vertices, H = 1; n = 0: nothing to move
   const int* perm;              // graphs
   int vec;                      // grids: quads of every user row are 16-byte aligned
 };
@@ -340,6 +340,7 @@ __global__ void __launch_bounds__(256) k_move_planes(const __grid_constant__ Pla
                                                      double lambda0, const SolveResult res) {
   if (!IN) gather_result(res);
   if (IN && reset && blockIdx.x == 0 && threadIdx.x == 0) scalars_reset(reset, lambda0);
+  if (ps.n == 0) return;
   const long long t0 = blockIdx.x * 256ll + threadIdx.x, step = gridDim.x * 256ll;
   auto move = [&](float* own, float* user) {
     if (IN) *own = *user;
@@ -371,6 +372,19 @@ __global__ void __launch_bounds__(256) k_move_planes(const __grid_constant__ Pla
   }
 }
 
+// Grids: a caller's plane that a kernel cannot address float by float (a byte offset
+// that is no multiple of 4, or memory CUDA does not know on this device) goes through a
+// copy, which takes any address and reports one that is not memory.
+bool addressable(const float* p) {
+  if (reinterpret_cast<uintptr_t>(p) % alignof(float) != 0) return false;
+  cudaPointerAttributes a = {};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return a.type != cudaMemoryTypeUnregistered && a.devicePointer == p;
+}
+
 opt_status copy_planes(const opt_problem* pb, PlaneDir dir, float* own, float* const* user, int n, cudaStream_t st,
                        Scalars* reset = nullptr, double lambda0 = 0.0, const SolveResult& res = SolveResult{}) {
   PlaneSet ps = {};
@@ -383,11 +397,23 @@ opt_status copy_planes(const opt_problem* pb, PlaneDir dir, float* own, float* c
   ps.P = grid ? pb->P : pb->V;
   ps.perm = grid ? nullptr : pb->d_perm;
   ps.vec = grid && pb->W % 4 == 0 && reinterpret_cast<uintptr_t>(own) % 16 == 0;
+  bool direct = true;
   for (int c = 0; c < n; ++c) {
     ps.user[c] = user[c];
     ps.vec = ps.vec && reinterpret_cast<uintptr_t>(user[c]) % 16 == 0;
+    direct = direct && (!grid || addressable(user[c]));
   }
-  const long long units = (long long)ps.W * ps.H / (ps.vec ? 4 : 1);
+  if (!direct) {
+    const size_t row = (size_t)pb->W * sizeof(float), pitch = (size_t)pb->P * sizeof(float);
+    for (int c = 0; c < n; ++c) {
+      float* o = own + c * pb->plane;
+      CK(dir == PlaneDir::In
+             ? cudaMemcpy2DAsync(o, pitch, user[c], row, row, pb->H, cudaMemcpyDeviceToDevice, st)
+             : cudaMemcpy2DAsync(user[c], row, o, pitch, row, pb->H, cudaMemcpyDeviceToDevice, st));
+    }
+    ps.n = 0;                     // the launch resets / gathers only
+  }
+  const long long units = ps.n ? (long long)ps.W * ps.H / (ps.vec ? 4 : 1) : 1;
   const unsigned blocks = (unsigned)std::max(1ll, std::min((units + 255) / 256, 16ll * pb->sms));
   if (dir == PlaneDir::In) k_move_planes<true><<<blocks, 256, 0, st>>>(ps, reset, lambda0, res);
   else k_move_planes<false><<<blocks, 256, 0, st>>>(ps, nullptr, 0.0, res);

@@ -1350,13 +1350,39 @@ __global__ void __launch_bounds__(NT) k64_move_planes(const __grid_constant__ Pl
       else ps.user[c][k] = ps.own[c * ps.n + k];
     }
 }
+// A caller's plane that a kernel cannot address double by double (an odd byte offset,
+// or memory CUDA does not know on this device) goes through a copy, which takes any
+// address and reports one that is not memory.
+bool addressable64(const double* p) {
+  if (reinterpret_cast<uintptr_t>(p) % alignof(double) != 0) return false;
+  cudaPointerAttributes a = {};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return a.type != cudaMemoryTypeUnregistered && a.devicePointer == p;
+}
 opt_status copy_x(opt_problem_f64* pb, bool in, cudaStream_t st, Scalars* reset = nullptr, double lambda0 = 0.0,
                   const SolveResult& res = SolveResult{}) {
   Planes64 ps = {};
-  for (int c = 0; c < pb->nx; ++c) ps.user[c] = pb->user_x[c];
+  bool direct = true;
+  for (int c = 0; c < pb->nx; ++c) {
+    ps.user[c] = pb->user_x[c];
+    direct = direct && addressable64(pb->user_x[c]);
+  }
   ps.own = pb->hp.x;
   ps.n = pb->hp.n;
   ps.planes = pb->nx;
+  if (!direct) {
+    const size_t bytes = (size_t)pb->hp.n * sizeof(double);
+    for (int c = 0; c < pb->nx; ++c) {
+      double* own = pb->hp.x + (size_t)c * pb->hp.n;
+      CK64(in ? cudaMemcpyAsync(own, pb->user_x[c], bytes, cudaMemcpyDeviceToDevice, st)
+              : cudaMemcpyAsync(pb->user_x[c], own, bytes, cudaMemcpyDeviceToDevice, st));
+    }
+    ps.planes = 0;                // the launch resets / gathers only
+    ps.n = 1;
+  }
   const unsigned blocks = (unsigned)std::max(1ll, std::min((ps.n + NT - 1) / NT, 8ll * pb->nblk));
   if (in) k64_move_planes<true><<<blocks, NT, 0, st>>>(ps, reset, lambda0, res);
   else k64_move_planes<false><<<blocks, NT, 0, st>>>(ps, nullptr, 0.0, res);
