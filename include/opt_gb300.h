@@ -198,7 +198,10 @@ typedef struct {
                                  fits on chip runs all iterations of an outer iteration in one
                                  launch (one thread-block cluster, or one block per SM), else
                                  two launches per iteration, as batches do; the same arithmetic.
-                                 A wait inside the launch is bounded (1 s): OPT_ERR_TIMEOUT.
+                                 The form over the device waits for its blocks with a limit (10 s
+                                 until the last one has found room beside other work on the
+                                 device, then 1 s): OPT_ERR_TIMEOUT; the cluster's blocks start
+                                 together and wait at the hardware's barrier.
                                  1 = single-reduction iteration, taken by matrix-free solves of
                                  OPT_ARAP_WARP_2D and OPT_POISSON_2D grids planned with 128-pixel
                                  tiles (other problems run form 0): it carries z = M^-1 r and
@@ -630,6 +633,23 @@ opt_status opt_selftest_grid_barrier(int32_t extra, int32_t rounds, int32_t* tim
  * and *timed_out = 1, leaving the context usable.  Synchronous.
  * OPT_ERR_INVALID_ARG for complete outside {0, 1} or a NULL pointer. */
 opt_status opt_selftest_staging_wait(int32_t complete, int32_t* timed_out);
+
+/* Self-test of the bounded exchanges of the on-chip PCG loop over the device (see
+ * opt_solve_params.persistent).  Two cooperative launches of 5 blocks that meet `rounds`
+ * times: kind 0 meetings, 1 the sums of the float32 loop, 2 those of the float64 loop
+ * (each after a meeting).  absent = 0: *timed_out = 0 and every total is right
+ * (OPT_ERR_NUMERIC otherwise).  absent = 1: one launch, in which one block does not take
+ * part; the others give up after 50 ms and *timed_out = 1, leaving the context usable.
+ * Synchronous.  OPT_ERR_INVALID_ARG for kind outside [0, 2], absent outside {0, 1}, rounds
+ * outside [1, 1000] or a NULL pointer. */
+opt_status opt_selftest_resident_exchange(int32_t kind, int32_t absent, int32_t rounds, int32_t* timed_out);
+
+/* Self-test: in the next solve of this problem that runs the on-chip loop over the device,
+ * one block does not take part, the others give up after 50 ms and the solve returns
+ * OPT_ERR_TIMEOUT; solves after it are normal.  Synchronous.  OPT_ERR_INVALID_ARG before
+ * the problem's first solve with that loop. */
+opt_status opt_selftest_lose_block(opt_problem* prob);
+opt_status opt_selftest_lose_block_f64(opt_problem_f64* prob);
 
 /* Human-readable name of a status code; never NULL. */
 const char* opt_status_str(opt_status s);

@@ -42,6 +42,19 @@ opt_status optgb::cuda_fail(cudaError_t e, const char* what) {
 
 void optgb::set_last_error(const std::string& text) { g_err = text; }
 
+// The counts and limits of a fresh exchange and empty slots; done when it returns, so
+// that the next solve finds them whatever its stream.
+opt_status optgb::reset_exchange(ResidentSync* d, cudaStream_t st, bool lose_block) {
+  ResidentSync head = {};
+  head.first_ns = lose_block ? kSelfTestLimitNs : kFirstLimitNs;
+  head.wait_ns = lose_block ? kSelfTestLimitNs : kBarrierLimitNs;
+  head.absent = lose_block;
+  cudaError_t e = cudaMemcpyAsync(d, &head, offsetof(ResidentSync, slot), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d->slot, 0xff, sizeof(d->slot), st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  return e == cudaSuccess ? OPT_OK : cuda_fail(e, "exchange slots");
+}
+
 namespace {
 
 #define CK(call)                                         \
@@ -556,7 +569,7 @@ opt_status resident_prepare(opt_problem* pb, int lm) {
   if (rp.blocks > 0) {
     if (!pb->d_rsync) {
       CKS(dalloc(pb, &pb->d_rsync, 1));
-      CK(cudaMemsetAsync(pb->d_rsync->slot, 0xff, sizeof(pb->d_rsync->slot), nullptr));
+      CKS(reset_exchange(pb->d_rsync, nullptr));
     }
     if (grid && !pb->d_cells) {
       CKS(dalloc(pb, &pb->d_cells, pb->h_cells.size()));
@@ -736,8 +749,7 @@ opt_status run_solve(opt_problem* pb, const opt_solve_params* prm_in, opt_report
   if (s.timeout) {
     if (pb->d_rsync) {
       // blocks gave up at different exchanges: back to empty slots
-      CK(cudaMemset(pb->d_rsync, 0, sizeof(ResidentSync)));
-      CK(cudaMemset(pb->d_rsync->slot, 0xff, sizeof(pb->d_rsync->slot)));
+      CKS(reset_exchange(pb->d_rsync, st));
     }
     return OPT_ERR_TIMEOUT;
   }
@@ -891,6 +903,32 @@ opt_status opt_selftest_staging_wait(int32_t complete, int32_t* timed_out) {
   if (e != cudaSuccess) return cuda_fail(e, "opt_selftest_staging_wait");
   *timed_out = h ? 1 : 0;
   return OPT_OK;
+}
+
+opt_status opt_selftest_resident_exchange(int32_t kind, int32_t absent, int32_t rounds, int32_t* timed_out) {
+  if (kind < 0 || kind > 2 || absent < 0 || absent > 1 || rounds < 1 || rounds > 1000 || !timed_out)
+    return OPT_ERR_INVALID_ARG;
+  *timed_out = 0;
+  opt_problem work;
+  ResidentSync* sy = nullptr;
+  int *d = nullptr, h[2] = {0, 0};
+  CKS(dalloc(&work, &sy, 1));
+  CKS(dalloc(&work, &d, 2));
+  CKS(reset_exchange(sy, nullptr, absent != 0));
+  // twice without a reset: the counts go on from launch to launch
+  for (int launch = 0; launch < (absent ? 1 : 2); ++launch) {
+    CK(kind == 2 ? launch_exchange_selftest64(sy, rounds, d, nullptr)
+                 : launch_exchange_selftest(sy, kind, rounds, d, nullptr));
+    CK(cudaMemcpy(h, d, sizeof(h), cudaMemcpyDeviceToHost));
+  }
+  *timed_out = h[0];
+  return h[1] ? OPT_ERR_NUMERIC : OPT_OK;
+}
+
+opt_status opt_selftest_lose_block(opt_problem* prob) {
+  if (!prob || !prob->d_rsync) return OPT_ERR_INVALID_ARG;
+  CK(cudaDeviceSynchronize());
+  return reset_exchange(prob->d_rsync, nullptr, true);
 }
 
 const char* opt_status_str(opt_status s) {

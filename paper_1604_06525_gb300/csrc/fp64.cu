@@ -44,6 +44,7 @@
 #include "opt_gb300.h"
 #include "meet.cuh"
 #include "opt_internal.cuh"
+#include "opt_launch.h"
 #include "opt_problem.h"
 
 using namespace optgb;
@@ -893,7 +894,7 @@ __device__ __forceinline__ bool meet_sum64(Meet& M, double acc, int cnt, double&
     const unsigned long long* p = sum_slot(M, k, on ? threadIdx.x : 0);
     unsigned long long b, t0 = 0;
     int ok = 1;
-    for (int spin = 0; (b = ld_relaxed(p)) == kEmpty && ok; ++spin) ok = !waited_too_long(spin, t0);
+    for (int spin = 0; (b = ld_relaxed(p)) == kEmpty && ok; ++spin) ok = !waited_too_long(spin, t0, M.limit);
     __threadfence();
     ok = __all_sync(0xffffffffu, ok);
     double t = on ? __longlong_as_double((long long)b) : 0.0;
@@ -913,6 +914,7 @@ __device__ __forceinline__ bool meet_sum64(Meet& M, double acc, int cnt, double&
 #pragma unroll
     for (int t = 1; t < NP; ++t) total += sg[t];
   }
+  M.limit = M.later;
   return ok != 0;
 }
 
@@ -922,7 +924,8 @@ __global__ void __launch_bounds__(RT, 1) k64_pcg_loop(P64 P, ResidentSync* sync,
   extern __shared__ double sh64[];
   Scalars* s = P.s;
   if (s->done || !s->pcg_active) return;       // the same for every block: none has met another
-  Meet M{sync, sync->meetings, 0u, sync->sums};
+  if (sync->absent && blockIdx.x + 1 == gridDim.x) return;
+  Meet M = meet_begin(sync);
   const double lam = P.lm ? s->lambda : 0.0;
   const int tid = threadIdx.x;
   const long long n = P.n, lo = (long long)blockIdx.x * per;
@@ -1026,6 +1029,24 @@ __global__ void __launch_bounds__(RT, 1) k64_pcg_loop(P64 P, ResidentSync* sync,
     s->pcg_iters += iters;
     if (!active) s->pcg_active = 0;
     if (nonfinite) s->nonfinite = 1;
+    sync->meetings = M.base + M.meetings * gridDim.x;
+    sync->sums = M.sums % 3u;
+  }
+}
+
+// Self-test: `rounds` sums, each after a meeting.
+__global__ void __launch_bounds__(RT, 1) k64_exchange_selftest(ResidentSync* sync, int rounds, int* out) {
+  if (sync->absent && blockIdx.x + 1 == gridDim.x) return;
+  Meet M = meet_begin(sync);
+  bool met = true;
+  for (int r = 1; r <= rounds && met; ++r) {
+    double total = 0.0;
+    met = meet_device(M) && meet_sum64(M, (double)r, RT, total);
+    if (met && threadIdx.x == 0 && total != (double)r * RT * gridDim.x) out[1] = 1;
+  }
+  if (threadIdx.x != 0) return;
+  if (!met) out[0] = 1;
+  if (met && blockIdx.x == 0) {
     sync->meetings = M.base + M.meetings * gridDim.x;
     sync->sums = M.sums % 3u;
   }
@@ -1266,9 +1287,7 @@ opt_status plan_loop(opt_problem_f64* pb) {
   pb->loop_blocks = (int)((pb->hp.n + per - 1) / per);
   pb->loop_smem = (int)bytes;
   CKS64(alloc64(pb, &pb->d_rsync, 1));
-  CK64(cudaMemset(pb->d_rsync, 0, sizeof(ResidentSync)));
-  CK64(cudaMemset(pb->d_rsync->slot, 0xff, sizeof(pb->d_rsync->slot)));
-  return OPT_OK;
+  return reset_exchange(pb->d_rsync, nullptr);
 }
 
 opt_status launch_loop(opt_problem_f64* pb, const P64& P, cudaStream_t st, int inner) {
@@ -1510,8 +1529,7 @@ opt_status run_solve64(opt_problem_f64* pb, const opt_solve_params* prm_in, opt_
   }
   if (s.timeout) {
     // blocks gave up at different meetings: back to empty slots
-    CK64(cudaMemset(pb->d_rsync, 0, sizeof(ResidentSync)));
-    CK64(cudaMemset(pb->d_rsync->slot, 0xff, sizeof(pb->d_rsync->slot)));
+    CKS64(reset_exchange(pb->d_rsync, st));
     return OPT_ERR_TIMEOUT;
   }
   if (s.nonfinite) return OPT_ERR_NUMERIC;
@@ -1549,6 +1567,11 @@ opt_status finish_create64(std::unique_ptr<opt_problem_f64>& pb, opt_problem_f64
 }
 
 }  // namespace
+
+cudaError_t optgb::launch_exchange_selftest64(ResidentSync* sync, int rounds, int* out, cudaStream_t st) {
+  void* args[] = {&sync, &rounds, &out};
+  return cudaLaunchCooperativeKernel((const void*)k64_exchange_selftest, dim3(5), dim3(RT), args, 0, st);
+}
 
 extern "C" {
 
@@ -1790,6 +1813,12 @@ opt_status opt_profile_pcg_f64(opt_problem_f64* pb, int32_t n_iters, void* strea
   ms[1] = ta / n_iters;
   ms[2] = tu / n_iters;
   return OPT_OK;
+}
+
+opt_status opt_selftest_lose_block_f64(opt_problem_f64* pb) {
+  if (!pb || !pb->d_rsync) return OPT_ERR_INVALID_ARG;
+  CK64(cudaDeviceSynchronize());
+  return reset_exchange(pb->d_rsync, nullptr, true);
 }
 
 opt_status opt_problem_info_f64(const opt_problem_f64* pb, int64_t* n_unknowns, int32_t* n_planes,

@@ -282,14 +282,20 @@ constexpr int RES_LANES = 4;          // threads per vertex where a block has fe
 constexpr int RES_CLUSTER = 16;       // blocks of the one-cluster form, at most
 // RES_D, RES_DC, RES_LIST: kept in shared memory; RES_Z: see Records (resident.cu)
 enum ResidentFlags : int { RES_D = 1, RES_DC = 2, RES_LIST = 4, RES_Z = 8 };
-// Exchange slots of one problem; the host fills slot with ones (empty) and the
-// rest with zeros before the first launch, and again after a timeout.
+// Exchange slots of one problem, set up by reset_exchange() before the first launch and
+// again after a timeout.  first_ns bounds the wait for the launch's first exchange, which
+// ends when its last block has found room beside whatever else runs on the device; from
+// then on all blocks are there and wait_ns bounds each wait.
+constexpr unsigned long long kFirstLimitNs = 10000000000ull;    // 10 s
 struct ResidentSync {
   unsigned int counter;         // arrivals at meetings, ever growing
   unsigned int pad0[31];
   unsigned int meetings;        // the counter's value between launches
   unsigned int sums;            // sums done so far (modulo the sets / tags of the loop that uses them)
-  unsigned int pad1[30];
+  unsigned int absent;          // self-test: the last block of the launch does not take part
+  unsigned int pad1;
+  unsigned long long first_ns, wait_ns;
+  unsigned int pad2[24];
   unsigned long long slot[3][RES_MAX_BLOCKS][16];   // a cache line each
 };
 struct ResidentPlan {

@@ -97,6 +97,11 @@ cudaError_t launch_resident_grid(int kind, const GridProb* probs, const int* cel
 cudaError_t launch_resident_graph(int kind, const MeshProb* probs, ResidentSync* sync, const ResidentPlan& rp,
                                   float4* rec, int inner, int step, cudaStream_t st);
 
+// Self-tests: `rounds` exchanges of 5 blocks (kind 0: meetings, 1: float32 sums; fp64.cu:
+// sums and meetings of the float64 loop).  out: [0] a wait ran out, [1] a total was wrong
+cudaError_t launch_exchange_selftest(ResidentSync* sync, int kind, int rounds, int* out, cudaStream_t st);
+cudaError_t launch_exchange_selftest64(ResidentSync* sync, int rounds, int* out, cudaStream_t st);
+
 // edge_plan.cu: the edges of a graph in the internal vertex order.  v0, v1: the
 // caller's; iperm: internal number of every caller vertex; e0, e1, isrc: E entries; orow,
 // irow: V + 1 zeros before the call; cursor: 2 (V + 1); degw: w_fit at handles, else 0,

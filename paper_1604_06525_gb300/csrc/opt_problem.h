@@ -166,6 +166,10 @@ struct opt_batch;
 namespace optgb {
 // api.cu: records a failed CUDA call for opt_last_error (OOM or CUDA status)
 opt_status cuda_fail(cudaError_t e, const char* what);
+// api.cu: sets the exchange slots of a resident PCG loop up, ordered on st and waited for;
+// lose_block (self-tests): one block of the next launch does not take part, short limits
+constexpr unsigned long long kSelfTestLimitNs = 50000000ull;     // 50 ms
+opt_status reset_exchange(ResidentSync* d, cudaStream_t st, bool lose_block = false);
 // api.cu: the calling thread's opt_last_error text
 void set_last_error(const std::string& text);
 // batch.cu (serving engine interface)

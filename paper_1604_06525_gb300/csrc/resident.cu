@@ -36,9 +36,10 @@
 // (2^-46 of the sum) say which sum it belongs to, so a slot needs no emptying and a
 // stale one is never taken for the next: a block stores sum k + 2 only after sum k
 // + 1, which every block reaches after reading those of k.  The counts go on from
-// launch to launch (sync->sums, sync->meetings).  Every wait is bounded (1 s); a
-// block that gives up flags s->timeout and returns, the others run into their own
-// limit, and the host resets the slots.
+// launch to launch (sync->sums, sync->meetings).  Every wait of the device-wide form is
+// bounded (ResidentSync); a block that gives up flags s->timeout and returns, the others
+// run into their own limit, and the host resets the slots.  The cluster form waits at the hardware's barrier, which has no limit
+// and needs none: its blocks start together and all take the same path.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -143,7 +144,8 @@ __device__ __forceinline__ bool meet_sum(Meet& M, F2 acc, F2& total) {
       const unsigned long long* p = &M.sy->slot[k & 1][on ? threadIdx.x : 0][0];
       unsigned long long b, t0 = 0;
       int ok = 1;
-      for (int spin = 0; (((b = ld_relaxed(p)) >> 32) & 3) != (k & 3) && ok; ++spin) ok = !waited_too_long(spin, t0);
+      for (int spin = 0; (((b = ld_relaxed(p)) >> 32) & 3) != (k & 3) && ok; ++spin)
+        ok = !waited_too_long(spin, t0, M.limit);
       if (FENCE) __threadfence();
       ok = __all_sync(0xffffffffu, ok);
       const F2 v = warp_sum_f2(on ? unpack(b & ~(3ull << 32)) : f2_zero());
@@ -160,6 +162,7 @@ __device__ __forceinline__ bool meet_sum(Meet& M, F2 acc, F2& total) {
       f2_add_f2(total, unpack(sg[t]));
       ok &= s_ok[t];
     }
+    M.limit = M.later;
     return ok != 0;
   }
 }
@@ -672,7 +675,8 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
   if (CL) pdl_begin();
   Scalars* s = pr.s;
   if (s->done || !s->pcg_active) return;      // the same for every block: none has passed an exchange
-  Meet M{sync, CL ? 0u : sync->meetings, 0u, CL ? 0u : sync->sums};
+  if (!CL && sync->absent && blockIdx.x + 1 == gridDim.x) return;
+  Meet M = CL ? Meet{} : meet_begin(sync);
   const int tid = threadIdx.x;
   const int u0 = blockIdx.x * rp.per, cnt = min(rp.per, rp.n - u0), cap = rp.per;
   const long long pl = rp.plane;
@@ -1010,6 +1014,29 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
   }
 }
 
+// Self-test: `rounds` meetings (kind 0) or sums, with and without ordered writes (kind 1).
+__global__ void __launch_bounds__(RT, 1) k_exchange_selftest(ResidentSync* sync, int kind, int rounds, int* out) {
+  if (sync->absent && blockIdx.x + 1 == gridDim.x) return;
+  Meet M = meet_begin(sync);
+  bool met = true;
+  for (int r = 1; r <= rounds && met; ++r) {
+    if (kind == 0) {
+      met = meet_device(M);
+      continue;
+    }
+    const F2 mine = {(float)r, 0.f};
+    F2 total = f2_zero();
+    met = r & 1 ? meet_sum<false, true>(M, mine, total) : meet_sum<false, false>(M, mine, total);
+    if (met && f2_to_double(total) != (double)r * RT * gridDim.x) out[1] = 1;
+  }
+  if (threadIdx.x != 0) return;
+  if (!met) out[0] = 1;
+  if (met && blockIdx.x == 0) {
+    sync->meetings = M.base + M.meetings * gridDim.x;
+    sync->sums = M.sums & 3u;
+  }
+}
+
 template <class K, bool CL>
 cudaError_t launch(const typename K::Prob* probs, const int* cells, ResidentSync* sync, const ResidentPlan& rp,
                    float4* rec, int inner, int step, int csn_out, cudaStream_t st) {
@@ -1202,6 +1229,11 @@ ResidentPlan resident_plan(int kind, int n, long long plane, int lm, const int* 
   if (!fill(d.sms, grid ? CELL : 64)) return ResidentPlan{};
   if (n <= RES_Z_UNITS) rp.flags |= RES_Z;
   return rp;
+}
+
+cudaError_t launch_exchange_selftest(ResidentSync* sync, int kind, int rounds, int* out, cudaStream_t st) {
+  void* args[] = {&sync, &kind, &rounds, &out};
+  return cudaLaunchCooperativeKernel((const void*)k_exchange_selftest, dim3(5), dim3(RT), args, 0, st);
 }
 
 cudaError_t launch_resident_grid(int kind, const GridProb* probs, const int* cells, ResidentSync* sync,
