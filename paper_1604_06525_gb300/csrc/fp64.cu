@@ -923,7 +923,9 @@ __global__ void __launch_bounds__(RT, 1) k64_pcg_loop(P64 P, ResidentSync* sync,
   constexpr int NX = K::NX;
   extern __shared__ double sh64[];
   Scalars* s = P.s;
-  if (s->done || !s->pcg_active) return;       // the same for every block: none has met another
+  // (the same for every block: none has met another; nothing waits after a launch whose
+  // exchanges failed)
+  if (s->done || !s->pcg_active || s->timeout) return;
   if (sync->absent && blockIdx.x + 1 == gridDim.x) return;
   Meet M = meet_begin(sync);
   const double lam = P.lm ? s->lambda : 0.0;

@@ -38,7 +38,8 @@
 // + 1, which every block reaches after reading those of k.  The counts go on from
 // launch to launch (sync->sums, sync->meetings).  Every wait of the device-wide form is
 // bounded (ResidentSync); a block that gives up flags s->timeout and returns, the others
-// run into their own limit, and the host resets the slots.  The cluster form waits at the hardware's barrier, which has no limit
+// run into their own limit, the later launches of the solve return at once, and the host
+// resets the slots.  The cluster form waits at the hardware's barrier, which has no limit
 // and needs none: its blocks start together and all take the same path.
 #include <algorithm>
 #include <cmath>
@@ -674,7 +675,9 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
   const typename K::Prob pr = probs[0];
   if (CL) pdl_begin();
   Scalars* s = pr.s;
-  if (s->done || !s->pcg_active) return;      // the same for every block: none has passed an exchange
+  // (the same for every block: none has passed an exchange; after a launch whose exchanges
+  // failed the counts no longer match, and the rest of the solve does not wait on them)
+  if (s->done || !s->pcg_active || s->timeout) return;
   if (!CL && sync->absent && blockIdx.x + 1 == gridDim.x) return;
   Meet M = CL ? Meet{} : meet_begin(sync);
   const int tid = threadIdx.x;
