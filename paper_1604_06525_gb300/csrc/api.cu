@@ -1131,7 +1131,7 @@ opt_status opt_problem_create_grid(const opt_grid_desc* d, const opt_solve_param
   up.add(q->d_chunks, chunks);
   q->h_chunks = chunks;
   q->nchunks = (int)chunks.size();
-  CKS(dalloc(q, &q->d_part, 4 * chunks.size()));   // up to three partials per chunk
+  CKS(dalloc(q, &q->d_part, 8 * chunks.size()));   // up to four Sums per chunk
   CKS(dalloc(q, &q->dg, 1));
   for (int k = 0; k < nx; ++k) q->user_x[k] = d->unknowns[k];
   q->h_mask = mask;
@@ -1837,7 +1837,7 @@ static opt_status rechunk(opt_problem* pb, int per) {
                                         : make_chunks_balanced(pb->ntiles, target, 0);
     if ((int)chunks.size() > pb->nchunks) {
       CKS(dalloc(pb, &pb->d_chunks, chunks.size()));
-      CKS(dalloc(pb, &pb->d_part, 4 * chunks.size()));
+      CKS(dalloc(pb, &pb->d_part, 8 * chunks.size()));
     }
     CKS(upload(pb->d_chunks, chunks));
     pb->h_chunks = chunks;

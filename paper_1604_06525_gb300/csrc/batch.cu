@@ -257,7 +257,7 @@ opt_status build_tables(opt_batch* b, int tpc) {
     if ((s = bupload(b->table_allocs, &g.d_probs, gp)) != OPT_OK) return s;
     if ((s = bupload(b->table_allocs, &g.d_chunks, chunks)) != OPT_OK) return s;
     if ((s = bupload(b->table_allocs, &g.d_tiles, tiles)) != OPT_OK) return s;
-    if ((s = balloc(b->table_allocs, &g.d_part, 4 * chunks.size())) != OPT_OK) return s;   // up to 4 partials
+    if ((s = balloc(b->table_allocs, &g.d_part, 8 * chunks.size())) != OPT_OK) return s;   // up to 4 Sums
     g.nchunks = (int)chunks.size();
     g.h_probs = gp;
   }

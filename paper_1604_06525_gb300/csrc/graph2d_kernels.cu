@@ -213,9 +213,9 @@ __global__ void __launch_bounds__(NT) k_wg_apply_pull(const MeshProb* __restrict
   }
   pdl_trigger();
   const F2 sums[1] = {acc};
-  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
-    F2 pq[1];
-    gather_pairs<1>(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, pq);
+  if (publish_sums<1>(part, blockIdx.x, sums, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
+    Sum pq[1];
+    gather_sums<1>(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, pq);
     if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
@@ -263,9 +263,9 @@ __global__ void __launch_bounds__(NT) k_wg_update(const MeshProb* __restrict__ p
   }
   pdl_trigger();
   const F2 sums[1] = {acc};
-  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
-    F2 rz[1];
-    gather_pairs<1>(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, rz);
+  if (publish_sums<1>(part, blockIdx.x, sums, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
+    Sum rz[1];
+    gather_sums<1>(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, rz);
     if (threadIdx.x == 0) finish_beta(s, rz[0]);
   }
 }

@@ -319,9 +319,9 @@ __global__ void __launch_bounds__(NT, MESH_PULL_MIN_BLOCKS) k_mesh_apply_pull(co
   }
   pdl_trigger();
   const F2 sums[1] = {acc};
-  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
-    F2 pq[1];
-    gather_pairs<1>(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, pq);
+  if (publish_sums<1>(part, blockIdx.x, sums, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
+    Sum pq[1];
+    gather_sums<1>(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, pq);
     if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
@@ -512,9 +512,9 @@ __global__ void __launch_bounds__(NT, MESH_TILED_MIN_BLOCKS) k_mesh_apply_tiled(
   (void)ibase;
   pdl_trigger();
   const F2 sums[1] = {acc};
-  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.tchunk_end - pr.tchunk_begin)) {
-    F2 pq[1];
-    gather_pairs<1>(part, pr.tchunk_begin, pr.tchunk_end, &s->counter, pq);
+  if (publish_sums<1>(part, blockIdx.x, sums, &s->counter, pr.tchunk_end - pr.tchunk_begin)) {
+    Sum pq[1];
+    gather_sums<1>(part, pr.tchunk_begin, pr.tchunk_end, &s->counter, pq);
     if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
@@ -562,9 +562,9 @@ __global__ void __launch_bounds__(NT) k_mesh_update(const MeshProb* __restrict__
   }
   pdl_trigger();
   const F2 sums[1] = {f2x2_fold(acc)};
-  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
-    F2 rz[1];
-    gather_pairs<1>(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, rz);
+  if (publish_sums<1>(part, blockIdx.x, sums, &s->counter, pr.vchunk_end - pr.vchunk_begin)) {
+    Sum rz[1];
+    gather_sums<1>(part, pr.vchunk_begin, pr.vchunk_end, &s->counter, rz);
     if (threadIdx.x == 0) finish_beta(s, rz[0]);
   }
 }

@@ -350,9 +350,9 @@ __global__ void __launch_bounds__(NT, 3) k_warp_apply(const GridProb* __restrict
     }
   }
   const F2 sums[1] = {acc};
-  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    F2 pq[1];
-    gather_pairs<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq);
+  if (publish_sums<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
+    Sum pq[1];
+    gather_sums<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq);
     if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
@@ -940,9 +940,9 @@ __device__ __forceinline__ void apply_wide_body(WideSmem& sm, const Chunk& ch, c
   }
   cp_async_wait_all();
   const F2 sums[1] = {f2x2_fold(acc)};
-  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    F2 pq[1];
-    gather_pairs<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq);
+  if (publish_sums<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
+    Sum pq[1];
+    gather_sums<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq);
     if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
@@ -1072,9 +1072,9 @@ __device__ __forceinline__ void fused_pending(const Chunk& ch, const GridProb& p
     }
   }
   const F2 none[4] = {f2_zero(), f2_zero(), f2_zero(), f2_zero()};
-  if (publish_pairs<4>(part, blockIdx.x, none, &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    F2 unused[4];
-    gather_pairs<4>(part, pr.chunk_begin, pr.chunk_end, &s->counter, unused);
+  if (publish_sums<4>(part, blockIdx.x, none, &s->counter, pr.chunk_end - pr.chunk_begin)) {
+    Sum unused[4];
+    gather_sums<4>(part, pr.chunk_begin, pr.chunk_end, &s->counter, unused);
     if (threadIdx.x == 0) s->alpha_f = 0.f;
   }
 }
@@ -1086,26 +1086,25 @@ __device__ __forceinline__ void fused_finish(const GridProb& pr, double* __restr
                                              const F2x2& acc_qz, const F2x2& acc_qw, const F2x2& acc_zr) {
   Scalars* s = pr.s;
   const F2 sums[4] = {f2x2_fold(acc_pq), f2x2_fold(acc_qz), f2x2_fold(acc_qw), f2x2_fold(acc_zr)};
-  if (publish_pairs<4>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    F2 v[4];
-    gather_pairs<4>(part, pr.chunk_begin, pr.chunk_end, &s->counter, v);
+  if (publish_sums<4>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
+    Sum v[4];
+    gather_sums<4>(part, pr.chunk_begin, pr.chunk_end, &s->counter, v);
     if (threadIdx.x == 0) {
-      const F2 pq = v[0], rz = v[3];
-      s->pq = f2_to_double(pq);
-      if (pq.hi > 0.f && isfinite(pq.hi) && rz.hi > 0.f && isfinite(rz.hi)) {
+      const Sum &pq = v[0], &rz = v[3];
+      s->pq = sum_double(pq);
+      if (pq.hi > 0.f && sum_finite(pq) && rz.hi > 0.f && sum_finite(rz)) {
         // alpha from the r.z of the stored z (as the two-pass form takes it);
         // the recurrence only carries r.z one iteration ahead, to set beta.  It
-        // cancels, so it is evaluated in float64.
-        const float af = f2_quot(rz, pq);
-        const double a = (double)af, rzd = f2_to_double(rz);
-        const double rz_next = fma(a * a, f2_to_double(v[2]), fma(-2.0 * a, f2_to_double(v[1]), rzd));
+        // cancels; it is evaluated in float64.
+        const float af = sum_quot(rz, pq);
+        const double a = (double)af, qz = sum_double(v[1]), qw = sum_double(v[2]), rzd = sum_double(rz);
+        const double rz_next = fma(a * a, qw, fma(-2.0 * a, qz, rzd));
         s->alpha_f = af;
         s->rz = rzd;
-        s->rz_hi = rz.hi;
-        s->rz_lo = rz.lo;
+        s->rz_sum = rz;
         s->pcg_iters += 1;
         if (rz_next > 0.0 && isfinite(rz_next)) {
-          s->beta_f = f2_quot(f2_from_double(rz_next), rz);
+          s->beta_f = sum_quot(sum_of(rz_next), rz);
         } else {
           s->pcg_active = 0;        // the step alpha p is still applied
           if (!isfinite(rz_next)) s->nonfinite = 1;
@@ -1113,7 +1112,7 @@ __device__ __forceinline__ void fused_finish(const GridProb& pr, double* __restr
       } else {
         s->alpha_f = 0.f;
         s->pcg_active = 0;
-        if (!isfinite(pq.hi) || !isfinite(rz.hi)) s->nonfinite = 1;
+        if (!sum_finite(pq) || !sum_finite(rz)) s->nonfinite = 1;
       }
     }
   }
@@ -2189,9 +2188,9 @@ __global__ void __launch_bounds__(NT, 3) k_poisson_apply(const GridProb* __restr
     }
   }
   const F2 sums[1] = {acc};
-  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    F2 pq[1];
-    gather_pairs<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq);
+  if (publish_sums<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
+    Sum pq[1];
+    gather_sums<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq);
     if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
@@ -2464,9 +2463,9 @@ __device__ __forceinline__ void k_poisson_apply_wide_body(PoisWideSmem& sm, cons
                            beta2, lam, pout, pl, acc);
   }
   const F2 sums[1] = {f2x2_fold(acc)};
-  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    F2 pq[1];
-    gather_pairs<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq);
+  if (publish_sums<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
+    Sum pq[1];
+    gather_sums<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, pq);
     if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
@@ -3026,9 +3025,9 @@ __device__ __forceinline__ void update_body(const Chunk& ch, const GridProb& pr,
     }
   }
   const F2 sums[1] = {f2x2_fold(acc)};
-  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
-    F2 rz[1];
-    gather_pairs<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, rz);
+  if (publish_sums<1>(part, blockIdx.x, sums, &s->counter, pr.chunk_end - pr.chunk_begin)) {
+    Sum rz[1];
+    gather_sums<1>(part, pr.chunk_begin, pr.chunk_end, &s->counter, rz);
     if (threadIdx.x == 0) finish_beta(s, rz[0]);
   }
 }

@@ -131,9 +131,9 @@ __global__ void __launch_bounds__(NT) k_csr_jtt(int nT, const int* __restrict__ 
     f2_add_prod(acc, pu, v);
   }
   const F2 sums[1] = {acc};
-  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, gridDim.x)) {
-    F2 pq[1];
-    gather_pairs<1>(part, 0, gridDim.x, &s->counter, pq);
+  if (publish_sums<1>(part, blockIdx.x, sums, &s->counter, gridDim.x)) {
+    Sum pq[1];
+    gather_sums<1>(part, 0, gridDim.x, &s->counter, pq);
     if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }
@@ -192,9 +192,9 @@ __global__ void __launch_bounds__(NT) k_jtj_spmv(int nT, const int* __restrict__
     f2_add_prod(acc, pu, v);
   }
   const F2 sums[1] = {acc};
-  if (publish_pairs<1>(part, blockIdx.x, sums, &s->counter, gridDim.x)) {
-    F2 pq[1];
-    gather_pairs<1>(part, 0, gridDim.x, &s->counter, pq);
+  if (publish_sums<1>(part, blockIdx.x, sums, &s->counter, gridDim.x)) {
+    Sum pq[1];
+    gather_sums<1>(part, 0, gridDim.x, &s->counter, pq);
     if (threadIdx.x == 0) finish_alpha(s, pq[0]);
   }
 }

@@ -19,8 +19,8 @@
 // on: each thread accumulates its terms as a compensated float32 pair (every
 // product split exactly by one FMA, every addition made error-free by TwoSum:
 // Ogita, Rump & Oishi's Dot2, see F2 below), warps combine the pairs in a fixed
-// shuffle order; the sums behind alpha and beta stay pairs to the end (see
-// publish_pairs), energies go on in float64 (the float64 pipe of this part is
+// shuffle order; the sums behind alpha and beta stay pairs to the end (see "sums above a
+// warp"), energies go on in float64 (the float64 pipe of this part is
 // narrow, so it is kept to the last levels).  Each block writes its partial to a
 // per-chunk slot, and the last block of a problem to arrive (atomic counter)
 // sums the problem's partials in chunk order, so the result does not depend on
@@ -52,6 +52,13 @@ constexpr int VT = 256;           // vertices per vertex tile (graph)
 constexpr int MT_HALO = 384;
 constexpr int MT_SLOTS = 2304;
 
+// A sum as an unevaluated float32 pair; big: what it stands for is 2^64 times that.  See
+// "sums above a warp".
+struct Sum {
+  float hi, lo;
+  int big;
+};
+
 // Device-resident scalars of one problem.  Written only by the single
 // finishing block of a reduction or by the one-thread LM decision kernel.
 struct __align__(16) Scalars {
@@ -67,7 +74,7 @@ struct __align__(16) Scalars {
   float alpha_f;      // alpha = rz / pq, rounded once to float
   float beta_f;       // beta  = rz' / rz
   float lambda_f;
-  float rz_hi, rz_lo; // rz as an unevaluated float32 pair (PCG loops; set with rz)
+  Sum rz_sum;         // rz as the PCG loops carry it (set with rz)
   int pcg_active;     // 0 once PCG broke down (rz == 0 or pq <= 0)
   int pcg_iters;      // completed PCG iterations in the current solve
   int accept;         // LM: the last trial step was accepted
@@ -79,6 +86,7 @@ struct __align__(16) Scalars {
   unsigned int counter;   // last-block counter
   unsigned int timeout;   // a bounded wait for a tensor copy ran out (the solve reports OPT_ERR_TIMEOUT)
   unsigned int misaligned;  // a staging area could not take tensor copies (the solve reports OPT_ERR_CUDA)
+  unsigned int pad1;
   double alpha_d;     // float64 solver: alpha = rz / pq
   double beta_d;      // float64 solver: beta  = rz' / rz
 };
@@ -499,15 +507,39 @@ __device__ __forceinline__ void gather_partials(const double* part, int cb, int 
 }
 
 // ---------------------------------------------------------------------------
-// PCG scalars: dot products carried as pairs to the end
+// sums above a warp
 // ---------------------------------------------------------------------------
-// The sums behind alpha and beta (p.q, r.z, ...) stay compensated pairs across
-// the warps and the blocks too.  alpha and beta are rounded to float32 once;
-// a pair (about 47 bits) carries them to that rounding as float64 does, and the
-// float64 tail it replaces was a serial chain of every launch: 64 cycles an
-// addition, 109 a shuffle level, 560 a division, about 3,000 cycles (1.5 us)
-// from the last block's partial sums to the published scalar against about 800
-// with pairs.  Energies and the LM decision stay in float64.
+// The dot products behind alpha and beta stay compensated pairs across the warps and the
+// blocks too: about 47 bits, of which alpha and beta, rounded to float32 once, keep 24.
+// In float64 every alpha and beta of the performance cases comes out the same, but its
+// tail is a serial chain (64 cycles an addition, 109 a shuffle level, 560 a division):
+// 1024^2 warp GN 4 x 20 2.10 against 2.06 ms, 64^2 0.33 against 0.28, level-7 mesh
+// LM 2 x 30 1.35 against 1.20.  Sums that float32 cannot hold go on in float64 and are
+// handed on as pairs of 2^-64 of them (big).  Energies and the LM decision are float64.
+//
+// A total that comes out as no number is formed again in float64 from what it was the
+// total of; a block's sum that float32 cannot hold is stored as kOver with 2^-64 of it
+// beside (nothing else of an ordinary sum is checked or carried).
+constexpr float kOver = __builtin_huge_valf();
+__device__ __forceinline__ Sum sum_zero() { return Sum{0.f, 0.f, 0}; }
+__device__ __forceinline__ bool sum_finite(const Sum& a) { return isfinite(a.hi); }
+__device__ __forceinline__ double sum_double(const Sum& a) {
+  double d = (double)a.hi + (double)a.lo;
+  if (a.big) d *= 0x1p64;
+  return d;
+}
+__device__ __forceinline__ Sum sum_of(double v) {
+  const int big = !(fabs(v) < 0x1p100);
+  if (big) v *= 0x1p-64;
+  const float hi = (float)v;
+  return Sum{hi, isfinite(hi) ? (float)(v - (double)hi) : 0.f, big};
+}
+// (out of line: reached by no ordinary sum)
+static __device__ __noinline__ Sum lanes_total64(double v, int hi, int lo) {
+  for (int o = hi / 2; o >= lo; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return sum_of(v);
+}
+static __device__ __noinline__ float sum_quot64(Sum a, Sum b) { return (float)(sum_double(a) / sum_double(b)); }
 __device__ __forceinline__ F2 f2_shfl_xor_add(F2 v, int o) {
   F2 w;
   w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
@@ -515,28 +547,25 @@ __device__ __forceinline__ F2 f2_shfl_xor_add(F2 v, int o) {
   f2_add_f2(v, w);
   return v;
 }
-__device__ __forceinline__ F2 f2_from_double(double d) {
-  const float hi = (float)d;
-  return F2{hi, isfinite(hi) ? (float)(d - (double)hi) : 0.f};
-}
-// a / b rounded to float32 (one correction step: the quotient of the leading
-// parts plus the remainder's; as the rounded float64 quotient unless that lies
-// within 2^-20 ulp of a rounding boundary)
-__device__ __forceinline__ float f2_quot(F2 a, F2 b) {
+// a / b rounded to float32: the quotient of the leading parts plus the remainder's, as the
+// rounded float64 quotient unless that lies within 2^-20 of a last place of a rounding
+// boundary; where an intermediate could leave float32's range, the float64 quotient.
+__device__ __forceinline__ float sum_quot(const Sum& a, const Sum& b) {
   const float q = __fdiv_rn(a.hi, b.hi);
   const float r = __fadd_rn(__fmaf_rn(-q, b.hi, a.hi), __fmaf_rn(-q, b.lo, a.lo));
   const float c = __fadd_rn(q, __fdiv_rn(r, b.hi));
-  return isfinite(c) ? c : q;
+  const bool mid = !(a.big | b.big) && fminf(fabsf(a.hi), fabsf(b.hi)) > 0x1p-90f && isfinite(c);
+  return mid ? c : sum_quot64(a, b);
 }
 
-// Stores this chunk's N partial pairs (N = 1: every other 8-byte slot of part, N =
-// 4: all) and reports whether this block is the last of its problem to do so.
-// Must be called by every thread of the block.
+// Stores this chunk's N sums in part (16 bytes of it each: a pair, and the pair of 2^-64 of
+// it where that is kOver; N = 4: the pairs of all four first) and reports whether this
+// block is the last of its problem to do so.  Must be called by every thread of the block.
 template <int N>
-__device__ __forceinline__ bool publish_pairs(double* part, int chunk, const F2 (&f)[N], unsigned int* counter,
-                                              unsigned int nchunks) {
+__device__ __forceinline__ bool publish_sums(double* part, int chunk, const F2 (&f)[N], unsigned int* counter,
+                                             unsigned int nchunks) {
   static_assert(NT == 256 && (N == 1 || N == 4), "one lane per warp and sum");
-  constexpr int NW = NT / 32, ST = N == 1 ? 2 : 4;
+  constexpr int NW = NT / 32;
   __shared__ F2 sw[N][NW];
   __shared__ int s_last;
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -550,8 +579,17 @@ __device__ __forceinline__ bool publish_pairs(double* part, int chunk, const F2 
     F2 v = l / NW < N ? sw[l / NW][l % NW] : f2_zero();
 #pragma unroll
     for (int o = NW / 2; o > 0; o >>= 1) v = f2_shfl_xor_add(v, o);
-    if (l / NW < N && l % NW == 0)
-      __stcg(reinterpret_cast<float2*>(part) + (long long)ST * chunk + l / NW, make_float2(v.hi, v.lo));
+    if (l / NW < N && l % NW == 0) {
+      float2* p = reinterpret_cast<float2*>(part) + (long long)2 * N * chunk + l / NW;
+      if (!isfinite(v.hi)) {
+        double d = 0.0;
+        for (int j = 0; j < NW; ++j) d += f2_to_double(sw[l / NW][j]);
+        d *= 0x1p-64;
+        __stcg(p + N, make_float2((float)d, (float)(d - (double)(float)d)));
+        v = F2{kOver, 0.f};
+      }
+      __stcg(p, make_float2(v.hi, v.lo));
+    }
     __syncwarp();
     if (l == 0) {
       __threadfence();
@@ -563,11 +601,23 @@ __device__ __forceinline__ bool publish_pairs(double* part, int chunk, const F2 
   return s_last != 0;
 }
 
+// Sum k of the chunks in float64, by a warp.
+template <int N>
+static __device__ __noinline__ Sum gather64(const double* part, int cb, int ce, int k) {
+  const float2* p = reinterpret_cast<const float2*>(part) + k;
+  double d = 0.0;
+  for (int c = cb + ((int)threadIdx.x & 31); c < ce; c += 32) {
+    const float2 t = __ldcg(p + (long long)2 * N * c), u = __ldcg(p + (long long)2 * N * c + N);
+    d += t.x == kOver ? ((double)u.x + (double)u.y) * 0x1p64 : (double)t.x + (double)t.y;
+  }
+  return lanes_total64(d, 32, 1);
+}
+
 // In the last block: the sums over chunks [cb, ce) (thread-strided in chunk
 // order, then a fixed tree); out is valid in thread 0; resets the counter.
 template <int N>
-__device__ __forceinline__ void gather_pairs(const double* part, int cb, int ce, unsigned int* counter, F2 (&out)[N]) {
-  constexpr int NW = NT / 32, ST = N == 1 ? 2 : 4;
+__device__ __forceinline__ void gather_sums(const double* part, int cb, int ce, unsigned int* counter, Sum (&out)[N]) {
+  constexpr int NW = NT / 32;
   __shared__ F2 g[N][NW];
   __threadfence();
   const float2* p = reinterpret_cast<const float2*>(part);
@@ -575,7 +625,7 @@ __device__ __forceinline__ void gather_pairs(const double* part, int cb, int ce,
   F2 v = f2_zero();
 #pragma unroll 4
   for (int c = cb + (int)threadIdx.x / N; c < ce; c += NT / N) {
-    const float2 t = __ldcg(p + (long long)ST * c + k);
+    const float2 t = __ldcg(p + (long long)2 * N * c + k);
     f2_add_f2(v, F2{t.x, t.y});
   }
 #pragma unroll
@@ -589,8 +639,8 @@ __device__ __forceinline__ void gather_pairs(const double* part, int cb, int ce,
     for (int o = NW / 2; o > 0; o >>= 1) t = f2_shfl_xor_add(t, o);
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-      out[j].hi = __shfl_sync(0xffffffffu, t.hi, j * NW);
-      out[j].lo = __shfl_sync(0xffffffffu, t.lo, j * NW);
+      out[j] = Sum{__shfl_sync(0xffffffffu, t.hi, j * NW), __shfl_sync(0xffffffffu, t.lo, j * NW), 0};
+      if (!sum_finite(out[j])) out[j] = gather64<N>(part, cb, ce, j);
     }
     if (l == 0) *counter = 0u;
   }
@@ -598,32 +648,32 @@ __device__ __forceinline__ void gather_pairs(const double* part, int cb, int ce,
 
 // alpha from the sum p.q of the last block (thread 0); p.q <= 0 or not finite
 // ends the loop.
-__device__ __forceinline__ void finish_alpha(Scalars* s, F2 pq) {
-  s->pq = f2_to_double(pq);
-  if (pq.hi > 0.f && isfinite(pq.hi)) {
-    s->alpha_f = f2_quot(F2{s->rz_hi, s->rz_lo}, pq);
+__device__ __forceinline__ void finish_alpha(Scalars* s, const Sum& pq) {
+  s->pq = sum_double(pq);
+  if (pq.hi > 0.f && sum_finite(pq)) {
+    s->alpha_f = sum_quot(s->rz_sum, pq);
   } else {
     s->alpha_f = 0.f;
     s->pcg_active = 0;
-    if (!isfinite(pq.hi)) s->nonfinite = 1;
+    if (!sum_finite(pq)) s->nonfinite = 1;
   }
 }
-// beta from the next r.z (thread 0 of the last block of a vector update)
-__device__ __forceinline__ void finish_beta(Scalars* s, F2 rz) {
-  s->beta_f = f2_quot(rz, F2{s->rz_hi, s->rz_lo});
-  s->rz = f2_to_double(rz);
-  s->rz_hi = rz.hi;
-  s->rz_lo = rz.lo;
-  s->pcg_iters += 1;
-  if (rz.hi == 0.f || !isfinite(rz.hi)) s->pcg_active = 0;
-  if (!isfinite(rz.hi)) s->nonfinite = 1;
+__device__ __forceinline__ void set_rz(Scalars* s, const Sum& rz) {
+  s->rz = sum_double(rz);
+  s->rz_sum = rz;
 }
 // r.z of PCGInit
 __device__ __forceinline__ void set_rz(Scalars* s, double rz) {
-  const F2 t = f2_from_double(rz);
   s->rz = rz;
-  s->rz_hi = t.hi;
-  s->rz_lo = t.lo;
+  s->rz_sum = sum_of(rz);
+}
+// beta from the next r.z (thread 0 of the last block of a vector update)
+__device__ __forceinline__ void finish_beta(Scalars* s, const Sum& rz) {
+  s->beta_f = sum_quot(rz, s->rz_sum);
+  set_rz(s, rz);
+  s->pcg_iters += 1;
+  if (rz.hi == 0.f || !sum_finite(rz)) s->pcg_active = 0;
+  if (!sum_finite(rz)) s->nonfinite = 1;
 }
 
 __device__ __forceinline__ bool finite_d(double v) { return isfinite(v); }

@@ -85,6 +85,33 @@ __device__ __forceinline__ unsigned long long pack(F2 a) {
 __device__ __forceinline__ F2 unpack(unsigned long long b) {
   return F2{__uint_as_float((unsigned)b), __uint_as_float((unsigned)(b >> 32))};
 }
+// A block's sum in its slot: two words that each carry the sum's number, so that each
+// says by itself whether it is there.
+__device__ __forceinline__ void st_slot(unsigned long long* p, F2 s, unsigned k) {
+  const unsigned long long tag = (unsigned long long)k << 32;
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(tag | __float_as_uint(s.hi)),
+               "l"(tag | __float_as_uint(s.lo))
+               : "memory");
+}
+__device__ __forceinline__ bool ld_slot(const unsigned long long* p, unsigned k, F2& s) {
+  unsigned long long a, b;
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+  s = F2{__uint_as_float((unsigned)a), __uint_as_float((unsigned)b)};
+  return (unsigned)(a >> 32) == k && (unsigned)(b >> 32) == k;
+}
+// 2^-64 of a block's sum that float32 cannot hold, by a whole warp (sw: its warps' pairs)
+static __device__ __noinline__ F2 block_total64(const F2* sw) {
+  const int l = threadIdx.x & 31;
+  const double d = [&] {
+    double v = l < RW ? f2_to_double(sw[l]) : 0.0;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v * 0x1p-64;
+  }();
+  return F2{(float)d, (float)(d - (double)(float)d)};
+}
+__device__ __forceinline__ double over_double(F2 v, F2 over) {
+  return v.hi == kOver ? f2_to_double(over) * 0x1p64 : f2_to_double(v);
+}
 
 // Meeting of all blocks: what any thread wrote to global memory before is
 // visible to every thread of every block after.  Returns false if a block did
@@ -102,68 +129,96 @@ __device__ __forceinline__ bool meet(Meet& M) {
 // every block.  FENCE: global writes are ordered too (a cluster's barrier always
 // does).
 template <bool CL, bool FENCE>
-__device__ __forceinline__ bool meet_sum(Meet& M, F2 acc, F2& total) {
-  __shared__ unsigned long long sw[RW];
+__device__ __forceinline__ bool meet_sum(Meet& M, F2 acc, Sum& total) {
+  __shared__ F2 sw[RW];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   acc = warp_sum_f2(acc);
-  if (l == 0) sw[w] = pack(acc);
+  if (l == 0) sw[w] = acc;
   __syncthreads();
   auto block_total = [&] {
-    F2 v = unpack(sw[l % RW]);
+    F2 v = sw[l % RW];
 #pragma unroll
     for (int o = RW / 2; o > 0; o >>= 1) v = f2_shfl_xor_add(v, o);
     return v;
   };
   M.sums += 1;
-  const unsigned k = M.sums;
+  const unsigned k = M.sums, n = gridDim.x;
   if (CL) {
-    __shared__ unsigned long long part[2][RES_CLUSTER];
-    const unsigned n = gridDim.x;
+    __shared__ unsigned long long part[2][RES_CLUSTER], over[2][RES_CLUSTER];
     if (w == 0) {
-      const F2 v = block_total();
+      F2 v = block_total();
+      if (!isfinite(v.hi)) {
+        const F2 o = block_total64(sw);
+        if (l < n) st_cluster(&over[k & 1][cluster_rank()], l, pack(o));
+        v = F2{kOver, 0.f};
+      }
       if (l < n) st_cluster(&part[k & 1][cluster_rank()], l, pack(v));
       __syncwarp();
     }
     cluster_meet();
-    total = l % RES_CLUSTER < n ? unpack(part[k & 1][l % RES_CLUSTER]) : f2_zero();
+    const int j = l % RES_CLUSTER;
+    F2 t = j < n ? unpack(part[k & 1][j]) : f2_zero();
 #pragma unroll
-    for (int o = RES_CLUSTER / 2; o > 0; o >>= 1) total = f2_shfl_xor_add(total, o);
+    for (int o = RES_CLUSTER / 2; o > 0; o >>= 1) t = f2_shfl_xor_add(t, o);
+    total = Sum{t.hi, t.lo, 0};
+    if (!sum_finite(total))
+      total = lanes_total64(l < n ? over_double(unpack(part[k & 1][l]), unpack(over[k & 1][l])) : 0.0, 32, 1);
     return true;
   } else {
-    constexpr int NP = RES_MAX_BLOCKS / 32;      // polling warps, one slot a thread
-    __shared__ unsigned long long sg[NP];
+    constexpr int NP = RES_MAX_BLOCKS / 32;       // polling warps, one slot a thread
+    __shared__ F2 sg[NP], so[NP];
     __shared__ int s_ok[NP];
+    unsigned long long (*const slot)[16] = M.sy->slot[k & 1];
     if (w == 0) {
-      const F2 v = block_total();
+      F2 v = block_total();
+      if (!isfinite(v.hi)) {
+        const F2 o = block_total64(sw);
+        if (l == 0) st_slot(&slot[blockIdx.x][2], o, k);
+        v = F2{kOver, 0.f};
+      }
       if (FENCE) __threadfence();
-      if (l == 0)
-        st_relaxed(&M.sy->slot[k & 1][blockIdx.x][0],
-                   (pack(v) & ~(3ull << 32)) | ((unsigned long long)(k & 3) << 32));
+      if (l == 0) st_slot(slot[blockIdx.x], v, k);
     }
     if (w < NP) {
-      const bool on = threadIdx.x < gridDim.x;
-      const unsigned long long* p = &M.sy->slot[k & 1][on ? threadIdx.x : 0][0];
-      unsigned long long b, t0 = 0;
+      const bool on = threadIdx.x < n;
+      const unsigned long long* p = slot[on ? threadIdx.x : 0];
+      F2 v;
+      unsigned long long t0 = 0;
       int ok = 1;
-      for (int spin = 0; (((b = ld_relaxed(p)) >> 32) & 3) != (k & 3) && ok; ++spin)
-        ok = !waited_too_long(spin, t0, M.limit);
+      for (int spin = 0; !ld_slot(p, k, v) && ok; ++spin) ok = !waited_too_long(spin, t0, M.limit);
       if (FENCE) __threadfence();
       ok = __all_sync(0xffffffffu, ok);
-      const F2 v = warp_sum_f2(on ? unpack(b & ~(3ull << 32)) : f2_zero());
+      F2 t = warp_sum_f2(on ? v : f2_zero());
+      if (!isfinite(__shfl_sync(0xffffffffu, t.hi, 0))) {
+        // a kOver among them, or too much in all: 2^-64 of the float64 sum beside kOver
+        F2 o = f2_zero();
+        t0 = 0;
+        int there = 1;
+        if (on && v.hi == kOver)
+          for (int spin = 0; !ld_slot(p + 2, k, o) && there; ++spin) there = !waited_too_long(spin, t0, M.limit);
+        ok = __all_sync(0xffffffffu, there) && ok;
+        double d = on ? over_double(v, o) : 0.0;
+        for (int b = 16; b > 0; b >>= 1) d += __shfl_xor_sync(0xffffffffu, d, b);
+        d *= 0x1p-64;
+        if (l == 0) so[w] = F2{(float)d, (float)(d - (double)(float)d)};
+        t = F2{kOver, 0.f};
+      }
       if (l == 0) {
-        sg[w] = pack(v);
+        sg[w] = t;
         s_ok[w] = ok;
       }
     }
     __syncthreads();
-    total = unpack(sg[0]);
+    M.limit = M.later;
+    F2 t = sg[0];
     int ok = s_ok[0];
 #pragma unroll
-    for (int t = 1; t < NP; ++t) {
-      f2_add_f2(total, unpack(sg[t]));
-      ok &= s_ok[t];
+    for (int j = 1; j < NP; ++j) {
+      f2_add_f2(t, sg[j]);
+      ok &= s_ok[j];
     }
-    M.limit = M.later;
+    total = Sum{t.hi, t.lo, 0};
+    if (!sum_finite(total)) total = lanes_total64(l < NP ? over_double(sg[l], so[l]) : 0.0, 32, 1);
     return ok != 0;
   }
 }
@@ -835,7 +890,7 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
       }
     }
   }
-  F2 rz = F2{s->rz_hi, s->rz_lo}, pq = f2_zero();   // the same values in every thread
+  Sum rz = s->rz_sum, pq = sum_zero();        // the same values in every thread
   int iters = 0, nonfinite = 0, active = 1;
   float alpha = 0.f, beta = 0.f;
   bool met = meet<CL>(M);
@@ -934,13 +989,13 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
       }
     }
     if (!(met = meet_sum<CL, false>(M, acc, pq))) break;
-    if (!(pq.hi > 0.f && isfinite(pq.hi))) {  // breakdown
+    if (!(pq.hi > 0.f && sum_finite(pq))) {   // breakdown
       alpha = 0.f;
       active = 0;
-      nonfinite = !isfinite(pq.hi);
+      nonfinite = !sum_finite(pq);
       break;
     }
-    alpha = f2_quot(rz, pq);
+    alpha = sum_quot(rz, pq);
     // delta += alpha p, r -= alpha q, r.z -> beta
     acc = f2_zero();
     for (int j = tid; j < cnt; j += RT) {
@@ -959,15 +1014,15 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
       }
       if (zrec) put_z(j, z);
     }
-    F2 rz2 = f2_zero();
+    Sum rz2 = sum_zero();
     met = zrec ? meet_sum<CL, true>(M, acc, rz2) : meet_sum<CL, false>(M, acc, rz2);
     if (!met) break;
     iters += 1;
-    beta = f2_quot(rz2, rz);
+    beta = sum_quot(rz2, rz);
     rz = rz2;
-    if (rz.hi == 0.f || !isfinite(rz.hi)) {
+    if (rz.hi == 0.f || !sum_finite(rz)) {
       active = 0;
-      nonfinite = !isfinite(rz.hi);
+      nonfinite = !sum_finite(rz);
       break;
     }
   }
@@ -1001,10 +1056,9 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
     }
   }
   if (blockIdx.x == 0 && tid == 0) {
-    s->rz = f2_to_double(rz);
-    s->rz_hi = rz.hi;
-    s->rz_lo = rz.lo;
-    s->pq = f2_to_double(pq);
+    s->rz = sum_double(rz);
+    s->rz_sum = rz;
+    s->pq = sum_double(pq);
     s->alpha_f = alpha;
     s->beta_f = beta;
     s->pcg_iters += iters;
@@ -1028,15 +1082,15 @@ __global__ void __launch_bounds__(RT, 1) k_exchange_selftest(ResidentSync* sync,
       continue;
     }
     const F2 mine = {(float)r, 0.f};
-    F2 total = f2_zero();
+    Sum total = sum_zero();
     met = r & 1 ? meet_sum<false, true>(M, mine, total) : meet_sum<false, false>(M, mine, total);
-    if (met && f2_to_double(total) != (double)r * RT * gridDim.x) out[1] = 1;
+    if (met && sum_double(total) != (double)r * RT * gridDim.x) out[1] = 1;
   }
   if (threadIdx.x != 0) return;
   if (!met) out[0] = 1;
   if (met && blockIdx.x == 0) {
     sync->meetings = M.base + M.meetings * gridDim.x;
-    sync->sums = M.sums & 3u;
+    sync->sums = M.sums;
   }
 }
 
