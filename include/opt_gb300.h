@@ -644,6 +644,10 @@ opt_status opt_selftest_staging_wait(int32_t complete, int32_t* timed_out);
  * outside [1, 1000] or a NULL pointer. */
 opt_status opt_selftest_resident_exchange(int32_t kind, int32_t absent, int32_t rounds, int32_t* timed_out);
 
+/* Self-test: the next device allocation of a float32 problem on this host thread is
+ * refused, as when memory has run out. */
+opt_status opt_selftest_refuse_allocation(void);
+
 /* Self-test: in the next solve of this problem that runs the on-chip loop over the device,
  * one block does not take part, the others give up after 50 ms and the solve returns
  * OPT_ERR_TIMEOUT; solves after it are normal.  Synchronous.  OPT_ERR_INVALID_ARG before

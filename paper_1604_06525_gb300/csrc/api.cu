@@ -178,7 +178,12 @@ cudaMemPool_t problem_pool() {
 // stream; planning ends with a synchronising copy before any other stream
 // touches it).  The many small ones of a plan share slabs.
 constexpr size_t kSlabBytes = 128 << 10, kSlabShare = 16 << 10;
+thread_local bool g_refuse_alloc = false;   // self-test: the next allocation is refused
 opt_status dalloc_bytes(opt_problem* pb, void** ptr, size_t bytes) {
+  if (g_refuse_alloc) {
+    g_refuse_alloc = false;
+    return cuda_fail(cudaErrorMemoryAllocation, "device allocation");
+  }
   cudaMemPool_t pool = problem_pool();
   cudaError_t e = pool ? cudaMallocFromPoolAsync(ptr, bytes, pool, nullptr) : cudaMalloc(ptr, bytes);
   if (e != cudaSuccess) return cuda_fail(e, "device allocation");
@@ -553,33 +558,68 @@ bool use_fused(const opt_problem* pb, const opt_solve_params& p) {
          pb->hg.zb != nullptr;
 }
 
-// Plans the resident PCG loop of a GN (lm = 0) / LM solve and allocates its
-// slots and records once (outside any capture).
-opt_status resident_prepare(opt_problem* pb, int lm) {
-  if (pb->rplanned[lm]) return OPT_OK;
-  const bool grid = is_grid(pb);
-  ResidentPlan rp;
-  if (grid) {
-    const long long n = (long long)pb->h_cells.size() * TW * TH;
-    // (records are indexed like the planes: a sparse mask on a huge image is left to the tiled kernels)
-    rp = n > (1 << 22) || pb->plane > (1 << 24) ? ResidentPlan{} : resident_plan(pb->kind, (int)n, pb->plane, lm, nullptr);
-  } else {
-    rp = resident_plan(pb->kind, pb->V, pb->plane, lm, pb->kind != K_VOLUME && pb->hm.sym ? pb->h_orow.data() : nullptr);
-  }
-  if (rp.blocks > 0) {
-    if (!pb->d_rsync) {
-      CKS(dalloc(pb, &pb->d_rsync, 1));
-      CKS(reset_exchange(pb->d_rsync, nullptr));
+// What the resident loop of the planned kinds of solve needs on the device.
+opt_status resident_alloc(opt_problem* pb) {
+  long long recs = 0;
+  for (const ResidentPlan& rp : pb->rplan)
+    if (rp.blocks > 0) recs = std::max(recs, rp.recs);
+  if (recs == 0) return OPT_OK;
+  CKS(dalloc(pb, &pb->d_rrec, resident_records(pb->kind, recs)));
+  CKS(dalloc(pb, &pb->d_rsync, 1));
+  CKS(reset_exchange(pb->d_rsync, nullptr));
+  if (is_grid(pb)) {
+    // cells ascend, so a cell's neighbours in its row are the next to it
+    const std::vector<int>& cells = pb->h_cells;
+    const int n = (int)cells.size();
+    std::vector<int4> at((size_t)n);
+    int first = 0;
+    for (int end = 0; first < n; first = end) {
+      while (end < n && cells[end] >> 16 == cells[first] >> 16) ++end;
+      for (int k = first; k < end; ++k)
+        at[k] = make_int4(first * TW * TH + (k - first) * TW, (end - first) * TW, 0, 0);
     }
-    if (grid && !pb->d_cells) {
-      CKS(dalloc(pb, &pb->d_cells, pb->h_cells.size()));
-      CKS(upload(pb->d_cells, pb->h_cells));
+    for (int k = 0, below = 0; k < n; ++k) {
+      while (below < n && cells[below] < cells[k] + (1 << 16)) ++below;
+      if (below == n || cells[below] != cells[k] + (1 << 16)) continue;
+      at[k].w = at[below].x;
+      at[below].z = at[k].x + (TH - 1) * at[k].y;
     }
-    if (!pb->d_rrec) CKS(dalloc(pb, &pb->d_rrec, resident_records(pb->kind, pb->plane)));
-    CK(cudaStreamSynchronize(nullptr));
+    Uploads up;
+    CKS(dalloc(pb, &pb->d_cells, cells.size()));
+    up.add(pb->d_cells, cells);
+    CKS(dalloc(pb, &pb->d_places, at.size()));
+    up.add(pb->d_places, at);
+    CKS(up.flush());
   }
-  pb->rplan[lm] = rp;
-  pb->rplanned[lm] = true;
+  CK(cudaStreamSynchronize(nullptr));
+  return OPT_OK;
+}
+
+// Plans the resident PCG loops of a GN and an LM solve and allocates their slots and
+// records once (outside any capture).  Where there is no memory for them, solves take
+// the launches.
+opt_status resident_prepare(opt_problem* pb) {
+  if (pb->rplanned) return OPT_OK;
+  for (int lm = 0; lm < 2; ++lm) {
+    if (is_grid(pb)) {
+      const long long n = (long long)pb->h_cells.size() * TW * TH;
+      // (nothing above 2^24 pixels has been measured on chip)
+      if (n <= (1 << 22) && pb->plane <= (1 << 24))
+        pb->rplan[lm] = resident_plan(pb->kind, (int)n, pb->plane, lm, nullptr);
+    } else {
+      pb->rplan[lm] = resident_plan(pb->kind, pb->V, pb->plane, lm,
+                                    pb->kind != K_VOLUME && pb->hm.sym ? pb->h_orow.data() : nullptr);
+    }
+  }
+  const std::string before = g_err;
+  const opt_status s = resident_alloc(pb);
+  if (s == OPT_ERR_OOM) {
+    g_err = before;
+    for (ResidentPlan& rp : pb->rplan) rp = ResidentPlan{};
+  } else if (s != OPT_OK) {
+    return s;
+  }
+  pb->rplanned = true;
   return OPT_OK;
 }
 
@@ -614,7 +654,7 @@ opt_status enqueue_solve(opt_problem* pb, const opt_solve_params& p, bool lm, cu
       CK(launch_grid_pcg_coop(grid_launch(pb, st), pb->d_gbar, 0, p.inner));
     } else if (resident) {
       const ResidentPlan& rp = pb->rplan[lm ? 1 : 0];
-      CK(is_grid(pb) ? launch_resident_grid(pb->kind, pb->dg, pb->d_cells, pb->d_rsync, rp, pb->d_rrec, p.inner,
+      CK(is_grid(pb) ? launch_resident_grid(pb->kind, pb->dg, pb->d_cells, pb->d_places, pb->d_rsync, rp, pb->d_rrec, p.inner,
                                             lm ? 0 : 1, csn_next, st)
                      : launch_resident_graph(pb->kind, pb->dm, pb->d_rsync, rp, pb->d_rrec, p.inner, lm ? 0 : 1, st));
     } else {
@@ -684,7 +724,7 @@ opt_status run_solve(opt_problem* pb, const opt_solve_params* prm_in, opt_report
   // descriptor's copy and one of two result copies less: about 25 us of every solve
   // (64^2 warp GN 4 x 10 295 -> 272 us; 28 x 108 mesh LM 1 x 7 174 -> 149 us).
   CKS(ensure_ehist(pb, p.outer + 1));
-  CKS(resident_prepare(pb, lm ? 1 : 0));
+  CKS(resident_prepare(pb));
   set_flags(pb, lm ? 1 : 0, p.use_precond, pb->d_Ehist);
   if (p.materialized || !desc_sent(pb)) {
     CK(cudaStreamSynchronize(st));
@@ -923,6 +963,11 @@ opt_status opt_selftest_resident_exchange(int32_t kind, int32_t absent, int32_t 
   }
   *timed_out = h[0];
   return h[1] ? OPT_ERR_NUMERIC : OPT_OK;
+}
+
+opt_status opt_selftest_refuse_allocation(void) {
+  g_refuse_alloc = true;
+  return OPT_OK;
 }
 
 opt_status opt_selftest_lose_block(opt_problem* prob) {

@@ -314,6 +314,7 @@ struct ResidentPlan {
   int slots;                    // graphs: table entries for edges that leave a block (0: no table)
   int lanes;                    // graphs: threads per vertex
   long long plane;              // plane stride
+  long long recs;               // direction records of one buffer (grids: one per unit, graphs: per plane element)
 };
 
 // ---------------------------------------------------------------------------

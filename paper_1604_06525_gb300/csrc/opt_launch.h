@@ -86,12 +86,13 @@ cudaError_t launch_barrier_selftest(GridBarrier* gb, int nblocks, unsigned int e
 
 // resident.cu: the PCG loop of one outer iteration in one launch with the state
 // on chip.  orow (graphs; NULL for voxel grids): host copy of the CSR rows.
-// cells (grids): the 32 x 8 pixel cells with an unknown, (row << 16) | column.
+// cells (grids): the 32 x 8 pixel cells with an unknown, (row << 16) | column, ascending;
+// places: of each cell, GridCtx::cell (resident.cu).
 // rec: resident_records() float4.  step: x += delta at the end (Gauss-Newton);
 // csn_out (wide warps): also cos / sin of the new theta.
 ResidentPlan resident_plan(int kind, int n, long long plane, int lm, const int* orow);
-size_t resident_records(int kind, long long plane);
-cudaError_t launch_resident_grid(int kind, const GridProb* probs, const int* cells, ResidentSync* sync,
+size_t resident_records(int kind, long long recs);
+cudaError_t launch_resident_grid(int kind, const GridProb* probs, const int* cells, const int4* places, ResidentSync* sync,
                                  const ResidentPlan& rp, float4* rec, int inner, int step, int csn_out,
                                  cudaStream_t st);
 cudaError_t launch_resident_graph(int kind, const MeshProb* probs, ResidentSync* sync, const ResidentPlan& rp,

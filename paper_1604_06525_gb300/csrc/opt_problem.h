@@ -71,7 +71,8 @@ struct opt_problem {
   // host mirrors of the work tables (batches build their combined tables from these)
   std::vector<int> h_tiles;
   std::vector<int> h_cells;             // 32 x 8 pixel cells holding an unmasked / free pixel
-  int* d_cells = nullptr;               // on the device where the resident loop may run
+  int* d_cells = nullptr;               // on the device where the resident loop may run,
+  int4* d_places = nullptr;             //   with where its and its neighbours' records are
   std::vector<optgb::Chunk> h_chunks, h_vch, h_ech, h_tch;
   // host copies kept for building the materialized Jacobian
   std::vector<unsigned char> h_mask;    // grid mask (empty = none)
@@ -109,10 +110,10 @@ struct opt_problem {
   // blocks that can be resident at once (0 = not available)
   optgb::GridBarrier* d_gbar = nullptr;
   int coop_cap = 0;
-  // resident PCG loop: plans of a GN and an LM solve (made at the first solve
-  // that may take it), exchange slots, direction records
+  // resident PCG loop: plans of a GN and an LM solve (made at the first solve),
+  // exchange slots, direction records
   optgb::ResidentPlan rplan[2] = {};
-  bool rplanned[2] = {false, false};
+  bool rplanned = false;
   optgb::ResidentSync* d_rsync = nullptr;
   float4* d_rrec = nullptr;
   cudaStream_t cap_stream = nullptr;
@@ -134,7 +135,7 @@ struct opt_problem {
     swap(nvchunks, o.nvchunks); swap(nechunks, o.nechunks); swap(d_tchunks, o.d_tchunks);
     swap(ntchunks, o.ntchunks); swap(tileable, o.tileable); swap(apply_form, o.apply_form); swap(chunking, o.chunking);
     swap(tile_w, o.tile_w); swap(has_grid_desc, o.has_grid_desc); swap(grid_desc, o.grid_desc);
-    swap(h_tiles, o.h_tiles); swap(h_cells, o.h_cells); swap(d_cells, o.d_cells); swap(h_chunks, o.h_chunks); swap(h_vch, o.h_vch); swap(h_ech, o.h_ech);
+    swap(h_tiles, o.h_tiles); swap(h_cells, o.h_cells); swap(d_cells, o.d_cells); swap(d_places, o.d_places); swap(h_chunks, o.h_chunks); swap(h_vch, o.h_vch); swap(h_ech, o.h_ech);
     swap(h_tch, o.h_tch);
     swap(h_mask, o.h_mask); swap(h_hpix, o.h_hpix); swap(h_e0, o.h_e0); swap(h_e1, o.h_e1); swap(h_orow, o.h_orow);
     swap(d_perm, o.d_perm); swap(csr, o.csr);

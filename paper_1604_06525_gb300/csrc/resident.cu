@@ -226,7 +226,10 @@ __device__ __forceinline__ bool meet_sum(Meet& M, F2 acc, Sum& total) {
 // ---------------------------------------------------------------------------
 // direction records
 // ---------------------------------------------------------------------------
-// NR float4 per pixel / vertex, in rec: two buffers of p and one of z = M^-1 r.
+// NR float4 per pixel / vertex, in rec: two buffers of p and one of z = M^-1 r.  Grids keep
+// them for the listed cells only, so that they take what the free pixels need and not what
+// the image does (a 4000^2 image would hold 770 MB): row by row of cells, and within one
+// the pixels row by row, as in the image without its other cells.
 // With RES_Z a neighbour forms the new direction itself, p = z + beta p_old, from
 // the z published before the exchange that yields beta: one exchange fewer per
 // iteration for twice the records read.  Without, p is published in a phase of
@@ -265,9 +268,13 @@ __device__ __forceinline__ float4 load_rec(const Records& R, long long k) {
 struct GridCtx {
   const GridProb& pr;
   const int* cells;
-  float2* csn;          // warp: cos / sin of theta, index y * P + x
-  int* idx;             // shared: plane index of each unit
+  int u0;
+  float4* geo;          // warp: cos / sin of theta and UrShape, by record
+  int* idx;             // shared: record of each unit
   int* flg;             // shared: neighbour flags of each unit
+  // shared, of each of the block's cells: the record of its first pixel, the records of a
+  // row of pixels, the first pixel's of the last row of the cell above and of the cell below
+  const int4* cell;
 };
 
 struct GridUnits {
@@ -282,7 +289,24 @@ struct GridUnits {
     y = (cc >> 16) * TH + (t >> 5);
     return x < pr.W && y < pr.H;
   }
-  static __device__ __forceinline__ int index(const GridCtx& c, int j) { return c.idx[j]; }
+  static __device__ __forceinline__ int record(const GridCtx& c, int j) {
+    const int4 ci = c.cell[j / CELL];
+    return ci.x + (j % CELL) / TW * ci.y + j % TW;
+  }
+  static __device__ __forceinline__ int index(const GridCtx& c, int j) {
+    int x, y;
+    locate(c, c.u0 + j, x, y);
+    return y * c.pr.P + x;
+  }
+  // the records left, right, above and below of unit j's
+  static __device__ __forceinline__ void near_records(const GridCtx& c, int j, int (&n)[4]) {
+    const int4 ci = c.cell[j / CELL];
+    const int i = c.idx[j], t = j % CELL;
+    n[0] = i - 1;
+    n[1] = i + 1;
+    n[2] = t >= TW ? i - ci.y : ci.z + t;
+    n[3] = t < CELL - TW ? i + ci.y : ci.w + t % TW;
+  }
 };
 
 struct WarpKind : GridUnits {
@@ -308,7 +332,7 @@ struct WarpKind : GridUnits {
     const int t = (y / TH) * pr.ntx + x / pr.tw;
     for (int h = pr.hbeg[t]; h < pr.hbeg[t + 1]; ++h)
       if (pr.hpix[h] == i) f |= 32;
-    c.idx[j] = i;
+    c.idx[j] = record(c, j);
     c.flg[j] = f;
     float cs, sn;
     if (pr.csn) {
@@ -317,27 +341,28 @@ struct WarpKind : GridUnits {
     } else {
       sincosf(pr.x[2 * pr.plane + i], &sn, &cs);
     }
-    c.csn[i] = make_float2(cs, sn);
+    c.geo[c.idx[j]] = make_float4(cs, sn, __ldg(pr.c + i), __ldg(pr.c + pr.plane + i));
     return true;
   }
   static __device__ __forceinline__ void publish(const GridCtx& c, int j, const float (&p)[NX], float4* dst) {
     dst[c.idx[j]] = make_float4(p[0], p[1], p[2], 0.f);
   }
   static __device__ __forceinline__ WarpPix pix(const GridCtx& c, const float4& p, int i) {
-    const float2 cs = c.csn[i];
-    return WarpPix{p.x, p.y, p.z, cs.x, cs.y, __ldg(c.pr.c + i), __ldg(c.pr.c + c.pr.plane + i)};
+    const float4 g = c.geo[i];
+    return WarpPix{p.x, p.y, p.z, g.x, g.y, g.z, g.w};
   }
   struct Near {
     WarpPix o, n[4];
   };
   static __device__ __forceinline__ void fetch(const GridCtx& c, int j, const Records& R, Near& N) {
     const int i = c.idx[j], f = c.flg[j];
-    const int off[4] = {-1, 1, -c.pr.P, c.pr.P};
+    int in[4];
+    near_records(c, j, in);
     N.o = pix(c, make_float4(0.f, 0.f, 0.f, 0.f), i);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const int in = (f >> k) & 1 ? i + off[k] : i;
-      N.n[k] = pix(c, load_rec(R, in), in);
+      const int n = (f >> k) & 1 ? in[k] : i;
+      N.n[k] = pix(c, load_rec(R, n), n);
     }
   }
   static __device__ __forceinline__ void rows(const GridCtx& c, int j, const float (&p)[NX], Near& N, float (&q)[NX]) {
@@ -370,10 +395,7 @@ struct PoissonKind : GridUnits {
     if (!locate(c, u, x, y)) return false;
     const int i = y * pr.P + x;
     const uint8_t* mk = pr.mask;
-    if (mk && mk[i]) {                    // fixed: no unknown
-      c.idx[j] = -2 - i;
-      return false;
-    }
+    if (mk && mk[i]) return false;        // fixed: no unknown
     int f = 0, S = 0;
     auto nb = [&](bool in, int o, int bit) {
       if (!in) return;
@@ -385,7 +407,7 @@ struct PoissonKind : GridUnits {
     nb(x + 1 < pr.W, 1, 2);
     nb(y > 0, -pr.P, 4);
     nb(y + 1 < pr.H, pr.P, 8);
-    c.idx[j] = i;
+    c.idx[j] = record(c, j);
     c.flg[j] = f | (S << 8);
     return true;
   }
@@ -396,10 +418,11 @@ struct PoissonKind : GridUnits {
     float4 n[4];
   };
   static __device__ __forceinline__ void fetch(const GridCtx& c, int j, const Records& R, Near& N) {
-    const int i = c.idx[j], f = c.flg[j];
-    const int off[4] = {-1, 1, -c.pr.P, c.pr.P};
+    const int f = c.flg[j];
+    int in[4];
+    near_records(c, j, in);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) N.n[k] = (f >> k) & 1 ? load_rec(R, i + off[k]) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = 0; k < 4; ++k) N.n[k] = (f >> k) & 1 ? load_rec(R, in[k]) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   static __device__ __forceinline__ void rows(const GridCtx& c, int j, const float (&p)[NX], Near& N, float (&q)[NX]) {
     const float S = (float)(c.flg[j] >> 8);
@@ -722,7 +745,8 @@ struct Lanes {
 
 template <class K, bool CL>
 __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* __restrict__ probs,
-                                                        const int* __restrict__ cells, ResidentSync* sync,
+                                                        const int* __restrict__ cells,
+                                                        const int4* __restrict__ places, ResidentSync* sync,
                                                         const ResidentPlan rp, float4* rec, int inner, int step,
                                                         int csn_out) {
   constexpr int NX = K::NX, NM = K::NM;
@@ -740,8 +764,8 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
   const long long pl = rp.plane;
   const bool zrec = (rp.flags & RES_Z) != 0, lm = pr.lm != 0;
   const float lam = lm ? s->lambda_f : 0.0f;
-  float4* const recp[2] = {rec, rec + (zrec ? K::NR * pl : 0)};
-  float4* const recz = rec + 2 * K::NR * pl;
+  float4* const recp[2] = {rec, rec + (zrec ? K::NR * rp.recs : 0)};
+  float4* const recz = rec + 2 * K::NR * rp.recs;
   float* cur = sh;
   auto take = [&](int words) { float* r = cur; cur += words; return r; };
   float* const sr = take(NX * cap);
@@ -812,7 +836,10 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
     } else {
       sp = take(NX * cap);
       idx = reinterpret_cast<int*>(take(cap));
-      return GridCtx{pr, cells, reinterpret_cast<float2*>(rec + 3 * pl), idx, flg};
+      int4* const cell = reinterpret_cast<int4*>(take(cap / CELL * 4));     // (16-byte aligned: cap is 256 k)
+      for (int k = tid; k < cnt / CELL; k += RT) cell[k] = places[u0 / CELL + k];
+      __syncthreads();
+      return GridCtx{pr, cells, u0, rec + 3 * rp.recs, idx, flg, cell};
     }
   }();
   // the vertices behind the entries of edges that leave the block
@@ -1095,7 +1122,7 @@ __global__ void __launch_bounds__(RT, 1) k_exchange_selftest(ResidentSync* sync,
 }
 
 template <class K, bool CL>
-cudaError_t launch(const typename K::Prob* probs, const int* cells, ResidentSync* sync, const ResidentPlan& rp,
+cudaError_t launch(const typename K::Prob* probs, const int* cells, const int4* places, ResidentSync* sync, const ResidentPlan& rp,
                    float4* rec, int inner, int step, int csn_out, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(rp.blocks);
@@ -1116,13 +1143,13 @@ cudaError_t launch(const typename K::Prob* probs, const int* cells, ResidentSync
   }
   cfg.attrs = attr;
   cfg.numAttrs = CL ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, k_pcg_resident<K, CL>, probs, cells, sync, rp, rec, inner, step, csn_out);
+  return cudaLaunchKernelEx(&cfg, k_pcg_resident<K, CL>, probs, cells, places, sync, rp, rec, inner, step, csn_out);
 }
 template <class K>
-cudaError_t launch(const typename K::Prob* probs, const int* cells, ResidentSync* sync, const ResidentPlan& rp,
+cudaError_t launch(const typename K::Prob* probs, const int* cells, const int4* places, ResidentSync* sync, const ResidentPlan& rp,
                    float4* rec, int inner, int step, int csn_out, cudaStream_t st) {
-  return rp.cluster ? launch<K, true>(probs, cells, sync, rp, rec, inner, step, csn_out, st)
-                    : launch<K, false>(probs, cells, sync, rp, rec, inner, step, csn_out, st);
+  return rp.cluster ? launch<K, true>(probs, cells, places, sync, rp, rec, inner, step, csn_out, st)
+                    : launch<K, false>(probs, cells, places, sync, rp, rec, inner, step, csn_out, st);
 }
 
 struct DeviceLimits {
@@ -1217,10 +1244,10 @@ Shape shape_of(int kind) {
 
 }  // namespace
 
-// float4 records the loop needs for planes of `plane` elements
-size_t resident_records(int kind, long long plane) {
+// float4 the loop needs for `recs` records in each buffer
+size_t resident_records(int kind, long long recs) {
   const Shape s = shape_of(kind);
-  return (size_t)(3 * s.NR) * plane + (kind == K_WARP ? plane / 2 + 1 : 0);
+  return (size_t)(3 * s.NR + (kind == K_WARP ? 1 : 0)) * recs;
 }
 
 #ifndef RES_CLUSTER_UNITS
@@ -1251,9 +1278,10 @@ ResidentPlan resident_plan(int kind, int n, long long plane, int lm, const int* 
     const long long want = std::max<long long>(least, (n + (long long)blocks - 1) / blocks);
     rp.per = (int)((want + quantum - 1) / quantum * quantum);
     rp.blocks = (n + rp.per - 1) / rp.per;
+    rp.recs = grid ? n : plane;
     const long long per = rp.per;
-    // r, q, M^-1, flags; the direction and what is derived from it
-    long long words = per * (2 * s.NX + s.NM + 1 + (s.NX - s.PT) + s.ND + (grid ? 1 : 0));
+    // r, q, M^-1, flags; the direction and what is derived from it; records and cells
+    long long words = per * (2 * s.NX + s.NM + 1 + (s.NX - s.PT) + s.ND + (grid ? 1 : 0)) + (grid ? per / CELL * 4 : 0);
     auto take = [&](long long w, int flag) {
       if (words + w > room) return false;
       words += w;
@@ -1293,20 +1321,20 @@ cudaError_t launch_exchange_selftest(ResidentSync* sync, int kind, int rounds, i
   return cudaLaunchCooperativeKernel((const void*)k_exchange_selftest, dim3(5), dim3(RT), args, 0, st);
 }
 
-cudaError_t launch_resident_grid(int kind, const GridProb* probs, const int* cells, ResidentSync* sync,
+cudaError_t launch_resident_grid(int kind, const GridProb* probs, const int* cells, const int4* places, ResidentSync* sync,
                                  const ResidentPlan& rp, float4* rec, int inner, int step, int csn_out,
                                  cudaStream_t st) {
-  return kind == K_WARP ? launch<WarpKind>(probs, cells, sync, rp, rec, inner, step, csn_out, st)
-                        : launch<PoissonKind>(probs, cells, sync, rp, rec, inner, step, 0, st);
+  return kind == K_WARP ? launch<WarpKind>(probs, cells, places, sync, rp, rec, inner, step, csn_out, st)
+                        : launch<PoissonKind>(probs, cells, places, sync, rp, rec, inner, step, 0, st);
 }
 
 cudaError_t launch_resident_graph(int kind, const MeshProb* probs, ResidentSync* sync, const ResidentPlan& rp,
                                   float4* rec, int inner, int step, cudaStream_t st) {
   switch (kind) {
-    case K_VOLUME: return launch<MeshKind<true>>(probs, nullptr, sync, rp, rec, inner, step, 0, st);
-    case K_WARPG: return launch<WarpGraphKind>(probs, nullptr, sync, rp, rec, inner, step, 0, st);
-    case K_EMBED: return launch<EmbeddedKind>(probs, nullptr, sync, rp, rec, inner, step, 0, st);
-    default: return launch<MeshKind<false>>(probs, nullptr, sync, rp, rec, inner, step, 0, st);
+    case K_VOLUME: return launch<MeshKind<true>>(probs, nullptr, nullptr, sync, rp, rec, inner, step, 0, st);
+    case K_WARPG: return launch<WarpGraphKind>(probs, nullptr, nullptr, sync, rp, rec, inner, step, 0, st);
+    case K_EMBED: return launch<EmbeddedKind>(probs, nullptr, nullptr, sync, rp, rec, inner, step, 0, st);
+    default: return launch<MeshKind<false>>(probs, nullptr, nullptr, sync, rp, rec, inner, step, 0, st);
   }
 }
 
