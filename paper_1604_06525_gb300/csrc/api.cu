@@ -1247,12 +1247,28 @@ static opt_status plan_edges(opt_problem& work, const opt_graph_desc* d, const s
     CK(cudaMemcpyAsync(v1, d->v1, (size_t)p.E * sizeof(int), cudaMemcpyDeviceToDevice, nullptr));
   }
   CKS(dalloc(&work, &p.cursor, 2 * ((size_t)p.V + 1)));
-  CKS(dalloc(&work, &p.flags, 2));
+  CKS(dalloc(&work, &p.flags, 3 + EDGE_LONG_ROWS));
+  p.long_rows = p.flags + 3;
   p.v0 = v0;
   p.v1 = v1;
   CK(launch_edge_plan(p, nullptr));
-  int flags[2];
+  int flags[3 + EDGE_LONG_ROWS];
   CK(cudaMemcpy(flags, p.flags, sizeof(flags), cudaMemcpyDeviceToHost));
+  if (!flags[0] && flags[2]) {
+    for (int k = 0; k < std::min(flags[2], EDGE_LONG_ROWS); ++k) {
+      const bool in = flags[3 + k] >= p.V;
+      const int v = flags[3 + k] - (in ? p.V : 0);
+      std::vector<int> at, row;
+      CKS(download(at, (in ? p.irow : p.orow) + v, 2));
+      int* list = (in ? p.isrc : p.e1) + at[0];
+      CKS(download(row, list, (size_t)(at[1] - at[0])));
+      std::sort(row.begin(), row.end());
+      CKS(upload(list, row));
+    }
+    CK(cudaMemset(p.flags + 1, 0, sizeof(int)));
+    CK(launch_edge_sym(p, nullptr));
+    CK(cudaMemcpy(flags, p.flags, sizeof(flags), cudaMemcpyDeviceToHost));
+  }
   sym = !flags[1];
   return flags[0] ? OPT_ERR_INVALID_ARG : OPT_OK;
 }
@@ -1393,7 +1409,7 @@ static opt_status create_graph_impl(const opt_graph_desc* d, int D, opt_problem*
   CKS(up.flush());
   bool sym = false;
   CKS(plan_edges(work, d, host_e0, host_e1, EdgePlan{nullptr, nullptr, dip, V, E, de0, de1, dorow, dirow, disrc, nullptr,
-                                                     dgw, d->w_reg, nullptr}, sym));
+                                                     dgw, d->w_reg, nullptr, nullptr}, sym));
   CKS(download(q->h_orow, dorow, (size_t)V + 1));
   q->h_vch = vch;
   q->h_ech = ech;

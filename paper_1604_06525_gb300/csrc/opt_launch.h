@@ -106,16 +106,20 @@ cudaError_t launch_exchange_selftest64(ResidentSync* sync, int rounds, int* out,
 // edge_plan.cu: the edges of a graph in the internal vertex order.  v0, v1: the
 // caller's; iperm: internal number of every caller vertex; e0, e1, isrc: E entries; orow,
 // irow: V + 1 zeros before the call; cursor: 2 (V + 1); degw: w_fit at handles, else 0,
-// before the call; flags (zeros): [0] an edge is no edge, [1] some edge is given one way.
+// before the call; flags (zeros): [0] an edge is no edge, [1] some edge is given one way, [2]
+// how many long rows there are; long_rows: the first EDGE_LONG_ROWS of them (a vertex, or V +
+// it for its in-edges), which the caller sorts, then asks for flags[1] again.
+constexpr int EDGE_LONG_ROWS = 64;
 struct EdgePlan {
   const int *v0, *v1, *iperm;
   int V, E;
   int *e0, *e1, *orow, *irow, *isrc, *cursor;
   float* degw;
   float w_reg;
-  int* flags;
+  int *flags, *long_rows;
 };
 cudaError_t launch_edge_plan(const EdgePlan& p, cudaStream_t st);
+cudaError_t launch_edge_sym(const EdgePlan& p, cudaStream_t st);
 
 // graph_kernels.cu
 void launch_mesh_init(const MeshLaunch& L, int k_outer, float dmin, float dmax);
