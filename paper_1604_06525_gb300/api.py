@@ -124,6 +124,7 @@ _SIGNATURES = [
     ("opt_selftest_grid_barrier", c_int32, [c_int32, c_int32, POINTER(c_int32)]),
     ("opt_selftest_staging_wait", c_int32, [c_int32, POINTER(c_int32)]),
     ("opt_selftest_resident_exchange", c_int32, [c_int32, c_int32, c_int32, POINTER(c_int32)]),
+    ("opt_selftest_footprint", c_int32, [c_void_p, POINTER(ctypes.c_size_t)]),
     ("opt_selftest_refuse_allocation", c_int32, []),
     ("opt_selftest_lose_block", c_int32, [c_void_p]),
     ("opt_selftest_lose_block_f64", c_int32, [c_void_p]),

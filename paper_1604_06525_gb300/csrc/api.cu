@@ -16,6 +16,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <initializer_list>
 #include <memory>
 #include <mutex>
 #include <numeric>
@@ -176,8 +177,11 @@ cudaMemPool_t problem_pool() {
 
 // Zero-filled device array owned by the problem (ordered on the legacy
 // stream; planning ends with a synchronising copy before any other stream
-// touches it).  The many small ones of a plan share slabs.
-constexpr size_t kSlabBytes = 128 << 10, kSlabShare = 16 << 10;
+// touches it).  Small ones share slabs, small enough that what is left of the last one
+// stays within what a server's estimate allows for tables; a plan that knows its sizes
+// reserves one block for all of them (level-5 mesh: 28 allocations in one).
+constexpr size_t kSlabBytes = 32 << 10, kSlabShare = 8 << 10;
+constexpr size_t room_of(size_t bytes) { return (std::max<size_t>(bytes, 1) + 255) / 256 * 256; }
 thread_local bool g_refuse_alloc = false;   // self-test: the next allocation is refused
 opt_status dalloc_bytes(opt_problem* pb, void** ptr, size_t bytes) {
   if (g_refuse_alloc) {
@@ -189,14 +193,18 @@ opt_status dalloc_bytes(opt_problem* pb, void** ptr, size_t bytes) {
   if (e != cudaSuccess) return cuda_fail(e, "device allocation");
   pb->allocs.push_back(*ptr);
   pb->pooled.push_back(pool != nullptr);
+  pb->bytes += bytes;
   e = cudaMemsetAsync(*ptr, 0, bytes, nullptr);
   return e == cudaSuccess ? OPT_OK : cuda_fail(e, "cudaMemsetAsync");
 }
 template <class T>
 opt_status dalloc(opt_problem* pb, T** ptr, size_t n) {
-  const size_t bytes = std::max<size_t>(n, 1) * sizeof(T), room = (bytes + 255) / 256 * 256;
+  const size_t bytes = std::max<size_t>(n, 1) * sizeof(T), room = room_of(bytes);
   void* p = nullptr;
-  if (room <= kSlabShare) {
+  if (room > pb->slab_left && room > kSlabShare) {
+    const opt_status s = dalloc_bytes(pb, &p, bytes);
+    if (s != OPT_OK) return s;
+  } else {
     if (pb->slab_left < room) {
       const opt_status s = dalloc_bytes(pb, &p, kSlabBytes);
       if (s != OPT_OK) return s;
@@ -206,11 +214,18 @@ opt_status dalloc(opt_problem* pb, T** ptr, size_t n) {
     p = pb->slab;
     pb->slab += room;
     pb->slab_left -= room;
-  } else {
-    const opt_status s = dalloc_bytes(pb, &p, bytes);
-    if (s != OPT_OK) return s;
   }
   *ptr = static_cast<T*>(p);
+  return OPT_OK;
+}
+opt_status dreserve(opt_problem* pb, std::initializer_list<size_t> bytes) {
+  size_t total = 0;
+  for (size_t b : bytes) total += room_of(b);
+  void* p = nullptr;
+  const opt_status s = dalloc_bytes(pb, &p, total);
+  if (s != OPT_OK) return s;
+  pb->slab = static_cast<char*>(p);
+  pb->slab_left = total;
   return OPT_OK;
 }
 
@@ -331,7 +346,6 @@ opt_status common_setup(opt_problem* pb) {
   CK(cudaStreamCreateWithFlags(&pb->cap_stream, cudaStreamNonBlocking));
   CK(cudaEventCreate(&pb->ev0));
   CK(cudaEventCreate(&pb->ev1));
-  CKS(dalloc(pb, &pb->d_s, 1));
   return OPT_OK;
 }
 
@@ -965,6 +979,12 @@ opt_status opt_selftest_resident_exchange(int32_t kind, int32_t absent, int32_t 
   return h[1] ? OPT_ERR_NUMERIC : OPT_OK;
 }
 
+opt_status opt_selftest_footprint(const opt_problem* prob, size_t* bytes) {
+  if (!prob || !bytes) return OPT_ERR_INVALID_ARG;
+  *bytes = prob->bytes;
+  return OPT_OK;
+}
+
 opt_status opt_selftest_refuse_allocation(void) {
   g_refuse_alloc = true;
   return OPT_OK;
@@ -1178,6 +1198,7 @@ opt_status opt_problem_create_grid(const opt_grid_desc* d, const opt_solve_param
   q->nchunks = (int)chunks.size();
   CKS(dalloc(q, &q->d_part, 8 * chunks.size()));   // up to four Sums per chunk
   CKS(dalloc(q, &q->dg, 1));
+  CKS(dalloc(q, &q->d_s, 1));
   for (int k = 0; k < nx; ++k) q->user_x[k] = d->unknowns[k];
   q->h_mask = mask;
   q->h_hpix = hpix;
@@ -1279,7 +1300,7 @@ static opt_status create_graph_impl(const opt_graph_desc* d, int D, opt_problem*
                                     const EmbedExtra* ed = nullptr) {
   // unknown planes, distinct-diagonal planes, geometry and vector records per vertex
   const int NXg = ed ? 12 : (D == 3 ? 6 : 3), NMg = ed ? 10 : (D == 3 ? 4 : 2);
-  const int NGR = ed ? 1 : (D == 3 ? 3 : 1), NVR = ed || D == 3 ? 3 : 1;
+  const int NGR = ed ? 1 : (D == 3 ? 3 : 1), NVR = ed ? 3 : (D == 3 ? 2 : 1);
   float* const* ux = ed ? ed->unknowns : d ? d->unknowns : nullptr;
   if (!out) return OPT_ERR_INVALID_ARG;
   *out = nullptr;
@@ -1365,6 +1386,14 @@ static opt_status create_graph_impl(const opt_graph_desc* d, int D, opt_problem*
   const size_t pl = (size_t)Vp;
   float *U = nullptr, *dgw = nullptr, *m = nullptr, *dc = nullptr, *dhtgt = nullptr;
   int *de0 = nullptr, *de1 = nullptr, *dhbeg = nullptr, *dhpix = nullptr;
+  {
+    const size_t f = sizeof(float) * pl, v1 = sizeof(int) * ((size_t)V + 1), e = sizeof(int) * (size_t)E;
+    CKS(dreserve(q, {NXg * f, D * f, f, NXg * f, NXg * f, NXg * f, 2 * NXg * f, NMg * f, NMg * f,
+                     sizeof(float4) * NGR * (size_t)V, sizeof(float4) * NVR * (size_t)V, v1, v1, v1, e, e, e,
+                     sizeof(int) * hbeg.size(), sizeof(int) * hpix.size(), sizeof(float) * hts.size(),
+                     sizeof(Chunk) * vch.size(), sizeof(Chunk) * ech.size(),
+                     2 * sizeof(double) * std::max(vch.size(), ech.size()), sizeof(MeshProb), sizeof(Scalars)}));
+  }
   CKS(dalloc(q, &q->x, NXg * pl));
   CKS(dalloc(q, &U, D * pl));
   CKS(dalloc(q, &dgw, pl));
@@ -1418,6 +1447,7 @@ static opt_status create_graph_impl(const opt_graph_desc* d, int D, opt_problem*
   q->nechunks = (int)ech.size();
   CKS(dalloc(q, &q->d_part, 2 * std::max(vch.size(), ech.size())));
   CKS(dalloc(q, &q->dm, 1));
+  CKS(dalloc(q, &q->d_s, 1));
   for (int k = 0; k < NXg; ++k) q->user_x[k] = ux[k];
   q->h_hpix = hpix;
 

@@ -18,7 +18,7 @@
 //             vertex only, (cos a_y, sin a_y, cos a_z, sin a_z)
 //                                                   written by PCGInit's vertex pass
 //   vrec[v] = x's displacement in PCGInit; (p_d, w) in applyJTJ, 2 float4;
-//             (x_d, U, delta_d) in the energies, 3 float4
+//             (x_d, U, delta_d but for its last component) in the energies, 2 float4
 //
 // ARAP mesh algebra per edge e = (a, b), v = U_a - U_b, d = O - U:
 //   r_e       = s_w [(d_a - d_b) + (v - R(A_a) v)]              (= Fig. 25)
@@ -573,8 +573,9 @@ __global__ void __launch_bounds__(NT) k_mesh_update(const MeshProb* __restrict__
 // energies and the outer update
 // ---------------------------------------------------------------------------
 // Vertex pass of the energies on edge lists: what the gather reads of a
-// neighbour, its displacement, rest position and (mode 1) displacement step,
-// in one record.  (A voxel's neighbours lie next to it in the planes.)
+// neighbour, its displacement, rest position and (mode 1) the first two components of
+// its displacement step, in one record; the third is read from its plane (a sector of its
+// own either way).  (A voxel's neighbours lie next to it in the planes.)
 __global__ void __launch_bounds__(NT) k_mesh_energy_v(const MeshProb* __restrict__ probs,
                                                       const Chunk* __restrict__ chunks, int mode) {
   const Chunk ch = chunks[blockIdx.x];
@@ -583,16 +584,15 @@ __global__ void __launch_bounds__(NT) k_mesh_energy_v(const MeshProb* __restrict
   if (mode == 1 && pr.s->done) return;
   const long long pl = pr.Vp;
   for (int v = ch.begin + threadIdx.x; v < ch.end; v += NT) {
-    float x[3], U[3], d[3] = {0.f, 0.f, 0.f};
+    float x[3], U[3], d[2] = {0.f, 0.f};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       x[c] = pr.x[c * pl + v];
       U[c] = __ldg(pr.U + c * pl + v);
-      if (mode == 1) d[c] = pr.d[c * pl + v];
+      if (mode == 1 && c < 2) d[c] = pr.d[c * pl + v];
     }
-    pr.vrec[3 * (size_t)v] = make_float4(x[0], x[1], x[2], U[0]);
-    pr.vrec[3 * (size_t)v + 1] = make_float4(U[1], U[2], d[0], d[1]);
-    if (mode == 1) pr.vrec[3 * (size_t)v + 2] = make_float4(d[2], 0.f, 0.f, 0.f);
+    pr.vrec[2 * (size_t)v] = make_float4(x[0], x[1], x[2], U[0]);
+    pr.vrec[2 * (size_t)v + 1] = make_float4(U[1], U[2], d[0], d[1]);
   }
 }
 
@@ -660,12 +660,12 @@ __global__ void __launch_bounds__(NT) k_mesh_energy(const MeshProb* __restrict__
           if (mode == 1) dd[c] = di[c] - pr.d[c * pl + j];
         }
       } else {
-        const float4 ra = pr.vrec[3 * (size_t)j], rb = pr.vrec[3 * (size_t)j + 1];
+        const float4 ra = pr.vrec[2 * (size_t)j], rb = pr.vrec[2 * (size_t)j + 1];
         d[0] = xi[0] - ra.x; d[1] = xi[1] - ra.y; d[2] = xi[2] - ra.z;
         v[0] = ui[0] - ra.w; v[1] = ui[1] - rb.x; v[2] = ui[2] - rb.y;
         if (mode == 1) {
           dd[0] = di[0] - rb.z; dd[1] = di[1] - rb.w;
-          dd[2] = di[2] - pr.vrec[3 * (size_t)j + 2].x;
+          dd[2] = di[2] - pr.d[2 * pl + j];
         }
       }
       float y[3], r[3];

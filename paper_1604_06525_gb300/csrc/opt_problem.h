@@ -104,7 +104,7 @@ struct opt_problem {
   std::vector<void*> allocs;
   std::vector<bool> pooled;             // allocs[k] came from the library's stream-ordered pool
   char* slab = nullptr;                 // what is left of the slab small allocations share
-  size_t slab_left = 0;
+  size_t slab_left = 0, bytes = 0;      // (bytes: allocated so far)
   int pcg_par = 0;
   // persistent PCG loop (wide warps): grid barrier state and the number of
   // blocks that can be resident at once (0 = not available)
@@ -144,7 +144,7 @@ struct opt_problem {
     swap(sent_hg, o.sent_hg); swap(sent_hm, o.sent_hm); swap(sent, o.sent);
     swap(user_x, o.user_x); swap(d_tmp, o.d_tmp); swap(d_jtf, o.d_jtf); swap(d_diag, o.d_diag);
     swap(x, o.x); swap(pbuf, o.pbuf); swap(dvec, o.dvec); swap(rvec, o.rvec); swap(qvec, o.qvec);
-    swap(allocs, o.allocs); swap(pooled, o.pooled); swap(slab, o.slab); swap(slab_left, o.slab_left); swap(pcg_par, o.pcg_par);
+    swap(allocs, o.allocs); swap(pooled, o.pooled); swap(slab, o.slab); swap(slab_left, o.slab_left); swap(bytes, o.bytes); swap(pcg_par, o.pcg_par);
     swap(rplan, o.rplan); swap(rplanned, o.rplanned); swap(d_rsync, o.d_rsync); swap(d_rrec, o.d_rrec);
     swap(d_gbar, o.d_gbar); swap(coop_cap, o.coop_cap); swap(cap_stream, o.cap_stream);
     swap(gexec, o.gexec); swap(gkey, o.gkey); swap(ev0, o.ev0); swap(ev1, o.ev1);
