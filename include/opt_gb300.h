@@ -647,7 +647,7 @@ opt_status opt_selftest_resident_exchange(int32_t kind, int32_t absent, int32_t 
 /* Self-test: device bytes a float32 problem has allocated so far. */
 opt_status opt_selftest_footprint(const opt_problem* prob, size_t* bytes);
 
-/* Self-test: the next device allocation of a float32 problem on this host thread is
+/* Self-test: the next device allocation of a float32 problem, on whichever host thread, is
  * refused, as when memory has run out. */
 opt_status opt_selftest_refuse_allocation(void);
 

@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <initializer_list>
@@ -182,12 +183,9 @@ cudaMemPool_t problem_pool() {
 // reserves one block for all of them (level-5 mesh: 28 allocations in one).
 constexpr size_t kSlabBytes = 32 << 10, kSlabShare = 8 << 10;
 constexpr size_t room_of(size_t bytes) { return (std::max<size_t>(bytes, 1) + 255) / 256 * 256; }
-thread_local bool g_refuse_alloc = false;   // self-test: the next allocation is refused
+std::atomic<bool> g_refuse_alloc{false};   // self-test: the next allocation is refused
 opt_status dalloc_bytes(opt_problem* pb, void** ptr, size_t bytes) {
-  if (g_refuse_alloc) {
-    g_refuse_alloc = false;
-    return cuda_fail(cudaErrorMemoryAllocation, "device allocation");
-  }
+  if (g_refuse_alloc.exchange(false)) return cuda_fail(cudaErrorMemoryAllocation, "device allocation");
   cudaMemPool_t pool = problem_pool();
   cudaError_t e = pool ? cudaMallocFromPoolAsync(ptr, bytes, pool, nullptr) : cudaMalloc(ptr, bytes);
   if (e != cudaSuccess) return cuda_fail(e, "device allocation");

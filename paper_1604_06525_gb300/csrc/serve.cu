@@ -140,7 +140,9 @@ opt_status write_back(opt_problem* pb, cudaStream_t st) {
 // at once, the longest first; each keeps its own status, the last CUDA error text goes
 // to the calling thread, and admission stays in arrival order.  Ten warps up to 826^2
 // and six meshes up to level 6: 6.9 ms one after the other, 4.7 ms on two threads, 4.5
-// on four, 4.7 on eight (the driver's lock).
+// on four, 4.7 on eight (the driver's lock).  Working memory of several plans at once is
+// more than the budget charges, so a request that found no memory beside the others is
+// planned again by itself.
 constexpr size_t kPlanThreads = 4;
 
 opt_status plan_one(ServeReq* r, const opt_solve_params& prm) {
@@ -191,6 +193,8 @@ void plan(const std::vector<ServeReq*>& admit, const opt_solve_params& prm, std:
   work(false);
   for (std::thread& t : threads) t.join();
   if (!err.empty()) set_last_error(err);
+  for (size_t i = 0; i < n; ++i)
+    if (status[i] == OPT_ERR_OOM) status[i] = plan_one(admit[i], prm);
 }
 
 opt_status copy_in(opt_problem* pb, cudaStream_t st) {

@@ -34,3 +34,20 @@ def test_planned_meshes_fit_their_estimate(case):
     assert g.lib.opt_selftest_footprint(g.h, ctypes.byref(used)) == 0
     assert used.value <= charged(prob.V, prob.v0.size, prob.handle_idx.size)
     g.close()
+
+
+def test_request_without_memory_beside_others_is_planned_alone():
+    import torch
+    from paper_1604_06525_gb300 import api
+    srv = api.Server(1 << 30, outer=2, inner=4, rel_tol=0.0)
+    tickets = [srv.submit(synth.warp_problem(40 + 9 * i, 33, 6, seed=i)) for i in range(4)]
+    tickets.append(srv.submit(synth.mesh_problem(2, seed=1, handle_frac=0.05)))
+    srv.lib.opt_selftest_refuse_allocation()              # one of the plans finds no memory
+    busy = True
+    while busy:
+        active, queued = srv.step()
+        busy = active + queued > 0
+    for t in tickets:
+        report, x = srv.poll(t)
+        assert report["outer_done"] == 2 and torch.isfinite(x).all()
+    srv.close()
