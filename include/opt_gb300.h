@@ -190,7 +190,14 @@ typedef struct {
                                  one launch per PCG kernel, measured faster on GB300 (a barrier
                                  costs more than a kernel boundary with programmatic dependent
                                  launch).  Same arithmetic either way.  A
-                                 barrier wait is bounded (1 s): OPT_ERR_TIMEOUT. */
+                                 barrier wait is bounded (1 s): OPT_ERR_TIMEOUT.
+                                 -1 = launches in any case.  A loop on chip over the device
+                                 takes up to one block of every SM, starts when the SMs it needs
+                                 are free and shares them with no other such loop: solves of
+                                 independent problems on streams of their own then run one
+                                 after the other, where launches interleave (500^2 warps, GN 4 x
+                                 15, 40 solves each on two threads: 57 ms, in launches 48 ms; one
+                                 thread alone 32 and 38 ms). */
     void* stream;             /* cudaStream_t; NULL = legacy default stream */
     int32_t pcg_form;         /* 0 (default) = the two-pass Jacobi-PCG iteration of Sec. 4.1
                                  (applyJTJ with p.q, then the vector update with r.z: two
@@ -587,7 +594,8 @@ opt_status opt_problem_create_graph_f64(const opt_graph_desc_f64* desc, const op
 opt_status opt_problem_destroy_f64(opt_problem_f64* prob);
 
 /* GN / LM exactly as opt_solve_gn / opt_solve_lm (params->materialized must
- * be 0; tile_w and persistent are ignored). */
+ * be 0; tile_w is ignored, and persistent but for -1, which keeps the PCG loop in launches
+ * where it would run on chip). */
 opt_status opt_solve_gn_f64(opt_problem_f64* prob, const opt_solve_params* params, opt_report* report);
 opt_status opt_solve_lm_f64(opt_problem_f64* prob, const opt_solve_params* params, opt_report* report);
 

@@ -559,7 +559,7 @@ opt_status check_params(const opt_solve_params& p, bool lm) {
 // for, matrix-free, on wide warp tiles, and every chunk's block fits on the
 // device at once.
 bool use_persistent(const opt_problem* pb, const opt_solve_params& p) {
-  return p.persistent && !p.materialized && p.inner > 0 && pb->d_gbar && pb->nchunks <= pb->coop_cap;
+  return p.persistent > 0 && !p.materialized && p.inner > 0 && pb->d_gbar && pb->nchunks <= pb->coop_cap;
 }
 
 // The single-reduction PCG iteration runs where asked for on warps and
@@ -636,10 +636,19 @@ opt_status resident_prepare(opt_problem* pb) {
 }
 
 // The resident loop serves the two-pass iteration (pcg_form 0, and form 1 on
-// problems without single-reduction buffers) of matrix-free solves.
+// problems without single-reduction buffers) of matrix-free solves, unless the caller
+// wants launches.  It is taken wherever the state fits: from three PCG iterations on it was
+// the faster route up to the largest states (us, loop / launches, GN 2 x 3 and 2 x 10: 64^2
+// warp 117 / 156 and 170 / 317, 600^2 warp 207 / 208 and 389 / 455, 1024^2 Poisson 191 /
+// 221 and 335 / 473, level-7 mesh 266 / 354 and 488 / 841, a sheet of 550^2 vertices 367 / 495 and
+// 749 / 1212, 50^3 volume 214 / 261 and 400 / 591; at the limit, a 700^2 warp, 240 / 226 and
+// 462 / 492).  With one iteration, where the state is loaded for one use, it is even below
+// 300^2 pixels and loses 10 % at 500^2 and 20 % at 700^2.
+bool want_resident(const opt_problem* pb, const opt_solve_params& p) {
+  return p.persistent >= 0 && !p.materialized && p.inner > 0 && !use_fused(pb, p) && !use_persistent(pb, p);
+}
 bool use_resident(const opt_problem* pb, const opt_solve_params& p, bool lm) {
-  return !p.materialized && p.inner > 0 && !use_fused(pb, p) && !use_persistent(pb, p) &&
-         pb->rplan[lm ? 1 : 0].blocks > 0;
+  return want_resident(pb, p) && pb->rplan[lm ? 1 : 0].blocks > 0;
 }
 
 opt_status enqueue_solve(opt_problem* pb, const opt_solve_params& p, bool lm, cudaStream_t st) {
@@ -736,7 +745,7 @@ opt_status run_solve(opt_problem* pb, const opt_solve_params* prm_in, opt_report
   // descriptor's copy and one of two result copies less: about 25 us of every solve
   // (64^2 warp GN 4 x 10 295 -> 272 us; 28 x 108 mesh LM 1 x 7 174 -> 149 us).
   CKS(ensure_ehist(pb, p.outer + 1));
-  CKS(resident_prepare(pb));
+  if (want_resident(pb, p)) CKS(resident_prepare(pb));
   set_flags(pb, lm ? 1 : 0, p.use_precond, pb->d_Ehist);
   if (p.materialized || !desc_sent(pb)) {
     CK(cudaStreamSynchronize(st));

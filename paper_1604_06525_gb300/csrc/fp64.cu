@@ -1434,7 +1434,7 @@ opt_status enqueue_solve64(opt_problem_f64* pb, const opt_solve_params& p, bool 
   for (int k = 0; k < p.outer; ++k) {
     k_rot(pb, st);
     k_init(pb, P, st, k, p.diag_min, p.diag_max);
-    if (pb->d_rsync && p.inner > 0) {
+    if (pb->d_rsync && p.inner > 0 && p.persistent >= 0) {
       CKS64(launch_loop(pb, P, st, p.inner));
     } else {
       for (int i = 0; i < p.inner; ++i) {
@@ -1480,7 +1480,7 @@ opt_status run_solve64(opt_problem_f64* pb, const opt_solve_params* prm_in, opt_
   if (p.use_graph) {
     const std::vector<double> key = {double(p.outer), double(p.inner), double(lm), double(p.use_precond),
                                      p.lambda0, p.lambda_min, p.lambda_max, p.diag_min, p.diag_max,
-                                     p.eta, p.rel_tol};
+                                     p.eta, p.rel_tol, double(p.persistent < 0)};
     if (!pb->gexec || key != pb->gkey) {
       if (pb->gexec) {
         cudaGraphExecDestroy(pb->gexec);
