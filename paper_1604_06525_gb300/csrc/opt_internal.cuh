@@ -286,7 +286,7 @@ __device__ __forceinline__ bool grid_sync(GridBarrier* gb, unsigned int expected
 // resident PCG loop (resident.cu)
 // ---------------------------------------------------------------------------
 constexpr int RES_MAX_BLOCKS = 160;
-constexpr int RES_LANES = 4;          // threads per vertex where a block has few of them
+constexpr int RES_LANES = 4;          // threads per voxel where a block has few of them
 constexpr int RES_CLUSTER = 16;       // blocks of the one-cluster form, at most
 // RES_D, RES_DC, RES_LIST: kept in shared memory; RES_Z: see Records (resident.cu)
 enum ResidentFlags : int { RES_D = 1, RES_DC = 2, RES_LIST = 4, RES_Z = 8 };
@@ -312,7 +312,7 @@ struct ResidentPlan {
   int flags;
   int cluster;                  // 1: one cluster, 0: cooperative launch over the device
   int slots;                    // graphs: table entries for edges that leave a block (0: no table)
-  int lanes;                    // graphs: threads per vertex
+  int lanes;                    // threads per voxel (else 1)
   long long plane;              // plane stride
   long long recs;               // direction records of one buffer (grids: one per unit, graphs: per plane element)
 };

@@ -443,9 +443,9 @@ struct PoissonKind : GridUnits {
 // (voxel grids, one-way edges, too many edges leave) neighbours are read from
 // their records, and lists hold vertices.
 //
-// A vertex is gathered by LANES threads where a block has few vertices: each
-// evaluates every LANES-th neighbour, and the terms are added in list order
-// whatever LANES is.
+// A voxel is gathered by RES_LANES threads where a block has few of them (see
+// resident_plan): each evaluates every RES_LANES-th neighbour, and the terms are added in
+// list order all the same.
 struct GraphCtx {
   const MeshProb& pr;
   int u0, cap, tab;
@@ -617,8 +617,8 @@ struct EmbeddedKind : GraphUnits {
   }
 };
 
-// The edge sums t of unit j (ok: there is one), by LANES consecutive threads of
-// a warp; all of them get the result.  Called by whole warps.
+// The edge sums t of unit j (ok: there is one), on voxel grids by LANES consecutive
+// threads of a warp; all of them get the result.  Called by whole warps.
 template <class K, int LANES>
 __device__ __forceinline__ void graph_sums(const GraphCtx& c, int j, bool ok, const typename K::Own& o,
                                            const Records& R, float (&t)[K::NT_]) {
@@ -690,47 +690,28 @@ __device__ __forceinline__ void graph_sums(const GraphCtx& c, int j, bool ok, co
   }
   const int o0 = ok ? c.row[j] : 0, deg = ok ? c.row[j + 1] - o0 : 0;
   const bool sym = pr.sym != 0;
-  if (LANES == 1) {
-    // two neighbours at a time: their records are in flight together
-    for (int k = 0; k < deg; k += 2) {
-      float d1[K::ND], g1[K::NS], d2[K::ND], g2[K::NS], v[NT_];
-      const bool two = k + 1 < deg;
-      const int e1 = c.lst[o0 + k], e2 = two ? c.lst[o0 + k + 1] : e1;
-      fetch(e1, d1, g1);
-      if (two) fetch(e2, d2, g2);
-      K::terms(pr, o, d1, g1, true, sym, v);
+  // two neighbours at a time: their records are in flight together
+  for (int k = 0; k < deg; k += 2) {
+    float d1[K::ND], g1[K::NS], d2[K::ND], g2[K::NS], v[NT_];
+    const bool two = k + 1 < deg;
+    const int e1 = c.lst[o0 + k], e2 = two ? c.lst[o0 + k + 1] : e1;
+    fetch(e1, d1, g1);
+    if (two) fetch(e2, d2, g2);
+    K::terms(pr, o, d1, g1, true, sym, v);
+#pragma unroll
+    for (int n = 0; n < NT_; ++n) t[n] += v[n];
+    if (two) {
+      K::terms(pr, o, d2, g2, true, sym, v);
 #pragma unroll
       for (int n = 0; n < NT_; ++n) t[n] += v[n];
-      if (two) {
-        K::terms(pr, o, d2, g2, true, sym, v);
-#pragma unroll
-        for (int n = 0; n < NT_; ++n) t[n] += v[n];
-      }
     }
-    if (!sym && ok) {
-      for (int k = pr.irow[c.u0 + j]; k < pr.irow[c.u0 + j + 1]; ++k) {
-        float v[NT_];
-        nbr(pr.isrc[k], false, true, v);
-#pragma unroll
-        for (int n = 0; n < NT_; ++n) t[n] += v[n];
-      }
-    }
-    return;
   }
-  const int most = __reduce_max_sync(0xffffffffu, deg);
-  for (int r = 0; r < most; r += LANES) {
-    float v[NT_];
-    const bool has = r + lane < deg;
+  if (!sym && ok) {
+    for (int k = pr.irow[c.u0 + j]; k < pr.irow[c.u0 + j + 1]; ++k) {
+      float v[NT_];
+      nbr(pr.isrc[k], false, true, v);
 #pragma unroll
-    for (int n = 0; n < NT_; ++n) v[n] = 0.f;
-    if (has) nbr(c.lst[o0 + r + lane], true, true, v);
-#pragma unroll
-    for (int s = 0; s < LANES; ++s) {
-#pragma unroll
-      for (int n = 0; n < NT_; ++n) {
-        const float a = __shfl_sync(0xffffffffu, v[n], s, LANES);
-        if (r + s < deg) t[n] += a;
-      }
+      for (int n = 0; n < NT_; ++n) t[n] += v[n];
     }
   }
 }
@@ -990,8 +971,12 @@ __global__ void __launch_bounds__(RT, 1) k_pcg_resident(const typename K::Prob* 
           }
         }
       };
-      if (rp.lanes > 1 && (K::G3 || pr.sym)) gather(Lanes<RES_LANES>{});
-      else gather(Lanes<1>{});
+      bool one = true;
+      if constexpr (K::G3) {
+        one = rp.lanes == 1;
+        if (!one) gather(Lanes<RES_LANES>{});
+      }
+      if (one) gather(Lanes<1>{});
     } else {
       // two pixels at a time: their neighbours' records are in flight together
       for (int j = tid; j < cnt; j += 2 * RT) {
@@ -1250,12 +1235,25 @@ size_t resident_records(int kind, long long recs) {
   return (size_t)(3 * s.NR + (kind == K_WARP ? 1 : 0)) * recs;
 }
 
+// Times below: LM 2 x 15, us.
+// Up to so many units one cluster takes the problem: it is as fast or faster for every
+// kind below (warp of 4,800 pixels 245 against 307 over the device, mesh of 642 vertices 293
+// / 315, of 2,562 310 / 331, sheet of 7,920 354 / 346, embedded 2,562 358 / 364, graph 7,650 288
+// / 324), and slower above where a unit is much work (mesh of 10,242 431 / 337, embedded
+// 527 / 388, volume 24^3 476 / 361; 15,360 pixels 318 / 311).
 #ifndef RES_CLUSTER_UNITS
 #define RES_CLUSTER_UNITS 8192
 #endif
+// Over the device, up to so many voxels a block RES_LANES threads share one: 26^3 373 against
+// 405 with one thread, 40^3 563 against 424.  (Edge lists lose: mesh of 2,562 350 / 310.)
 #ifndef RES_LANE_UNITS
 #define RES_LANE_UNITS 256
 #endif
+// Over the device, up to so many units z goes through records (RES_Z): one meeting an
+// iteration less for twice the records read.  Sheet of 32,040 366 against 375 without, mesh
+// of 10,242 346 / 365, graph 328 / 338, pixels equal; still 1 to 4 % at 62,500; far above the
+// reads cost more (LM / GN 2 x 30: embedded 163,842 3.02 / 1.97 ms, Poisson of 315,000 pixels 699 /
+// 614).
 #ifndef RES_Z_UNITS
 #define RES_Z_UNITS 32768
 #endif
@@ -1289,7 +1287,7 @@ ResidentPlan resident_plan(int kind, int n, long long plane, int lm, const int* 
       return true;
     };
     if (words > room) return false;
-    rp.lanes = !grid && per <= RES_LANE_UNITS ? RES_LANES : 1;
+    rp.lanes = 1;
     if (orow) {
       int most = 0;
       for (int b = 0; b < rp.blocks; ++b)
@@ -1313,6 +1311,7 @@ ResidentPlan resident_plan(int kind, int n, long long plane, int lm, const int* 
   }
   if (!fill(d.sms, grid ? CELL : 64)) return ResidentPlan{};
   if (n <= RES_Z_UNITS) rp.flags |= RES_Z;
+  if (kind == K_VOLUME && rp.per <= RES_LANE_UNITS) rp.lanes = RES_LANES;
   return rp;
 }
 
