@@ -573,12 +573,20 @@ bool use_fused(const opt_problem* pb, const opt_solve_params& p) {
 // What the resident loop of the planned kinds of solve needs on the device.
 opt_status resident_alloc(opt_problem* pb) {
   long long recs = 0;
-  for (const ResidentPlan& rp : pb->rplan)
-    if (rp.blocks > 0) recs = std::max(recs, rp.recs);
+  bool wide = false;                    // over the device: exchanges through memory
+  for (const ResidentPlan& rp : pb->rplan) {
+    if (rp.blocks == 0) continue;
+    recs = std::max(recs, rp.recs);
+    wide = wide || !rp.cluster;
+  }
   if (recs == 0) return OPT_OK;
-  CKS(dalloc(pb, &pb->d_rrec, resident_records(pb->kind, recs)));
-  CKS(dalloc(pb, &pb->d_rsync, 1));
-  CKS(reset_exchange(pb->d_rsync, nullptr));
+  const size_t nrec = resident_records(pb->kind, recs), nc = is_grid(pb) ? pb->h_cells.size() : 0;
+  CKS(dreserve(pb, {sizeof(float4) * nrec, wide ? sizeof(ResidentSync) : 0, sizeof(int) * nc, sizeof(int4) * nc}));
+  CKS(dalloc(pb, &pb->d_rrec, nrec));
+  if (wide) {
+    CKS(dalloc(pb, &pb->d_rsync, 1));
+    CKS(reset_exchange(pb->d_rsync, nullptr));
+  }
   if (is_grid(pb)) {
     // cells ascend, so a cell's neighbours in its row are the next to it
     const std::vector<int>& cells = pb->h_cells;
