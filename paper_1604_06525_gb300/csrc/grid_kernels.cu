@@ -12,9 +12,9 @@
 //     delta = 0, float64 r.z and E        k_warp_init(_wide), k_poisson_init(_wide)
 //   Two-pass PCG iteration (Sec. 4.1, 4.2):
 //     applyJTJ with the direction p = z + beta p_old (halo included),
-//     q = (J^T J + lambda D) p, float64 p.q -> alpha
+//     q = (J^T J + lambda D) p, p.q -> alpha
 //                                          k_warp_apply(_wide), k_poisson_apply(_wide)
-//     vector update delta += alpha p, r -= alpha q, z = M^-1 r, float64 r.z -> beta
+//     vector update delta += alpha p, r -= alpha q, z = M^-1 r, r.z -> beta
 //                                          k_grid_update
 //   Single-reduction PCG iteration (128-pixel tiles): the update of the
 //     previous iteration, the direction, applyJTJ and p.q, q.z, q.M^-1 q, r.z
@@ -1079,9 +1079,40 @@ __device__ __forceinline__ void fused_pending(const Chunk& ch, const GridProb& p
   }
 }
 
+// alpha, the next r.z and beta of a single-reduction iteration from p.q, q.z, q.M^-1 q
+// and r.z (or the end of the loop on a breakdown).  alpha comes from the r.z of the stored
+// z (as the two-pass form takes it); the recurrence only carries r.z one iteration ahead,
+// to set beta.  It cancels; it is evaluated in float64.
+__device__ __forceinline__ void fused_scalars(Scalars* s, const Sum& pq, double qz, double qw, const Sum& rz, double pqd,
+                                              double rzd) {
+  s->pq = pqd;
+  if (pq.hi > 0.f && sum_finite(pq) && rz.hi > 0.f && sum_finite(rz)) {
+    const float af = sum_quot(rz, pq);
+    const double a = (double)af;
+    const double rz_next = fma(a * a, qw, fma(-2.0 * a, qz, rzd));
+    s->alpha_f = af;
+    s->rz = rzd;
+    s->rz_sum = rz;
+    s->pcg_iters += 1;
+    if (rz_next > 0.0 && isfinite(rz_next)) {
+      s->beta_f = sum_quot(sum_of(rz_next), rz);
+    } else {
+      s->pcg_active = 0;        // the step alpha p is still applied
+      if (!isfinite(rz_next)) s->nonfinite = 1;
+    }
+  } else {
+    s->alpha_f = 0.f;
+    s->pcg_active = 0;
+    if (!sum_finite(pq) || !sum_finite(rz)) s->nonfinite = 1;
+  }
+}
+static __device__ __noinline__ void fused_scalars64(Scalars* s, Sum pq, Sum qz, Sum qw, Sum rz) {
+  fused_scalars(s, pq, sum_double(qz), sum_double(qw), rz, sum_double(pq), sum_double(rz));
+}
+
 // End of a single-reduction iteration: the block's four compensated sums
 // (p.q, q.z, q.M^-1 q, r.z) published; the last block of the problem sets
-// alpha, the next r.z and beta (or ends the loop on a breakdown).
+// alpha, the next r.z and beta.
 __device__ __forceinline__ void fused_finish(const GridProb& pr, double* __restrict__ part, const F2x2& acc_pq,
                                              const F2x2& acc_qz, const F2x2& acc_qw, const F2x2& acc_zr) {
   Scalars* s = pr.s;
@@ -1090,29 +1121,11 @@ __device__ __forceinline__ void fused_finish(const GridProb& pr, double* __restr
     Sum v[4];
     gather_sums<4>(part, pr.chunk_begin, pr.chunk_end, &s->counter, v);
     if (threadIdx.x == 0) {
-      const Sum &pq = v[0], &rz = v[3];
-      s->pq = sum_double(pq);
-      if (pq.hi > 0.f && sum_finite(pq) && rz.hi > 0.f && sum_finite(rz)) {
-        // alpha from the r.z of the stored z (as the two-pass form takes it);
-        // the recurrence only carries r.z one iteration ahead, to set beta.  It
-        // cancels; it is evaluated in float64.
-        const float af = sum_quot(rz, pq);
-        const double a = (double)af, qz = sum_double(v[1]), qw = sum_double(v[2]), rzd = sum_double(rz);
-        const double rz_next = fma(a * a, qw, fma(-2.0 * a, qz, rzd));
-        s->alpha_f = af;
-        s->rz = rzd;
-        s->rz_sum = rz;
-        s->pcg_iters += 1;
-        if (rz_next > 0.0 && isfinite(rz_next)) {
-          s->beta_f = sum_quot(sum_of(rz_next), rz);
-        } else {
-          s->pcg_active = 0;        // the step alpha p is still applied
-          if (!isfinite(rz_next)) s->nonfinite = 1;
-        }
+      if (__builtin_expect(v[0].big | v[1].big | v[2].big | v[3].big, 0)) {
+        fused_scalars64(s, v[0], v[1], v[2], v[3]);
       } else {
-        s->alpha_f = 0.f;
-        s->pcg_active = 0;
-        if (!sum_finite(pq) || !sum_finite(rz)) s->nonfinite = 1;
+        const auto d = [](const Sum& a) { return f2_to_double(F2{a.hi, a.lo}); };
+        fused_scalars(s, v[0], d(v[1]), d(v[2]), v[3], d(v[0]), d(v[3]));
       }
     }
   }
@@ -1391,7 +1404,8 @@ __device__ __forceinline__ void fused_wide_body(FusedSmem& sm, const Chunk& ch, 
         }
       }
       // w = M^-1 q and the three inner products; z of the own pixels comes
-      // back from the stores of phase 2 (this thread's own writes)
+      // back from phase 2 (this thread's own writes): from the staging planes a
+      // lattice leaves free, else from its stores
       if (!LAT) {
         m0 = ld4(pr.m + i);
         m1 = ld4(pr.m + pl + i);
@@ -2961,7 +2975,7 @@ __global__ void __launch_bounds__(NT, 2) k_poisson_energy(const GridProb* __rest
 // ---------------------------------------------------------------------------
 // shared grid passes
 // ---------------------------------------------------------------------------
-// delta += alpha p, r -= alpha q, z = M^-1 r, float64 r.z -> beta.
+// delta += alpha p, r -= alpha q, z = M^-1 r, r.z -> beta.
 // Float4 stream over the tile rows (a tile row is 32 floats = 128 B of each
 // plane; the pitch keeps rows 16-byte aligned and the pitch padding holds
 // zeros in every vector).  All loads of a quad are issued before any use.
