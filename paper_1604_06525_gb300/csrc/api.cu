@@ -44,15 +44,21 @@ opt_status optgb::cuda_fail(cudaError_t e, const char* what) {
 
 void optgb::set_last_error(const std::string& text) { g_err = text; }
 
-// The counts and limits of a fresh exchange and empty slots; done when it returns, so
-// that the next solve finds them whatever its stream.
+// The counts and limits of a fresh exchange and empty slots.
+static __global__ void k_set_exchange(ResidentSync* d, int lose_block) {
+  unsigned int* w = reinterpret_cast<unsigned int*>(d);
+  constexpr int head = offsetof(ResidentSync, slot) / 4, words = sizeof(ResidentSync) / 4;
+  for (int k = threadIdx.x; k < words; k += blockDim.x) w[k] = k < head ? 0u : ~0u;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  d->first_ns = lose_block ? kSelfTestLimitNs : kFirstLimitNs;
+  d->wait_ns = lose_block ? kSelfTestLimitNs : kBarrierLimitNs;
+  d->absent = lose_block;
+}
+// (done when it returns, so that the next solve finds them whatever its stream)
 opt_status optgb::reset_exchange(ResidentSync* d, cudaStream_t st, bool lose_block) {
-  ResidentSync head = {};
-  head.first_ns = lose_block ? kSelfTestLimitNs : kFirstLimitNs;
-  head.wait_ns = lose_block ? kSelfTestLimitNs : kBarrierLimitNs;
-  head.absent = lose_block;
-  cudaError_t e = cudaMemcpyAsync(d, &head, offsetof(ResidentSync, slot), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d->slot, 0xff, sizeof(d->slot), st);
+  k_set_exchange<<<1, 512, 0, st>>>(d, lose_block);
+  cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   return e == cudaSuccess ? OPT_OK : cuda_fail(e, "exchange slots");
 }
@@ -581,17 +587,19 @@ opt_status resident_alloc(opt_problem* pb) {
   }
   if (recs == 0) return OPT_OK;
   const size_t nrec = resident_records(pb->kind, recs), nc = is_grid(pb) ? pb->h_cells.size() : 0;
-  CKS(dreserve(pb, {sizeof(float4) * nrec, wide ? sizeof(ResidentSync) : 0, sizeof(int) * nc, sizeof(int4) * nc}));
+  CKS(dreserve(pb, {sizeof(float4) * nrec, wide ? sizeof(ResidentSync) : 0, sizeof(int) * 5 * nc}));
   CKS(dalloc(pb, &pb->d_rrec, nrec));
   if (wide) {
     CKS(dalloc(pb, &pb->d_rsync, 1));
-    CKS(reset_exchange(pb->d_rsync, nullptr));
+    k_set_exchange<<<1, 512>>>(pb->d_rsync, 0);
+    CK(cudaGetLastError());
   }
   if (is_grid(pb)) {
     // cells ascend, so a cell's neighbours in its row are the next to it
     const std::vector<int>& cells = pb->h_cells;
     const int n = (int)cells.size();
-    std::vector<int4> at((size_t)n);
+    std::vector<int> table((size_t)5 * n);          // places, then cells
+    int4* at = reinterpret_cast<int4*>(table.data());
     int first = 0;
     for (int end = 0; first < n; first = end) {
       while (end < n && cells[end] >> 16 == cells[first] >> 16) ++end;
@@ -604,12 +612,12 @@ opt_status resident_alloc(opt_problem* pb) {
       at[k].w = at[below].x;
       at[below].z = at[k].x + (TH - 1) * at[k].y;
     }
-    Uploads up;
-    CKS(dalloc(pb, &pb->d_cells, cells.size()));
-    up.add(pb->d_cells, cells);
-    CKS(dalloc(pb, &pb->d_places, at.size()));
-    up.add(pb->d_places, at);
-    CKS(up.flush());
+    std::copy(cells.begin(), cells.end(), table.begin() + 4 * (size_t)n);
+    int* dev = nullptr;
+    CKS(dalloc(pb, &dev, table.size()));
+    CKS(upload(dev, table));
+    pb->d_places = reinterpret_cast<int4*>(dev);
+    pb->d_cells = dev + 4 * (size_t)n;
   }
   CK(cudaStreamSynchronize(nullptr));
   return OPT_OK;
