@@ -42,13 +42,15 @@ METRIC = "PCG iters/s and % HBM roofline; batched solves/s and p99 latency vs pl
 UNIT = "PCG iters/s"
 W_BENCH, H_BENCH, HANDLES, OUTER, INNER = 1024, 1024, 64, 20, 20
 # algorithmic bytes per pixel (float32 planes, each touched once per launch)
-BYTES_APPLY_WARP = 64      # read r 12, M^-1 8, p_old 12, cos/sin 8 (a pixel lattice: no UrShape); write p 12, q 12
+BYTES_APPLY_WARP = 64      # unmasked pixel lattice under GN, as the headline: read r 12, M^-1 8, p_old 12, cos/sin 8 (no UrShape);
+#                            write p 12, q 12
 BYTES_UPDATE_WARP = 80     # read delta 12, p 12, r 12, q 12, M^-1 8; write delta 12, r 12
 BYTES_INIT_WARP = 56       # as a solve runs it from the second outer iteration on (cos / sin of theta written by
 #                            the previous outer update): read dx, dy 8, cos/sin 8, UrShape 8; write r 12, M^-1 8,
 #                            delta 12 (GN)
 # single-reduction PCG iteration (pcg_form = 1), one launch per PCG iteration
-BYTES_FUSED_WARP = 104     # read z 12, w 12, p_old 12, cos/sin 8, delta 12 (a lattice under GN: no UrShape, M^-1 formed);
+BYTES_FUSED_WARP = 104     # unmasked pixel lattice under GN: read z 12, w 12, p_old 12, cos/sin 8, delta 12 (no
+#                            UrShape, M^-1 formed);
 #                            write z 12, w 12, p 12, delta 12
 BYTES_FIN_WARP = 36        # the last iteration's step: read delta 12, p 12; write delta 12
 PCG_FORM = 1               # the headline's PCG iteration: 1 single-reduction, 0 two-pass
@@ -1018,7 +1020,7 @@ def run_ours(args):
         "config": {"workload": f"ARAP image warping {W_BENCH}x{H_BENCH} (3 unknowns/pixel, {HANDLES} handles), "
                                f"GN {OUTER} outer x {INNER} PCG, Jacobi, matrix-free, one CUDA graph per solve",
                    "parallelism": "replicas" if world > 1 else "single GPU",
-                   "l2": "flushed between steps (512 MB write)", "precision": "f32 vectors, f64 dots/energies",
+                   "l2": "flushed between steps (512 MB write)", "precision": "f32 vectors, dots as compensated f32 pairs, f64 energies",
                    "chunking": chunking, "tile_w": head_cfg["tile_w"],
                    "pcg_form": ("single-reduction: one launch per PCG iteration (p.q, q.z, q.M^-1 q, r.z in "
                                 "one reduction)" if fused else "two-pass: applyJTJ + vector update"),

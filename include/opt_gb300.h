@@ -25,8 +25,10 @@
  *    host synchronise that stream.  One problem must not be used from two
  *    host threads or two streams at once.
  *  - Arithmetic: residuals, Jacobian entries, J^T J p and vector updates run
- *    in float32; PCG dot products (alpha, beta), energies and the LM gain
- *    ratio run in float64.
+ *    in float32; energies and the LM gain ratio run in float64.  PCG dot
+ *    products are compensated float32 pairs (about 47 bits; in float64 where
+ *    float32's range ends), from which alpha and beta are rounded to float32
+ *    once: the same alpha and beta as from float64 sums in every measured solve.
  *  - Errors: every call returns an opt_status; no exception crosses the ABI.
  *    OPT_ERR_INVALID_ARG leaves the problem unchanged.  OPT_ERR_CUDA means a
  *    CUDA call failed (the message is in opt_last_error()).
@@ -320,7 +322,7 @@ opt_status opt_pcg_get_state(opt_problem* prob, float* delta, float* r, float* p
 /* q = (J^T J + lambda * D) p at the caller's current unknowns (Sec. 4.2
  * applyJTJ without the factor 2 that cancels).  p, q: device, dense layout of
  * the unknowns (excluded Poisson pixels must hold p = 0).  pq (host, may be
- * NULL) receives p.q in float64. */
+ * NULL) receives p.q (a compensated float32 sum, about 47 bits). */
 opt_status opt_apply_jtj(opt_problem* prob, const float* p, float* q, double lambda, double* pq);
 
 /* J^T F and diag(J^T J) at the caller's current unknowns (Sec. 4.2 evalJTF).
@@ -367,7 +369,12 @@ opt_status opt_problem_set_chunking(opt_problem* prob, int32_t units_per_block);
  * with tile tables and each tile width (32, 128) of a grid (see
  * opt_problem_get_config); keeps the fastest combination and returns its
  * granularity in *chosen and its per-iteration time in *best_ms (host, either
- * may be NULL).  Leaves the PCG state of its last timed run.  A grid whose
+ * may be NULL).  What it times and chooses are launches: they serve batches and
+ * the server, pcg_form 1, persistent = -1, and problems whose state does not fit
+ * on chip.  A solve whose loop runs on chip issues none of them, so *best_ms is
+ * not its iteration; of the choices it keeps the tile width for its other kernels
+ * (up to 3 % of such a solve, 32 against 128 pixels, either way).  The same holds
+ * for opt_profile_pcg.  Leaves the PCG state of its last timed run.  A grid whose
  * other tile width wins is re-planned in place: autotune a problem before
  * building a batch over it, not while a batch holds it. */
 opt_status opt_problem_autotune(opt_problem* prob, int32_t* chosen, float* best_ms);
@@ -382,11 +389,12 @@ opt_status opt_problem_info(const opt_problem* prob, int64_t* n_unknowns, int32_
  * default), apply_form = how an ARAP mesh forms J^T J p (1: one block per
  * vertex tile with the tile's halo staged in shared memory, every residual of
  * the tile evaluated once; 0: the two-pass vertex gather; -1: not an ARAP mesh
- * with tile tables; a solve whose loop runs on chip uses neither).  opt_problem_autotune chooses all three: the form and
- * granularity of a mesh, the granularity and tile width of a grid (the other
- * width is planned afresh from the creation descriptor, whose arrays must
- * still be valid, and kept if faster).  Results agree across configurations
- * to float rounding (the sums are compensated, see Sec. 4.1 PCG). */
+ * with tile tables; a solve whose loop runs on chip uses neither granularity
+ * nor form).  opt_problem_autotune chooses all three: the form and granularity
+ * of a mesh, the granularity and tile width of a grid (the other width is
+ * planned afresh from the creation descriptor, whose arrays must still be
+ * valid, and kept if faster).  Results agree across configurations to float
+ * rounding (the sums are compensated, see Sec. 4.1 PCG). */
 opt_status opt_problem_get_config(const opt_problem* prob, int32_t* tile_w, int32_t* chunking,
                                   int32_t* apply_form);
 

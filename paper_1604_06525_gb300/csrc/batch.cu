@@ -8,7 +8,7 @@
 // never straddle two problems.  Each phase (PCGInit, applyJTJ, vector update,
 // outer update, energies) is one launch per energy kind covering all members;
 // members advance in lock-step through the same outer / inner counts, and every
-// float64 scalar (alpha, beta, energies, LM damping) stays per problem on the
+// scalar (alpha, beta, energies, LM damping) stays per problem on the
 // device.  The whole batched solve is captured once as a CUDA graph.
 //
 // The chunk granularity (tiles per chunk) is picked by a small autotuner that

@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(NT) k_ed_apply_v(const MeshProb* __restrict__ 
 }
 
 // Gather pass: q_i = (fit + damping) p_i + own edge rows + incoming edge
-// rows + constraint rows, float64 p.q -> alpha.
+// rows + constraint rows, p.q -> alpha.
 __global__ void __launch_bounds__(NT) k_ed_apply_pull(const MeshProb* __restrict__ probs,
                                                       const Chunk* __restrict__ chunks,
                                                       double* __restrict__ part) {
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(NT) k_ed_apply_pull(const MeshProb* __restrict
   }
 }
 
-// delta += alpha p, r -= alpha q, z = M^-1 r, float64 r.z -> beta.
+// delta += alpha p, r -= alpha q, z = M^-1 r, r.z -> beta.
 // The update streams twelve planes per array: in two groups of six unknowns
 // (all loads of a group before its stores) it fits 64 registers and runs 4
 // blocks per SM; loading all twelve first took 186 registers (one block per

@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(NT) k_wg_apply_v(const MeshProb* __restrict__ 
 // Gather pass: q_i = (fit + damping) p_i + sum over out-edges (i, j) of the own
 // rows s_w J_e p (displacement) and g . J_e p (angle) + sum over in-edges
 // (j, i) of -s_w J_e p (displacement), J_e p = s_w (p_a,d - p_b,d) + g p_a,t;
-// float64 p.q -> alpha.
+// p.q -> alpha.
 __global__ void __launch_bounds__(NT) k_wg_apply_pull(const MeshProb* __restrict__ probs,
                                                       const Chunk* __restrict__ chunks,
                                                       double* __restrict__ part) {
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(NT) k_wg_apply_pull(const MeshProb* __restrict
   }
 }
 
-// delta += alpha p, r -= alpha q, z = M^-1 r, float64 r.z -> beta; four
+// delta += alpha p, r -= alpha q, z = M^-1 r, r.z -> beta; four
 // vertices per thread, all loads first.
 __global__ void __launch_bounds__(NT) k_wg_update(const MeshProb* __restrict__ probs,
                                                   const Chunk* __restrict__ chunks,

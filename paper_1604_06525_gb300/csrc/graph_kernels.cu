@@ -38,7 +38,7 @@
 // Per outer iteration (PCGInit): k_mesh_init_v (quaternions, axes, records),
 // k_mesh_init_pull (J^T F, diag, M^-1, r, delta, float64 r.z and E).
 // Per PCG iteration: k_mesh_apply_v (p = z + beta p into the planes, p_d and w
-// into the records), k_mesh_apply_pull (J^T J p + fit + damping, float64 p.q ->
+// into the records), k_mesh_apply_pull (J^T J p + fit + damping, p.q ->
 // alpha), k_mesh_update (vector update -> beta).
 #include "opt_internal.cuh"
 #include "mesh_algebra.cuh"
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(NT) k_mesh_apply_v(const MeshProb* __restrict_
 
 // Gather pass: q_i = (fit + damping) p_i + sum over out-edges (i, j) of the
 // own rows s_w J_e p (displacement) and the torque rows (angles) + sum over
-// in-edges (j, i) of -s_w J_e p (displacement); float64 p.q -> alpha.  The
+// in-edges (j, i) of -s_w J_e p (displacement); p.q -> alpha.  The
 // kernel is bound by its dependent index -> record loads, so it is compiled for
 // MESH_PULL_MIN_BLOCKS resident blocks per SM.
 template <bool G3>
@@ -519,7 +519,7 @@ __global__ void __launch_bounds__(NT, MESH_TILED_MIN_BLOCKS) k_mesh_apply_tiled(
   }
 }
 
-// delta += alpha p, r -= alpha q, z = M^-1 r, float64 r.z -> beta; four
+// delta += alpha p, r -= alpha q, z = M^-1 r, r.z -> beta; four
 // vertices per thread, all loads first.
 __global__ void __launch_bounds__(NT) k_mesh_update(const MeshProb* __restrict__ probs,
                                                     const Chunk* __restrict__ chunks,

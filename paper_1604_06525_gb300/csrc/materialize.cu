@@ -13,7 +13,7 @@
 //
 // Per PCG iteration: direction update p = M^-1 r + beta p over the non-empty
 // unknowns, t = J p (one thread per row), q = J^T t + lambda D p with a
-// float64 p.q reduction (one thread per unknown), then the shared vector
+// p.q reduction (one thread per unknown), then the shared vector
 // update of the matrix-free path.
 #include <cuda_runtime.h>
 
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(NT) k_csr_jp(int R, const int* __restrict__ rp
   }
 }
 
-// q = J^T t (+ lambda D p), one thread per non-empty unknown; float64 p.q -> alpha.
+// q = J^T t (+ lambda D p), one thread per non-empty unknown; p.q -> alpha.
 __global__ void __launch_bounds__(NT) k_csr_jtt(int nT, const int* __restrict__ t_unk, const int* __restrict__ t_ptr,
                                                 const int* __restrict__ t_row, const float* __restrict__ t_val,
                                                 const float* __restrict__ t, const float* __restrict__ p,
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(NT) k_jtj_assemble(int nT, const int* __restri
   }
 }
 
-// q = A p (+ lambda D p) over the non-empty unknowns; float64 p.q -> alpha.
+// q = A p (+ lambda D p) over the non-empty unknowns; p.q -> alpha.
 __global__ void __launch_bounds__(NT) k_jtj_spmv(int nT, const int* __restrict__ t_unk, const int* __restrict__ a_ptr,
                                                  const int* __restrict__ a_col, const float* __restrict__ a_val,
                                                  const float* __restrict__ p, float* __restrict__ q,

@@ -190,10 +190,10 @@ void batch_enqueue_lm_round(opt_batch* b, const opt_solve_params& p, cudaStream_
 // Copies the members' scalars and the records of the first `rounds` rounds
 // (round-major) to the host; synchronises the stream.
 opt_status batch_read_scalars(opt_batch* b, Scalars* host_out, RoundRec* rounds_out, int rounds, cudaStream_t st);
-// api.cu: caller planes (dense rows for grids, caller vertex order for
-// graphs) <-> internal planes
 // api.cu: h_e0 / h_e1 from the device, where not there yet
 opt_status host_edges(opt_problem* pb);
+// api.cu: caller planes (dense rows for grids, caller vertex order for
+// graphs) <-> internal planes
 opt_status copy_planes_in(const opt_problem* pb, float* internal, float* const* user, int n, cudaStream_t st);
 opt_status copy_planes_out(const opt_problem* pb, float* const* user, const float* internal, int n,
                            cudaStream_t st);

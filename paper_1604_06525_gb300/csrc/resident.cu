@@ -32,9 +32,9 @@
 // alpha and beta are the same and with them every iterate.  (Only the mesh
 // energies' records with RES_Z carry w = w(z) + beta w(p_old) in place of w(p).)
 //
-// Slots: two sets, used in turn; the two lowest bits of a stored pair's low part
-// (2^-46 of the sum) say which sum it belongs to, so a slot needs no emptying and a
-// stale one is never taken for the next: a block stores sum k + 2 only after sum k
+// Slots: two sets, used in turn; both words of a stored pair carry the sum's number, so
+// a slot needs no emptying and a stale one is never taken for the next: a block stores
+// sum k + 2 only after sum k
 // + 1, which every block reaches after reading those of k.  The counts go on from
 // launch to launch (sync->sums, sync->meetings).  Every wait of the device-wide form is
 // bounded (ResidentSync); a block that gives up flags s->timeout and returns, the others

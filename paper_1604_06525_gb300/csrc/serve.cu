@@ -17,7 +17,8 @@
 //      stored for opt_server_poll, and their memory returns to the budget.
 // Every member follows exactly the LM sequence of opt_solve_lm with the same
 // parameters, so its result equals the one-at-a-time solve up to float
-// rounding (batch reductions run per problem in the same order).
+// rounding (a member's sums are split by the group it is in, see one_wave_tiles in
+// batch.cu, and a solo solve's by the blocks of its loop on chip; all are compensated).
 #include <cuda_runtime.h>
 
 #include <algorithm>
