@@ -409,8 +409,8 @@ __global__ void __launch_bounds__(256) k_move_planes(const __grid_constant__ Pla
 }
 
 // Grids: a caller's plane that a kernel cannot address float by float (a byte offset
-// that is no multiple of 4, or memory CUDA does not know on this device) goes through a
-// copy, which takes any address and reports one that is not memory.
+// that is no multiple of 4, another device's memory, or memory CUDA does not know) goes
+// through a copy, which takes any address and reports one that is not memory.
 bool addressable(const float* p) {
   if (reinterpret_cast<uintptr_t>(p) % alignof(float) != 0) return false;
   cudaPointerAttributes a = {};
@@ -418,7 +418,9 @@ bool addressable(const float* p) {
     (void)cudaGetLastError();
     return false;
   }
-  return a.type != cudaMemoryTypeUnregistered && a.devicePointer == p;
+  int dev = -1;
+  const bool here = a.type != cudaMemoryTypeDevice || (cudaGetDevice(&dev) == cudaSuccess && a.device == dev);
+  return a.type != cudaMemoryTypeUnregistered && here && a.devicePointer == p;
 }
 
 opt_status copy_planes(const opt_problem* pb, PlaneDir dir, float* own, float* const* user, int n, cudaStream_t st,

@@ -1372,7 +1372,7 @@ __global__ void __launch_bounds__(NT) k64_move_planes(const __grid_constant__ Pl
     }
 }
 // A caller's plane that a kernel cannot address double by double (an odd byte offset,
-// or memory CUDA does not know on this device) goes through a copy, which takes any
+// another device's memory, or memory CUDA does not know) goes through a copy, which takes any
 // address and reports one that is not memory.
 bool addressable64(const double* p) {
   if (reinterpret_cast<uintptr_t>(p) % alignof(double) != 0) return false;
@@ -1381,7 +1381,9 @@ bool addressable64(const double* p) {
     (void)cudaGetLastError();
     return false;
   }
-  return a.type != cudaMemoryTypeUnregistered && a.devicePointer == p;
+  int dev = -1;
+  const bool here = a.type != cudaMemoryTypeDevice || (cudaGetDevice(&dev) == cudaSuccess && a.device == dev);
+  return a.type != cudaMemoryTypeUnregistered && here && a.devicePointer == p;
 }
 opt_status copy_x(opt_problem_f64* pb, bool in, cudaStream_t st, Scalars* reset = nullptr, double lambda0 = 0.0,
                   const SolveResult& res = SolveResult{}) {
