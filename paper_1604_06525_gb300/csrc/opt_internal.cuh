@@ -514,8 +514,8 @@ __device__ __forceinline__ void gather_partials(const double* part, int cb, int 
 // blocks too: about 47 bits, of which alpha and beta, rounded to float32 once, keep 24.
 // In float64 every alpha and beta of the performance cases comes out the same, but its
 // tail is a serial chain (64 cycles an addition, 109 a shuffle level, 560 a division):
-// 1024^2 warp GN 4 x 20 2.10 against 2.06 ms, 64^2 0.33 against 0.28, level-7 mesh
-// LM 2 x 30 1.35 against 1.20.  Sums that float32 cannot hold go on in float64 and are
+// 1024^2 warp GN 4 x 20 2.09 against 2.03 ms, 64^2 0.33 against 0.28, level-7 mesh
+// LM 2 x 30 1.35 against 1.18.  Sums that float32 cannot hold go on in float64 and are
 // handed on as pairs of 2^-64 of them (big).  Energies and the LM decision are float64.
 //
 // A total that comes out as no number is formed again in float64 from what it was the
